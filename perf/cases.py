@@ -270,3 +270,68 @@ def tolerance(case):
     # The fast mode may resolve correlations that agree to 2^-15 either way: the library's own arg-max
     # variants differ in up to 0.08 % of the indices (every later pick of such a row among them).
     return {"rel": 0.03, "max": 0.99, "differ": 0.003}
+
+
+# ---------------------------------------------------------------------------------------
+# the same results from 64-bit sums in plain torch
+# ---------------------------------------------------------------------------------------
+
+def _pursuit64(D, X, s):
+    """Matching pursuit of the rows of X over the atoms of D, all in 64 bits."""
+    D, idx, coef = D.double(), [], []
+    for x in X.split(max(64, (1 << 26) // D.shape[0])):
+        R, picks, cs = x.double(), [], []
+        for _ in range(s):
+            corr = R @ D.T
+            n = corr.abs().argmax(dim=1)
+            c = corr.gather(1, n[:, None])
+            R = R - c * D[n]
+            picks.append(n)
+            cs.append(c)
+        idx.append(torch.stack(picks, 1))
+        coef.append(torch.cat(cs, 1))
+    return torch.cat(idx), torch.cat(coef)
+
+
+def _rows64(D, idx, coef, group=1 << 16):
+    """The rows that codes stand for."""
+    return torch.cat([(c.double()[:, :, None] * D[i]).sum(1) for i, c in zip(idx.split(group), coef.split(group))])
+
+
+def _ints(idx):
+    return idx.view(torch.int16).long() & 0xFFFF
+
+
+def exact(case, seed):
+    """run()'s outputs in 64 bits.  None where they hang on the fast mode's picks: it resolves near-ties
+    in 16 bits, either way, and every later number of such a row follows from its picks."""
+    kind, s = case["kind"], case["s"]
+    if kind in ("roundtrip", "host") or case.get("encode") is True or (kind in ("encode", "train") and case["mode"] == "fast"):
+        return None
+    st = prepare(case, seed)
+    if kind == "decode":
+        B, T, d = case["B"], case["T"], case["d"]
+        Dk, Dv, Q = st["Dk"].double(), st["Dv"].double(), st["Q"].double()
+        out, weights = [], []
+        for b in range(B):
+            K = _rows64(Dk, _ints(st["k_idx"][b]), st["k_coef"][b], 1 << 14)
+            w = torch.softmax(Q[b] @ K.T / math.sqrt(d), dim=-1)
+            weights.append(w)
+            out.append(w @ _rows64(Dv, _ints(st["v_idx"][b]), st["v_coef"][b], 1 << 14))
+        return torch.stack(out), torch.stack(weights)
+    if kind == "restore":
+        D = st["D"].half().double() if case["handle"] else st["D"].double()
+        return _rows64(D, _ints(st["idx"]), st["coef"], 1 << 14)
+    idx, coef = _pursuit64(st["D"], st["X"], s)
+    if kind == "encode":
+        return idx, coef
+    # one step of gradient descent on ||X - X_hat||^2 + beta ||D D^T - I||^2 / N^2, then unit atoms
+    D, N = st["D"].double(), case["N"]
+    grad, loss = torch.zeros_like(D), 0.0
+    for x, i, c in zip(st["X"].split(1 << 14), idx.split(1 << 14), coef.split(1 << 14)):
+        e = x.double() - _rows64(D, i, c)
+        loss = loss + (e * e).sum()
+        grad.index_add_(0, i.reshape(-1), (-2.0 * c[:, :, None] * e[:, None, :]).reshape(-1, D.shape[1]))
+    G = D @ D.T - torch.eye(N, dtype=D.dtype, device=D.device)
+    W = D - 1e-5 * (grad + 0.1 * 4.0 / N ** 2 * (G @ D))
+    return torch.nn.functional.normalize(W, dim=1), torch.stack([loss, (G * G).sum() / N ** 2])
