@@ -1,0 +1,580 @@
+// Correctness-mode matching pursuit (paper Eq. 2-4) on the tensor cores for up to one tile of 128
+// rows per SM: the dictionary is split across the CTAs that share a row tile.
+//
+// A CTA of encode_exact_tc.cu holds two row tiles and sweeps the whole dictionary, so a call of a
+// few rows leaves all but a few SMs idle and takes s whole sweeps all the same.  Here the grid is
+// (row tiles) x (slices of the dictionary), at most one CTA per SM, and all s iterations run in one
+// launch.  Per iteration
+//   - every CTA loads the bf16 high and low parts of its tile's 128 residual rows (64 KB from the
+//     L2), multiplies them with its slice by the same three bf16 products per correlation, and
+//     every thread keeps the four largest keys of its half row (drain as in encode_exact_tc.cu);
+//   - the keys go to a scratch array, the CTAs of the row tile meet (counter in global memory,
+//     bounded wait);
+//   - the rows of the tile are dealt out to its CTAs, eight lanes settle a row: the largest key
+//     over all slices, everything inside the band re-scored in fp64, fp64 coefficient and residual
+//     update; the new high and low parts go back to the scratch array and the CTAs meet again.
+// The fp64 rows, bands and parts live in L2-resident scratch.  The dictionary stages of the next
+// iteration are fetched while the rows are being settled.
+//
+// What bounds it: with few rows the chain of dependent steps (A load, MMA, drain, meeting, settle,
+// meeting: about 8 us an iteration), with many the MMAs, 3072 cycles per 256 atoms and row tile.
+// The grid is launched cooperatively whenever a row tile has more than one CTA, so all CTAs that
+// wait for one another are resident.
+#include "exact_tc_common.cuh"
+
+namespace csr {
+namespace {
+
+using namespace exact_tc;
+
+constexpr int NT = 320;
+constexpr int EPI = 256;                                  // epilogue threads
+constexpr int PRODUCER_WARP = 8;
+constexpr int MMA_WARP = 9;
+constexpr uint32_t TMEM_COLS = 512;
+constexpr int UNIT = 64;                                  // atoms per TMA box; slices are whole units
+constexpr int MAX_SLICES = TILE_M;                        // at most one CTA per row
+constexpr int CAND = 16;                                  // candidates a row may have before the whole dictionary is re-scored
+
+// Keys of one row over one column half of a slice: the four largest and the atoms of the first three.
+struct __align__(8) Entry {
+    uint32_t k[4];
+    uint32_t n01, n2;
+};
+
+template <int D_>
+struct GridSmem {
+    static constexpr int kStages = D_ == 128 ? 4 : 5;
+    static constexpr int kATileBytes = TILE_M * D_ * 2;
+    static constexpr int kStageBytes = TILE_N * STAGE_CH * 2;
+    alignas(1024) uint8_t A[2][kATileBytes];              // [high, low]
+    alignas(1024) uint8_t B[kStages][kStageBytes];
+    Entry ent[2 * (2 * TILE_M)];                          // entries of the rows this CTA settles (rows x 2 slices <= 2 (127 + slices))
+    uint16_t cand[EPI / 8][CAND];
+    int n_cand[EPI / 8];
+    uint32_t unknown[TILE_M / 32];                        // rows settled here whose candidates are not all known
+    float limit[TILE_M];                                  // ... from which fp32 value on an atom can be the pick
+    int found_n[TILE_M];                                  // ... and what the search of the whole dictionary found
+    Rescored found[EPI / 32];
+    uint64_t full_b[kStages];
+    uint64_t empty_b[kStages];
+    uint64_t acc_full[2];
+    uint64_t acc_empty[2];
+    uint64_t res_ready;
+    uint64_t drained;
+    uint32_t tmem_base;
+    volatile uint32_t abort;
+};
+
+struct GridArgs {
+    const float* D;
+    const void* X;
+    int x_dtype;
+    int64_t ldx, M;
+    int N, s;
+    uint16_t* out_idx;
+    void* out_coef;
+    int coef_dtype;
+    int64_t ldc;
+    double* Rd;             // [tiles * 128][d] fp64 residual rows
+    uint32_t* Rh;           // [tiles * 128][d / 2] bf16 high parts, two channels per word
+    uint32_t* Rl;           // low parts
+    float* band;            // [tiles * 128]
+    Entry* entries;         // [tiles][128][2 * slices]
+    uint32_t* counters;     // [tiles * 32], zero at launch
+    int slices;
+    uint32_t* status;
+    uint32_t* diag;
+    unsigned long long wait_limit_ns;
+};
+
+// The CTAs of a row tile meet: everything their epilogue threads wrote before is visible to all of
+// them afterwards.  All 256 epilogue threads call; returns false to all when any has given up.
+__device__ __forceinline__ bool meet(uint32_t* counter, uint32_t target, int slices, bool ok, const WaitCtx& w) {
+    if (epilogue_barrier_any(!ok || *w.abort != 0)) return false;
+    if (slices > 1) {
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(counter, 1u);
+            uint32_t seen;
+            unsigned long long t0 = 0;
+            bool in = false;
+            for (uint32_t it = 0; it < (1u << 28); ++it) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
+                if (seen >= target) {
+                    in = true;
+                    break;
+                }
+                if ((it & 63u) == 0) {
+                    if (*w.abort) break;
+                    const unsigned long long t = globaltimer_ns();
+                    if (t0 == 0) t0 = t;
+                    if (t - t0 > w.limit_ns || w.limit_ns == 0) break;
+                }
+            }
+            if (!in) {
+                *w.abort = 1;
+                atomicOr(w.status, kStatusTimeout);
+            }
+            __threadfence();
+        }
+        if (epilogue_barrier_any(*w.abort != 0)) return false;
+    }
+    return true;
+}
+
+template <int D_>
+__global__ void __launch_bounds__(NT, 1)
+encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid_constant__ CUtensorMap tmap_lo, const GridArgs a) {
+    using S = GridSmem<D_>;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    if ((smem_u32(smem_raw) & 1023u) != 0) {              // the swizzled tiles need this; never seen otherwise
+        if (threadIdx.x == 0) atomicOr(a.status, kStatusLayout);
+        return;
+    }
+    S& sm = *reinterpret_cast<S*>(smem_raw);
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int slices = a.slices;
+    const int tile = blockIdx.x / slices, slice = blockIdx.x % slices;
+    const int units = (a.N + UNIT - 1) / UNIT;
+    const int u0 = static_cast<int>(static_cast<int64_t>(units) * slice / slices);
+    const int u1 = static_cast<int>(static_cast<int64_t>(units) * (slice + 1) / slices);
+    const int n_first = u0 * UNIT, width = (u1 - u0) * UNIT;   // this CTA's atoms (slices <= units: never empty)
+    const int T = (width + TILE_N - 1) / TILE_N;          // accumulator tiles of a sweep, the last 64 .. 256 wide
+    constexpr int KH = D_ / STAGE_CH;
+    constexpr int KSTEPS = STAGE_CH / UMMA_K;
+    constexpr int STAGES = S::kStages;
+    constexpr int NSTG = 2 * KH;
+    const WaitCtx wc{&sm.abort, a.status, a.wait_limit_ns};
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < STAGES; ++i) {
+            mbar_init(&sm.full_b[i], 1);
+            mbar_init(&sm.empty_b[i], 1);
+        }
+        for (int t = 0; t < 2; ++t) {
+            mbar_init(&sm.acc_full[t], 1);
+            mbar_init(&sm.acc_empty[t], 8);
+        }
+        mbar_init(&sm.res_ready, EPI);
+        mbar_init(&sm.drained, 1);
+        sm.abort = 0;
+        fence_barrier_init();
+    }
+    if (warp == MMA_WARP) {
+        tmem_alloc(&sm.tmem_base, TMEM_COLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = sm.tmem_base;
+
+    if (warp == PRODUCER_WARP) {
+        // ------------------------------ TMA producer ------------------------------
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_hi)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_lo)) : "memory");
+            uint32_t p = 0;
+            bool ok = true;
+            for (int g = 0; g < a.s && ok; ++g) {
+                for (int t = 0; t < T && ok; ++t) {
+                    const int w = min(TILE_N, width - t * TILE_N);
+                    for (int hp = 0; hp < NSTG; ++hp, ++p) {
+                        const int stage = p % STAGES;
+                        if (!wait_bounded_suspended(&sm.empty_b[stage], ((p / STAGES) & 1) ^ 1, wc, 2000)) {
+                            ok = false;
+                            break;
+                        }
+                        // atoms past N arrive as zeros and count as bytes
+                        mbar_expect_tx(&sm.full_b[stage], static_cast<uint32_t>(w) * STAGE_CH * 2);
+                        for (int u = 0; u < w / UNIT; ++u)
+                            tma_load_2d(&sm.B[stage][u * (UNIT * STAGE_CH * 2)], (hp & 1) ? &tmap_lo : &tmap_hi, (hp >> 1) * STAGE_CH,
+                                        n_first + t * TILE_N + u * UNIT, &sm.full_b[stage]);
+                    }
+                }
+            }
+            if (!ok) {                                    // let the copies already issued land
+                const uint32_t first = p > STAGES ? p - STAGES : 0;
+                for (uint32_t qq = first; qq < p; ++qq) {
+                    const unsigned long long t0 = globaltimer_ns();
+                    while (!mbar_try_wait(&sm.full_b[qq % STAGES], (qq / STAGES) & 1))
+                        if (globaltimer_ns() - t0 > 20000000ull) break;
+                }
+            }
+        }
+    } else if (warp == MMA_WARP) {
+        // ------------------------------ MMA issuer ------------------------------
+        if (lane == 0) {
+            uint32_t p = 0, accn = 0;
+            bool ok = true;
+            for (int g = 0; g < a.s && ok; ++g) {
+                if (!wait_bounded(&sm.res_ready, g & 1, wc)) {
+                    ok = false;
+                    break;
+                }
+                for (int t = 0; t < T && ok; ++t, ++accn, p += NSTG) {
+                    const int acc = accn & 1;             // the accumulators take the tiles in turn
+                    const uint32_t idesc = instr_desc_bf16(TILE_M, min(TILE_N, width - t * TILE_N));
+                    if (!wait_bounded(&sm.acc_empty[acc], ((accn >> 1) & 1) ^ 1, wc)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t d_tmem = tmem_base + acc * TILE_N;
+                    for (int hp = 0; hp < NSTG; ++hp) {
+                        const uint32_t ps = p + hp;
+                        const int stage = ps % STAGES;
+                        const int h = hp >> 1;
+                        if (!wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
+                        const uint64_t ah = make_smem_desc(smem_u32(&sm.A[0][h * (TILE_M * 128)]));
+                        const uint64_t al = make_smem_desc(smem_u32(&sm.A[1][h * (TILE_M * 128)]));
+#pragma unroll
+                        for (int k = 0; k < KSTEPS; ++k) {
+                            const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
+                            umma_bf16(d_tmem, ah + off, b0 + off, idesc, (hp | k) ? 1u : 0u);
+                        }
+                        if ((hp & 1) == 0) {              // high parts of the atoms: the low parts of the rows meet them too
+#pragma unroll
+                            for (int k = 0; k < KSTEPS; ++k) {
+                                const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
+                                umma_bf16(d_tmem, al + off, b0 + off, idesc, 1u);
+                            }
+                        }
+                        umma_commit(&sm.empty_b[stage]);
+                    }
+                    if (ok) umma_commit(&sm.acc_full[acc]);
+                }
+            }
+            if (!ok) {
+                umma_commit(&sm.drained);
+                const unsigned long long t0 = globaltimer_ns();
+                while (!mbar_try_wait(&sm.drained, 0))
+                    if (globaltimer_ns() - t0 > 20000000ull) break;
+            }
+        }
+    } else {
+        // ------------------------------ epilogue ------------------------------
+        constexpr int CH = D_ / 8;                        // channels per lane when eight lanes share a row
+        const int q = warp & 3, half = warp >> 2;         // TMEM lane quarter, column half
+        const int r_own = q * 32 + lane;                  // the row of the tile whose correlations this thread sees
+        const int l8 = lane & 7, grp = lane >> 3;
+        const int group = warp * 4 + grp;
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+        const int64_t row_base = static_cast<int64_t>(tile) * TILE_M;
+        const int rows_here = static_cast<int>(a.M - row_base < TILE_M ? a.M - row_base : TILE_M);   // >= 1
+        // rows settled here: slice, slice + slices, ...; the k-th by warp k % 8, lane group k / 8 % 4, pass k / 32
+        const int n_own = rows_here > slice ? (rows_here - slice + slices - 1) / slices : 0;
+        const int n_ent = 2 * slices;                     // entries of a row
+        uint32_t* counter = a.counters + tile * 32;
+        uint32_t target = 0;
+        bool ok = true;
+        uint32_t accn = 0;
+        // An fp64 row, its parts and its band to the scratch arrays, by the eight lanes of a row (all lanes
+        // of the warp call; only those with `has` write).
+        auto put_row = [&](const double (&R)[CH], int64_t row, bool has) {
+            double n0 = 0.0, n1 = 0.0;
+#pragma unroll
+            for (int k = 0; k < CH / 2; ++k) {
+                n0 = fma(R[2 * k], R[2 * k], n0);
+                n1 = fma(R[2 * k + 1], R[2 * k + 1], n1);
+            }
+            const double nn = group8_sum(n0 + n1);
+            if (!has) return;
+#pragma unroll
+            for (int k = 0; k < CH / 2; ++k) {
+                uint32_t hi, lo;
+                split_pair(R[2 * k], R[2 * k + 1], hi, lo);
+                __stcg(reinterpret_cast<double2*>(a.Rd + row * D_) + 8 * k + l8, make_double2(R[2 * k], R[2 * k + 1]));
+                __stcg(a.Rh + row * (D_ / 2) + 8 * k + l8, hi);
+                __stcg(a.Rl + row * (D_ / 2) + 8 * k + l8, lo);
+            }
+            if (l8 == 0) __stcg(a.band + row, kBandRel * sqrtf(static_cast<float>(nn)) * 1.001f);
+        };
+        // ---- R_0 = x ----
+        for (int k0 = 0; k0 < n_own; k0 += EPI / 8) {
+            const int k = k0 + grp * 8 + warp;
+            const bool has = k < n_own;
+            const int64_t row = row_base + slice + (has ? k : 0) * slices;
+            double R[CH];
+#pragma unroll
+            for (int c = 0; c < CH / 2; ++c) load_x2(a.X, a.x_dtype, row * a.ldx + 2 * (8 * c + l8), R[2 * c], R[2 * c + 1]);
+            put_row(R, row, has);
+        }
+        ok = meet(counter, target += slices, slices, ok, wc);
+
+        for (int g = 0; g < a.s && ok; ++g) {
+            // ---- the residual's parts into the operand tiles (rows past M: zeros, once) ----
+            constexpr int CPR = D_ / 8;                   // 16-byte chunks of a row
+            constexpr int PER = 2 * TILE_M * CPR / EPI;
+            uint4 v[PER];
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int f = threadIdx.x + u * EPI;
+                const int part = f / (TILE_M * CPR), r = f / CPR % TILE_M, c = f % CPR;
+                v[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (r < rows_here) v[u] = __ldcg(reinterpret_cast<const uint4*>((part ? a.Rl : a.Rh) + (row_base + r) * (D_ / 2)) + c);
+            }
+            const float band_own = r_own < rows_here ? __ldcg(a.band + row_base + r_own) : 0.f;
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int f = threadIdx.x + u * EPI;
+                const int part = f / (TILE_M * CPR), r = f / CPR % TILE_M, c = f % CPR;
+                if (g == 0 || r < rows_here) *reinterpret_cast<uint4*>(&sm.A[part][swz_off(r, c)]) = v[u];
+            }
+            fence_proxy_async_smem();
+            mbar_arrive(&sm.res_ready);
+
+            // ---- sweep of this slice: top four keys of this thread's half row ----
+            Top4 top{0u, 0u, 0u, 0u, 0u, 0u, 0u};
+            const float fband = band_own > 0.f ? band_own * 1.0625f : -1.f;
+            for (int t = 0; t < T; ++t, ++accn) {
+                const int acc = accn & 1;
+                bool got = wait_bounded(&sm.acc_full[acc], (accn >> 1) & 1, wc);
+                got = __all_sync(FULL, got);
+                if (!got) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const int w = min(TILE_N, width - t * TILE_N);
+                const uint32_t ta = taddr + acc * TILE_N + half * (w / 2);
+                const uint32_t id = static_cast<uint32_t>(2 * t + half);
+                uint64_t* back = &sm.acc_empty[acc];
+                drain(ta, w / UNIT, top, id, fband, back, lane);
+            }
+            if (ok && r_own < rows_here) {
+                auto atom = [&](uint32_t key, uint32_t id) {      // (an empty key's place is never used)
+                    const int t = static_cast<int>(id >> 1), w = min(TILE_N, width - t * TILE_N);
+                    return static_cast<uint32_t>(n_first + t * TILE_N + static_cast<int>(id & 1) * (w / 2) + 127 - static_cast<int>(key & 127u)) & 0xFFFFu;
+                };
+                uint2* e = reinterpret_cast<uint2*>(a.entries + ((row_base + r_own) * n_ent + 2 * slice + half));
+                __stcg(e + 0, make_uint2(top.k0, top.k1));
+                __stcg(e + 1, make_uint2(top.k2, top.k3));
+                __stcg(e + 2, make_uint2(atom(top.k0, top.i0) | (atom(top.k1, top.i1) << 16), atom(top.k2, top.i2)));
+            }
+            ok = meet(counter, target += slices, slices, ok, wc);
+            if (!ok) break;
+
+            // ---- settle this CTA's rows ----
+            if (threadIdx.x < TILE_M / 32) sm.unknown[threadIdx.x] = 0u;
+            for (int f = threadIdx.x; f < n_own * n_ent; f += EPI) {
+                const uint2* e = reinterpret_cast<const uint2*>(a.entries + ((row_base + slice + f / n_ent * slices) * n_ent + f % n_ent));
+                const uint2 e0 = __ldcg(e), e1 = __ldcg(e + 1), e2 = __ldcg(e + 2);
+                uint2* d = reinterpret_cast<uint2*>(&sm.ent[f]);
+                d[0] = e0;
+                d[1] = e1;
+                d[2] = e2;
+            }
+            epilogue_barrier();
+#pragma unroll 1
+            for (int round = 0; round < 2; ++round) {
+                if (round == 1) {
+                    epilogue_barrier();
+                    if ((sm.unknown[0] | sm.unknown[1] | sm.unknown[2] | sm.unknown[3]) == 0u) break;
+#pragma unroll 1
+                    for (int w = 0; w < TILE_M / 32; ++w)
+                        for (uint32_t left = sm.unknown[w]; left; left &= left - 1) {
+                            const int k = w * 32 + __ffs(left) - 1;
+                            const int nr = rescore_row<D_>(a.D, a.N, a.Rd + (row_base + slice + k * slices) * D_, sm.limit[k], sm.found, warp, lane);
+                            if (threadIdx.x == 0) sm.found_n[k] = nr;
+                        }
+                    epilogue_barrier();
+                }
+#pragma unroll 1
+                for (int k0 = 0; k0 < n_own; k0 += EPI / 8) {
+                    const int k = k0 + grp * 8 + warp;
+                    bool has = k < n_own;
+                    if (round == 1) has = has && ((sm.unknown[k >> 5] >> (k & 31)) & 1u);
+                    if (!__any_sync(FULL, has)) continue;
+                    const int kk = k < n_own ? k : 0;         // (lane groups without a row repeat one and write nothing)
+                    const int64_t row = row_base + slice + kk * slices;
+                    double R[CH];
+#pragma unroll
+                    for (int c = 0; c < CH / 2; ++c) {
+                        const double2 x = __ldcg(reinterpret_cast<const double2*>(a.Rd + row * D_) + 8 * c + l8);
+                        R[2 * c] = x.x;
+                        R[2 * c + 1] = x.y;
+                    }
+                    const float band = __ldcg(a.band + row);
+                    const Entry* ent = &sm.ent[kk * n_ent];
+                    uint32_t kmax = 0;
+                    for (int e = l8; e < n_ent; e += 8) kmax = max(kmax, ent[e].k[0]);
+                    kmax = max(kmax, __shfl_xor_sync(FULL, kmax, 1));
+                    kmax = max(kmax, __shfl_xor_sync(FULL, kmax, 2));
+                    kmax = max(kmax, __shfl_xor_sync(FULL, kmax, 4));
+                    const float v0 = __uint_as_float(kmax & kKeyMask);
+                    const bool some = v0 > 0.f && a.N > 1;    // else: an all-zero sweep (or NaN) picks atom 0
+                    if (l8 == 0) sm.n_cand[group] = 0;
+                    __syncwarp();
+                    bool full = some && !(v0 > band);
+                    if (some) {
+                        for (int e = l8; e < n_ent; e += 8) {
+                            if (v0 - __uint_as_float(ent[e].k[0] & kKeyMask) > band) continue;
+#pragma unroll
+                            for (int i = 0; i < 3; ++i) {
+                                const uint32_t key = ent[e].k[i];
+                                const uint32_t n = i == 0 ? ent[e].n01 & 0xFFFFu : i == 1 ? ent[e].n01 >> 16 : ent[e].n2;
+                                if (key != 0u && !(v0 - __uint_as_float(key & kKeyMask) > band) && n < static_cast<uint32_t>(a.N)) {
+                                    const int slot = atomicAdd(&sm.n_cand[group], 1);
+                                    if (slot < CAND) sm.cand[group][slot] = static_cast<uint16_t>(n);
+                                }
+                            }
+                            // four of a half slice inside the band: there may be more
+                            if (ent[e].k[3] != 0u && !(v0 - __uint_as_float(ent[e].k[3] & kKeyMask) > band)) full = true;
+                        }
+                    }
+                    __syncwarp();
+                    int cnt = some ? sm.n_cand[group] : 0;
+                    full = full || cnt > CAND || (some && cnt == 0);
+                    full = ((__ballot_sync(FULL, full) >> (8 * grp)) & 0xFFu) != 0;
+                    int n = cnt > 0 ? sm.cand[group][0] : 0;
+                    if (round == 1) {                         // searched for by all warps: nothing left to decide
+                        n = has ? sm.found_n[kk] : 0;
+                        full = false;
+                        cnt = 0;
+                    } else if (full && has) {                 // left for the second round
+                        if (l8 == 0) {
+                            atomicOr(&sm.unknown[k >> 5], 1u << (k & 31));
+                            sm.limit[k] = v0 - 1.5f * band;
+                        }
+                        has = false;
+                    }
+                    const bool cmp = !full && cnt > 1;        // several candidates: their fp64 correlations decide, the lowest atom among equals
+                    if (__any_sync(FULL, cmp)) {
+                        const int most = static_cast<int>(__reduce_max_sync(FULL, cmp ? static_cast<unsigned>(cnt) : 0u));
+                        double cbest = -1.0;
+                        int nbest = n;
+#pragma unroll 1
+                        for (int ci = 0; ci < most; ++ci) {
+                            const int nc = cmp ? sm.cand[group][min(ci, cnt - 1)] : n;
+                            float ax[CH];
+                            load_atom<CH>(a.D + static_cast<int64_t>(nc) * D_, l8, ax);
+                            const double cc = fabs(group8_sum(slice_dot<CH>(R, ax)));
+                            if (cc > cbest || (cc == cbest && nc < nbest)) {
+                                cbest = cc;
+                                nbest = nc;
+                            }
+                        }
+                        if (cmp) n = nbest;
+                    }
+                    float at[CH];
+                    load_atom<CH>(a.D + static_cast<int64_t>(n) * D_, l8, at);
+                    const double c = group8_sum(slice_dot<CH>(R, at));
+#ifdef CSR_DEBUG_CHECKS
+                    if (l8 == 0 && has && cnt == 1 && band > 0.f)   // as in encode_exact_tc.cu
+                        atomicMax(a.diag, __float_as_uint(fabsf(v0 - static_cast<float>(fabs(c))) / (band / kBandRel)));
+#endif
+                    if (l8 == 0 && has) {
+                        a.out_idx[row * a.ldc + g] = static_cast<uint16_t>(n);
+                        const float cf = static_cast<float>(c);
+                        if (a.coef_dtype == CSR_DTYPE_F16)
+                            reinterpret_cast<__half*>(a.out_coef)[row * a.ldc + g] = __float2half_rn(cf);
+                        else
+                            reinterpret_cast<float*>(a.out_coef)[row * a.ldc + g] = cf;
+                    }
+                    if (g + 1 < a.s) {
+#pragma unroll
+                        for (int c2 = 0; c2 < CH; ++c2) R[c2] = fma(-c, static_cast<double>(at[c2]), R[c2]);
+                        put_row(R, row, has);
+                    }
+                }
+            }
+            if (g + 1 < a.s) ok = meet(counter, target += slices, slices, ok, wc);
+        }
+    }
+
+    // ------------------------------ teardown ------------------------------
+    tc_fence_before();
+    __syncthreads();
+    if (warp == MMA_WARP) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, TMEM_COLS);
+    }
+}
+
+size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+int tiles_of(int64_t M) { return static_cast<int>((M + TILE_M - 1) / TILE_M); }
+
+template <int D_>
+int run(const CUtensorMap& mh, const CUtensorMap& ml, const GridArgs& g, int grid, cudaStream_t stream) {
+    const size_t smem = sizeof(GridSmem<D_>);
+    cudaError_t e = cudaFuncSetAttribute(encode_exact_grid_kernel<D_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = g.slices > 1 ? 1 : 0;                  // a lone CTA per row tile waits for nobody
+    e = cudaLaunchKernelEx(&cfg, encode_exact_grid_kernel<D_>, mh, ml, g);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return kGridLaunchRefused;                        // nothing ran: the caller takes the other engine
+    }
+    return CSR_OK;
+}
+
+}  // namespace
+
+int exact_grid_slices(int64_t M, int N) {
+    const int tiles = tiles_of(M), units = (N + UNIT - 1) / UNIT;
+    if (tiles < 1 || tiles > sm_count()) return 0;
+    int s = sm_count() / tiles;
+    if (s > units) s = units;
+    return s < MAX_SLICES ? s : MAX_SLICES;
+}
+
+size_t exact_grid_scratch_bytes(int64_t M, int d, int N) {
+    const size_t rows = (size_t)tiles_of(M) * TILE_M;
+    return rows * d * 8 + 2 * rows * d * 2 + align256(rows * 4) + align256(rows * 2 * exact_grid_slices(M, N) * sizeof(Entry));
+}
+size_t exact_grid_counter_words(int64_t M) { return (size_t)tiles_of(M) * 32; }
+
+int launch_encode_exact_grid(const EncodeArgs& a, void* hi, void* lo, void* scratch, uint32_t* counters, uint32_t* status,
+                             uint32_t* diag) {
+    const size_t rows = (size_t)tiles_of(a.M) * TILE_M;
+    char* p = static_cast<char*>(scratch);
+    GridArgs g;
+    g.D = a.D;
+    g.X = a.X;
+    g.x_dtype = a.x_dtype;
+    g.ldx = a.ldx;
+    g.M = a.M;
+    g.N = a.N;
+    g.s = a.s;
+    g.out_idx = a.out_idx;
+    g.out_coef = a.out_coef;
+    g.coef_dtype = a.coef_dtype;
+    g.ldc = a.ld_code;
+    g.Rd = reinterpret_cast<double*>(p);
+    p += rows * a.d * 8;
+    g.Rh = reinterpret_cast<uint32_t*>(p);
+    p += rows * a.d * 2;
+    g.Rl = reinterpret_cast<uint32_t*>(p);
+    p += rows * a.d * 2;
+    g.band = reinterpret_cast<float*>(p);
+    p += align256(rows * 4);
+    g.entries = reinterpret_cast<Entry*>(p);
+    g.counters = counters;
+    g.slices = exact_grid_slices(a.M, a.N);
+    g.status = status;
+    g.diag = diag;
+    g.wait_limit_ns = options().wait_limit_ns;
+    CUtensorMap mh, ml;
+    if (int rc = part_map(&mh, hi, a.N, a.d, UNIT)) return rc;
+    if (int rc = part_map(&ml, lo, a.N, a.d, UNIT)) return rc;
+    const int grid = tiles_of(a.M) * g.slices;
+    return a.d == 128 ? run<128>(mh, ml, g, grid, a.stream) : run<64>(mh, ml, g, grid, a.stream);
+}
+
+}  // namespace csr
