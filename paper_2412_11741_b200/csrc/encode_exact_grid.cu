@@ -206,27 +206,29 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        const uint32_t tmem_d = warp_uniform(tmem_base);
+        {
             uint32_t p = 0, accn = 0;
             bool ok = true;
             for (int g = 0; g < a.s && ok; ++g) {
-                if (!wait_bounded(&sm.res_ready, g & 1, wc)) {
+                if (!warp_wait_bounded(&sm.res_ready, g & 1, wc)) {
                     ok = false;
                     break;
                 }
                 for (int t = 0; t < T && ok; ++t, ++accn, p += NSTG) {
                     const int acc = accn & 1;             // the accumulators take the tiles in turn
                     const uint32_t idesc = instr_desc_bf16(TILE_M, min(TILE_N, width - t * TILE_N));
-                    if (!wait_bounded(&sm.acc_empty[acc], ((accn >> 1) & 1) ^ 1, wc)) {
+                    if (!warp_wait_bounded(&sm.acc_empty[acc], ((accn >> 1) & 1) ^ 1, wc)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t d_tmem = tmem_base + acc * TILE_N;
+                    const uint32_t d_tmem = tmem_d + acc * TILE_N;
                     for (int hp = 0; hp < NSTG; ++hp) {
                         const uint32_t ps = p + hp;
                         const int stage = ps % STAGES;
                         const int h = hp >> 1;
-                        if (!wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
+                        if (!warp_wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
                             ok = false;
                             break;
                         }

@@ -155,12 +155,14 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        const uint32_t tmem_d = warp_uniform(tmem_base);
+        {
             uint32_t p = 0, accn = 0, steps = 0;
             bool ok = true;
             for (int64_t pair = blockIdx.x; pair < n_pairs && ok; pair += gridDim.x) {
                 for (int g = 0; g < s && ok; ++g, ++steps) {
-                    if (!wait_bounded_suspended(&sm.res_ready, steps & 1, wc, 4000)) {
+                    if (!warp_wait_bounded_suspended(&sm.res_ready, steps & 1, wc, 4000)) {
                         ok = false;
                         break;
                     }
@@ -177,17 +179,17 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                                     const int stage = ps % STAGES;
                                     const int h = hp >> 1;
                                     const bool low = hp & 1;      // this stage holds low parts of the atoms
-                                    if (tile == 0 && !wait_bounded_suspended(&sm.full_b[stage], (ps / STAGES) & 1, wc, 1000)) {
+                                    if (tile == 0 && !warp_wait_bounded_suspended(&sm.full_b[stage], (ps / STAGES) & 1, wc, 1000)) {
                                         ok = false;
                                         break;
                                     }
-                                    if (hp == 0 && !wait_bounded_suspended(&sm.acc_empty[tile], (accn & 1) ^ 1, wc, 1000)) {
+                                    if (hp == 0 && !warp_wait_bounded_suspended(&sm.acc_empty[tile], (accn & 1) ^ 1, wc, 1000)) {
                                         ok = false;
                                         break;
                                     }
                                     tc_fence_after();
                                     const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
-                                    const uint32_t d_tmem = tmem_base + tile * TILE_N;
+                                    const uint32_t d_tmem = tmem_d + tile * TILE_N;
                                     const uint64_t ah = make_smem_desc(smem_u32(&sm.A[tile][0][h * (TILE_M * 128)]));
                                     const uint64_t al = make_smem_desc(smem_u32(&sm.A[tile][1][h * (TILE_M * 128)]));
 #pragma unroll

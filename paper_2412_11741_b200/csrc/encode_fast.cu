@@ -537,28 +537,30 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0 && CL == 2) {
+        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        const uint32_t tmem_d = warp_uniform(tmem_base);
+        if constexpr (CL == 2) {
             // one row tile; the CTA's dictionary tiles go to the two accumulators in turn
             uint32_t p = 0, accn[2] = {0u, 0u};
             bool ok = true;
             for (int g = 0; g < s && ok; ++g) {
-                if (!wait_bounded(&sm.res_ready[0], g & 1, wc)) {
+                if (!warp_wait_bounded(&sm.res_ready[0], g & 1, wc)) {
                     ok = false;
                     break;
                 }
                 int j = 0;
                 for (int t = t_begin; t < T && ok; t += t_step, p += KH, ++j) {
                     const int acc = j & 1;
-                    if (!wait_bounded(&sm.acc_empty[acc], (accn[acc] & 1) ^ 1, wc)) {
+                    if (!warp_wait_bounded(&sm.acc_empty[acc], (accn[acc] & 1) ^ 1, wc)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t d_tmem = tmem_base + acc * TILE_N;
+                    const uint32_t d_tmem = tmem_d + acc * TILE_N;
 #pragma unroll
                     for (int h = 0; h < KH; ++h) {
                         const uint32_t ps = p + h;
                         const int stage = ps % STAGES;
-                        if (!wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
+                        if (!warp_wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
                             ok = false;
                             break;
                         }
@@ -584,27 +586,27 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                 while (!mbar_try_wait(&sm.drained, 0))
                     if (globaltimer_ns() - t0 > 20000000ull) break;
             }
-        } else if (lane == 0) {
+        } else {
             uint32_t p = 0, accn = 0, steps = 0;
             bool ok = true;
             for (int64_t pair = pair_first; pair < n_pairs && ok; pair += pair_step) {
                 for (int g = 0; g < s && ok; ++g, ++steps) {
                     for (int t = t_begin; t < T && ok; t += t_step, p += KH, ++accn) {
                         for (int tile = 0; tile < 2 && ok; ++tile) {
-                            if (t == t_begin && !wait_bounded(&sm.res_ready[tile], steps & 1, wc)) {
+                            if (t == t_begin && !warp_wait_bounded(&sm.res_ready[tile], steps & 1, wc)) {
                                 ok = false;
                                 break;
                             }
-                            if (!wait_bounded(&sm.acc_empty[tile], (accn & 1) ^ 1, wc)) {
+                            if (!warp_wait_bounded(&sm.acc_empty[tile], (accn & 1) ^ 1, wc)) {
                                 ok = false;
                                 break;
                             }
-                            const uint32_t d_tmem = tmem_base + tile * TILE_N;
+                            const uint32_t d_tmem = tmem_d + tile * TILE_N;
 #pragma unroll
                             for (int h = 0; h < KH; ++h) {
                                 const uint32_t ps = p + h;
                                 const int stage = ps % STAGES;
-                                if (tile == 0 && !wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
+                                if (tile == 0 && !warp_wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
                                     ok = false;
                                     break;
                                 }

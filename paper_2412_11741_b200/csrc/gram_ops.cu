@@ -160,17 +160,19 @@ gram_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
             }
         }
     } else if (warp == MMA_WARP) {
-        if (lane == 0) {
-            bool ok = wait_bounded(&sm.a_full, 0, wc);
+        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        const uint32_t tmem_d = warp_uniform(tmem_base);
+        {
+            bool ok = warp_wait_bounded(&sm.a_full, 0, wc);
             uint32_t n = 0;
             for (int jt = jt0; jt < jt1 && ok; ++jt, ++n) {
                 const int b = n & 1;
-                if (!wait_bounded(&sm.b_full[b], (n >> 1) & 1, wc) || !wait_bounded(&sm.acc_empty[b], ((n >> 1) & 1) ^ 1, wc)) {
+                if (!warp_wait_bounded(&sm.b_full[b], (n >> 1) & 1, wc) || !warp_wait_bounded(&sm.acc_empty[b], ((n >> 1) & 1) ^ 1, wc)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + b * GM;
+                const uint32_t d_tmem = tmem_d + b * GM;
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb) {
                     const uint64_t ah = make_smem_desc(smem_u32(&sm.A[0][kb][0])), al = make_smem_desc(smem_u32(&sm.A[1][kb][0]));
@@ -334,12 +336,14 @@ grad_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constant__ 
             }
         }
     } else if (warp == MMA_WARP) {
-        if (lane == 0) {
+        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        const uint32_t tmem_d = warp_uniform(tmem_base);
+        {
             bool ok = true;
             uint32_t p = 0;
             for (int kb = kb0; kb < kb1 && ok; ++kb, ++p) {
                 const int st = p % GRAD_STAGES;
-                if (!wait_bounded(&sm.full[st], (p / GRAD_STAGES) & 1, wc)) {
+                if (!warp_wait_bounded(&sm.full[st], (p / GRAD_STAGES) & 1, wc)) {
                     ok = false;
                     break;
                 }
@@ -349,9 +353,9 @@ grad_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constant__ 
 #pragma unroll
                 for (int k = 0; k < KBLK / 16; ++k) {
                     const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                    umma_bf16(tmem_base, ah + off, bh + off, kIdesc, (p | k) ? 1u : 0u);
-                    umma_bf16(tmem_base, ah + off, bl + off, kIdesc, 1u);
-                    umma_bf16(tmem_base, al + off, bh + off, kIdesc, 1u);
+                    umma_bf16(tmem_d, ah + off, bh + off, kIdesc, (p | k) ? 1u : 0u);
+                    umma_bf16(tmem_d, ah + off, bl + off, kIdesc, 1u);
+                    umma_bf16(tmem_d, al + off, bh + off, kIdesc, 1u);
                 }
                 umma_commit(&sm.empty[st]);
             }

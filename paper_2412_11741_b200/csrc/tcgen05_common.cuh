@@ -129,22 +129,34 @@ __device__ __forceinline__ void tmem_relinquish() {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 operands, fp32 accumulate.
+// D[tmem] (+)= A[smem] * B[smem]^T, bf16 operands, fp32 accumulate.  The whole warp calls, converged, with
+// the same arguments, and one elected lane issues: in code that only lane 0 runs, every MMA first has
+// to move its descriptors to the uniform registers the instruction takes, 116 cycles a piece, 168
+// when the other warps are busy too, more than the 128 x 256 x 16 MMA itself takes.  Measured, 128
+// MMAs in a row per SM with eight warps reading tensor memory: 178 cycles per MMA from lane 0,
+// 139 with the election (128 is the tensor core's own rate).
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(
         "{\n"
-        ".reg .pred p;\n"
+        ".reg .pred p, e;\n"
+        "elect.sync _|e, 0xffffffff;\n"
         "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
         "}\n" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// The mbarrier gets one arrival once every tcgen05.mma issued so far by this thread is done.
+// The mbarrier gets one arrival once every tcgen05.mma issued so far by the elected lane is done (the
+// whole warp calls, as above).
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+    asm volatile(
+        "{\n"
+        ".reg .pred e;\n"
+        "elect.sync _|e, 0xffffffff;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(smem_u32(bar))
+        : "memory");
 }
 // Waits for this thread's outstanding tcgen05.ld.  The registers are passed through the
 // statement so that no use of them can be scheduled ahead of the wait.
@@ -243,6 +255,16 @@ __device__ __forceinline__ bool wait_bounded_suspended(uint64_t* bar, uint32_t p
     atomicOr(w.status, kStatusTimeout);
     return false;
 }
+
+// The waits of a warp that stays converged (every lane polls; the answer is the same for all).
+__device__ __forceinline__ bool warp_wait_bounded(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
+    return __all_sync(0xffffffffu, wait_bounded(bar, parity, w));
+}
+__device__ __forceinline__ bool warp_wait_bounded_suspended(uint64_t* bar, uint32_t parity, const WaitCtx& w, uint32_t suspend_ns) {
+    return __all_sync(0xffffffffu, wait_bounded_suspended(bar, parity, w, suspend_ns));
+}
+// A value every lane of the warp holds, as one the compiler knows to be uniform.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // The same wait on a barrier that other CTAs of the cluster arrive on.
 __device__ __forceinline__ bool wait_bounded_cluster(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
