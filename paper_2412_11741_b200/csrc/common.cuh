@@ -134,12 +134,14 @@ struct AttnArgs {
     float* out;
     cudaStream_t stream;
 };
-// `scratch` holds attn_scratch_bytes() bytes: the fp32 array of per-atom partial products
-// ([B][N][H] for the scores, [B][pieces][H][N] for the value mix).
-size_t attn_scratch_bytes(int B, int H, int N, int64_t T);
+// `scratch`: the function's *_scratch_bytes(), 16-byte aligned.
+size_t key_scores_scratch_bytes(int B, int H, int N, int64_t T);
+size_t value_mix_scratch_bytes(int B, int H, int N, int64_t T);
+size_t decode_attention_scratch_bytes(int B, int H, int Nk, int Nv, int64_t T);
 int launch_key_scores(const AttnArgs& a, float* scratch);
 int launch_value_mix(const AttnArgs& a, float* scratch);
-int launch_softmax_rows(float* S, int64_t rows, int64_t T, cudaStream_t stream);   // in place, fp32
+// Both with a softmax over the tokens between: k.out holds the scores and then the weights (v.Q is not read).
+int launch_decode_attention(const AttnArgs& k, const AttnArgs& v, void* scratch);
 
 // Gradient step of the dictionary on one batch whose codes (idx, fp32 coef, dense [M][s])
 // are given; losses[0] = L_MSE, losses[1] = L_div of the dictionary before the update.

@@ -643,7 +643,7 @@ int csr_key_scores(const void* D, int N, int d, const void* Q, int q_dtype, int 
                static_cast<cudaStream_t>(stream)};
     if (B == 0 || T == 0) return CSR_OK;
     void* base = nullptr;
-    if (int rc = ensure_work(attn_scratch_bytes(B, H, N, T), &base, a.stream)) return rc;
+    if (int rc = ensure_work(key_scores_scratch_bytes(B, H, N, T), &base, a.stream)) return rc;
     return launch_key_scores(a, static_cast<float*>(align_up(static_cast<char*>(base) + kStatusBytes, 1024)));
 }
 
@@ -655,7 +655,7 @@ int csr_value_mix(const void* D, int N, int d, const float* W, int B, int H, con
                static_cast<cudaStream_t>(stream)};
     if (B == 0) return CSR_OK;
     void* base = nullptr;
-    if (int rc = ensure_work(attn_scratch_bytes(B, H, N, T), &base, a.stream)) return rc;
+    if (int rc = ensure_work(value_mix_scratch_bytes(B, H, N, T), &base, a.stream)) return rc;
     return launch_value_mix(a, static_cast<float*>(align_up(static_cast<char*>(base) + kStatusBytes, 1024)));
 }
 
@@ -664,11 +664,15 @@ int csr_decode_attention(const void* Dk, int Nk, const void* Dv, int Nv, int d, 
                          int sv, int coef_dtype, int64_t T, float scale, float* weights, float* out, void* stream) {
     if (T == 0 && B > 0) return fail(CSR_ERR_INVALID_ARG, "attention over an empty cache (T = 0) is undefined");
     if (int rc = check_attn(Dv, Nv, d, weights, B, H, v_idx, v_coef, coef_dtype, T, sv, out)) return rc;
-    if (int rc = csr_key_scores(Dk, Nk, d, Q, q_dtype, B, H, k_idx, k_coef, coef_dtype, T, sk, scale, weights, stream))
-        return rc;
+    if (int rc = check_attn(Dk, Nk, d, Q, B, H, k_idx, k_coef, coef_dtype, T, sk, weights)) return rc;
+    if (!valid_x_dtype(q_dtype)) return fail(CSR_ERR_INVALID_ARG, "q_dtype must be F32, BF16 or F16");
     if (B == 0) return CSR_OK;
-    if (int rc = launch_softmax_rows(weights, (int64_t)B * H, T, static_cast<cudaStream_t>(stream))) return rc;
-    return csr_value_mix(Dv, Nv, d, weights, B, H, v_idx, v_coef, coef_dtype, T, sv, out, stream);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    AttnArgs k{static_cast<const float*>(Dk), Nk, d, Q, q_dtype, B, H, k_idx, k_coef, coef_dtype, T, sk, scale, weights, st};
+    AttnArgs v{static_cast<const float*>(Dv), Nv, d, nullptr, CSR_DTYPE_F32, B, H, v_idx, v_coef, coef_dtype, T, sv, 1.0f, out, st};
+    void* base = nullptr;
+    if (int rc = ensure_work(decode_attention_scratch_bytes(B, H, Nk, Nv, T), &base, st)) return rc;
+    return launch_decode_attention(k, v, align_up(static_cast<char*>(base) + kStatusBytes, 1024));
 }
 
 int csr_dict_train_step(const csr_train_params_t* p) {
