@@ -22,7 +22,7 @@ namespace csr {
 namespace {
 
 constexpr int NT = 256;
-constexpr int RW = 16;                                    // rows per unit of a warp
+constexpr int RW = 16;                                    // most rows per unit of a warp
 constexpr int PP = 2;                                     // passes (rows) a lane works on together
 constexpr int INFLIGHT = 4;                               // gathers per row issued before their first use
 
@@ -115,14 +115,14 @@ __device__ __forceinline__ void store_out(void* out, int out_dtype, int64_t off,
     }
 }
 
-// Codes of rows [row0, row0 + RW) into the warp's shared memory as [RW][s].  `fast`: the unit lies
-// inside dense, 16-byte aligned code arrays, so it is one contiguous run per array and moves with
-// cp.async; otherwise element by element (row strides, the ragged last unit).
+// Codes of rows [row0, row0 + rows) into the warp's shared memory as [rows][s].  `fast`: a whole unit inside
+// dense, 16-byte aligned code arrays, so it is one contiguous run per array and moves with cp.async;
+// otherwise element by element (row strides, the ragged last unit).
 __device__ __forceinline__ void stage_codes(uint16_t* s_idx, unsigned char* s_coef, const uint16_t* __restrict__ idx,
                                             const void* __restrict__ coef, int cbytes, int64_t ldc, int64_t row0, int rows,
                                             int s, bool fast, int lane) {
     if (fast) {
-        const int n_i = RW * s * 2 / 16, n_c = RW * s * cbytes / 16;
+        const int n_i = rows * s * 2 / 16, n_c = rows * s * cbytes / 16;
         const char* gi = reinterpret_cast<const char*>(idx + row0 * s);
         const char* gc = static_cast<const char*>(coef) + row0 * s * cbytes;
         for (int q = lane; q < n_i; q += 32) cp_async16(reinterpret_cast<char*>(s_idx) + 16 * q, gi + 16 * q);
@@ -227,17 +227,55 @@ __device__ __forceinline__ void rows_by_four(const uint4* __restrict__ Dl, const
     }
 }
 
-template <int D_, bool F16>
+// The same for s a multiple of three (six entries per row is what a 4-byte-per-entry budget of 24 bytes
+// gives): three steps per trip, no step of four left half empty.
+template <int CH, int LPR, typename P, bool COEF16>
+__device__ __forceinline__ void rows_by_three(const uint4* __restrict__ Dl, const uint16_t* ci, const unsigned char* cc, int s,
+                                              int N, const int (&r)[PP], float (&acc)[PP][CH], [[maybe_unused]] uint32_t* status) {
+    constexpr bool RAW16 = COEF16 && CH == 8;
+    using CoefT = typename std::conditional<RAW16, uint16_t, float>::type;
+    const int nmax = N - 1;
+    for (int g0 = 0; g0 < s; g0 += 3) {
+        uint4 v[PP][3];
+        CoefT c[PP][3];
+#pragma unroll
+        for (int w = 0; w < PP; ++w)
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+                const int o = r[w] * s + g0 + u;
+                const int i = ci[o];
+#ifdef CSR_DEBUG_CHECKS
+                if (i > nmax) atomicOr(status, kStatusBounds);
+#endif
+                if constexpr (RAW16)
+                    c[w][u] = reinterpret_cast<const uint16_t*>(cc)[o];
+                else if constexpr (COEF16)
+                    c[w][u] = __half2float(reinterpret_cast<const __half*>(cc)[o]);
+                else
+                    c[w][u] = reinterpret_cast<const float*>(cc)[o];
+                v[w][u] = __ldg(Dl + static_cast<uint32_t>(min(i, nmax) * LPR));
+            }
+#pragma unroll
+        for (int w = 0; w < PP; ++w)
+#pragma unroll
+            for (int u = 0; u < 3; ++u) P::axpy(acc[w], c[w][u], v[w][u]);
+    }
+}
+
+// How the entries of a row are taken: four at a time (s a multiple of four), three at a time, or with
+// every step tested.  A kernel of its own for each: together they need more registers than the fp32
+// variant's four CTAs per SM leave.
+enum class By { Any, Four, Three };
+
+template <int D_, bool F16, By BY>
 __global__ void __launch_bounds__(NT, F16 ? 3 : 4)
 reconstruct_kernel(const void* __restrict__ Dict, const uint16_t* __restrict__ idx, const void* __restrict__ coef,
                    int coef_dtype, int64_t ldc, int64_t M, int N, int s, void* __restrict__ X_hat, int out_dtype,
-                   int64_t ldxh, int dense_codes, uint32_t* status) {
+                   int64_t ldxh, int dense_codes, int rw, uint32_t* status) {
     using P = Piece<F16>;
     constexpr int CH = P::CH;                             // channels per lane
     constexpr int LPR = D_ / CH;                          // lanes per row: 32, 16 or 8
     constexpr int RPP = 32 / LPR;                         // rows per warp pass
-    constexpr int PASSES = RW / RPP;                      // passes per unit: 16, 8 or 4
-    static_assert(PASSES % PP == 0, "passes are taken PP at a time");
     extern __shared__ __align__(16) unsigned char smem[];
     const int cbytes = coef_dtype == CSR_DTYPE_F16 ? 2 : 4;
     const int stride_i = RW * s * 2, stride_c = RW * s * cbytes;      // multiples of 16 bytes
@@ -248,86 +286,109 @@ reconstruct_kernel(const void* __restrict__ Dict, const uint16_t* __restrict__ i
 
     const int sub = lane / LPR, l = lane % LPR;
     const uint4* Dl = static_cast<const uint4*>(Dict) + l;  // this lane's 16 bytes of atom 0; an atom row is LPR pieces
-    const int64_t n_units = (M + RW - 1) / RW;
+    const int64_t n_units = (M + rw - 1) / rw;            // units of rw rows
     const int64_t unit_step = (int64_t)gridDim.x * (NT / 32);
-    const bool by_four = (s & 3) == 0;
 
-    auto unit_fast = [&](int64_t u) { return dense_codes && (u + 1) * RW <= M; };
+    auto unit_fast = [&](int64_t u) { return dense_codes && (u + 1) * rw <= M; };
     int64_t u = (int64_t)blockIdx.x * (NT / 32) + warp;
     int buf = 0;
-    if (u < n_units) stage_codes(s_idx(0), s_coef(0), idx, coef, cbytes, ldc, u * RW, (int)min((int64_t)RW, M - u * RW), s, unit_fast(u), lane);
+    if (u < n_units) stage_codes(s_idx(0), s_coef(0), idx, coef, cbytes, ldc, u * rw, (int)min((int64_t)rw, M - u * rw), s, unit_fast(u), lane);
     cp_async_commit();
     for (; u < n_units; u += unit_step, buf ^= 1) {
         const int64_t nu = u + unit_step;
         if (nu < n_units)
-            stage_codes(s_idx(buf ^ 1), s_coef(buf ^ 1), idx, coef, cbytes, ldc, nu * RW, (int)min((int64_t)RW, M - nu * RW), s,
+            stage_codes(s_idx(buf ^ 1), s_coef(buf ^ 1), idx, coef, cbytes, ldc, nu * rw, (int)min((int64_t)rw, M - nu * rw), s,
                         unit_fast(nu), lane);
         cp_async_commit();
         cp_async_wait<1>();                               // this unit's codes have landed (the next may be in flight)
         __syncwarp();
         const uint16_t* ci = s_idx(buf);
         const unsigned char* cc = s_coef(buf);
-        const bool whole = (u + 1) * RW <= M;
+        const int rows = (int)min((int64_t)rw, M - u * rw);
 #pragma unroll 1
-        for (int p = 0; p < PASSES; p += PP) {
+        for (int p = 0; p * RPP < rows; p += PP) {
             int r[PP];
             bool valid[PP];
             float acc[PP][CH];
 #pragma unroll
             for (int w = 0; w < PP; ++w) {
                 r[w] = (p + w) * RPP + sub;               // row inside the unit
-                valid[w] = u * RW + r[w] < M;
+                valid[w] = r[w] < rows;
+                if (BY != By::Any) r[w] = min(r[w], rows - 1);   // (a row past the end repeats the last one and is not stored)
 #pragma unroll
                 for (int k = 0; k < CH; ++k) acc[w][k] = 0.f;
             }
-            if (whole && by_four) {
+            if constexpr (BY == By::Four) {
                 if (cbytes == 2)
                     rows_by_four<CH, LPR, P, true>(Dl, ci, cc, s, N, r, acc, status);
                 else
                     rows_by_four<CH, LPR, P, false>(Dl, ci, cc, s, N, r, acc, status);
+            } else if constexpr (BY == By::Three) {
+                if (cbytes == 2)
+                    rows_by_three<CH, LPR, P, true>(Dl, ci, cc, s, N, r, acc, status);
+                else
+                    rows_by_three<CH, LPR, P, false>(Dl, ci, cc, s, N, r, acc, status);
             } else {
                 rows_generic<CH, LPR, P>(Dl, ci, cc, cbytes, s, N, r, valid, acc, status);
             }
 #pragma unroll
             for (int w = 0; w < PP; ++w)
-                if (valid[w]) store_out<CH>(X_hat, out_dtype, (u * RW + r[w]) * ldxh + l * CH, acc[w]);
+                if (valid[w]) store_out<CH>(X_hat, out_dtype, (u * rw + r[w]) * ldxh + l * CH, acc[w]);
         }
         __syncwarp();                                      // the buffer may be refilled
     }
     cp_async_wait<0>();
 }
 
-template <int D_, bool F16>
-int launch_t(const ReconstructArgs& a, const void* dict) {
+template <int D_, bool F16, By BY>
+int launch_by(const ReconstructArgs& a, const void* dict) {
+    auto kernel = reconstruct_kernel<D_, F16, BY>;
     const int cbytes = a.coef_dtype == CSR_DTYPE_F16 ? 2 : 4;
     const size_t smem = (size_t)(NT / 32) * 2 * RW * a.s * (2 + cbytes);
-    const int64_t n_blocks = ((a.M + RW - 1) / RW + NT / 32 - 1) / (NT / 32);
     static int ctas_per_sm[64] = {};                       // per device; what the occupancy calculator says for smem = 0
     int dev = 0;
     cudaGetDevice(&dev);
     dev = (dev >= 0 && dev < 64) ? dev : 0;
     int per_sm = ctas_per_sm[dev];
     if (per_sm == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reconstruct_kernel<D_, F16>, NT, 0) != cudaSuccess || per_sm < 1)
-            per_sm = 4;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, 0) != cudaSuccess || per_sm < 1) per_sm = 4;
         ctas_per_sm[dev] = per_sm;
     }
     // shared memory may hold fewer CTAs than the registers do (227 KB per SM)
     int fit = smem ? (int)((size_t)(227 * 1024) / (smem + 1024)) : per_sm;
     if (fit < 1) fit = 1;
     const int64_t cap = (int64_t)sm_count() * (per_sm < fit ? per_sm : fit);
+    // Rows per unit: 16, or 8 or 4 where that leaves a warp at least a tenth fewer rows in all (a last round of
+    // units that few warps have): 77777 rows are 1.03 rounds of 16 on 4736 warps, two rounds, or five
+    // rounds of 4: 34.9 -> 20.6 us (s = 6, N = 5001, fp32 atoms; with the steps of three).  Longer units are
+    // better otherwise (2^20 rows, s = 8, fp16 atoms: 126 us in units of 16, 140 in units of 4).  Eight rows of codes end on a 16-byte boundary in any case, four if s is
+    // even; a trip of a warp takes 32 / lanes per row * PP rows.
+    constexpr int trip = 32 / (D_ / Piece<F16>::CH) * PP;
+    const int64_t warps = cap * (NT / 32);
+    auto rows_of_a_warp = [&](int w) { return ((a.M + w - 1) / w + warps - 1) / warps * w; };
+    int rw = RW;
+    for (int w : {8, 4})
+        if (w >= trip && (w == 8 || a.s % 2 == 0) && 10 * rows_of_a_warp(w) <= 9 * rows_of_a_warp(rw)) rw = w;
+    const int64_t n_blocks = ((a.M + rw - 1) / rw + NT / 32 - 1) / (NT / 32);
     const int grid = (int)(n_blocks < cap ? n_blocks : cap);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(reconstruct_kernel<D_, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     }
     const uintptr_t pi = reinterpret_cast<uintptr_t>(a.idx), pc = reinterpret_cast<uintptr_t>(a.coef);
     const int dense = a.ld_code == a.s && pi % 16 == 0 && pc % 16 == 0;
-    reconstruct_kernel<D_, F16><<<grid, NT, smem, a.stream>>>(dict, a.idx, a.coef, a.coef_dtype, a.ld_code, a.M, a.N, a.s,
-                                                              a.X_hat, a.out_dtype, a.ld_xhat, dense, a.status);
+    kernel<<<grid, NT, smem, a.stream>>>(dict, a.idx, a.coef, a.coef_dtype, a.ld_code, a.M, a.N, a.s, a.X_hat, a.out_dtype, a.ld_xhat,
+                                         dense, rw, a.status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "reconstruct launch: %s", cudaGetErrorString(e));
     return CSR_OK;
+}
+
+template <int D_, bool F16>
+int launch_t(const ReconstructArgs& a, const void* dict) {
+    if (a.s % 4 == 0) return launch_by<D_, F16, By::Four>(a, dict);
+    if (a.s % 3 == 0) return launch_by<D_, F16, By::Three>(a, dict);
+    return launch_by<D_, F16, By::Any>(a, dict);
 }
 
 }  // namespace
