@@ -84,28 +84,27 @@ extern "C" {
  *                        (a) sweep on the tcgen05 tensor cores, residual and atoms each
  *                        split into a bf16 high and low part, three bf16 products per
  *                        correlation accumulated in fp32 (band 2^-12 * ||R||): the default
- *                        for 2048 rows or more where the library-owned scratch is in use (no
- *                        caller workspace;
- *                        about 4 * N * d + 2048 * d * min(ceil(M / 256), SMs) bytes of it);
+ *                        wherever the library-owned scratch is in use (no caller workspace;
+ *                        about 4 * N * d + 2048 * d * min(ceil(M / 256), SMs) bytes of it).
+ *                        Whole waves of pairs of 128-row tiles run with one CTA per pair;
+ *                        fewer rows, and what is left over, with the dictionary split
+ *                        across the CTAs of one cooperative launch (the same codes);
  *                        (b) fp32 operands and fp32 accumulation on the plain ALUs (band
  *                        1.6e-5 * ||R||), one CTA per 64 rows, no scratch: taken when a
  *                        caller workspace is given;
- *                        (c) with few rows (the vectors one decoding step adds: fewer than
- *                        2048) the plain-ALU sweep with the
- *                        dictionary split across the SMs instead of the rows, two launches
- *                        per iteration; library-owned scratch, not taken when a caller
- *                        workspace is given.
+ *                        (c) the plain-ALU sweep for few rows with the dictionary split
+ *                        across the SMs, two launches per iteration, library-owned
+ *                        scratch: the option "exact_engine" = 1.
  *   CSR_MODE_BF16_FAST   correlations on the tcgen05 tensor cores with bf16 operands
  *                        (residual and atoms rounded to bf16) and fp32 accumulation.
  *                        Near-tied picks may differ from an fp64 evaluation; the mean
  *                        reconstruction error does not, down to a floor of about
  *                        2^-8 * ||x|| (the residual is carried in bf16); use the exact
- *                        mode for errors below 1e-2 * ||x||.  With few rows (at most half
- *                        as many pairs of 128-row tiles as SMs) the dictionary is split
- *                        across the CTAs of thread-block clusters that share the rows,
- *                        still one launch, with identical codes; where clusters cannot be
- *                        launched and the library-owned scratch is in use, across CTAs
- *                        with one sweep and one pick launch per iteration.
+ *                        mode for errors below 1e-2 * ||x||.  Few rows, and what is left
+ *                        over after whole waves of pairs of 128-row tiles, run as single
+ *                        row tiles whose dictionary sweep is split across the CTAs of a
+ *                        thread-block cluster where that is faster: the same codes, no
+ *                        scratch.
  *                        (csr_set_option can force each of these paths.)
  */
 #define CSR_MODE_FP32_EXACT 0
@@ -413,10 +412,11 @@ int csr_dict_check_norms(const void* D, int N, int d, float tol, void* stream, f
  * to drive every code path, measurements to compare them).  All paths return the same codes.
  *   "fast_group"     0 (default: the library chooses) or 1, 2, 4, 8: atoms per arg-max group
  *                    of the fast encoder's sweep;
- *   "fast_split"     0 (default: few rows split the dictionary across thread-block
- *                    clusters, else across CTAs with a launch pair per iteration),
+ *   "fast_split"     0 (default: single row tiles, split across thread-block clusters, for few
+ *                    and left-over rows),
  *                    1 = always one CTA per pair of row tiles over the whole dictionary,
- *                    2 = no clusters;
+ *                    2 = no clusters (few rows: a launch pair per iteration in the library's
+ *                    scratch);
  *   "exact_split"    0 (default: the exact mode splits the dictionary for few rows), 1 = never;
  *   "exact_engine"   0 (default: the exact mode's tensor-core encoders), 1 = plain-ALU encoders only,
  *                    2 = the tensor-core encoder of pairs of row tiles whatever the number of rows;

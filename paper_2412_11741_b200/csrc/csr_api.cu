@@ -330,7 +330,7 @@ int encode_device(const csr_encode_params_t* p, bool shared_scratch = true, cons
     a.stream = static_cast<cudaStream_t>(p->stream);
     const Options opt = options();
     if (p->mode == CSR_MODE_FP32_EXACT) {
-        // Both the few-rows encoder and the tensor-core encoder need scratch, which comes from
+        // The tensor-core encoders and the few-rows plain-ALU encoder need scratch, which comes from
         // the library-owned buffer only (a caller workspace is sized for the fast mode, and two
         // encodes in flight must not share it): otherwise the row-tile encoder runs.
         const bool own = shared_scratch && !p->workspace;
@@ -361,11 +361,9 @@ int encode_device(const csr_encode_params_t* p, bool shared_scratch = true, cons
         cudaError_t e = cudaMemsetAsync(status, 0, sizeof(uint32_t), a.stream);
         if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
     }
-    // few rows: the cluster path needs no scratch; its fallback (a launch pair per iteration)
-    // does, and gets it from the library-owned buffer only (a caller workspace is sized for
-    // the bf16 copy)
-    const bool split = shared_scratch && !p->workspace && !prepared && encode_fast_split_applies(p->M, p->N) &&
-                       opt.fast_split != 1;
+    // few rows without clusters (an option): a launch pair per iteration, whose scratch comes from the
+    // library-owned buffer only (a caller workspace is sized for the bf16 copy)
+    const bool split = shared_scratch && !p->workspace && !prepared && opt.fast_split == 2 && encode_fast_split_applies(p->M, p->N);
     const size_t dict_b = (encode_fast_workspace_bytes(p->d, p->N) + 1023) / 1024 * 1024;
     const size_t split_b = split ? encode_fast_split_scratch_bytes(p->M, p->d, p->N) : 0;
     if (p->dict || prepared) {

@@ -42,21 +42,16 @@
 // after which the CTA raises a flag in the status word, lets its copies land, frees
 // its TMEM and exits.
 //
-// Few rows (the vectors one decoding step adds) would leave all but a few SMs idle, each of
-// them sweeping the whole dictionary s times.  Three instantiations of the kernel cover
-// that case (template argument CL):
-//   CL = 0  the kernel above; with n_splits > 1 it sweeps only a slice of the dictionary for
-//           ONE iteration and leaves the rows' maxima to split_pick_kernel (a launch pair
-//           per iteration: the fallback where clusters cannot be launched);
-//   CL = 1  n_splits CTAs form a thread-block cluster, hold the same pair of row tiles and
-//           each sweep a slice; after every sweep the rows' maxima are exchanged through
-//           distributed shared memory (st.async credited to the peers' mbarriers: gather at
-//           the CTA that merges a row, merged value back to everyone) and every CTA makes
-//           the same pick and update, so all s iterations run in one launch;
-//   CL = 2  the same with at most 128 rows in all: both accumulators and both epilogue warp
-//           groups serve the one row tile, and the other row tile's shared memory holds
-//           exchange buffers large enough for a one-hop all-to-all.
-// The codes are the same bits in every case.
+// Few rows (the vectors one decoding step adds, a short prompt, what is left over after whole waves of
+// pairs) would leave most SMs idle, each of the others sweeping the whole dictionary s times.  A
+// second instantiation (template argument ONE) works on single row tiles: n_splits CTAs (1, 2, 4, 8 or
+// 16, a thread-block cluster) hold the same tile and each sweep a slice of the dictionary, both
+// accumulators and both epilogue warp groups serving the one tile; after every sweep the rows' maxima
+// are exchanged through distributed shared memory in one hop (st.async credited to the peers'
+// mbarriers, into the other row tile's memory) and every CTA makes the same pick and update, so all
+// s iterations run in one launch.  plan_rows() says which rows run how; the codes are the same bits in
+// every case.  (Where clusters must not be used, n_splits > 1 without ONE sweeps a slice for one
+// iteration and leaves the rows' maxima to split_pick_kernel: a launch pair per iteration.)
 #include <cuda.h>
 
 #include <mutex>
@@ -101,13 +96,12 @@ struct FastSmem {
     uint64_t acc_empty[2];
     uint64_t res_ready[2];
     uint64_t drained;
-    uint64_t pair_bar;                                 // CL == 2: second warp group's result is in xout
-    uint64_t pick_bar;                                 // CL == 2: the rows' picks are in xin (for the second group)
-    uint64_t xbar[2];                                  // cluster exchange: gathered / merged, one phase per iteration each
-    unsigned long long xin[2 * TILE_M];                // cluster exchange: (key, ~tile) of the rows this CTA merges, per source CTA
-                                                       // (CL == 2: the rows' winning atoms, for the second warp group)
-    unsigned long long xout[2 * TILE_M];               // cluster exchange: merged (key, ~tile) of every row
-                                                       // (CL == 2: the second warp group's maxima)
+    // ONE:
+    uint64_t pair_bar;                                 // the second warp group's maxima are in xout
+    uint64_t pick_bar;                                 // the rows' winning atoms are in pick_n0 (for the second group)
+    uint64_t xbar;                                     // every CTA's maxima have arrived, one phase per iteration
+    unsigned long long xout[TILE_M];
+    int pick_n0[TILE_M];
     uint32_t tmem_base;
     volatile uint32_t abort;
 };
@@ -426,7 +420,7 @@ split_pick_kernel(const uint16_t* __restrict__ Db, int N, uint4* __restrict__ Rb
 // ---------------------------------------------------------------------------------------
 // the encoder
 // ---------------------------------------------------------------------------------------
-template <int D_, int G, int CL>
+template <int D_, int G, bool ONE>
 __global__ void __launch_bounds__(NT, 1)
 encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* __restrict__ Db,
                    const void* __restrict__ X, int x_dtype, int64_t ldx, int64_t M, int N, int s,
@@ -440,20 +434,15 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int T = (N + TILE_N - 1) / TILE_N;                // dictionary tiles per sweep (the last may be half)
-    const int64_t n_pairs = (M + 2 * TILE_M - 1) / (2 * TILE_M);
-    // Few rows (n_splits > 1): n_splits CTAs share one pair of row tiles, CTA j sweeping the
-    // dictionary tiles j, j + n_splits, ...
-    //  - CL: the n_splits CTAs are one thread-block cluster and run all s iterations.
-    //    After each sweep every row's best (key, tile) is max-reduced into every CTA's shared
-    //    memory, every CTA then makes the same pick and the same residual update on its own
-    //    copy of the rows, and CTA 0 of the cluster writes the codes.
-    //    CL == 2: at most TILE_M rows in all (one decoding step of a small batch).  Only the
-    //    first row tile exists; the two accumulators take the CTA's dictionary tiles in turn
-    //    and the second group of epilogue warps drains the second accumulator for the same
-    //    rows; the unused second row tile holds the exchange buffers, large enough for every
-    //    CTA to hear from every CTA directly (one hop).
-    //  - otherwise ONE iteration per launch (s == 1 is passed): each row's best (key, tile) goes
-    //    to `partial` and the pick kernel takes over.
+    const int64_t n_pairs = ONE ? (M + TILE_M - 1) / TILE_M : (M + 2 * TILE_M - 1) / (2 * TILE_M);   // (ONE: single tiles)
+    // n_splits > 1: n_splits CTAs share the rows, CTA j sweeping the dictionary tiles j, j + n_splits, ...
+    //  - ONE: they are one thread-block cluster, hold the same single row tile and run all s
+    //    iterations.  Only the first row tile exists; the two accumulators take the CTA's
+    //    dictionary tiles in turn and the second group of epilogue warps drains the second
+    //    accumulator for the same rows; the unused second row tile holds the exchange buffers, large
+    //    enough for every CTA to hear from every CTA directly.  CTA 0 of the cluster writes the codes.
+    //  - otherwise ONE iteration per launch (s == 1 is passed) on pairs of row tiles: each row's
+    //    best (key, tile) goes to `partial` and the pick kernel takes over.
     const int t_begin = n_splits > 1 ? (int)(blockIdx.x % n_splits) : 0;
     const int t_step = n_splits > 1 ? n_splits : 1;
     const int64_t pair_first = n_splits > 1 ? blockIdx.x / n_splits : blockIdx.x;
@@ -473,19 +462,12 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
             mbar_init(&sm.acc_full[t], 1);
             mbar_init(&sm.acc_empty[t], 4);
             // (with one tile of rows both warp groups update rows of it)
-            mbar_init(&sm.res_ready[t], CL == 2 ? 2 * TILE_M : TILE_M);
+            mbar_init(&sm.res_ready[t], ONE ? 2 * TILE_M : TILE_M);
         }
         mbar_init(&sm.drained, 1);
-        if constexpr (CL == 1) {
-            // one phase per iteration: this thread arms it with the bytes the peers will send
-            mbar_init(&sm.xbar[0], 1);
-            mbar_init(&sm.xbar[1], 1);
-            mbar_expect_tx(&sm.xbar[0], 2 * TILE_M * 8);
-            mbar_expect_tx(&sm.xbar[1], 2 * TILE_M * 8);
-        }
-        if constexpr (CL == 2) {
-            mbar_init(&sm.xbar[0], 1);
-            mbar_expect_tx(&sm.xbar[0], static_cast<uint32_t>(n_splits) * TILE_M * 8);
+        if constexpr (ONE) {
+            mbar_init(&sm.xbar, 1);
+            mbar_expect_tx(&sm.xbar, static_cast<uint32_t>(n_splits) * TILE_M * 8);
             mbar_init(&sm.pair_bar, TILE_M);
             mbar_init(&sm.pick_bar, TILE_M);
         }
@@ -501,7 +483,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
     tc_fence_after();
     const uint32_t tmem_base = sm.tmem_base;
     // no CTA touches a peer's barrier or words before every peer has set them up
-    if constexpr (CL) cluster_sync_all();
+    if constexpr (ONE) cluster_sync_all();
 
     if (warp == PRODUCER_WARP) {
         // ------------------------------ TMA producer ------------------------------
@@ -539,7 +521,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         // ------------------------------ MMA issuer ------------------------------
         // (the whole warp runs this, one elected lane issues: see umma_bf16)
         const uint32_t tmem_d = warp_uniform(tmem_base);
-        if constexpr (CL == 2) {
+        if constexpr (ONE) {
             // one row tile; the CTA's dictionary tiles go to the two accumulators in turn
             uint32_t p = 0, accn[2] = {0u, 0u};
             bool ok = true;
@@ -638,7 +620,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
     } else {
         // ------------------------------ epilogue ------------------------------
         const int acc = warp >> 2;                        // the accumulator this warp drains
-        const int tile = CL == 2 ? 0 : acc;               // the row tile its rows belong to
+        const int tile = ONE ? 0 : acc;               // the row tile its rows belong to
         const int q = warp & 3;
         const int r = q * 32 + lane;                      // row inside the tile == TMEM lane
         const int slot = tile * TILE_M + r;               // row inside the CTA's pair
@@ -649,14 +631,14 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         uint32_t accn = 0;
         [[maybe_unused]] uint32_t xn = 0;
         bool ok = true;
-        const bool writes_codes = !CL || t_begin == 0;
+        const bool writes_codes = !ONE || t_begin == 0;
         for (int64_t pair = pair_first; pair < n_pairs && ok; pair += pair_step) {
-            const int64_t m = pair * (2 * TILE_M) + slot;
+            const int64_t m = pair * (ONE ? TILE_M : 2 * TILE_M) + slot;
             const bool valid = m < M;
             uint32_t row_mask = 0xffffffffu;
-            if constexpr (CL) row_mask = __ballot_sync(0xffffffffu, valid);
+            if constexpr (ONE) row_mask = __ballot_sync(0xffffffffu, valid);
             // ---- R_0 = x, rounded to bf16, into the operand tile ----
-            if (CL == 2 && acc == 1) {
+            if (ONE && acc == 1) {
                 // the second warp group has no rows of its own
             } else if (x_dtype == CSR_DTYPE_BF16) {
                 const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(X) + m * ldx);
@@ -706,7 +688,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                 // ---- sweep: running arg-max of |correlation| over all atom tiles ----
                 uint32_t best_key = 0, best_t = 0;
                 [[maybe_unused]] int n0_other = 0;
-                for (int t = t_begin + (CL == 2 ? acc * t_step : 0); t < T; t += (CL == 2 ? 2 : 1) * t_step, ++accn) {
+                for (int t = t_begin + (ONE ? acc * t_step : 0); t < T; t += (ONE ? 2 : 1) * t_step, ++accn) {
                     bool got = wait_bounded(&sm.acc_full[acc], accn & 1, wc);
                     got = __all_sync(0xffffffffu, got);
                     if (!got) {
@@ -751,11 +733,11 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                     }
                 }
                 if (!ok) break;
-                if (!CL && partial) {                       // split sweep: the pick kernel takes over
+                if (!ONE && partial) {                       // split sweep: the pick kernel takes over
                     if (valid) partial[m * n_splits + t_begin] = make_uint2(best_key, best_t);
                     continue;
                 }
-                if constexpr (CL == 2) {
+                if constexpr (ONE) {
                     // ---- the row's best over this CTA's tiles (both accumulators), then over the
                     // whole dictionary: every CTA sends its (key, ~tile) of the row to every CTA.
                     // The entries are double-buffered by iteration: a peer writes iteration g + 2's
@@ -765,7 +747,6 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                     // (a CTA with a single dictionary tile has no use for the second group, which
                     // would otherwise run ahead of the first: nothing paces it but its sweep)
                     const bool two_groups = t_begin + t_step < T;
-                    int* pick_n0 = reinterpret_cast<int*>(&sm.xin[0]);
                     bool got = true;
                     if (acc == 1) {
                         if (two_groups) {
@@ -777,18 +758,18 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                     } else if (two_groups) {
                         got = wait_bounded(&sm.pair_bar, xn & 1, wc);
                     }
-                    if (got && acc == 0) {
-                        if (two_groups) {
-                            const unsigned long long other = *reinterpret_cast<volatile unsigned long long*>(&sm.xout[r]);
-                            mine = other > mine ? other : mine;
-                        }
+                    if (got && acc == 0 && two_groups) {
+                        const unsigned long long other = *reinterpret_cast<volatile unsigned long long*>(&sm.xout[r]);
+                        mine = other > mine ? other : mine;
+                    }
+                    if (got && acc == 0 && n_splits > 1) {
                         constexpr int XMAX = FastSmem<D_>::kATileBytes / (2 * TILE_M * 8);   // CTAs the buffers hold
                         unsigned long long* xg = reinterpret_cast<unsigned long long*>(&sm.A[1][0]) + (xn & 1) * XMAX * TILE_M;
-                        const uint32_t dst = smem_u32(&xg[t_begin * TILE_M + r]), bar = smem_u32(&sm.xbar[0]);
+                        const uint32_t dst = smem_u32(&xg[t_begin * TILE_M + r]), bar = smem_u32(&sm.xbar);
                         for (int c = 0; c < n_splits; ++c) st_async_u64(map_to_cta(dst, c), mine, map_to_cta(bar, c));
-                        got = wait_bounded_cluster(&sm.xbar[0], xn & 1, wc);
+                        got = wait_bounded_cluster(&sm.xbar, xn & 1, wc);
                         if (got) {
-                            if (r == 0) mbar_expect_tx(&sm.xbar[0], static_cast<uint32_t>(n_splits) * TILE_M * 8);
+                            if (r == 0) mbar_expect_tx(&sm.xbar, static_cast<uint32_t>(n_splits) * TILE_M * 8);
                             unsigned long long top = 0ull;
                             for (int c = 0; c < n_splits; ++c) {
                                 const unsigned long long v = *reinterpret_cast<volatile unsigned long long*>(&xg[c * TILE_M + r]);
@@ -806,63 +787,19 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                     best_key = static_cast<uint32_t>(mine >> 32);
                     best_t = 0xFFFFFFFFu - static_cast<uint32_t>(mine);
                     if (acc == 0) {
-                        pick_n0[r] = candidate_start<G>(best_key, best_t, N, status);
+                        sm.pick_n0[r] = candidate_start<G>(best_key, best_t, N, status);
                         mbar_arrive(&sm.pick_bar);
                         row_mask &= 0x0000FFFFu;
                     } else {
-                        n0_other = *reinterpret_cast<volatile int*>(&pick_n0[r]);
+                        n0_other = *reinterpret_cast<volatile int*>(&sm.pick_n0[r]);
                         row_mask &= 0xFFFF0000u;
                     }
-                }
-                if constexpr (CL == 1) {
-                    // ---- every CTA of the cluster learns the row's best over the whole dictionary:
-                    // the highest key and, among equal keys, the lowest tile.  Row i of the pair is
-                    // merged by CTA i % n_splits: gather there, merge, send the result to everyone.
-                    // Both buffers are single.  An entry of xin is overwritten by a peer that has
-                    // seen this iteration's merged rows from all of this CTA's merging threads,
-                    // each of which read its entries first; an entry of xout is overwritten by a
-                    // peer that has received the next iteration's key from the one thread that
-                    // reads it. ----
-                    const unsigned long long mine =
-                        (static_cast<unsigned long long>(best_key) << 32) | (0xFFFFFFFFu - best_t);
-                    const int per_cta = 2 * TILE_M / n_splits;        // rows merged by one CTA
-                    {
-                        const uint32_t o = static_cast<uint32_t>(slot % n_splits);
-                        st_async_u64(map_to_cta(smem_u32(&sm.xin[t_begin * per_cta + slot / n_splits]), o), mine,
-                                     map_to_cta(smem_u32(&sm.xbar[0]), o));
-                    }
-                    bool got = true;
-                    if (slot < per_cta) {
-                        got = wait_bounded_cluster(&sm.xbar[0], xn & 1, wc);
-                        if (got) {
-                            if (slot == 0) mbar_expect_tx(&sm.xbar[0], 2 * TILE_M * 8);       // the next iteration's
-                            unsigned long long top = 0ull;
-                            for (int c = 0; c < n_splits; ++c) {
-                                const unsigned long long v =
-                                    *reinterpret_cast<volatile unsigned long long*>(&sm.xin[c * per_cta + slot]);
-                                top = v > top ? v : top;
-                            }
-                            const uint32_t dst = smem_u32(&sm.xout[slot * n_splits + t_begin]), bar = smem_u32(&sm.xbar[1]);
-                            for (int c = 0; c < n_splits; ++c) st_async_u64(map_to_cta(dst, c), top, map_to_cta(bar, c));
-                        }
-                    }
-                    if (got) got = wait_bounded_cluster(&sm.xbar[1], xn & 1, wc);
-                    got = __all_sync(0xffffffffu, got);
-                    if (!got) {
-                        ok = false;
-                        break;
-                    }
-                    if (slot == 0) mbar_expect_tx(&sm.xbar[1], 2 * TILE_M * 8);               // the next iteration's
-                    const unsigned long long all = *reinterpret_cast<volatile unsigned long long*>(&sm.xout[slot]);
-                    ++xn;
-                    best_key = static_cast<uint32_t>(all >> 32);
-                    best_t = 0xFFFFFFFFu - static_cast<uint32_t>(all);
                 }
                 // ---- pick, signed coefficient, residual update ----
                 const int gi = g & (CODE_BLOCK - 1);
                 int n0 = candidate_start<G>(best_key, best_t, N, status);
-                if (CL == 2 && acc == 1) n0 = n0_other;
-                if constexpr (CL)
+                if (ONE && acc == 1) n0 = n0_other;
+                if constexpr (ONE)
                     pick_and_update<D_, G, true>(Atile, q, lane, Db, n0, g + 1 < s, code_idx, code_coef, gi, row_mask);
                 else
                     pick_and_update<D_, G>(Atile, q, lane, Db, n0, g + 1 < s, code_idx, code_coef, gi);
@@ -872,7 +809,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                 }
                 __syncwarp();
                 // ---- flush the collected codes eight at a time ----
-                if ((gi == CODE_BLOCK - 1 || g == s - 1) && valid && writes_codes && (CL != 2 || (lane < 16) == (acc == 0))) {
+                if ((gi == CODE_BLOCK - 1 || g == s - 1) && valid && writes_codes && (!ONE || (lane < 16) == (acc == 0))) {
                     const int g0 = g - gi;
                     const int64_t o = m * ldc + g0;
                     if (gi == CODE_BLOCK - 1 && vec_codes) {
@@ -916,7 +853,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         tmem_dealloc(tmem_base, TMEM_COLS);
     }
     // a CTA's shared memory must outlive its peers' last writes to it
-    if constexpr (CL) cluster_sync_all();
+    if constexpr (ONE) cluster_sync_all();
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -965,18 +902,16 @@ int max_clusters(int cluster_ctas) {
     if (cached[cluster_ctas] == 0) {
         const size_t smem = sizeof(FastSmem<D_>) + 1024;
         int n = 0;
-        bool good = cudaFuncSetAttribute(encode_fast_kernel<D_, G, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        bool good = cudaFuncSetAttribute(encode_fast_kernel<D_, G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem) == cudaSuccess;
         if (good && cluster_ctas > 8)
-            good = cudaFuncSetAttribute(encode_fast_kernel<D_, G, 1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                       cudaSuccess &&
-                   cudaFuncSetAttribute(encode_fast_kernel<D_, G, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                       cudaSuccess;
+            good = cudaFuncSetAttribute(encode_fast_kernel<D_, G, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                   cudaSuccess;
         if (good) {
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute attr[1];
             cluster_config<D_, G>(cfg, attr, cluster_ctas, cluster_ctas, smem, 0);
-            good = cudaOccupancyMaxActiveClusters(&n, encode_fast_kernel<D_, G, 1>, &cfg) == cudaSuccess;
+            good = cudaOccupancyMaxActiveClusters(&n, encode_fast_kernel<D_, G, true>, &cfg) == cudaSuccess;
         }
         if (!good) {
             cudaGetLastError();                        // a refusal is an answer, not a failure of the call
@@ -987,47 +922,36 @@ int max_clusters(int cluster_ctas) {
     return cached[cluster_ctas] > 0 ? cached[cluster_ctas] : 0;
 }
 
+// Pairs of row tiles, one CTA each over the whole dictionary (n_splits = 0), or one iteration of the
+// split without clusters; or, with `tile_splits` > 0, single row tiles, tile_splits CTAs each.
 template <int D_, int G>
-int launch(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status, int n_splits,
-           uint2* partial, int cluster_grid = 0) {
+int launch(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status, int n_splits, uint2* partial,
+           int tile_splits = 0) {
     const size_t smem = sizeof(FastSmem<D_>) + 1024;
-    // at most one tile of rows in all: the clustered kernel that spends both accumulators on it
-    const bool one_tile = cluster_grid > 0 && a.M <= TILE_M && n_splits <= FastSmem<D_>::kATileBytes / (2 * TILE_M * 8);
-    cudaError_t e =
-        cluster_grid > 0
-            ? cudaFuncSetAttribute(one_tile ? encode_fast_kernel<D_, G, 2> : encode_fast_kernel<D_, G, 1>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-            : cudaFuncSetAttribute(encode_fast_kernel<D_, G, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kernel = tile_splits > 0 ? encode_fast_kernel<D_, G, true> : encode_fast_kernel<D_, G, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    const int64_t n_pairs = (a.M + 2 * TILE_M - 1) / (2 * TILE_M);
-    const int grid = n_splits > 1 ? (int)(n_pairs * n_splits)
-                                  : (int)(n_pairs < (int64_t)sm_count() ? n_pairs : (int64_t)sm_count());
     // keys keep the magnitude bits above the group tag; with G == 1 the key is built from the
     // raw value, so the mask clears the sign bit as well
     const uint32_t key_mask = (G == 1 ? 0x7FFFFFFFu : 0xFFFFFFFFu) & ~static_cast<uint32_t>(TILE_N / G - 1);
     // 16-byte code stores need eight codes per flush and 16-byte aligned rows in both arrays
     const uintptr_t ci = reinterpret_cast<uintptr_t>(a.out_idx), cc = reinterpret_cast<uintptr_t>(a.out_coef);
     const int vec_codes = (a.s % 8 == 0) && (a.ld_code % 8 == 0) && (ci % 16 == 0) && (cc % 16 == 0);
-    const unsigned long long wait_limit = options().wait_limit_ns;
-    if (cluster_grid > 0) {
-        // n_splits CTAs per cluster, cluster_grid CTAs in all
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        cluster_config<D_, G>(cfg, attr, n_splits, cluster_grid, smem, a.stream);
-        e = cudaLaunchKernelEx(&cfg, one_tile ? encode_fast_kernel<D_, G, 2> : encode_fast_kernel<D_, G, 1>, tmap, Db, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx,
-                               a.out_coef, a.coef_dtype, a.ld_code, vec_codes, key_mask, status, n_splits,
-                               static_cast<uint2*>(nullptr), wait_limit);
-        if (e != cudaSuccess) {
-            // refused at launch (nothing ran): the caller takes another path
-            cudaGetLastError();
-            return kClusterLaunchRefused;
-        }
-        return CSR_OK;
+    const int64_t n_pairs = (a.M + 2 * TILE_M - 1) / (2 * TILE_M), n_tiles = (a.M + TILE_M - 1) / TILE_M;
+    const int grid = tile_splits > 0 ? (int)(n_tiles * tile_splits)
+                     : n_splits > 1  ? (int)(n_pairs * n_splits)
+                                     : (int)(n_pairs < (int64_t)sm_count() ? n_pairs : (int64_t)sm_count());
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cluster_config<D_, G>(cfg, attr, tile_splits > 1 ? tile_splits : 1, grid, smem, a.stream);
+    if (tile_splits <= 1) cfg.numAttrs = 0;
+    e = cudaLaunchKernelEx(&cfg, kernel, tmap, Db, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx, a.out_coef, a.coef_dtype,
+                           a.ld_code, vec_codes, key_mask, status, tile_splits > 0 ? tile_splits : n_splits, partial,
+                           options().wait_limit_ns);
+    if (e != cudaSuccess && tile_splits > 1) {             // refused at launch (nothing ran): the caller takes another path
+        cudaGetLastError();
+        return kClusterLaunchRefused;
     }
-    encode_fast_kernel<D_, G, 0><<<grid, NT, smem, a.stream>>>(tmap, Db, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx,
-                                                           a.out_coef, a.coef_dtype, a.ld_code, vec_codes, key_mask,
-                                                           status, n_splits, partial, wait_limit);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "encode_fast launch: %s", cudaGetErrorString(e));
     return CSR_OK;
 }
@@ -1044,93 +968,97 @@ int group_size(int d, int N) {
     return 1;
 }
 
+// How M rows are run: `pair_rows` of them as whole waves of pairs of row tiles, one CTA per pair, then up
+// to two launches of single row tiles with splits[k] CTAs per tile.  A pair shares each dictionary
+// stage between its two tiles and is the cheapest way to fill the chip; single tiles spread what
+// does not.  The estimates are fits of this kernel's measured time per iteration in us (M from 64 to
+// 28000, N from 512 to 16384, s = 8): pairs 3.3 + 1.55 per 256-atom tile of the dictionary (d = 64: 3.0
+// + 1.05), single tiles 4.1 + 0.75 per tile of the CTA's slice (d = 64: 3.2 + 0.48).  Some of it, in us
+// per call of 8 iterations at N = 1024 / 8192, d = 128, this plan against clusters of up to 16 CTAs
+// on pairs of row tiles: 64 rows 35 / 45 against 47 / 45; 1100 rows 37 / 58 against 54 / 74; 4160 rows
+// 40 / 83 against 56 / 140; 9400 rows 45 / 131 against 68 / 233; 18900 rows 54 / 227 against 70 / 237.
+struct RowPlan {
+    int64_t pair_rows;
+    int64_t tile_rows[2];
+    int splits[2];
+};
+template <int D_, int G>
+RowPlan plan_rows(int64_t M, int N) {
+    const int T = (N + TILE_N - 1) / TILE_N;
+    const int64_t sms = sm_count(), wave = sms * 2 * TILE_M;
+    const int64_t rest = M % wave, tiles = (rest + TILE_M - 1) / TILE_M;
+    constexpr float kPair0 = D_ == 128 ? 3.3f : 3.0f, kPair1 = D_ == 128 ? 1.55f : 1.05f;
+    constexpr float kTile0 = D_ == 128 ? 4.1f : 3.2f, kTile1 = D_ == 128 ? 0.75f : 0.48f;
+    constexpr int kMost = FastSmem<D_>::kATileBytes / (2 * TILE_M * 8);       // the exchange buffers bound the cluster
+    // n row tiles in one launch: the best number of CTAs per tile
+    auto best_split = [&](int64_t n, float* cost) {
+        int best = 1;
+        *cost = (float)((n + sms - 1) / sms) * (kTile0 + kTile1 * T);
+        for (int ns = 2; ns <= kMost && ns <= T; ns *= 2) {
+            const int nc = max_clusters<D_, G>(ns);
+            if (nc < 1) continue;
+            const float c = (float)((n + nc - 1) / nc) * (kTile0 + kTile1 * ((T + ns - 1) / ns));
+            if (c < *cost) {
+                *cost = c;
+                best = ns;
+            }
+        }
+        return best;
+    };
+    RowPlan p{M, {0, 0}, {0, 0}};
+    if (tiles == 0) return p;
+    float least = kPair0 + kPair1 * T, cost;
+    const int one = best_split(tiles, &cost);
+    if (cost < least) {
+        least = cost;
+        p = RowPlan{M - rest, {rest, 0}, {one, 0}};
+    }
+    if (tiles > sms) {                                     // a whole wave of single tiles, then the others over the whole chip
+        const int two = best_split(tiles - sms, &cost);
+        cost += kTile0 + kTile1 * T;
+        if (cost < least) p = RowPlan{M - rest, {sms * TILE_M, rest - sms * TILE_M}, {1, two}};
+    }
+    return p;
+}
+
+template <int D_, int G>
+int launch_planned(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status) {
+    // (the option forces pairs only)
+    const RowPlan p = options().fast_split == 0 ? plan_rows<D_, G>(a.M, a.N) : RowPlan{a.M, {0, 0}, {0, 0}};
+    auto rows_from = [&](int64_t r0, int64_t m) {
+        EncodeArgs b = a;
+        b.X = static_cast<const char*>(a.X) + (size_t)r0 * a.ldx * dtype_size(a.x_dtype);
+        b.out_idx = a.out_idx + r0 * a.ld_code;
+        b.out_coef = static_cast<char*>(a.out_coef) + (size_t)r0 * a.ld_code * (a.coef_dtype == CSR_DTYPE_F16 ? 2 : 4);
+        b.M = m;
+        return b;
+    };
+    if (p.pair_rows)
+        if (int rc = launch<D_, G>(rows_from(0, p.pair_rows), tmap, Db, status, 0, nullptr)) return rc;
+    int64_t r0 = p.pair_rows;
+    for (int k = 0; k < 2; ++k) {
+        if (p.tile_rows[k] == 0) continue;
+        const EncodeArgs b = rows_from(r0, p.tile_rows[k]);
+        int rc = launch<D_, G>(b, tmap, Db, status, 0, nullptr, p.splits[k]);
+        if (rc == kClusterLaunchRefused) rc = launch<D_, G>(b, tmap, Db, status, 0, nullptr, 1);
+        if (rc != CSR_OK) return rc;
+        r0 += p.tile_rows[k];
+    }
+    return CSR_OK;
+}
+
 template <int D_>
 int launch_d(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status) {
     switch (group_size(D_, a.N)) {
-        case 1: return launch<D_, 1>(a, tmap, Db, status, 0, nullptr);
-        case 2: return launch<D_, 2>(a, tmap, Db, status, 0, nullptr);
-        case 8: return launch<D_, 8>(a, tmap, Db, status, 0, nullptr);
-        default: return launch<D_, 4>(a, tmap, Db, status, 0, nullptr);
+        case 1: return launch_planned<D_, 1>(a, tmap, Db, status);
+        case 2: return launch_planned<D_, 2>(a, tmap, Db, status);
+        case 8: return launch_planned<D_, 8>(a, tmap, Db, status);
+        default: return launch_planned<D_, 4>(a, tmap, Db, status);
     }
 }
 
-// Few rows, one launch: clusters of CTAs share a pair of row tiles.  Picks the cluster size
-// whose modelled time per iteration (about 1.6 us per 256-atom tile swept plus about 3.5 us
-// for the exchange and the pick, over as many rounds as the device needs to hold all pairs)
-// is lowest, and returns 0 when one CTA per pair over the whole dictionary (about 1.55 us
-// per tile, measured) is no slower, or when the estimate exceeds `budget_us` (what another
-// path is expected to take).  *grid gets the CTAs to launch.
-template <int D_, int G>
-int cluster_split(int64_t M, int N, float budget_us, int* grid) {
-    const int64_t n_pairs = (M + 2 * TILE_M - 1) / (2 * TILE_M);
-    const int T = (N + TILE_N - 1) / TILE_N;
-    if (n_pairs < 1 || T < 2) return 0;
-    float best = 0.f;
-    int best_ns = 0;
-    for (int ns = 16; ns >= 2; ns >>= 1) {
-        if (ns > T) continue;
-        // one tile of rows: the exchange buffers (the unused row tile) bound the cluster size
-        if (M <= TILE_M && ns > FastSmem<D_>::kATileBytes / (2 * TILE_M * 8)) continue;
-        const int nc = max_clusters<D_, G>(ns);
-        if (nc < 1) continue;
-        const int64_t rounds = (n_pairs + nc - 1) / nc;
-        const float est = (float)rounds * (1.6f * ((T + ns - 1) / ns) + 3.5f);
-        if (best_ns == 0 || est < best) {
-            best = est;
-            best_ns = ns;
-            *grid = (int)(n_pairs < nc ? n_pairs : nc) * ns;
-        }
-    }
-    if (best_ns == 0 || best > budget_us) return 0;
-    const int64_t whole_rounds = (n_pairs + sm_count() - 1) / sm_count();
-    return (float)whole_rounds * 1.55f * T > 1.15f * best ? best_ns : 0;
-}
-
-template <int D_>
-int launch_clustered_g(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status, float budget_us,
-                       bool* done);
-
-// *done says whether the clustered launch took the job; a launch the driver refuses leaves
-// it to the other paths.
-template <int D_>
-int launch_clustered(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status, float budget_us,
-                     bool* done) {
-    const int rc = launch_clustered_g<D_>(a, tmap, Db, status, budget_us, done);
-    if (rc == kClusterLaunchRefused) {
-        *done = false;
-        return CSR_OK;
-    }
-    return rc;
-}
-
-template <int D_>
-int launch_clustered_g(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status, float budget_us,
-                       bool* done) {
-    int grid = 0, ns = 0;
-    *done = false;
-    switch (group_size(D_, a.N)) {
-        case 1:
-            if ((ns = cluster_split<D_, 1>(a.M, a.N, budget_us, &grid)) == 0) return CSR_OK;
-            *done = true;
-            return launch<D_, 1>(a, tmap, Db, status, ns, nullptr, grid);
-        case 2:
-            if ((ns = cluster_split<D_, 2>(a.M, a.N, budget_us, &grid)) == 0) return CSR_OK;
-            *done = true;
-            return launch<D_, 2>(a, tmap, Db, status, ns, nullptr, grid);
-        case 8:
-            if ((ns = cluster_split<D_, 8>(a.M, a.N, budget_us, &grid)) == 0) return CSR_OK;
-            *done = true;
-            return launch<D_, 8>(a, tmap, Db, status, ns, nullptr, grid);
-        default:
-            if ((ns = cluster_split<D_, 4>(a.M, a.N, budget_us, &grid)) == 0) return CSR_OK;
-            *done = true;
-            return launch<D_, 4>(a, tmap, Db, status, ns, nullptr, grid);
-    }
-}
-
-// Few rows: how many CTAs share a pair of row tiles (1 = the whole dictionary per CTA);
-// *per_iter_us gets the modelled time of one iteration.
-int split_count(int64_t M, int N, float* per_iter_us = nullptr) {
+// Without clusters: how many CTAs share a pair of row tiles (1 = the whole dictionary per CTA).
+int split_count(int64_t M, int N) {
     const int64_t n_pairs = (M + 2 * TILE_M - 1) / (2 * TILE_M);
     const int T = (N + TILE_N - 1) / TILE_N;
     if (n_pairs < 1 || n_pairs * 2 > sm_count() || T < 2) return 1;
@@ -1140,7 +1068,6 @@ int split_count(int64_t M, int N, float* per_iter_us = nullptr) {
     // Worth it only if an iteration's sweep over all T tiles by one CTA (about 1.55 us per
     // tile, measured) outlasts two launches (about 12 us) plus the sweep of a slice.
     const float whole = 1.55f * T, sliced = 12.f + 1.6f * ((T + ns - 1) / ns);
-    if (per_iter_us) *per_iter_us = sliced;
     return whole > 1.2f * sliced ? ns : 1;
 }
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
@@ -1237,18 +1164,7 @@ int launch_encode_fast_prepared(const EncodeArgs& a, const void* dict_bf16, uint
     if (r != CUDA_SUCCESS) return fail(CSR_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
 
     const uint16_t* Db = static_cast<const uint16_t*>(workspace);
-    // few rows: one launch of CTA clusters that share the dictionary (needs no scratch) ...
-    // (unless the launch-per-iteration split below, which can spread a pair of row tiles over more
-    // than 16 CTAs, is expected to be faster: very large dictionaries)
-    if (options().fast_split == 0) {
-        float budget = 3.0e38f;
-        if (split_scratch && split_count(a.M, a.N, &budget) <= 1) budget = 3.0e38f;
-        bool done = false;
-        const int rc = a.d == 128 ? launch_clustered<128>(a, tmap, Db, status, budget, &done)
-                                  : launch_clustered<64>(a, tmap, Db, status, budget, &done);
-        if (rc != CSR_OK || done) return rc;
-    }
-    // ... else, with scratch, a sweep launch and a pick launch per iteration
+    // no clusters wanted: with scratch, a sweep launch and a pick launch per iteration
     if (split_scratch) {
         if (a.d == 128) return run_split<128>(a, tmap, Db, status, split_scratch);
         return run_split<64>(a, tmap, Db, status, split_scratch);

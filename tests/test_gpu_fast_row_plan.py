@@ -1,0 +1,62 @@
+"""The fast encoder's plan of a call's rows (whole waves of pairs of row tiles, then single row tiles with
+one or more CTAs each): the codes are those of pairs only, bit for bit, around the sizes where the
+plan changes (one row, one tile, one tile per SM, a wave of pairs, what is left over)."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def csr():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import paper_2412_11741_b200 as m
+    return m
+
+
+def _np(t):
+    return t.contiguous().view(torch.int16).cpu().numpy()
+
+
+@pytest.mark.parametrize("d,N", [(128, 200), (128, 1024), (128, 2500), (64, 600), (64, 9000)])
+@pytest.mark.parametrize("M", [1, 127, 129, 1025, 4160, 9473, 18944, 18945, 26000, 37888, 38000, 60000])
+def test_plan_gives_the_codes_of_pairs(csr, d, N, M):
+    g = torch.Generator(device=DEV).manual_seed(M + N)
+    D = torch.nn.functional.normalize(torch.randn(N, d, device=DEV, generator=g), dim=1).contiguous()
+    X = torch.randn(M, d, device=DEV, generator=g).to(torch.bfloat16)
+    if N > 600:
+        D[N - 1], X[0] = D[5], 3.0 * D[5].to(torch.bfloat16)
+    X[M // 2] = 0.0
+    out_i = torch.full((M + 1, 3), -1, dtype=torch.int16, device=DEV).view(torch.uint16)
+    out_c = torch.full((M + 1, 3), 7.0, device=DEV)
+    csr.csr_encode_ex(D, X, 3, out_idx=out_i[:M], out_coef=out_c[:M])
+    assert csr.csr_device_status() == csr.CSR_OK
+    csr.csr_set_option("fast_split", 1)
+    try:
+        idx, coef = csr.csr_encode_ex(D, X, 3, coef_dtype=torch.float32)
+    finally:
+        csr.csr_set_option("fast_split", 0)
+    assert csr.csr_device_status() == csr.CSR_OK
+    assert np.array_equal(_np(out_i)[:M], _np(idx)) and torch.equal(out_c[:M], coef)
+    assert np.all(_np(out_i)[M] == -1) and bool((out_c[M] == 7.0).all())
+
+
+def test_single_tiles_bounded_wait_runs_out_and_recovers(csr):
+    g = torch.Generator(device=DEV).manual_seed(4)
+    D = torch.nn.functional.normalize(torch.randn(4096, 128, device=DEV, generator=g), dim=1).contiguous()
+    for M in (100, 3000, 15000):
+        X = torch.randn(M, 128, device=DEV, generator=g).to(torch.bfloat16)
+        want = csr.csr_encode_ex(D, X, 4)
+        assert csr.csr_device_status() == csr.CSR_OK
+        csr.csr_set_option("wait_limit_ns", 0)
+        try:
+            csr.csr_encode_ex(D, X, 4)
+            assert csr.csr_device_status() == csr.CSR_ERR_TIMEOUT
+        finally:
+            csr.csr_set_option("wait_limit_ns", 2_000_000_000)
+        got = csr.csr_encode_ex(D, X, 4)
+        assert csr.csr_device_status() == csr.CSR_OK
+        assert np.array_equal(_np(got[0]), _np(want[0])) and torch.equal(got[1], want[1])
