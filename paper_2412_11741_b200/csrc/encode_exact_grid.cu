@@ -49,9 +49,10 @@ struct GridSmem {
     static constexpr int kStageBytes = TILE_N * STAGE_CH * 2;
     alignas(1024) uint8_t A[2][kATileBytes];              // [high, low]
     alignas(1024) uint8_t B[kStages][kStageBytes];
-    Entry ent[2 * (2 * TILE_M)];                          // entries of the rows this CTA settles (rows x 2 slices <= 2 (127 + slices))
-    uint16_t cand[EPI / 8][CAND];
-    int n_cand[EPI / 8];
+    // of the rows settled here: the largest key, the atoms inside the band, their number
+    uint32_t top_key[TILE_M];
+    uint16_t cand[TILE_M][CAND];
+    int n_cand[TILE_M];
     uint32_t unknown[TILE_M / 32];                        // rows settled here whose candidates are not all known
     float limit[TILE_M];                                  // ... from which fp32 value on an atom can be the pick
     int found_n[TILE_M];                                  // ... and what the search of the whole dictionary found
@@ -266,7 +267,6 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
         const int q = warp & 3, half = warp >> 2;         // TMEM lane quarter, column half
         const int r_own = q * 32 + lane;                  // the row of the tile whose correlations this thread sees
         const int l8 = lane & 7, grp = lane >> 3;
-        const int group = warp * 4 + grp;
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
         const int64_t row_base = static_cast<int64_t>(tile) * TILE_M;
         const int rows_here = static_cast<int>(a.M - row_base < TILE_M ? a.M - row_base : TILE_M);   // >= 1
@@ -363,17 +363,65 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
             ok = meet(counter, target += slices, slices, ok, wc);
             if (!ok) break;
 
-            // ---- settle this CTA's rows ----
+            // ---- this CTA's rows: largest key over all slices, then what lies inside its band ----
+            // (an entry per thread and trip, at most two trips: rows x 2 slices <= 2 (127 + slices))
+            constexpr int TRIPS = 2;
+            Entry mine[TRIPS];
+            float band_of[TRIPS];
             if (threadIdx.x < TILE_M / 32) sm.unknown[threadIdx.x] = 0u;
-            for (int f = threadIdx.x; f < n_own * n_ent; f += EPI) {
-                const uint2* e = reinterpret_cast<const uint2*>(a.entries + ((row_base + slice + f / n_ent * slices) * n_ent + f % n_ent));
-                const uint2 e0 = __ldcg(e), e1 = __ldcg(e + 1), e2 = __ldcg(e + 2);
-                uint2* d = reinterpret_cast<uint2*>(&sm.ent[f]);
-                d[0] = e0;
-                d[1] = e1;
-                d[2] = e2;
+            if (threadIdx.x < TILE_M) {
+                sm.top_key[threadIdx.x] = 0u;
+                sm.n_cand[threadIdx.x] = 0;
+            }
+#pragma unroll
+            for (int u = 0; u < TRIPS; ++u) {
+                const int f = threadIdx.x + u * EPI;
+                mine[u] = Entry{{0u, 0u, 0u, 0u}, 0u, 0u};
+                band_of[u] = 0.f;
+                if (f < n_own * n_ent) {
+                    const int64_t row = row_base + slice + f / n_ent * slices;
+                    const uint2* e = reinterpret_cast<const uint2*>(a.entries + (row * n_ent + f % n_ent));
+                    const uint2 e0 = __ldcg(e), e1 = __ldcg(e + 1), e2 = __ldcg(e + 2);
+                    mine[u] = Entry{{e0.x, e0.y, e1.x, e1.y}, e2.x, e2.y};
+                    band_of[u] = __ldcg(a.band + row);
+                }
             }
             epilogue_barrier();
+#pragma unroll
+            for (int u = 0; u < TRIPS; ++u) {
+                const int f = threadIdx.x + u * EPI;
+                if (f < n_own * n_ent) atomicMax(&sm.top_key[f / n_ent], mine[u].k[0]);
+            }
+            epilogue_barrier();
+#pragma unroll
+            for (int u = 0; u < TRIPS; ++u) {
+                const int f = threadIdx.x + u * EPI;
+                if (f >= n_own * n_ent) continue;
+                const int k = f / n_ent;
+                const float v0 = __uint_as_float(sm.top_key[k] & kKeyMask), band = band_of[u];
+                if (!(v0 > 0.f) || a.N == 1 || v0 - __uint_as_float(mine[u].k[0] & kKeyMask) > band) continue;
+                // four of a half slice inside the band: there may be more; a band above everything: anything may be the pick
+                bool full = !(v0 > band) || (mine[u].k[3] != 0u && !(v0 - __uint_as_float(mine[u].k[3] & kKeyMask) > band));
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const uint32_t key = mine[u].k[i];
+                    const uint32_t n = i == 0 ? mine[u].n01 & 0xFFFFu : i == 1 ? mine[u].n01 >> 16 : mine[u].n2;
+                    if (key != 0u && !(v0 - __uint_as_float(key & kKeyMask) > band) && n < static_cast<uint32_t>(a.N)) {
+                        const int slot = atomicAdd(&sm.n_cand[k], 1);
+                        if (slot < CAND)
+                            sm.cand[k][slot] = static_cast<uint16_t>(n);
+                        else
+                            full = true;
+                    }
+                }
+                if (full) {
+                    atomicOr(&sm.unknown[k >> 5], 1u << (k & 31));
+                    sm.limit[k] = v0 - 1.5f * band;       // (every writer of a row writes the same)
+                }
+            }
+            epilogue_barrier();
+
+            // ---- settle them, rows with unknown candidates in a second round ----
 #pragma unroll 1
             for (int round = 0; round < 2; ++round) {
                 if (round == 1) {
@@ -404,57 +452,25 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                         R[2 * c + 1] = x.y;
                     }
                     const float band = __ldcg(a.band + row);
-                    const Entry* ent = &sm.ent[kk * n_ent];
-                    uint32_t kmax = 0;
-                    for (int e = l8; e < n_ent; e += 8) kmax = max(kmax, ent[e].k[0]);
-                    kmax = max(kmax, __shfl_xor_sync(FULL, kmax, 1));
-                    kmax = max(kmax, __shfl_xor_sync(FULL, kmax, 2));
-                    kmax = max(kmax, __shfl_xor_sync(FULL, kmax, 4));
-                    const float v0 = __uint_as_float(kmax & kKeyMask);
-                    const bool some = v0 > 0.f && a.N > 1;    // else: an all-zero sweep (or NaN) picks atom 0
-                    if (l8 == 0) sm.n_cand[group] = 0;
-                    __syncwarp();
-                    bool full = some && !(v0 > band);
-                    if (some) {
-                        for (int e = l8; e < n_ent; e += 8) {
-                            if (v0 - __uint_as_float(ent[e].k[0] & kKeyMask) > band) continue;
-#pragma unroll
-                            for (int i = 0; i < 3; ++i) {
-                                const uint32_t key = ent[e].k[i];
-                                const uint32_t n = i == 0 ? ent[e].n01 & 0xFFFFu : i == 1 ? ent[e].n01 >> 16 : ent[e].n2;
-                                if (key != 0u && !(v0 - __uint_as_float(key & kKeyMask) > band) && n < static_cast<uint32_t>(a.N)) {
-                                    const int slot = atomicAdd(&sm.n_cand[group], 1);
-                                    if (slot < CAND) sm.cand[group][slot] = static_cast<uint16_t>(n);
-                                }
-                            }
-                            // four of a half slice inside the band: there may be more
-                            if (ent[e].k[3] != 0u && !(v0 - __uint_as_float(ent[e].k[3] & kKeyMask) > band)) full = true;
-                        }
-                    }
-                    __syncwarp();
-                    int cnt = some ? sm.n_cand[group] : 0;
-                    full = full || cnt > CAND || (some && cnt == 0);
-                    full = ((__ballot_sync(FULL, full) >> (8 * grp)) & 0xFFu) != 0;
-                    int n = cnt > 0 ? sm.cand[group][0] : 0;
-                    if (round == 1) {                         // searched for by all warps: nothing left to decide
+                    const float v0 = __uint_as_float(sm.top_key[kk] & kKeyMask);
+                    const bool open = (sm.unknown[kk >> 5] >> (kk & 31)) & 1u;
+                    int cnt = min(sm.n_cand[kk], CAND);   // none: an all-zero sweep (or NaN, or one atom) picks atom 0
+                    int n = cnt > 0 ? sm.cand[kk][0] : 0;
+                    if (round == 1) {                     // searched for by all warps: nothing left to decide
                         n = has ? sm.found_n[kk] : 0;
-                        full = false;
                         cnt = 0;
-                    } else if (full && has) {                 // left for the second round
-                        if (l8 == 0) {
-                            atomicOr(&sm.unknown[k >> 5], 1u << (k & 31));
-                            sm.limit[k] = v0 - 1.5f * band;
-                        }
+                    } else if (open) {
                         has = false;
+                        cnt = min(cnt, 1);
                     }
-                    const bool cmp = !full && cnt > 1;        // several candidates: their fp64 correlations decide, the lowest atom among equals
+                    const bool cmp = cnt > 1;        // several candidates: their fp64 correlations decide, the lowest atom among equals
                     if (__any_sync(FULL, cmp)) {
                         const int most = static_cast<int>(__reduce_max_sync(FULL, cmp ? static_cast<unsigned>(cnt) : 0u));
                         double cbest = -1.0;
                         int nbest = n;
 #pragma unroll 1
                         for (int ci = 0; ci < most; ++ci) {
-                            const int nc = cmp ? sm.cand[group][min(ci, cnt - 1)] : n;
+                            const int nc = cmp ? sm.cand[kk][min(ci, cnt - 1)] : n;
                             float ax[CH];
                             load_atom<CH>(a.D + static_cast<int64_t>(nc) * D_, l8, ax);
                             const double cc = fabs(group8_sum(slice_dot<CH>(R, ax)));
