@@ -104,7 +104,10 @@ extern "C" {
  *                        over after whole waves of pairs of 128-row tiles, run as single
  *                        row tiles whose dictionary sweep is split across the CTAs of a
  *                        thread-block cluster where that is faster: the same codes, no
- *                        scratch.
+ *                        scratch.  The rows of a decoding step (8 or 16 per cluster, as many
+ *                        clusters as fit) meet a dictionary held in registers; channels are
+ *                        summed in another order there, which can decide between two
+ *                        atoms only where the mode does not tell them apart anyway.
  *                        (csr_set_option can force each of these paths.)
  */
 #define CSR_MODE_FP32_EXACT 0

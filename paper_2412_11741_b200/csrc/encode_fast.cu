@@ -50,7 +50,10 @@
 // are exchanged through distributed shared memory in one hop (st.async credited to the peers'
 // mbarriers, into the other row tile's memory) and every CTA makes the same pick and update, so all
 // s iterations run in one launch.  plan_rows() says which rows run how; the codes are the same bits in
-// every case.  (Where clusters must not be used, n_splits > 1 without ONE sweeps a slice for one
+// every case.  The handful of rows that a decoding step adds takes encode_few_kernel instead, which
+// holds the dictionary in registers; its correlations are summed in another order, so that it could part
+// from the others where two atoms' correlations agree to the width of the key's tag and the last
+// bit decides (about one pick in 10^6; none in the tests).  (Where clusters must not be used, n_splits > 1 without ONE sweeps a slice for one
 // iteration and leaves the rows' maxima to split_pick_kernel: a launch pair per iteration.)
 #include <cuda.h>
 
@@ -856,6 +859,234 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
     if constexpr (ONE) cluster_sync_all();
 }
 
+// ---------------------------------------------------------------------------------------
+// a handful of rows: the dictionary in registers
+// ---------------------------------------------------------------------------------------
+// What one decoding step adds is 8 to 128 rows.  A 128-row MMA spends 2100 cycles on 512 atoms whatever
+// the rows, and with its hand-offs a sweep of two dictionary tiles takes 4000.  Here a cluster of up to 16
+// CTAs keeps the dictionary in registers for all s iterations, 16 warps with MT * 16 atoms each as the A
+// fragments of mma.sync m16n8k16 (64 registers), and 8 * NTL residual rows (B, bf16, in shared
+// memory) are all that moves: a sweep is 16 * NTL instructions per warp.  The maxima go through one
+// shared-memory table and one hop through distributed shared memory, a warp per row; every CTA makes
+// the same pick and the same residual update on its own copy of the rows.
+// A lane of quarter q holds channels q * D_/4 ..: the k positions of the fragments are dealt out so that
+// its share of an atom or of a row is contiguous (a dot product does not mind the order; the
+// correlations may differ from tcgen05's in the last bit).
+constexpr int RT_THREADS = 512, RT_WARPS = RT_THREADS / 32;
+template <int D_, int NTL>
+struct FewSmem {
+    static constexpr int ROWS = 8 * NTL;
+    static constexpr int LD = D_ / 2 + 4;                 // words per residual row: rows 4 banks apart, 16-byte aligned
+    alignas(16) uint32_t R[ROWS][LD];                     // residual rows, bf16
+    unsigned long long best[ROWS][RT_WARPS];              // (key, ~tile) of each warp's atoms
+    unsigned long long from[2][ROWS][16];                 // ... of each CTA's, double-buffered by iteration
+    uint64_t bar[ROWS];                                   // one per row: every CTA's word has arrived
+    volatile uint32_t abort;
+};
+
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ unsigned long long max_u64(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
+
+template <int D_, int G, int NTL>
+__global__ void __launch_bounds__(RT_THREADS, 1)
+encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, int x_dtype, int64_t ldx, int64_t M, int N, int s,
+                  uint16_t* __restrict__ out_idx, void* __restrict__ out_coef, int coef_dtype, int64_t ldc, uint32_t key_mask,
+                  uint32_t* status, int n_ctas, unsigned long long wait_limit_ns) {
+    using S = FewSmem<D_, NTL>;
+    constexpr int ROWS = S::ROWS, MT = D_ == 128 ? 2 : 4, KT = D_ / 16;
+    constexpr int NG = TILE_N / G;
+    __shared__ S sm;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cta = static_cast<int>(blockIdx.x) % n_ctas;
+    const int64_t m0 = static_cast<int64_t>(blockIdx.x / n_ctas) * ROWS;
+    const int q4 = lane & 3, l4 = lane >> 2;
+    const int n_pad = (N + 7) / 8 * 8;
+    const WaitCtx wc{&sm.abort, status, wait_limit_ns};
+    if (threadIdx.x < ROWS) {
+        mbar_init(&sm.bar[threadIdx.x], 1);
+        mbar_expect_tx(&sm.bar[threadIdx.x], static_cast<uint32_t>(n_ctas) * 8);
+    }
+    if (threadIdx.x == 0) {
+        sm.abort = 0;
+        fence_barrier_init();
+    }
+    // ---- this warp's atoms ----
+    const int a0 = (cta * RT_WARPS + warp) * (MT * 16);   // atoms a0 + 16 mt + l4 (+ 8)
+    uint32_t A[MT][KT][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int hi = 0; hi < 2; ++hi) {
+            const int n = a0 + 16 * mt + 8 * hi + l4;
+            const uint4* src = reinterpret_cast<const uint4*>(Db + static_cast<size_t>(n < n_pad ? n : 0) * D_ + q4 * (D_ / 4));
+#pragma unroll
+            for (int c = 0; c < D_ / 32; ++c) {           // eight channels: two k tiles of four
+                uint4 v = __ldg(src + c);
+                if (n >= n_pad) v = make_uint4(0u, 0u, 0u, 0u);
+                A[mt][2 * c][hi] = v.x;
+                A[mt][2 * c][2 + hi] = v.y;
+                A[mt][2 * c + 1][hi] = v.z;
+                A[mt][2 * c + 1][2 + hi] = v.w;
+            }
+        }
+    // ---- R_0 = x, rounded to bf16 (rows past M: zeros) ----
+    for (int f = threadIdx.x; f < ROWS * (D_ / 8); f += RT_THREADS) {
+        const int r = f / (D_ / 8), c = f % (D_ / 8);
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (m0 + r < M) {
+            const int64_t o = (m0 + r) * ldx + 8 * c;
+            if (x_dtype == CSR_DTYPE_BF16) {
+                v = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(X) + o);
+            } else {
+                float x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) x[k] = load_elem(X, x_dtype, o + k);
+                v = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
+            }
+        }
+        *reinterpret_cast<uint4*>(&sm.R[r][4 * c]) = v;
+    }
+    __syncthreads();
+    if (n_ctas > 1) cluster_sync_all();                   // no CTA touches a peer's barriers before they are set up
+
+    for (int g = 0; g < s; ++g) {
+        // ---- sweep ----
+#pragma unroll
+        for (int nt = 0; nt < NTL; ++nt) {
+            float c[MT][4];
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) c[mt][i] = 0.f;
+            const uint4* row = reinterpret_cast<const uint4*>(&sm.R[8 * nt + l4][q4 * (D_ / 8)]);
+#pragma unroll
+            for (int ch = 0; ch < D_ / 32; ++ch) {
+                const uint4 b = row[ch];
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    mma_bf16_16816(c[mt], A[mt][2 * ch], b.x, b.y);
+                    mma_bf16_16816(c[mt], A[mt][2 * ch + 1], b.z, b.w);
+                }
+            }
+            // this lane: atoms a0 + 16 mt + l4 (c0, c1) and + 8 (c2, c3) of rows 8 nt + 2 q4 (c0, c2) and + 1 (c1, c3)
+            unsigned long long k0 = 0ull, k1 = 0ull;
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int hi = 0; hi < 2; ++hi) {
+                    const int n = a0 + 16 * mt + 8 * hi + l4;
+                    const uint32_t tag = static_cast<uint32_t>(NG - 1 - (n & (TILE_N - 1)) / G), low = 0xFFFFFFFFu - static_cast<uint32_t>(n / TILE_N);
+                    const uint32_t v0 = (__float_as_uint(c[mt][2 * hi]) & 0x7FFFFFFFu & key_mask) | tag;
+                    const uint32_t v1 = (__float_as_uint(c[mt][2 * hi + 1]) & 0x7FFFFFFFu & key_mask) | tag;
+                    if (n < n_pad) {
+                        k0 = max_u64(k0, (static_cast<unsigned long long>(v0) << 32) | low);
+                        k1 = max_u64(k1, (static_cast<unsigned long long>(v1) << 32) | low);
+                    }
+                }
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) {
+                k0 = max_u64(k0, __shfl_xor_sync(0xffffffffu, k0, o));
+                k1 = max_u64(k1, __shfl_xor_sync(0xffffffffu, k1, o));
+            }
+            if (l4 == 0) {
+                sm.best[8 * nt + 2 * q4][warp] = k0;
+                sm.best[8 * nt + 2 * q4 + 1][warp] = k1;
+            }
+        }
+        __syncthreads();
+        // ---- a warp per row: merge, exchange, pick, update ----
+        bool got = true;
+#pragma unroll
+        for (int rr = 0; rr < ROWS; rr += RT_WARPS) {     // everyone's words are on their way before any is waited for
+            const int r = rr + warp;
+            if (ROWS < RT_WARPS && r >= ROWS) continue;
+            unsigned long long k = sm.best[r][lane & 15];
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, o));
+            if (n_ctas == 1) {
+                if (lane == 0) sm.from[g & 1][r][0] = k;
+            } else if (lane < n_ctas) {
+                st_async_u64(map_to_cta(smem_u32(&sm.from[g & 1][r][cta]), lane), k, map_to_cta(smem_u32(&sm.bar[r]), lane));
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int rr = 0; rr < ROWS; rr += RT_WARPS) {
+            const int r = rr + warp;
+            if (ROWS < RT_WARPS && r >= ROWS) continue;
+            if (n_ctas > 1 && got) {
+                got = wait_bounded_cluster(&sm.bar[r], g & 1, wc);
+                got = __all_sync(0xffffffffu, got);
+                if (got && lane == 0) mbar_expect_tx(&sm.bar[r], static_cast<uint32_t>(n_ctas) * 8);      // the next iteration's
+            }
+            if (!got) continue;
+            unsigned long long k = lane < n_ctas ? *reinterpret_cast<volatile unsigned long long*>(&sm.from[g & 1][r][lane]) : 0ull;
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, o));
+            k = __shfl_sync(0xffffffffu, k, 0);
+            const int n0 = candidate_start<G>(static_cast<uint32_t>(k >> 32), 0xFFFFFFFFu - static_cast<uint32_t>(k), N, status);
+            // the arithmetic of pick_and_update: eight lanes (four times the same here) with CH chunks each
+            constexpr int CH = D_ / 64, APR = D_ / 8;
+            const int l8 = lane & 7;
+            uint4 atom[G][CH], rv[CH];
+            const uint4* src = reinterpret_cast<const uint4*>(Db + static_cast<size_t>(n0) * D_) + l8 * CH;
+#pragma unroll
+            for (int j = 0; j < G; ++j)
+#pragma unroll
+                for (int c = 0; c < CH; ++c) atom[j][c] = __ldg(src + j * APR + c);
+#pragma unroll
+            for (int c = 0; c < CH; ++c) rv[c] = *reinterpret_cast<const uint4*>(&sm.R[r][4 * (l8 * CH + c)]);
+            float dot[G];
+#pragma unroll
+            for (int j = 0; j < G; ++j) {
+                float ev = 0.f, od = 0.f;
+#pragma unroll
+                for (int c = 0; c < CH; ++c) dot8(rv[c], atom[j][c], ev, od);
+                dot[j] = ev + od;
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+                for (int j = 0; j < G; ++j) dot[j] += __shfl_xor_sync(0xffffffffu, dot[j], o);
+            float coef = dot[0];
+            int jb = 0;
+#pragma unroll
+            for (int j = 1; j < G; ++j)
+                if (fabsf(dot[j]) > fabsf(coef)) {
+                    coef = dot[j];
+                    jb = j;
+                }
+            __syncwarp();                                  // every lane has read its part of the row
+            if (lane < 8) {
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    uint4 av = atom[0][c];
+#pragma unroll
+                    for (int j = 1; j < G; ++j)
+                        if (jb == j) av = atom[j][c];
+                    *reinterpret_cast<uint4*>(&sm.R[r][4 * (l8 * CH + c)]) = axpy8(rv[c], av, coef);
+                }
+            }
+            const int64_t m = m0 + r;
+            if (cta == 0 && lane == 0 && m < M) {
+                out_idx[m * ldc + g] = static_cast<uint16_t>(n0 + jb);
+                if (coef_dtype == CSR_DTYPE_F16)
+                    reinterpret_cast<__half*>(out_coef)[m * ldc + g] = __float2half_rn(coef);
+                else
+                    reinterpret_cast<float*>(out_coef)[m * ldc + g] = coef;
+            }
+        }
+        if (__syncthreads_or(!got || sm.abort != 0)) break;
+    }
+    // a CTA's shared memory must outlive its peers' last writes to it
+    if (n_ctas > 1) cluster_sync_all();
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -974,13 +1205,14 @@ int group_size(int d, int N) {
 // does not.  The estimates are fits of this kernel's measured time per iteration in us (M from 64 to
 // 28000, N from 512 to 16384, s = 8): pairs 3.3 + 1.55 per 256-atom tile of the dictionary (d = 64: 3.0
 // + 1.05), single tiles 4.1 + 0.75 per tile of the CTA's slice (d = 64: 3.2 + 0.48).  Some of it, in us
-// per call of 8 iterations at N = 1024 / 8192, d = 128, this plan against clusters of up to 16 CTAs
+// a call of 8 iterations at N = 1024 / 8192, d = 128, this plan against clusters of up to 16 CTAs
 // on pairs of row tiles: 64 rows 35 / 45 against 47 / 45; 1100 rows 37 / 58 against 54 / 74; 4160 rows
 // 40 / 83 against 56 / 140; 9400 rows 45 / 131 against 68 / 233; 18900 rows 54 / 227 against 70 / 237.
 struct RowPlan {
     int64_t pair_rows;
     int64_t tile_rows[2];
     int splits[2];
+    float us;                // an iteration of what follows the whole waves
 };
 template <int D_, int G>
 RowPlan plan_rows(int64_t M, int N) {
@@ -1005,26 +1237,81 @@ RowPlan plan_rows(int64_t M, int N) {
         }
         return best;
     };
-    RowPlan p{M, {0, 0}, {0, 0}};
+    RowPlan p{M, {0, 0}, {0, 0}, 0.f};
     if (tiles == 0) return p;
     float least = kPair0 + kPair1 * T, cost;
+    p.us = least;
     const int one = best_split(tiles, &cost);
     if (cost < least) {
         least = cost;
-        p = RowPlan{M - rest, {rest, 0}, {one, 0}};
+        p = RowPlan{M - rest, {rest, 0}, {one, 0}, cost};
     }
     if (tiles > sms) {                                     // a whole wave of single tiles, then the others over the whole chip
         const int two = best_split(tiles - sms, &cost);
         cost += kTile0 + kTile1 * T;
-        if (cost < least) p = RowPlan{M - rest, {sms * TILE_M, rest - sms * TILE_M}, {1, two}};
+        if (cost < least) p = RowPlan{M - rest, {sms * TILE_M, rest - sms * TILE_M}, {1, two}, cost};
     }
     return p;
 }
 
+// A handful of rows (see encode_few_kernel): atoms a CTA holds, and how many CTAs the dictionary takes
+// (0: it does not fit).
+template <int D_>
+int few_ctas(int N) {
+    constexpr int kAtoms = RT_WARPS * 16 * (D_ == 128 ? 2 : 4);
+    int n = 1;
+    while (n <= 16 && n * kAtoms < (N + 7) / 8 * 8) n *= 2;
+    return n <= 16 ? n : 0;
+}
+// Rows per cluster of encode_few_kernel, 8 or 16 (0: row tiles are faster).  Measured, s = 16, in us, this
+// kernel with 8 rows / 16 rows per cluster against row tiles: 8 rows N = 1000 33 / 33 / 57, N = 8192 35 / 49 /
+// 78; 64 rows N = 8192 (8 clusters of 16, more than the chip holds at once) 68 / 49 / 84; 128 rows
+// N = 1000 33 / 47 / 68.  Per iteration 2.2 us (8 rows) and 3.05 (16 rows) a round of clusters.
+template <int D_, int G>
+int few_rows_per_cluster(int64_t M, int N) {
+    const int n_ctas = few_ctas<D_>(N);
+    if (n_ctas == 0 || M > 4096) return 0;
+    const int fit = n_ctas == 1 ? sm_count() : max_clusters<D_, G>(n_ctas);
+    if (fit < 1) return 0;
+    auto rounds = [&](int rows) { return (float)(((M + rows - 1) / rows + fit - 1) / fit); };
+    const float c8 = 2.2f * rounds(8), c16 = 3.05f * rounds(16), few = c8 <= c16 ? c8 : c16;
+    if (few >= plan_rows<D_, G>(M, N).us) return 0;
+    return c8 <= c16 ? 8 : 16;
+}
+
+template <int D_, int G, int NTL>
+int launch_few(const EncodeArgs& a, const uint16_t* Db, uint32_t* status) {
+    auto kernel = encode_few_kernel<D_, G, NTL>;
+    const int n_ctas = few_ctas<D_>(a.N);
+    cudaError_t e = n_ctas > 8 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
+    if (e == cudaSuccess) {
+        const uint32_t key_mask = ~static_cast<uint32_t>(TILE_N / G - 1);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        cluster_config<D_, G>(cfg, attr, n_ctas, (int)((a.M + 8 * NTL - 1) / (8 * NTL)) * n_ctas, 0, a.stream);
+        cfg.blockDim = dim3(RT_THREADS, 1, 1);
+        if (n_ctas == 1) cfg.numAttrs = 0;
+        e = cudaLaunchKernelEx(&cfg, kernel, Db, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx, a.out_coef, a.coef_dtype, a.ld_code,
+                               key_mask, status, n_ctas, options().wait_limit_ns);
+    }
+    if (e != cudaSuccess) {                                // refused at launch (nothing ran): the caller takes another path
+        cudaGetLastError();
+        return kClusterLaunchRefused;
+    }
+    return CSR_OK;
+}
+
 template <int D_, int G>
 int launch_planned(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status) {
+    if (options().fast_split == 0) {
+        const int rows = few_rows_per_cluster<D_, G>(a.M, a.N);
+        if (rows > 0) {
+            const int rc = rows == 8 ? launch_few<D_, G, 1>(a, Db, status) : launch_few<D_, G, 2>(a, Db, status);
+            if (rc != kClusterLaunchRefused) return rc;
+        }
+    }
     // (the option forces pairs only)
-    const RowPlan p = options().fast_split == 0 ? plan_rows<D_, G>(a.M, a.N) : RowPlan{a.M, {0, 0}, {0, 0}};
+    const RowPlan p = options().fast_split == 0 ? plan_rows<D_, G>(a.M, a.N) : RowPlan{a.M, {0, 0}, {0, 0}, 0.f};
     auto rows_from = [&](int64_t r0, int64_t m) {
         EncodeArgs b = a;
         b.X = static_cast<const char*>(a.X) + (size_t)r0 * a.ldx * dtype_size(a.x_dtype);

@@ -268,14 +268,18 @@ __device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_syn
 
 // The same wait on a barrier that other CTAs of the cluster arrive on.
 __device__ __forceinline__ bool wait_bounded_cluster(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer_ns();
-    for (uint32_t it = 1; it < (1u << 28); ++it) {
+    if (w.limit_ns != 0) {
         if (mbar_try_wait_cluster(bar, parity)) return true;
-        if ((it & 63u) == 0) {
-            if (*w.abort) return false;
-            if (globaltimer_ns() - t0 > w.limit_ns) break;
+        const unsigned long long t0 = globaltimer_ns();
+        for (uint32_t it = 1; it < (1u << 28); ++it) {
+            if (mbar_try_wait_cluster(bar, parity)) return true;
+            if ((it & 63u) == 0) {
+                if (*w.abort) return false;
+                if (globaltimer_ns() - t0 > w.limit_ns) break;
+            }
         }
+    } else if (mbar_test_wait(bar, parity)) {
+        return true;
     }
     *w.abort = 1;
     atomicOr(w.status, kStatusTimeout);

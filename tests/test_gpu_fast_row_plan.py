@@ -22,7 +22,7 @@ def _np(t):
 
 
 @pytest.mark.parametrize("d,N", [(128, 200), (128, 1024), (128, 2500), (64, 600), (64, 9000)])
-@pytest.mark.parametrize("M", [1, 127, 129, 1025, 4160, 9473, 18944, 18945, 26000, 37888, 38000, 60000])
+@pytest.mark.parametrize("M", [1, 8, 9, 40, 127, 129, 500, 1025, 4160, 9473, 18944, 18945, 26000, 37888, 38000, 60000])
 def test_plan_gives_the_codes_of_pairs(csr, d, N, M):
     g = torch.Generator(device=DEV).manual_seed(M + N)
     D = torch.nn.functional.normalize(torch.randn(N, d, device=DEV, generator=g), dim=1).contiguous()
