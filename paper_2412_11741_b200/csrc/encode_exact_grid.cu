@@ -95,8 +95,8 @@ __device__ __forceinline__ bool meet(uint32_t* counter, uint32_t target, int sli
     if (epilogue_barrier_any(!ok || *w.abort != 0)) return false;
     if (slices > 1) {
         if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(counter, 1u);
+            // (release: what the CTA's other threads wrote before the barrier above goes with it)
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
             uint32_t seen;
             unsigned long long t0 = 0;
             bool in = false;
@@ -117,7 +117,6 @@ __device__ __forceinline__ bool meet(uint32_t* counter, uint32_t target, int sli
                 *w.abort = 1;
                 atomicOr(w.status, kStatusTimeout);
             }
-            __threadfence();
         }
         if (epilogue_barrier_any(*w.abort != 0)) return false;
     }

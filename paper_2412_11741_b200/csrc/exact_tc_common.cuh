@@ -65,24 +65,26 @@ struct Top4Thr {
 };
 static __device__ __noinline__ Top4Thr insert_group(Top4 q, float thr, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, uint32_t v4,
                                                     uint32_t v5, uint32_t v6, uint32_t v7, uint32_t tag, uint32_t id, float band) {
-    float a[8] = {fabsf(__uint_as_float(v0)), fabsf(__uint_as_float(v1)), fabsf(__uint_as_float(v2)), fabsf(__uint_as_float(v3)),
-                  fabsf(__uint_as_float(v4)), fabsf(__uint_as_float(v5)), fabsf(__uint_as_float(v6)), fabsf(__uint_as_float(v7))};
+    // Keys whose last three bits are the place in the group (a lower column wins among equals); the
+    // chains are kept short: a call is waited for, two warps per scheduler cannot cover it.
+    uint32_t k[8] = {v0, v1, v2, v3, v4, v5, v6, v7};
+#pragma unroll
+    for (int j = 0; j < 8; ++j) k[j] = (k[j] & kKeyMask) | static_cast<uint32_t>(7 - j);
+    const uint32_t rest = tag - 7u;                       // tags of a group are consecutive, the last a multiple of eight
 #pragma unroll 1
     for (int trip = 0; trip < 8; ++trip) {
-        const float gm = absmax3(absmax3(a[0], a[1], a[2]), absmax3(a[3], a[4], a[5]), fmaxf(a[6], a[7]));
-        if (!(gm >= thr)) break;
-        uint32_t pos = 7u;                                // of the largest magnitude left (the lowest column among equals)
-#pragma unroll
-        for (int j = 6; j >= 0; --j) pos = a[j] == gm ? static_cast<uint32_t>(j) : pos;
-        const uint32_t key = (__float_as_uint(gm) & kKeyMask) | (tag - pos);
-        if (gm > __uint_as_float(q.k0 & kKeyMask) + band)
+        const uint32_t a = __vimax3_u32(k[0], k[1], k[2]), b = __vimax3_u32(k[3], k[4], k[5]);
+        const uint32_t best = max(__vimax3_u32(k[6], k[7], a), b);
+        const float val = __uint_as_float(best & kKeyMask);
+        if (!(val >= thr)) break;
+        const uint32_t key = best | rest;
+        if (val > __uint_as_float(q.k0 & kKeyMask) + band)
             q = Top4{key, 0u, 0u, 0u, id, 0u, 0u};
         else
             top4_insert(q, key, id);
         thr = __uint_as_float(q.k0 & kKeyMask) - band;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) a[j] = pos == static_cast<uint32_t>(j) ? 0.f : a[j];
-        if (!(thr > 0.f)) thr = fmaxf(thr, 1e-45f);       // (a spent value is not seen again)
+        for (int j = 0; j < 8; ++j) k[j] = k[j] == best ? 0u : k[j];
     }
     return Top4Thr{q, thr};
 }
