@@ -54,7 +54,7 @@ struct GridSmem {
     uint16_t cand[TILE_M][CAND];
     int n_cand[TILE_M];
     uint32_t unknown[TILE_M / 32];                        // rows settled here whose candidates are not all known
-    float limit[TILE_M];                                  // ... from which fp32 value on an atom can be the pick
+    float limit[TILE_M];                                  // ... from which |correlation| / ||R|| on an atom can be the pick
     int found_n[TILE_M];                                  // ... and what the search of the whole dictionary found
     Rescored found[EPI / 32];
     uint64_t full_b[kStages];
@@ -78,9 +78,9 @@ struct GridArgs {
     int coef_dtype;
     int64_t ldc;
     double* Rd;             // [tiles * 128][d] fp64 residual rows
-    uint32_t* Rh;           // [tiles * 128][d / 2] bf16 high parts, two channels per word
+    uint32_t* Rh;           // [tiles * 128][d / 2] bf16 high parts of the scaled rows, two channels per word
     uint32_t* Rl;           // low parts
-    float* band;            // [tiles * 128]
+    float* band;            // [tiles * 128] of the scaled rows
     Entry* entries;         // [tiles][128][2 * slices]
     uint32_t* counters;     // [tiles * 32], zero at launch
     int slices;
@@ -276,26 +276,22 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
         uint32_t target = 0;
         bool ok = true;
         uint32_t accn = 0;
-        // An fp64 row, its parts and its band to the scratch arrays, by the eight lanes of a row (all lanes
+        // An fp64 row, the parts of its scaled form and its band to the scratch arrays, by the eight lanes of a row (all lanes
         // of the warp call; only those with `has` write).
         auto put_row = [&](const double (&R)[CH], int64_t row, bool has) {
-            double n0 = 0.0, n1 = 0.0;
-#pragma unroll
-            for (int k = 0; k < CH / 2; ++k) {
-                n0 = fma(R[2 * k], R[2 * k], n0);
-                n1 = fma(R[2 * k + 1], R[2 * k + 1], n1);
-            }
-            const double nn = group8_sum(n0 + n1);
+            const double nn = group8_sum(norm2_share<CH>(R));
             if (!has) return;
+            float band;
+            const double scale = row_scale(nn, band);
 #pragma unroll
             for (int k = 0; k < CH / 2; ++k) {
                 uint32_t hi, lo;
-                split_pair(R[2 * k], R[2 * k + 1], hi, lo);
+                split_pair(R[2 * k] * scale, R[2 * k + 1] * scale, hi, lo);
                 __stcg(reinterpret_cast<double2*>(a.Rd + row * D_) + 8 * k + l8, make_double2(R[2 * k], R[2 * k + 1]));
                 __stcg(a.Rh + row * (D_ / 2) + 8 * k + l8, hi);
                 __stcg(a.Rl + row * (D_ / 2) + 8 * k + l8, lo);
             }
-            if (l8 == 0) __stcg(a.band + row, kBandRel * sqrtf(static_cast<float>(nn)) * 1.001f);
+            if (l8 == 0) __stcg(a.band + row, band);
         };
         // ---- R_0 = x ----
         for (int k0 = 0; k0 < n_own; k0 += EPI / 8) {
@@ -415,7 +411,7 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                 }
                 if (full) {
                     atomicOr(&sm.unknown[k >> 5], 1u << (k & 31));
-                    sm.limit[k] = v0 - 1.5f * band;       // (every writer of a row writes the same)
+                    sm.limit[k] = relative_limit(v0, band);   // (every writer of a row writes the same)
                 }
             }
             epilogue_barrier();
@@ -484,8 +480,9 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                     load_atom<CH>(a.D + static_cast<int64_t>(n) * D_, l8, at);
                     const double c = group8_sum(slice_dot<CH>(R, at));
 #ifdef CSR_DEBUG_CHECKS
-                    if (l8 == 0 && has && cnt == 1 && band > 0.f)   // as in encode_exact_tc.cu
-                        atomicMax(a.diag, __float_as_uint(fabsf(v0 - static_cast<float>(fabs(c))) / (band / kBandRel)));
+                    const double nr = sqrt(group8_sum(norm2_share<CH>(R)));   // as in encode_exact_tc.cu
+                    if (l8 == 0 && has && cnt == 1 && band > 0.f)
+                        atomicMax(a.diag, __float_as_uint(fabsf(v0 / (band / (kBandRel * 1.001f)) - static_cast<float>(fabs(c) / nr))));
 #endif
                     if (l8 == 0 && has) {
                         a.out_idx[row * a.ldc + g] = static_cast<uint16_t>(n);

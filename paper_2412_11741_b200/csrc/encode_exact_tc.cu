@@ -10,8 +10,8 @@
 //
 // One persistent CTA per SM owns two tiles of 128 rows for all s iterations:
 //   - the fp64 residuals live in a per-CTA scratch area in global memory (256 KB, L2 resident);
-//     their bf16 high and low parts are the tcgen05.mma A operands in shared memory (K-major,
-//     128-byte swizzle, 2 row tiles x 2 parts);
+//     the bf16 high and low parts of the row, scaled by a power of two to a norm in [1, 2), are the
+//     tcgen05.mma A operands in shared memory (K-major, 128-byte swizzle, 2 row tiles x 2 parts);
 //   - the dictionary's high and low parts (two bf16 arrays made once per call) stream through a
 //     ring of 32 KB stages fetched by TMA: 64 channels of 256 atoms of one part per stage.  A
 //     stage of high parts feeds four groups of MMAs (both parts of both row tiles), a stage of low
@@ -248,10 +248,11 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
 #pragma unroll
                     for (int k = 0; k < CH; ++k) R[k] = 0.0;
                 }
-                double nn = store_residual<CH>(R, Rd_cta + static_cast<int64_t>(own_tile * TILE_M + r) * D_, Ahi, Alo, r, l8);
-                nn = group8_sum(nn);
-                const float nn_o = static_cast<float>(__shfl_sync(FULL, nn, (lane & 3) * 8));
-                if ((lane >> 2) == p) band = kBandRel * sqrtf(nn_o) * 1.001f;
+                float b;
+                const double scale = row_scale(group8_sum(norm2_share<CH>(R)), b);
+                store_residual<CH>(R, scale, Rd_cta + static_cast<int64_t>(own_tile * TILE_M + r) * D_, Ahi, Alo, r, l8);
+                const float b_o = __shfl_sync(FULL, b, (lane & 3) * 8);
+                if ((lane >> 2) == p) band = b_o;
             }
             fence_proxy_async_smem();
             mbar_arrive(&sm.res_ready);
@@ -366,7 +367,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                         float* limit = reinterpret_cast<float*>(lists + 8);
                         Rescored* found = reinterpret_cast<Rescored*>(lists + 8 + ROWS);
                         if (lane == 0) lists[warp] = unknown;
-                        if (my_flags & 64) limit[warp * 32 + lane] = v0 - 1.5f * band;
+                        if (my_flags & 64) limit[warp * 32 + lane] = relative_limit(v0, band);
                         if (!epilogue_barrier_any(unknown != 0)) break;
 #pragma unroll 1
                         for (int w = 0; w < 8; ++w)
@@ -430,8 +431,9 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
 #ifdef CSR_DEBUG_CHECKS
                         {   // largest |tensor-core value - fp64 value| / ||R|| seen, as float bits
                             const float vbo = __shfl_sync(FULL, v0, src), bo = __shfl_sync(FULL, band, src);
+                            const double nr = sqrt(group8_sum(norm2_share<CH>(R)));
                             if (l8 == 0 && m < M && has && round == 0 && (flags & (flags - 1)) == 0 && bo > 0.f) {
-                                const float rel = fabsf(vbo - static_cast<float>(fabs(c))) / (bo / kBandRel);
+                                const float rel = fabsf(vbo / (bo / (kBandRel * 1.001f)) - static_cast<float>(fabs(c) / nr));
                                 atomicMax(diag, __float_as_uint(rel));
                             }
                         }
@@ -445,15 +447,15 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                                 reinterpret_cast<float*>(out_coef)[m * ldc + g] = cf;
                         }
                         if (g + 1 < s) {
-                            double nn = 0.0;
                             if (has) {
 #pragma unroll
                                 for (int k = 0; k < CH; ++k) R[k] = fma(-c, static_cast<double>(a[k]), R[k]);
-                                nn = store_residual<CH>(R, Rrow, Ahi, Alo, r, l8);
                             }
-                            nn = group8_sum(nn);
-                            const float nn_o = static_cast<float>(__shfl_sync(FULL, nn, (lane & 3) * 8));
-                            if ((lane >> 2) == p && ((todo >> lane) & 1u)) band = kBandRel * sqrtf(nn_o) * 1.001f;
+                            float b;
+                            const double scale = row_scale(group8_sum(norm2_share<CH>(R)), b);
+                            if (has) store_residual<CH>(R, scale, Rrow, Ahi, Alo, r, l8);
+                            const float b_o = __shfl_sync(FULL, b, (lane & 3) * 8);
+                            if ((lane >> 2) == p && ((todo >> lane) & 1u)) band = b_o;
                         }
                         n = n_nx;
                         flags = flags_nx;

@@ -234,25 +234,48 @@ __device__ __forceinline__ void split_pair(double r0, double r1, uint32_t& hi, u
     lo = static_cast<uint32_t>(__bfloat16_as_ushort(l0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(l1)) << 16);
 }
 
-// Writes this lane's CH residual values: fp64 to the scratch row (`row`: its first element), bf16
-// high and low parts into the operand tiles.  Returns the lane's share of ||R||^2.
+// This lane's share of ||R||^2.
 template <int CH>
-__device__ __forceinline__ double store_residual(const double (&R)[CH], double* __restrict__ row, uint8_t* Ahi, uint8_t* Alo,
-                                                 int r, int l8) {
+__device__ __forceinline__ double norm2_share(const double (&R)[CH]) {
     double n0 = 0.0, n1 = 0.0;
 #pragma unroll
     for (int k = 0; k < CH / 2; ++k) {
-        reinterpret_cast<double2*>(row)[8 * k + l8] = make_double2(R[2 * k], R[2 * k + 1]);
         n0 = fma(R[2 * k], R[2 * k], n0);
         n1 = fma(R[2 * k + 1], R[2 * k + 1], n1);
+    }
+    return n0 + n1;
+}
+
+// What a row is multiplied by before it is split into parts, from its ||R||^2: the power of two that brings
+// ||R|| into [1, 2), so that the parts, the sweep's values and the band keep their precision at any
+// norm (the keys of a sweep are only compared with one another and with the band, all in the same
+// unit, and a power of two leaves every bit of them as it is).  `band` gets the undecided zone in that
+// unit: 0 for a row of zeros; Inf or NaN, and no scaling, for a row that is not finite.
+__device__ __forceinline__ double row_scale(double nn, float& band) {
+    const int e = (__double2hiint(nn) >> 20) & 0x7FF;
+    const double scale = e == 0 || e == 0x7FF ? 1.0 : __hiloint2double((1023 - ((e - 1023) >> 1)) << 20, 0);
+    band = e == 0 ? 0.f : kBandRel * sqrtf(static_cast<float>(nn * scale * scale)) * 1.001f;
+    return scale;
+}
+// From which |correlation| on, relative to ||R||, an atom can be the pick, for a sweep whose largest value was `v0`
+// (both in the sweep's unit): that value less the band, and half a band for the search's fp32 rounding.
+__device__ __forceinline__ float relative_limit(float v0, float band) { return (v0 - 1.5f * band) * (kBandRel * 1.001f / band); }
+
+// Writes this lane's CH residual values: fp64 to the scratch row (`row`: its first element), bf16 high and
+// low parts of `scale` times them into the operand tiles.
+template <int CH>
+__device__ __forceinline__ void store_residual(const double (&R)[CH], double scale, double* __restrict__ row, uint8_t* Ahi, uint8_t* Alo,
+                                               int r, int l8) {
+#pragma unroll
+    for (int k = 0; k < CH / 2; ++k) {
+        reinterpret_cast<double2*>(row)[8 * k + l8] = make_double2(R[2 * k], R[2 * k + 1]);
         uint32_t hi, lo;
-        split_pair(R[2 * k], R[2 * k + 1], hi, lo);
+        split_pair(R[2 * k] * scale, R[2 * k + 1] * scale, hi, lo);
         // channels 2 (8 k + l8), +1: 16-byte chunk 2 k + l8 / 4 of the row, word l8 % 4 of it
         const uint32_t off = swz_off(r, 2 * k + (l8 >> 2)) + (l8 & 3) * 4;
         *reinterpret_cast<uint32_t*>(Ahi + off) = hi;
         *reinterpret_cast<uint32_t*>(Alo + off) = lo;
     }
-    return n0 + n1;
 }
 
 // Elements `off` and `off + 1` of X widened to fp64.
@@ -276,9 +299,9 @@ __device__ __forceinline__ void load_x2(const void* X, int x_dtype, int64_t off,
 
 // Arg-max of |R . d_n| over the atoms [n0, n1) for one row, by one warp (all lanes call): its share
 // of a row that has more atoms inside the band than the sweep kept track of.  The true arg-max has
-// an fp32 value of at least `thresh` (the tensor-core maximum less the band and the fp32
-// rounding), so an fp32 pass collects those atoms, one per lane, and their fp64 correlations
-// decide, the lowest atom among equal values.  More than 32 candidates (copies of one atom): every
+// an fp32 value of at least `thresh` times ||R|| (see relative_limit), so an fp32 pass over the row
+// divided by its norm collects those atoms, one per lane, and their fp64 correlations decide, the
+// lowest atom among equal values.  More than 32 candidates (copies of one atom): every
 // atom is scored in fp64.  Returns the value (negative: no candidate) and the atom in `bn`.
 // The pass is bound by the latency of the atoms' loads, 16 atoms at a time, eight lanes each.
 template <int D_>
@@ -286,12 +309,19 @@ static __device__ __noinline__ double rescore_part(const float* __restrict__ D, 
                                                    int* bn) {
     constexpr int QV = D_ / 32;                           // 16-byte loads per lane and atom
     const int l8 = lane & 7, grp = lane >> 3;
+    double nn = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4 * QV; ++k) {
+        const double r = __ldcg(Rrow + ((k >> 2) * 8 + l8) * 4 + (k & 3));
+        nn = fma(r, r, nn);
+    }
+    const double inv = 1.0 / sqrt(group8_sum(nn));
     float4 rf[QV];
 #pragma unroll
     for (int k = 0; k < QV; ++k) {
         const double* r = Rrow + (8 * k + l8) * 4;
-        rf[k] = make_float4(static_cast<float>(__ldcg(r)), static_cast<float>(__ldcg(r + 1)), static_cast<float>(__ldcg(r + 2)),
-                            static_cast<float>(__ldcg(r + 3)));
+        rf[k] = make_float4(static_cast<float>(__ldcg(r) * inv), static_cast<float>(__ldcg(r + 1) * inv),
+                            static_cast<float>(__ldcg(r + 2) * inv), static_cast<float>(__ldcg(r + 3) * inv));
     }
     int mine = 0, count = 0;
 #pragma unroll 1
