@@ -46,7 +46,9 @@ template <int HGP>
 __host__ __device__ constexpr int ctas_per_sm() {
     return HGP <= 2 ? 2 : 1;
 }
-constexpr float kNegInf = -INFINITY;
+// Where a row's running maximum starts: finite, so that exp(score - maximum) adds nothing for a score of -Inf and
+// NaN for one of NaN (from -Inf on, fmaxf and the difference would lose a NaN that came first).
+constexpr float kLowest = -3.402823466e38f;
 
 __device__ __forceinline__ float load_coef(const void* coef, int coef_dtype, int64_t off) {
     return coef_dtype == CSR_DTYPE_F16 ? __half2float(reinterpret_cast<const __half*>(coef)[off])
@@ -551,7 +553,7 @@ key_scores_kernel(const float* P, int N, int H, const uint16_t* __restrict__ idx
             if constexpr (STATS) {
 #pragma unroll
                 for (int h = 0; h < HGP; ++h) {
-                    m[h] = kNegInf;
+                    m[h] = kLowest;
                     l[h] = 0.f;
                 }
             }
@@ -595,8 +597,7 @@ key_scores_kernel(const float* P, int N, int H, const uint16_t* __restrict__ idx
 #pragma unroll
                 for (int h = 0; h < HGP; ++h) {
                     const float mn = fmaxf(m[h], acc[h]);
-                    // (-inf - -inf would be NaN: a row's -inf entries add nothing to its sum)
-                    l[h] = mn == kNegInf ? l[h] : l[h] * __expf(m[h] - mn) + __expf(acc[h] - mn);
+                    l[h] = l[h] * __expf(m[h] - mn) + __expf(acc[h] - mn);
                     m[h] = mn;
                 }
             }
@@ -614,16 +615,16 @@ key_scores_kernel(const float* P, int N, int H, const uint16_t* __restrict__ idx
                 for (int h = 0; h < HGP; ++h) {
                     float mw = m[h];
                     for (int o = 16; o; o >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o));
-                    float lw = mw == kNegInf ? l[h] : l[h] * __expf(m[h] - mw);
+                    float lw = l[h] * __expf(m[h] - mw);
                     for (int o = 16; o; o >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o);
                     if ((threadIdx.x & 31) == 0) red[warp][h] = make_float2(mw, lw);
                 }
                 __syncthreads();
                 if (threadIdx.x < HGP) {
                     const int h = threadIdx.x;
-                    float mx = kNegInf, sum = 0.f;
+                    float mx = kLowest, sum = 0.f;
                     for (int q = 0; q < NTHR / 32; ++q) mx = fmaxf(mx, red[q][h].x);
-                    for (int q = 0; q < NTHR / 32; ++q) sum += mx == kNegInf ? red[q][h].y : red[q][h].y * __expf(red[q][h].x - mx);
+                    for (int q = 0; q < NTHR / 32; ++q) sum += red[q][h].y * __expf(red[q][h].x - mx);
                     const int slot = blockIdx.x - rg.owner(bg * rg.chunks);
                     st.ml[(bg * st.slots + slot) * HGP + h] = make_float2(mx, sum);
                 }
@@ -712,9 +713,9 @@ value_scatter_kernel(int N, float* W, int B, int H, const uint16_t* __restrict__
             if (threadIdx.x < HGP) {                       // (a handful of slots: one thread per head)
                 const int slots = rg.owner((bg + 1) * rg.chunks - 1) - rg.owner(bg * rg.chunks) + 1;
                 const float2* ml = st.ml + bg * st.slots * HGP + threadIdx.x;
-                float mx = kNegInf, sum = 0.f;
+                float mx = kLowest, sum = 0.f;
                 for (int q = 0; q < slots; ++q) mx = fmaxf(mx, ml[q * HGP].x);
-                for (int q = 0; q < slots; ++q) sum += mx == kNegInf ? ml[q * HGP].y : ml[q * HGP].y * __expf(ml[q * HGP].x - mx);
+                for (int q = 0; q < slots; ++q) sum += ml[q * HGP].y * __expf(ml[q * HGP].x - mx);
                 row_max[threadIdx.x] = mx;
                 row_inv[threadIdx.x] = 1.0f / sum;
             }

@@ -101,3 +101,20 @@ def test_overlapped_launches_in_a_cuda_graph(csr):
             torch.cuda.synchronize()
             assert torch.equal(out, o) and torch.equal(w, ww)
     del graph
+
+
+@pytest.mark.parametrize("T,at", [(2, 0), (900, 0), (900, 512), (900, 700), (4099, 3071)])
+@pytest.mark.parametrize("B,H,s", [(3, 4, 8), (40, 2, 6)])
+def test_one_nan_or_infinite_score_is_softmaxed_like_any_other(csr, B, H, s, T, at):
+    """One token's key coefficient is NaN, another stream's is infinite (scores of +Inf and -Inf, by the sign of q . d):
+    the weights are NaN where the softmax of the scores is, wherever in the row the token stands."""
+    Dk, Dv, Q, (ki, kc), (vi, vc) = _inputs(B, H, T, 300, 200, 64, s, s, torch.float32, torch.float16)
+    kc[0, at, 1], kc[2, at, 3] = float("nan"), float("inf")
+    out, w = csr.csr_decode_attention(Dk, Dv, Q, ki, kc, vi, vc, 0.125)
+    scores = csr.csr_key_scores(Dk, Q, ki, kc, 0.125)
+    assert bool(scores[0, :, at].isnan().all()) and bool(scores[2, :, at].isinf().all()) and not bool(scores[1].isnan().any())
+    want = torch.softmax(scores.double(), -1)
+    assert bool(w[0].isnan().all()) and bool(out[0].isnan().all())
+    assert torch.equal(w.isnan(), want.isnan())
+    # the exponentials' few ulp, and their arguments' rounding
+    torch.testing.assert_close(w.double(), want, rtol=2e-5, atol=1e-30, equal_nan=True)
