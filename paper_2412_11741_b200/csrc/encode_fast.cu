@@ -487,6 +487,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
     const uint32_t tmem_base = sm.tmem_base;
     // no CTA touches a peer's barrier or words before every peer has set them up
     if constexpr (ONE) cluster_sync_all();
+    [[maybe_unused]] uint32_t x_phases = 0;                 // phases of xbar that thread 0 has waited out
 
     if (warp == PRODUCER_WARP) {
         // ------------------------------ TMA producer ------------------------------
@@ -772,7 +773,10 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                         for (int c = 0; c < n_splits; ++c) st_async_u64(map_to_cta(dst, c), mine, map_to_cta(bar, c));
                         got = wait_bounded_cluster(&sm.xbar, xn & 1, wc);
                         if (got) {
-                            if (r == 0) mbar_expect_tx(&sm.xbar, static_cast<uint32_t>(n_splits) * TILE_M * 8);
+                            if (r == 0) {
+                                mbar_expect_tx(&sm.xbar, static_cast<uint32_t>(n_splits) * TILE_M * 8);
+                                ++x_phases;
+                            }
                             unsigned long long top = 0ull;
                             for (int c = 0; c < n_splits; ++c) {
                                 const unsigned long long v = *reinterpret_cast<volatile unsigned long long*>(&xg[c * TILE_M + r]);
@@ -855,8 +859,13 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         tc_fence_after();
         tmem_dealloc(tmem_base, TMEM_COLS);
     }
-    // a CTA's shared memory must outlive its peers' last writes to it
-    if constexpr (ONE) cluster_sync_all();
+    // A CTA's shared memory must outlive its peers' last writes to it: a CTA that has done all iterations
+    // has waited for every one of them, one that has given up has not.
+    if constexpr (ONE) {
+        cluster_sync_all();
+        if (sm.abort != 0 && threadIdx.x == 0 && n_splits > 1)
+            let_words_land(&sm.xbar, x_phases, static_cast<uint32_t>(n_splits) * TILE_M * 8);
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -954,6 +963,8 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
     __syncthreads();
     if (n_ctas > 1) cluster_sync_all();                   // no CTA touches a peer's barriers before they are set up
 
+    uint32_t phases = 0;                                  // of this warp's row's barrier, waited out
+    static_assert(ROWS <= RT_WARPS, "a warp has at most one row");
     for (int g = 0; g < s; ++g) {
         // ---- sweep ----
 #pragma unroll
@@ -1023,6 +1034,7 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
                 got = wait_bounded_cluster(&sm.bar[r], g & 1, wc);
                 got = __all_sync(0xffffffffu, got);
                 if (got && lane == 0) mbar_expect_tx(&sm.bar[r], static_cast<uint32_t>(n_ctas) * 8);      // the next iteration's
+                if (got) ++phases;
             }
             if (!got) continue;
             unsigned long long k = lane < n_ctas ? *reinterpret_cast<volatile unsigned long long*>(&sm.from[g & 1][r][lane]) : 0ull;
@@ -1083,8 +1095,11 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
         }
         if (__syncthreads_or(!got || sm.abort != 0)) break;
     }
-    // a CTA's shared memory must outlive its peers' last writes to it
-    if (n_ctas > 1) cluster_sync_all();
+    // a CTA's shared memory must outlive its peers' last writes to it, also when it has given up
+    if (n_ctas > 1) {
+        cluster_sync_all();
+        if (sm.abort != 0 && lane == 0 && warp < ROWS) let_words_land(&sm.bar[warp], phases, static_cast<uint32_t>(n_ctas) * 8);
+    }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,

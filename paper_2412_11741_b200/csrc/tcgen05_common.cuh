@@ -286,5 +286,19 @@ __device__ __forceinline__ bool wait_bounded_cluster(uint64_t* bar, uint32_t par
     return false;
 }
 
+// A CTA that has given up must stay until what its peers have sent it has landed: the cluster barrier does
+// not wait for st.async.  One thread calls this after the cluster barrier that every CTA passes when it
+// sends no more; `phase`: the barrier's first phase not waited out, `bytes` its transaction count.  A
+// peer can be one phase ahead, no further (it would need this CTA's words).  A phase that some peer
+// never sent for does not complete: what was sent for it has 20 ms to land.
+__device__ __forceinline__ void let_words_land(uint64_t* bar, uint32_t phase, uint32_t bytes) {
+    const unsigned long long t0 = globaltimer_ns();
+    for (int k = 0; k < 2; ++k, ++phase) {
+        for (uint32_t it = 0; !mbar_try_wait_cluster(bar, phase & 1); ++it)
+            if (globaltimer_ns() - t0 > 20000000ull || it >= (1u << 28)) return;
+        if (k == 0) mbar_expect_tx(bar, bytes);
+    }
+}
+
 }  // namespace tc
 }  // namespace csr

@@ -60,3 +60,28 @@ def test_single_tiles_bounded_wait_runs_out_and_recovers(csr):
         got = csr.csr_encode_ex(D, X, 4)
         assert csr.csr_device_status() == csr.CSR_OK
         assert np.array_equal(_np(got[0]), _np(want[0])) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("M,N,d,s", [(8, 8192, 128, 6), (120, 3000, 64, 5), (40, 1000, 128, 4), (1500, 4096, 128, 4), (3000, 2048, 64, 4)])
+def test_clusters_that_give_up_leave_no_words_behind(csr, M, N, d, s):
+    """The CTAs of a cluster write into one another's shared memory.  Calls that give up at once, each followed
+    at once on the same SMs by a whole call: that one's codes are right every time."""
+    g = torch.Generator(device=DEV).manual_seed(M)
+    D = torch.nn.functional.normalize(torch.randn(N, d, device=DEV, generator=g), dim=1).contiguous()
+    X = torch.randn(M, d, device=DEV, generator=g).to(torch.bfloat16)
+    want_i, want_c = csr.csr_encode_ex(D, X, s)
+    assert csr.csr_device_status() == csr.CSR_OK
+    gave_up = torch.zeros(1, dtype=torch.int32, device=DEV)
+    whole = []
+    try:
+        for _ in range(8):
+            csr.csr_set_option("wait_limit_ns", 0)
+            csr.csr_encode_ex(D, X, s, dev_status=gave_up)
+            csr.csr_set_option("wait_limit_ns", 2_000_000_000)
+            whole.append(csr.csr_encode_ex(D, X, s))
+    finally:
+        csr.csr_set_option("wait_limit_ns", 2_000_000_000)
+    assert csr.csr_device_status() == csr.CSR_OK          # of the whole calls: the others have a word of their own
+    assert int(gave_up.item()) != 0
+    for idx, coef in whole:
+        assert np.array_equal(_np(idx), _np(want_i)) and torch.equal(coef, want_c)
