@@ -668,10 +668,11 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 // pass over the unit's weights and coefficients gives, per head, S = sum |w_t| and
 // U = max over tokens of sum_g |coef[t][g]| (a token's entries may all name one atom); no
 // table entry can exceed S * U in magnitude, and the scale is the power
-// of two that maps S * U to at most 2^29, which leaves the rounding of the individual terms
-// (half a unit each) far inside the 32-bit range.  Each term w * coef is rounded once to
-// fp32, as a floating-point accumulation would, and once to the grid, whose step is
-// 2^-29 * S * U or finer.  A unit whose S or U is not finite falls back to fp32 atomics, so
+// of two that maps S * U to at most 2^30; the roundings of the individual terms, half a unit
+// each, add at most 2^29 (a unit has no more than 2^30 terms) and stay inside the 32-bit
+// range.  Each term w * coef is rounded once to fp32, as a floating-point accumulation would,
+// and once to the grid, whose step is between 2^-30 and 2^-29 of S * U: it grows with the tokens of a
+// unit (see plan_split).  A unit whose S or U is not finite falls back to fp32 atomics, so
 // that NaN and Inf still reach the output.
 // STATS: W holds scores; the first pass makes them weights (softmax over the row, from the statistics the
 // scores kernel left) and reads no codes: U is there already.
@@ -757,7 +758,7 @@ value_scatter_kernel(int N, float* W, int B, int H, const uint16_t* __restrict__
         }
         umax = block_max(umax, red);
         float scale[HGP], inv_scale[HGP];
-        // (the half-unit roundings of the terms must stay far inside the range too)
+        // (the half-unit roundings of the terms must stay inside the range too)
         bool fixed_point = umax < INFINITY && (c1 - c0) * NTHR * static_cast<int64_t>(s) <= (1ll << 30);
 #pragma unroll
         for (int h = 0; h < HGP; ++h) {
@@ -765,7 +766,7 @@ value_scatter_kernel(int N, float* W, int B, int H, const uint16_t* __restrict__
             const float bound = S * umax;
             if (!(bound < INFINITY)) fixed_point = false;                 // Inf or NaN
             int e = 0;
-            if (bound > 0.f) e = 29 - (ilogbf(bound) + 1);                // 2^e * bound <= 2^29
+            if (bound > 0.f) e = 30 - (ilogbf(bound) + 1);                // 2^e * bound <= 2^30
             e = e > 96 ? 96 : e < -96 ? -96 : e;
             scale[h] = ldexpf(1.f, e);
             inv_scale[h] = ldexpf(1.f, -e);
@@ -864,6 +865,11 @@ Split plan_split(int B, int H, int N, int64_t T) {
     // pieces of a stream's tokens for the value scatter: a unit per SM, no more than there are chunks (each
     // unit's table is cleared, stored and read back by ad_kernel)
     int64_t k = sms / ((int64_t)B * p.groups);
+    // ... but at least half as many as a stream has SMs, down to units of 2048 tokens: a unit's grid step grows
+    // with its share of the weights, and however many groups the heads are cut into, the step stays at
+    // what one group per stream has with 2^29 for the grid's range
+    const int64_t fine = (p.chunks + 1) / 2, share = sms / B, least = ((share < fine ? share : fine) + 1) / 2;
+    if (k < least) k = least;
     if (k > p.chunks) k = p.chunks;
     p.pieces = k < 1 ? 1 : (int)k;
     return p;

@@ -118,3 +118,22 @@ def test_one_nan_or_infinite_score_is_softmaxed_like_any_other(csr, B, H, s, T, 
     assert torch.equal(w.isnan(), want.isnan())
     # the exponentials' few ulp, and their arguments' rounding
     torch.testing.assert_close(w.double(), want, rtol=2e-5, atol=1e-30, equal_nan=True)
+
+
+@pytest.mark.parametrize("B,H,T,N,d,s,unit", [(10, 64, 16384, 500, 64, 8, 2048), (18, 64, 6000, 9000, 128, 16, 1024), (4, 32, 9000, 24000, 64, 8, 1024)])
+def test_value_grid_does_not_coarsen_with_the_number_of_head_groups(csr, B, H, T, N, d, s, unit):
+    """`unit`: the tokens of a piece when all SMs share the streams' tokens and a piece takes all heads.  A grid of 29 bits
+    over such a piece's bound has steps of at most 2^-28 S U (the scale is a power of two); T s terms, each half a
+    step off at most, give an output this error in the root mean square."""
+    _, Dv, _, _, (vi, vc) = _inputs(B, H, T, 2, N, d, 1, s, torch.float32, torch.float16)
+    g = torch.Generator(device=DEV).manual_seed(N)
+    W = torch.rand(B, H, T, device=DEV, generator=g)
+    W /= W.sum(-1, keepdim=True)
+    out = csr.csr_value_mix(Dv, W, vi, vc)
+    for b in (0, B - 1):
+        ref = W[b].double() @ _rows(Dv, vi[b], vc[b])
+        U = float(vc[b].double().abs().sum(-1).max())
+        S = float(torch.stack([w.sum(-1).max() for w in W[b].double().split(unit, dim=-1)]).max())
+        bound = 2.0 ** -28 * S * U * math.sqrt(T * s / (12.0 * d))
+        rms = float((out[b] - ref).pow(2).mean().sqrt())
+        assert rms <= bound + 1e-6 * float(ref.pow(2).mean().sqrt()), (rms, bound)
