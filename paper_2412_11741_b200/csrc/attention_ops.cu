@@ -615,7 +615,7 @@ key_scores_kernel(const float* P, int N, int H, const uint16_t* __restrict__ idx
                 for (int h = 0; h < HGP; ++h) {
                     float mw = m[h];
                     for (int o = 16; o; o >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o));
-                    float lw = l[h] * __expf(m[h] - mw);
+                    float lw = l[h] * expf(m[h] - mw);
                     for (int o = 16; o; o >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o);
                     if ((threadIdx.x & 31) == 0) red[warp][h] = make_float2(mw, lw);
                 }
@@ -624,7 +624,7 @@ key_scores_kernel(const float* P, int N, int H, const uint16_t* __restrict__ idx
                     const int h = threadIdx.x;
                     float mx = kLowest, sum = 0.f;
                     for (int q = 0; q < NTHR / 32; ++q) mx = fmaxf(mx, red[q][h].x);
-                    for (int q = 0; q < NTHR / 32; ++q) sum += red[q][h].y * __expf(red[q][h].x - mx);
+                    for (int q = 0; q < NTHR / 32; ++q) sum += red[q][h].y * expf(red[q][h].x - mx);
                     const int slot = blockIdx.x - rg.owner(bg * rg.chunks);
                     st.ml[(bg * st.slots + slot) * HGP + h] = make_float2(mx, sum);
                 }
@@ -716,7 +716,7 @@ value_scatter_kernel(int N, float* W, int B, int H, const uint16_t* __restrict__
                 const float2* ml = st.ml + bg * st.slots * HGP + threadIdx.x;
                 float mx = kLowest, sum = 0.f;
                 for (int q = 0; q < slots; ++q) mx = fmaxf(mx, ml[q * HGP].x);
-                for (int q = 0; q < slots; ++q) sum += ml[q * HGP].y * __expf(ml[q * HGP].x - mx);
+                for (int q = 0; q < slots; ++q) sum += ml[q * HGP].y * expf(ml[q * HGP].x - mx);
                 row_max[threadIdx.x] = mx;
                 row_inv[threadIdx.x] = 1.0f / sum;
             }

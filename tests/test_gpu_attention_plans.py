@@ -137,3 +137,12 @@ def test_value_grid_does_not_coarsen_with_the_number_of_head_groups(csr, B, H, T
         bound = 2.0 ** -28 * S * U * math.sqrt(T * s / (12.0 * d))
         rms = float((out[b] - ref).pow(2).mean().sqrt())
         assert rms <= bound + 1e-6 * float(ref.pow(2).mean().sqrt()), (rms, bound)
+
+
+@pytest.mark.parametrize("B,H,T,N,s", [(64, 4, 16384, 8192, 16), (8, 4, 4099, 8192, 16), (3, 64, 8000, 4096, 8)])
+def test_weights_of_a_row_add_up_to_one_on_average(csr, B, H, T, N, s):
+    """A row's weights share the error of its sum of exponentials, which is put together from parts with maxima of their
+    own.  Roundings go either way: over the rows, the weights' sums miss 1 by less than half an fp32 ulp."""
+    Dk, Dv, Q, (ki, kc), (vi, vc) = _inputs(B, H, T, N, N, 128, s, s, torch.float32, torch.float16)
+    _, w = csr.csr_decode_attention(Dk, Dv, Q, ki, kc, vi, vc, 2.0 / math.sqrt(128))
+    assert abs(float((w.double().sum(-1) - 1.0).mean())) < 2.0 ** -24
