@@ -963,7 +963,7 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
     __syncthreads();
     if (n_ctas > 1) cluster_sync_all();                   // no CTA touches a peer's barriers before they are set up
 
-    uint32_t phases = 0;                                  // of this warp's row's barrier, waited out
+    uint32_t phases = 0;                                  // set on giving up: of this warp's row's barrier, waited out
     static_assert(ROWS <= RT_WARPS, "a warp has at most one row");
     for (int g = 0; g < s; ++g) {
         // ---- sweep ----
@@ -1034,7 +1034,6 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
                 got = wait_bounded_cluster(&sm.bar[r], g & 1, wc);
                 got = __all_sync(0xffffffffu, got);
                 if (got && lane == 0) mbar_expect_tx(&sm.bar[r], static_cast<uint32_t>(n_ctas) * 8);      // the next iteration's
-                if (got) ++phases;
             }
             if (!got) continue;
             unsigned long long k = lane < n_ctas ? *reinterpret_cast<volatile unsigned long long*>(&sm.from[g & 1][r][lane]) : 0ull;
@@ -1093,7 +1092,10 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
                     reinterpret_cast<float*>(out_coef)[m * ldc + g] = coef;
             }
         }
-        if (__syncthreads_or(!got || sm.abort != 0)) break;
+        if (__syncthreads_or(!got || sm.abort != 0)) {
+            phases = g + (got ? 1 : 0);
+            break;
+        }
     }
     // a CTA's shared memory must outlive its peers' last writes to it, also when it has given up
     if (n_ctas > 1) {
