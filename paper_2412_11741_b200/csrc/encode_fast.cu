@@ -985,20 +985,39 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
                 }
             }
             // this lane: atoms a0 + 16 mt + l4 (c0, c1) and + 8 (c2, c3) of rows 8 nt + 2 q4 (c0, c2) and + 1 (c1, c3)
-            unsigned long long k0 = 0ull, k1 = 0ull;
+            unsigned long long k0, k1;
+            auto largest = [&]() {
+                k0 = k1 = 0ull;
 #pragma unroll
-            for (int mt = 0; mt < MT; ++mt)
+                for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-                for (int hi = 0; hi < 2; ++hi) {
-                    const int n = a0 + 16 * mt + 8 * hi + l4;
-                    const uint32_t tag = static_cast<uint32_t>(NG - 1 - (n & (TILE_N - 1)) / G), low = 0xFFFFFFFFu - static_cast<uint32_t>(n / TILE_N);
-                    const uint32_t v0 = (__float_as_uint(c[mt][2 * hi]) & 0x7FFFFFFFu & key_mask) | tag;
-                    const uint32_t v1 = (__float_as_uint(c[mt][2 * hi + 1]) & 0x7FFFFFFFu & key_mask) | tag;
-                    if (n < n_pad) {
-                        k0 = max_u64(k0, (static_cast<unsigned long long>(v0) << 32) | low);
-                        k1 = max_u64(k1, (static_cast<unsigned long long>(v1) << 32) | low);
+                    for (int hi = 0; hi < 2; ++hi) {
+                        const int n = a0 + 16 * mt + 8 * hi + l4;
+                        const uint32_t tag = static_cast<uint32_t>(NG - 1 - (n & (TILE_N - 1)) / G), low = 0xFFFFFFFFu - static_cast<uint32_t>(n / TILE_N);
+                        const uint32_t v0 = (__float_as_uint(c[mt][2 * hi]) & 0x7FFFFFFFu & key_mask) | tag;
+                        const uint32_t v1 = (__float_as_uint(c[mt][2 * hi + 1]) & 0x7FFFFFFFu & key_mask) | tag;
+                        if (n < n_pad) {
+                            k0 = max_u64(k0, (static_cast<unsigned long long>(v0) << 32) | low);
+                            k1 = max_u64(k1, (static_cast<unsigned long long>(v1) << 32) | low);
+                        }
                     }
+            };
+            largest();
+            if constexpr (G > 1) {
+                // A key above those of Inf is a NaN's, which only rows that are not finite have.  As in group_key, the NaNs
+                // of a group count only where all of it is NaN.
+                constexpr uint32_t kInfKey = 0x7F800000u | (NG - 1);
+                if (__any_sync(0xffffffffu, max(static_cast<uint32_t>(k0 >> 32), static_cast<uint32_t>(k1 >> 32)) > kInfKey)) {
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+#pragma unroll
+                            for (int o = 4; o < 4 * G; o <<= 1)
+                                c[mt][i] = fmaxf(fabsf(c[mt][i]), fabsf(__shfl_xor_sync(0xffffffffu, c[mt][i], o)));
+                    largest();
                 }
+            }
 #pragma unroll
             for (int o = 4; o < 32; o <<= 1) {
                 k0 = max_u64(k0, __shfl_xor_sync(0xffffffffu, k0, o));

@@ -85,3 +85,28 @@ def test_clusters_that_give_up_leave_no_words_behind(csr, M, N, d, s):
     assert int(gave_up.item()) != 0
     for idx, coef in whole:
         assert np.array_equal(_np(idx), _np(want_i)) and torch.equal(coef, want_c)
+
+
+@pytest.mark.parametrize("d,N", [(64, 1000), (64, 2304), (64, 5000), (128, 1000)])
+@pytest.mark.parametrize("M", [8, 50, 200])
+def test_rows_that_are_not_finite_get_the_codes_of_pairs_too(csr, d, N, M):
+    """An infinite channel makes an atom's correlation infinite, or NaN where the atom does not use the channel: groups of
+    atoms with some NaNs and with nothing but NaNs."""
+    g = torch.Generator(device=DEV).manual_seed(M + N)
+    D = torch.randn(N, d, device=DEV, generator=g)
+    D[::3, 5] = 0.0
+    D[40:64, 5] = 0.0
+    D = torch.nn.functional.normalize(D, dim=1).contiguous()
+    X = torch.randn(M, d, device=DEV, generator=g)
+    X[1, 5], X[3, 5], X[4] = float("inf"), -float("inf"), float("nan")
+    X[6, 4], X[6, 5] = float("inf"), -float("inf")
+    X = X.to(torch.bfloat16)
+    idx, coef = csr.csr_encode_ex(D, X, 4, coef_dtype=torch.float32)
+    csr.csr_set_option("fast_split", 1)
+    try:
+        idx2, coef2 = csr.csr_encode_ex(D, X, 4, coef_dtype=torch.float32)
+    finally:
+        csr.csr_set_option("fast_split", 0)
+    assert csr.csr_device_status() == csr.CSR_OK
+    assert np.array_equal(_np(idx), _np(idx2))
+    assert bool(((coef == coef2) | (coef.isnan() & coef2.isnan())).all())
