@@ -382,10 +382,11 @@ int csr_reconstruct_host(const csr_reconstruct_params_t* p);
  *     atoms of 128 channels, a 2 MiB bf16 copy);
  *     larger dictionaries are rejected with CSR_ERR_UNSUPPORTED.
  *   - The first call on a device looks up the array's device address, once, with that
- *     device current.  That lookup (and the first launch of each kernel) makes the CUDA
- *     runtime load the part of the library image that holds the array, which is when the
- *     2 MiB + 2 KiB are taken from that GPU's memory, to be held until the process exits.
- *     Make one call per device and per shape class (many rows; few rows) at start-up and
+ *     device current.  That lookup makes the CUDA runtime load the part of the library image
+ *     that holds the array, which is when the 2 MiB + 2 KiB are taken from that GPU's memory,
+ *     to be held until the process exits.  The first call for a d and N also loads the code
+ *     of the kernels that serve them, those for every number of rows.
+ *     Make one call per device and dictionary shape, of any number of rows, at start-up and
  *     before any stream capture begins; later calls take nothing from device memory.
  *   - All calls on a device share the one array, and it keeps what the last call wrote.
  *     Each call rewrites the dictionary copy in full and zeroes its status word before

@@ -82,6 +82,8 @@ int launch_encode_fast(const EncodeArgs& a, void* workspace, uint32_t* status);
 size_t encode_fast_workspace_bytes(int d, int N);
 // fp32 -> fp16 copy of D (round to nearest even), same [N][d] layout: the de-sparse kernel's gather source.
 int launch_dict_to_f16(const float* D, int N, int d, void* dst, cudaStream_t stream);
+// Loads the code of all kernels that launch_encode_fast may launch for this d and N, once per device.
+int load_fast_kernels(int d, int N);
 // The two halves of launch_encode_fast: build the bf16 copy once, encode against it many times.
 int prepare_fast_dictionary(const float* D, int N, int d, void* workspace, cudaStream_t stream);
 // Whole waves of pairs of row tiles, then single row tiles with one or more CTAs each (clusters that

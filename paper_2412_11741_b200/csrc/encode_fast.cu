@@ -57,6 +57,7 @@
 // iteration and leaves the rows' maxima to split_pick_kernel: a launch pair per iteration.)
 #include <cuda.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -1457,6 +1458,42 @@ int prepare_fast_dictionary(const float* D, int N, int d, void* workspace, cudaS
         e = cudaMemsetAsync(static_cast<char*>(workspace) + (size_t)N * d * 2, 0, (size_t)(n_pad - N) * d * 2, stream);
         if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
     }
+    return CSR_OK;
+}
+
+// Has the runtime load the code of every kernel that a call of any number of rows may launch for this d and
+// N (it loads a kernel when that is first asked for, and its code takes device memory).
+template <int D_>
+static int load_kernels(int G) {
+    auto load = [](auto... kernels) {
+        cudaFuncAttributes at;
+        cudaError_t e = cudaFuncGetAttributes(&at, dict_to_bf16_kernel);
+        for (const void* k : {reinterpret_cast<const void*>(kernels)...})
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, k);
+        return e;
+    };
+    auto of = [&](auto g) {
+        constexpr int g_ = decltype(g)::value;
+        return load(encode_fast_kernel<D_, g_, false>, encode_fast_kernel<D_, g_, true>, encode_few_kernel<D_, g_, 1>,
+                    encode_few_kernel<D_, g_, 2>);
+    };
+    using std::integral_constant;
+    const cudaError_t e = G == 1   ? of(integral_constant<int, 1>{})
+                          : G == 2 ? of(integral_constant<int, 2>{})
+                          : G == 8 ? of(integral_constant<int, 8>{})
+                                   : of(integral_constant<int, 4>{});
+    return e == cudaSuccess ? CSR_OK : fail(CSR_ERR_CUDA, "loading the encoder's kernels: %s", cudaGetErrorString(e));
+}
+int load_fast_kernels(int d, int N) {
+    static std::atomic<uint32_t> loaded[64];              // per device, a bit for each d and group size
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || dev < 0 || dev >= 64) return fail(CSR_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
+    const int G = group_size(d, N);
+    const uint32_t bit = static_cast<uint32_t>(G) << (d == 128 ? 8 : 0);
+    if (loaded[dev].load() & bit) return CSR_OK;
+    if (int rc = d == 128 ? load_kernels<128>(G) : load_kernels<64>(G)) return rc;
+    loaded[dev].fetch_or(bit);
     return CSR_OK;
 }
 

@@ -10,8 +10,9 @@
 // library image, and no call here calls an allocating routine.  The image's device data is
 // placed by the CUDA runtime when the module that holds it is first used on a device (with
 // lazy module loading: at the first call of this entry point there, which looks the array
-// up; the first launch of each kernel loads its code the same way), so the first call on a
-// device belongs to start-up; from the second call on nothing is taken from device memory.
+// up).  A kernel's code is loaded the same way; which kernels a call launches depends on its number of
+// rows, so the first call for a dictionary shape asks for all of them.  The first call on a device
+// and for a shape belongs to start-up; later ones take nothing from device memory, whatever their rows.
 // Every GPU that has made that first call holds the bytes until the process exits.
 #include <mutex>
 
@@ -77,6 +78,7 @@ extern "C" int csr_encode_static(const void* D, const void* X, int64_t M, int d,
 
     void* base = nullptr;
     if (int rc = static_scratch(&base)) return rc;
+    if (int rc = load_fast_kernels(d, N)) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // The status word must start at zero; the dictionary copy is rewritten in full by every call.
     uint32_t* status = dev_status ? dev_status : static_cast<uint32_t*>(base);
