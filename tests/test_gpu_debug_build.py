@@ -103,3 +103,36 @@ def test_tensor_core_correlations_stay_far_inside_the_band():
     assert res.returncode == 0, res.stdout + res.stderr
     worst = float([l for l in res.stdout.splitlines() if l.startswith("TCERR")][0].split(" ", 1)[1])
     assert 0.0 < worst < 2.0 ** -14, worst
+
+
+CHILD_SPLIT = r'''
+import sys
+import torch
+sys.path.insert(0, %(root)r)
+import paper_2412_11741_b200 as csr
+from paper_2412_11741_b200 import workloads as wl
+
+# rows and atoms that give the split engine slices of one 64-column box, of two and three, and of several tiles
+worst = 0.0
+for w, rows in ((wl.gqa_long(tokens=64), (16, 128, 700, 3000, 8192)), (wl.dict_sweep(4096, d=64, M=8192), (100, 1500, 8192)),
+                (wl.dict_sweep(1024, M=8192), (128, 600, 2500))):
+    D = torch.from_numpy(w.D).to("cuda:0")
+    X = torch.from_numpy(w.X).to("cuda:0").to(torch.bfloat16)
+    for M in rows:
+        x = X[torch.linspace(0, X.shape[0] - 1, M, device=X.device).long()].contiguous()
+        csr.csr_encode_ex(D, x, w.s, mode=csr.CSR_MODE_FP32_EXACT)
+        assert csr.csr_device_status() == csr.CSR_OK, csr.csr_last_error_string()
+        worst = max(worst, csr.csr_debug_read("exact_tensor_error"))
+print("TCERR", repr(worst))
+'''
+
+
+def test_split_engine_correlations_stay_far_inside_the_band():
+    """The same bound for the engine that splits the dictionary (the default up to one row tile per SM)."""
+    from paper_2412_11741_b200 import build
+    lib = build.build(debug=True)
+    env = dict(os.environ, CSR_LIBRARY_PATH=lib)
+    res = subprocess.run([sys.executable, "-c", CHILD_SPLIT % {"root": ROOT}], env=env, capture_output=True, text=True, timeout=900)
+    assert res.returncode == 0, res.stdout + res.stderr
+    worst = float([l for l in res.stdout.splitlines() if l.startswith("TCERR")][0].split(" ", 1)[1])
+    assert 0.0 < worst < 2.0 ** -14, worst
