@@ -84,11 +84,14 @@ extern "C" {
  *                        (a) sweep on the tcgen05 tensor cores, residual and atoms each
  *                        split into a bf16 high and low part, three bf16 products per
  *                        correlation accumulated in fp32 (band 2^-12 * ||R||): the default
- *                        wherever the library-owned scratch is in use (no caller workspace;
- *                        about 4 * N * d + 2048 * d * min(ceil(M / 256), SMs) bytes of it).
+ *                        wherever the library-owned scratch is in use (no caller workspace).
  *                        Whole waves of pairs of 128-row tiles run with one CTA per pair;
  *                        fewer rows, and what is left over, with the dictionary split
- *                        across the CTAs of one cooperative launch (the same codes);
+ *                        across the CTAs of one cooperative launch (the same codes).
+ *                        Scratch: about 4 * N * d bytes, and the larger of
+ *                        2048 * d * min(ceil(M / 256), SMs) (pairs) and, for the rows that
+ *                        run split (at most 128 * SMs in a launch, rounded up to 128),
+ *                        12 * d + 48 * min(SMs / (rows / 128), ceil(N / 64), 128) bytes a row;
  *                        (b) fp32 operands and fp32 accumulation on the plain ALUs (band
  *                        1.6e-5 * ||R||), one CTA per 64 rows, no scratch: taken when a
  *                        caller workspace is given;
@@ -107,8 +110,10 @@ extern "C" {
  *                        scratch.  The rows of a decoding step (8 or 16 per cluster, as many
  *                        clusters as fit) meet a dictionary held in registers; channels are
  *                        summed in another order there, which can decide between two
- *                        atoms only where the mode does not tell them apart anyway.
- *                        (csr_set_option can force each of these paths.)
+ *                        atoms only where the mode does not tell them apart anyway (about
+ *                        one pick in 10^6), so that a row's codes may depend on how many rows
+ *                        share its call.  csr_set_option("fast_split", 1) gives codes that do
+ *                        not.  (It can force each of these paths.)
  */
 #define CSR_MODE_FP32_EXACT 0
 #define CSR_MODE_BF16_FAST 1
@@ -225,7 +230,7 @@ int csr_pack_coefficients(const float* coef32, int64_t n, void* coef16, void* st
  * fp16 for the de-sparse kernel (params.dict of csr_reconstruct_ex).  The fast mode works on a
  * bf16 copy of D which the encode calls
  * otherwise rebuild in scratch memory on every call (one extra launch of a few
- * microseconds: measured 83 -> 80 us on a 4160-row call, nothing on large ones).  A
+ * microseconds: measured 48 -> 43 us on a 4160-row call, nothing on large ones).  A
  * dictionary is fixed for a layer's lifetime, so the copy can be made once and the encode
  * calls then need no scratch for it: csr_dict_create allocates it (cudaMalloc, N rounded up to 8
  * atoms of d bf16 values), converts D on `stream` and returns a handle; an encode call whose
@@ -413,7 +418,9 @@ int csr_dict_check_norms(const void* D, int N, int d, float tol, void* stream, f
 
 /*
  * Process-wide tuning and diagnostic switches; none is needed in normal use (tests use them
- * to drive every code path, measurements to compare them).  All paths return the same codes.
+ * to drive every code path, measurements to compare them).  The exact mode's paths all return the
+ * same codes; so do the fast mode's with "fast_split" 1 or 2 and one "fast_group" (see
+ * CSR_MODE_BF16_FAST for the rows of a decoding step).
  *   "fast_group"     0 (default: the library chooses) or 1, 2, 4, 8: atoms per arg-max group
  *                    of the fast encoder's sweep;
  *   "fast_split"     0 (default: single row tiles, split across thread-block clusters, for few

@@ -89,7 +89,8 @@ int prepare_fast_dictionary(const float* D, int N, int d, void* workspace, cudaS
 // Whole waves of pairs of row tiles, then single row tiles with one or more CTAs each (clusters that
 // share the dictionary's sweep): no scratch.  With `split_scratch` (encode_fast_split_scratch_bytes(),
 // 256-byte aligned) few rows run without clusters instead, one sweep launch and one pick launch
-// per iteration.  Identical codes.
+// per iteration.  Identical codes, but for the rows of a decoding step, whose correlations may be summed
+// in another order (see encode_few_kernel).
 int launch_encode_fast_prepared(const EncodeArgs& a, const void* dict_bf16, uint32_t* status, void* split_scratch);
 bool encode_fast_split_applies(int64_t M, int N);
 size_t encode_fast_split_scratch_bytes(int64_t M, int d, int N);

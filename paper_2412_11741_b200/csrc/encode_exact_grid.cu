@@ -17,7 +17,7 @@
 // iteration are fetched while the rows are being settled.
 //
 // What bounds it: with few rows the chain of dependent steps (A load, MMA, drain, meeting, settle,
-// meeting: about 8 us an iteration), with many the MMAs, 3072 cycles per 256 atoms and row tile.
+// meeting: 10 to 11 us an iteration at 16 to 128 rows, N = 8192), with many the MMAs, 3072 cycles per 256 atoms and row tile.
 // The grid is launched cooperatively whenever a row tile has more than one CTA, so all CTAs that
 // wait for one another are resident.
 #include "exact_tc_common.cuh"

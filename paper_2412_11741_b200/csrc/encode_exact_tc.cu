@@ -529,11 +529,12 @@ int run(const EncodeArgs& a, const CUtensorMap& mh, const CUtensorMap& ml, doubl
 // A wave of pairs takes the time of two waves of single row tiles (the tensor cores bound both),
 // a row tile split over c CTAs 1/c of one.  Whole waves of pairs come first (they read the
 // dictionary half as often); the last, partial one is replaced wherever that saves at least a
-// quarter of it.  Measured at N = 4096, s = 8, d = 128 in us, this plan against pairs only: 2048 rows
-// 165 / 715, 9472 300 / 723, 18944 432 / 750, 20000 589 / 750, 24224 704 / 750, 27648 734 / 750 (where
-// the second launch would not split its tiles any more, pairs are as good and are taken), 37888 750.
-// Few rows at N = 8192, s = 16: 16 rows 203 us, 128 rows 234 us, 512 rows 259 us, against 332-598,
-// 478-873 and 1520 us for the plain-ALU encoder with its launch pair per iteration.
+// quarter of it.  Measured at N = 4096, s = 8, d = 128 in us (cold caches, the dictionary's split and the
+// launches included), this plan against pairs only: 2048 rows 155 / 744, 9472 284 / 747, 18944
+// 415 / 753, 20000 540 / 755, 24224 652 / 759, 27648 691 / 759 (where the second launch would not split
+// its tiles any more, pairs are as good and are taken), 37888 769.  Few rows at N = 8192, s = 16: 16 rows
+// 157 us, 128 rows 189, 512 rows 237, 4096 rows 511, against 474, 339, 1672 and 6567 for the plain-ALU
+// encoder with its launch pair per iteration and 2090 to 2350 for pairs.
 struct Plan {
     int64_t pair_rows;
     int64_t grid_rows[2];

@@ -1303,7 +1303,10 @@ int few_ctas(int N) {
 // Rows per cluster of encode_few_kernel, 8 or 16 (0: row tiles are faster).  Measured, s = 16, in us, this
 // kernel with 8 rows / 16 rows per cluster against row tiles: 8 rows N = 1000 33 / 33 / 57, N = 8192 35 / 49 /
 // 78; 64 rows N = 8192 (8 clusters of 16, more than the chip holds at once) 68 / 49 / 84; 128 rows
-// N = 1000 33 / 47 / 68.  Per iteration 2.2 us (8 rows) and 3.05 (16 rows) a round of clusters.
+// N = 1000 33 / 47 / 68.  Per iteration 2.2 us (8 rows) and 3.05 (16 rows) a round of clusters, at d = 64 (a
+// warp holds twice the atoms, half the channels) as at d = 128: 8 rows N = 1000 35 / 51 / 51, 512 rows
+// N = 1000 35 / 51 / 57, 128 rows N = 4096 43 / 59 / 76, 512 rows N = 4096 80 / 61 / 76, 128 rows N = 8192
+// 80 / 60 / 90, 256 rows N = 8192 117 / 115 / 92 (d = 64, cold caches).
 template <int D_, int G>
 int few_rows_per_cluster(int64_t M, int N) {
     const int n_ctas = few_ctas<D_>(N);

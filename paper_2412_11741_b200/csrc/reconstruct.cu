@@ -2,13 +2,14 @@
 //
 // HBM traffic per row is 4*s bytes of codes in and d * sizeof(out) bytes out; the s atom rows a
 // row needs are gathered from the dictionary, which is a few MB and stays in L2, so from about
-// s = 4 up the kernel is bound by the L2 -> SM gather (s * d * sizeof(atom) bytes per row), not
-// by HBM.  Two things follow:
+// s = 4 up the kernel is bound by the L2 -> SM gather (s * d * sizeof(atom) bytes per row) or, with
+// fp16 atoms up to about s = 8, by instruction issue (0.71 per cycle at s = 8; 139 us for 2^20 rows at
+// N = 8192, 132 at N = 512, where the L1 holds the dictionary), not by HBM.  Two things follow:
 //   - the atoms can be gathered from the fp16 copy of a prepared dictionary (csr_dict_create)
 //     instead of the fp32 master: half the gathered bytes, and with fp16 coefficients (the
 //     stored form) the products need no unpacking at all: fma.rn.f32.f16 multiplies two fp16
 //     values exactly and accumulates in fp32;
-//   - what is left is latency: every warp works on units of 16 consecutive rows whose codes it
+//   - what is left is latency: every warp works on units of 16 (or 8 or 4) consecutive rows whose codes it
 //     stages through its own piece of shared memory with cp.async one unit ahead (one coalesced
 //     stream instead of a dependent load per row; no block-wide barrier anywhere), and it keeps
 //     the gathers of several rows in flight: every lane moves 16 bytes of an atom, so an atom
@@ -360,9 +361,10 @@ int launch_by(const ReconstructArgs& a, const void* dict) {
     const int64_t cap = (int64_t)sm_count() * (per_sm < fit ? per_sm : fit);
     // Rows per unit: 16, or 8 or 4 where that leaves a warp at least a tenth fewer rows in all (a last round of
     // units that few warps have): 77777 rows are 1.03 rounds of 16 on 4736 warps, two rounds, or five
-    // rounds of 4: 34.9 -> 20.6 us (s = 6, N = 5001, fp32 atoms; with the steps of three).  Longer units are
-    // better otherwise (2^20 rows, s = 8, fp16 atoms: 126 us in units of 16, 140 in units of 4).  Eight rows of codes end on a 16-byte boundary in any case, four if s is
-    // even; a trip of a warp takes 32 / lanes per row * PP rows.
+    // rounds of 4: 24.6 us in units of 16, 22.6 in units of 4 (s = 6, N = 5001, fp32 atoms, cold caches; both
+    // with the steps of three).  Longer units are better otherwise (2^20 rows, s = 8, fp16 atoms, N = 8192: 131 us
+    // in units of 16, 166 in units of 4).  Eight rows of codes end on a 16-byte boundary in any case, four if s
+    // is even; a trip of a warp takes 32 / lanes per row * PP rows.
     constexpr int trip = 32 / (D_ / Piece<F16>::CH) * PP;
     const int64_t warps = cap * (NT / 32);
     auto rows_of_a_warp = [&](int w) { return ((a.M + w - 1) / w + warps - 1) / warps * w; };
