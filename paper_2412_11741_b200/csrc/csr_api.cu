@@ -312,9 +312,11 @@ int ensure_side_streams(DeviceBuffers** out) {
 // Runs one encode on device pointers.  `shared_scratch` = false keeps the call off the parts of
 // the library-owned buffer that two encodes in flight would both write.  `prepared` (fast mode
 // only) is a bf16 copy of D made by the caller of this function: no conversion is enqueued.
-int encode_device(const csr_encode_params_t* p, bool shared_scratch = true, const void* prepared = nullptr) {
+// `load`: see EncodeArgs.
+int encode_device(const csr_encode_params_t* p, bool shared_scratch = true, const void* prepared = nullptr, float load = 1.f) {
     if (p->M == 0) return CSR_OK;
     EncodeArgs a;
+    a.load = load;
     a.D = static_cast<const float*>(p->D);
     a.X = p->X;
     a.x_dtype = p->x_dtype;
@@ -564,6 +566,13 @@ int csr_encode_grouped(const csr_encode_params_t* problems, int count) {
         if (int rc = ensure_side_streams(&b)) return rc;
         std::lock_guard<std::mutex> group_lock(g_group_mu);
         cudaStream_t main = static_cast<cudaStream_t>(problems[i].stream);
+        // (a problem shares the GPU with those on the other streams, one on each at a time)
+        int64_t rows = 0;
+        for (int k = i; k < j; ++k) rows += problems[k].M;
+        auto load = [&](const csr_encode_params_t& q) {
+            const float all = static_cast<float>(rows) / static_cast<float>(q.M);
+            return all < kSideStreams + 1 ? all : static_cast<float>(kSideStreams + 1);
+        };
         cudaError_t e = cudaEventRecord(b->fork, main);
         bool used[kSideStreams] = {};
         int rc = CSR_OK;
@@ -573,9 +582,9 @@ int csr_encode_grouped(const csr_encode_params_t* problems, int count) {
             used[sidx] = true;
             csr_encode_params_t q = problems[k];
             q.stream = b->side[sidx];
-            if (e == cudaSuccess) rc = encode_device(&q, false);
+            if (e == cudaSuccess) rc = encode_device(&q, false, nullptr, load(q));
         }
-        if (rc == CSR_OK && e == cudaSuccess) rc = encode_device(&problems[i], false);
+        if (rc == CSR_OK && e == cudaSuccess) rc = encode_device(&problems[i], false, nullptr, load(problems[i]));
         // join whatever was forked, also after a failure: the caller's stream must not run ahead
         for (int sidx = 0; sidx < kSideStreams; ++sidx) {
             if (!used[sidx]) continue;

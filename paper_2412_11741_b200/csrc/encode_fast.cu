@@ -1245,14 +1245,22 @@ int group_size(int d, int N) {
 // a call of 8 iterations at N = 1024 / 8192, d = 128, this plan against clusters of up to 16 CTAs
 // on pairs of row tiles: 64 rows 35 / 45 against 47 / 45; 1100 rows 37 / 58 against 54 / 74; 4160 rows
 // 40 / 83 against 56 / 140; 9400 rows 45 / 131 against 68 / 233; 18900 rows 54 / 227 against 70 / 237.
+// Problems side by side (a grouped call) share the chip: a plan that gives each all of it has their
+// clusters wait for one another.  Measured in us, two / four problems, d = 128, s = 16, planned for the whole
+// chip against for their share of it: 128 rows N = 4096 96 / 143 against 83 / 86; 1024 rows N = 1024 95 / 187
+// against 74 / 85, N = 8192 214 / 321 against 155 / 161; 9472 rows N = 1024 167 / 327 against 102 / 156.
 struct RowPlan {
     int64_t pair_rows;
     int64_t tile_rows[2];
     int splits[2];
     float us;                // an iteration of what follows the whole waves
 };
+// Rounds in which the GPU gets through n units of a call, `cap` at a time, with `load` times as many rows in flight.
+int64_t rounds_of(int64_t n, int64_t cap, float load) {
+    return (static_cast<int64_t>(ceilf(static_cast<float>(n) * load - 1e-3f)) + cap - 1) / cap;
+}
 template <int D_, int G>
-RowPlan plan_rows(int64_t M, int N) {
+RowPlan plan_rows(int64_t M, int N, float load) {
     const int T = (N + TILE_N - 1) / TILE_N;
     const int64_t sms = sm_count(), wave = sms * 2 * TILE_M;
     const int64_t rest = M % wave, tiles = (rest + TILE_M - 1) / TILE_M;
@@ -1262,11 +1270,11 @@ RowPlan plan_rows(int64_t M, int N) {
     // n row tiles in one launch: the best number of CTAs per tile
     auto best_split = [&](int64_t n, float* cost) {
         int best = 1;
-        *cost = (float)((n + sms - 1) / sms) * (kTile0 + kTile1 * T);
+        *cost = (float)rounds_of(n, sms, load) * (kTile0 + kTile1 * T);
         for (int ns = 2; ns <= kMost && ns <= T; ns *= 2) {
             const int nc = max_clusters<D_, G>(ns);
             if (nc < 1) continue;
-            const float c = (float)((n + nc - 1) / nc) * (kTile0 + kTile1 * ((T + ns - 1) / ns));
+            const float c = (float)rounds_of(n, nc, load) * (kTile0 + kTile1 * ((T + ns - 1) / ns));
             if (c < *cost) {
                 *cost = c;
                 best = ns;
@@ -1276,7 +1284,7 @@ RowPlan plan_rows(int64_t M, int N) {
     };
     RowPlan p{M, {0, 0}, {0, 0}, 0.f};
     if (tiles == 0) return p;
-    float least = kPair0 + kPair1 * T, cost;
+    float least = (float)rounds_of((tiles + 1) / 2, sms, load) * (kPair0 + kPair1 * T), cost;
     p.us = least;
     const int one = best_split(tiles, &cost);
     if (cost < least) {
@@ -1285,7 +1293,7 @@ RowPlan plan_rows(int64_t M, int N) {
     }
     if (tiles > sms) {                                     // a whole wave of single tiles, then the others over the whole chip
         const int two = best_split(tiles - sms, &cost);
-        cost += kTile0 + kTile1 * T;
+        cost += (float)rounds_of(sms, sms, load) * (kTile0 + kTile1 * T);
         if (cost < least) p = RowPlan{M - rest, {sms * TILE_M, rest - sms * TILE_M}, {1, two}, cost};
     }
     return p;
@@ -1308,14 +1316,14 @@ int few_ctas(int N) {
 // N = 1000 35 / 51 / 57, 128 rows N = 4096 43 / 59 / 76, 512 rows N = 4096 80 / 61 / 76, 128 rows N = 8192
 // 80 / 60 / 90, 256 rows N = 8192 117 / 115 / 92 (d = 64, cold caches).
 template <int D_, int G>
-int few_rows_per_cluster(int64_t M, int N) {
+int few_rows_per_cluster(int64_t M, int N, float load) {
     const int n_ctas = few_ctas<D_>(N);
     if (n_ctas == 0 || M > 4096) return 0;
     const int fit = n_ctas == 1 ? sm_count() : max_clusters<D_, G>(n_ctas);
     if (fit < 1) return 0;
-    auto rounds = [&](int rows) { return (float)(((M + rows - 1) / rows + fit - 1) / fit); };
+    auto rounds = [&](int rows) { return (float)rounds_of((M + rows - 1) / rows, fit, load); };
     const float c8 = 2.2f * rounds(8), c16 = 3.05f * rounds(16), few = c8 <= c16 ? c8 : c16;
-    if (few >= plan_rows<D_, G>(M, N).us) return 0;
+    if (few >= plan_rows<D_, G>(M, N, load).us) return 0;
     return c8 <= c16 ? 8 : 16;
 }
 
@@ -1344,14 +1352,14 @@ int launch_few(const EncodeArgs& a, const uint16_t* Db, uint32_t* status) {
 template <int D_, int G>
 int launch_planned(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uint32_t* status) {
     if (options().fast_split == 0) {
-        const int rows = few_rows_per_cluster<D_, G>(a.M, a.N);
+        const int rows = few_rows_per_cluster<D_, G>(a.M, a.N, a.load);
         if (rows > 0) {
             const int rc = rows == 8 ? launch_few<D_, G, 1>(a, Db, status) : launch_few<D_, G, 2>(a, Db, status);
             if (rc != kClusterLaunchRefused) return rc;
         }
     }
     // (the option forces pairs only)
-    const RowPlan p = options().fast_split == 0 ? plan_rows<D_, G>(a.M, a.N) : RowPlan{a.M, {0, 0}, {0, 0}, 0.f};
+    const RowPlan p = options().fast_split == 0 ? plan_rows<D_, G>(a.M, a.N, a.load) : RowPlan{a.M, {0, 0}, {0, 0}, 0.f};
     auto rows_from = [&](int64_t r0, int64_t m) {
         EncodeArgs b = a;
         b.X = static_cast<const char*>(a.X) + (size_t)r0 * a.ldx * dtype_size(a.x_dtype);

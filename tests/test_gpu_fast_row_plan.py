@@ -110,3 +110,26 @@ def test_rows_that_are_not_finite_get_the_codes_of_pairs_too(csr, d, N, M):
     assert csr.csr_device_status() == csr.CSR_OK
     assert np.array_equal(_np(idx), _np(idx2))
     assert bool(((coef == coef2) | (coef.isnan() & coef2.isnan())).all())
+
+
+@pytest.mark.parametrize("d,N,rows", [(128, 4096, (128, 128)), (128, 1024, (512, 40, 9472, 1025)), (64, 2500, (9000, 9000, 9000, 9000)),
+                                      (128, 2000, (30000, 8, 700)), (64, 1000, (1024,) * 6), (128, 300, (40000, 38000))])
+def test_grouped_problems_get_the_codes_of_pairs(csr, d, N, rows):
+    """Problems side by side plan for their share of the GPU: other splits than alone, the same codes."""
+    g = torch.Generator(device=DEV).manual_seed(sum(rows))
+    problems, want = [], []
+    for M in rows:
+        D = torch.nn.functional.normalize(torch.randn(N, d, device=DEV, generator=g), dim=1).contiguous()
+        X = torch.randn(M, d, device=DEV, generator=g).to(torch.bfloat16)
+        problems.append((D, X, 3, torch.full((M, 3), -1, dtype=torch.int16, device=DEV).view(torch.uint16),
+                         torch.full((M, 3), 7.0, dtype=torch.float16, device=DEV), csr.csr_dict_create(D)))
+    csr.csr_set_option("fast_split", 1)
+    try:
+        want = [csr.csr_encode_ex(D, X, s) for D, X, s, _, _, _ in problems]
+    finally:
+        csr.csr_set_option("fast_split", 0)
+    csr.csr_encode_grouped(problems)
+    assert csr.csr_device_status() == csr.CSR_OK
+    for (_, _, _, idx, coef, h), (i, c) in zip(problems, want):
+        assert np.array_equal(_np(idx), _np(i)) and torch.equal(coef, c)
+        csr.csr_dict_destroy(h)
