@@ -463,9 +463,14 @@ int csr_debug_checks(void);
 /*
  * Quantities only a checked build records (CSR_ERR_UNSUPPORTED otherwise); reading one
  * synchronises the device and resets it.
- *   "exact_tensor_error"  the largest | tensor-core correlation - fp64 correlation | / ||R||
- *                         over the picks the exact mode's tensor-core encoder took without
- *                         re-scoring since the last read (must stay below half the band).
+ * Both over the picks the exact mode's tensor-core encoders took without re-scoring since the last
+ * read:
+ *   "exact_tensor_error"  the largest | tensor-core correlation - fp64 correlation of the same 16-bit
+ *                         operands | relative to ||R|| and the largest norm of an atom: what the
+ *                         tensor cores' fp32 sums add (the operands' rounding is bounded by norms that
+ *                         the encoder takes);
+ *   "exact_band_use"      the largest | tensor-core correlation - fp64 correlation | relative to half
+ *                         the band that decided the pick (must stay below 1).
  */
 int csr_debug_read(const char* name, double* value);
 

@@ -58,24 +58,23 @@ bool encode_exact_split_applies(int64_t M, int N);
 size_t encode_exact_split_scratch_bytes(int64_t M, int d, int N);
 int launch_encode_exact_split(const EncodeArgs& a, void* scratch);
 
-// The same picks with the sweep on the tensor cores (three bf16 products per correlation bound
-// it to a band; rows inside the band are re-scored in fp64).  `scratch`:
+// The same picks with the sweep on the tensor cores (an fp16 product bounds every correlation
+// to a band; rows inside the band are re-scored in fp64).  `scratch`:
 // encode_exact_tc_scratch_bytes() bytes, 1024-byte aligned; `status` receives kStatusTimeout;
-// `diag` is a device word that a build with CSR_DEBUG_CHECKS raises to the largest error of a
-// tensor-core correlation seen, relative to ||R|| (float bits).
+// `diag`: two device words that a build with CSR_DEBUG_CHECKS raises (see csr_debug_read; float bits).
 // Up to one row tile per SM the dictionary is split across the CTAs of one launch
 // (encode_exact_grid.cu); more rows run as whole waves of pairs of row tiles, one CTA each, and
 // what is left over the same way as few rows.  `pairs_only`: pairs of row tiles whatever M is.
 size_t encode_exact_tc_scratch_bytes(int64_t M, int d, int N);
 int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status, uint32_t* diag, bool pairs_only);
 // The split engine's pieces: CTAs per row tile (0: too many rows), scratch, counter words (zeroed by the
-// caller), launch on the dictionary's bf16 parts; kGridLaunchRefused when the driver refuses it.
+// caller), launch on the dictionary's scaled fp16 copy and its bounds; kGridLaunchRefused when the driver refuses it.
 constexpr int kGridLaunchRefused = 1;                      // internal: not a CSR_ERR_* code
 int exact_grid_slices(int64_t M, int N);
 size_t exact_grid_scratch_bytes(int64_t M, int d, int N);
 size_t exact_grid_counter_words(int64_t M);
-int launch_encode_exact_grid(const EncodeArgs& a, void* hi, void* lo, void* scratch, uint32_t* counters, uint32_t* status,
-                             uint32_t* diag);
+int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* dict_parts, int n_parts, void* scratch, uint32_t* counters,
+                             uint32_t* status, uint32_t* diag);
 
 // tcgen05 bf16 matching pursuit.  `workspace` holds the bf16 copy of D (N*d*2 bytes,
 // 1024-byte aligned); `status` is a device word that receives kStatusTimeout.

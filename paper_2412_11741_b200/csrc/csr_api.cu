@@ -63,7 +63,7 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 constexpr size_t kStatusBytes = 256;
-constexpr int kDiagWord = 2;              // word of the status block a checked build raises (see csr_debug_read)
+constexpr int kDiagWord = 2;              // first of the words of the status block a checked build raises (see csr_debug_read)
 constexpr uint32_t kDictMagic = 0x43535244u;   // "CSRD"
 
 // Library-owned, grow-only device buffers of one device.
@@ -971,7 +971,8 @@ int csr_set_option(const char* name, int64_t value) {
 
 int csr_debug_read(const char* name, double* value) {
     if (!name || !value) return fail(CSR_ERR_INVALID_ARG, "name or value is NULL");
-    if (strcmp(name, "exact_tensor_error") != 0) return fail(CSR_ERR_INVALID_ARG, "unknown quantity '%s'", name);
+    [[maybe_unused]] const int which = !strcmp(name, "exact_tensor_error") ? 0 : !strcmp(name, "exact_band_use") ? 1 : -1;
+    if (which < 0) return fail(CSR_ERR_INVALID_ARG, "unknown quantity '%s'", name);
 #ifndef CSR_DEBUG_CHECKS
     return fail(CSR_ERR_UNSUPPORTED, "only a library built with CSR_DEBUG_CHECKS records '%s'", name);
 #else
@@ -986,7 +987,7 @@ int csr_debug_read(const char* name, double* value) {
     }
     float v = 0.f;
     if (work) {
-        uint32_t* word = static_cast<uint32_t*>(work) + kDiagWord;
+        uint32_t* word = static_cast<uint32_t*>(work) + kDiagWord + which;
         e = cudaMemcpy(&v, word, sizeof(float), cudaMemcpyDeviceToHost);
         if (e == cudaSuccess) e = cudaMemset(word, 0, sizeof(uint32_t));
         if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "diagnostic read: %s", cudaGetErrorString(e));

@@ -5,19 +5,20 @@
 // few rows leaves all but a few SMs idle and takes s whole sweeps all the same.  Here the grid is
 // (row tiles) x (slices of the dictionary), at most one CTA per SM, and all s iterations run in one
 // launch.  Per iteration
-//   - every CTA loads the bf16 high and low parts of its tile's 128 residual rows (64 KB from the
-//     L2), multiplies them with its slice by the same three bf16 products per correlation, and
-//     every thread keeps the four largest keys of its half row (drain as in encode_exact_tc.cu);
+//   - every CTA loads its tile's 128 residual rows as fp16 (32 KB from the L2), multiplies them with
+//     its slice by the same fp16 product per correlation, and every thread keeps the five
+//     largest keys of its half row (drain as in encode_exact_tc.cu);
 //   - the keys go to a scratch array, the CTAs of the row tile meet (counter in global memory,
 //     bounded wait);
 //   - the rows of the tile are dealt out to its CTAs, eight lanes settle a row: the largest key
 //     over all slices, everything inside the band re-scored in fp64, fp64 coefficient and residual
-//     update; the new high and low parts go back to the scratch array and the CTAs meet again.
-// The fp64 rows, bands and parts live in L2-resident scratch.  The dictionary stages of the next
+//     update; the new fp16 rows go back to the scratch array and the CTAs meet again.
+// The fp64 rows, bands and fp16 rows live in L2-resident scratch.  The dictionary stages of the next
 // iteration are fetched while the rows are being settled.
 //
 // What bounds it: with few rows the chain of dependent steps (A load, MMA, drain, meeting, settle,
-// meeting: 10 to 11 us an iteration at 16 to 128 rows, N = 8192), with many the MMAs, 3072 cycles per 256 atoms and row tile.
+// meeting: 9 to 10 us an iteration at 16 to 128 rows, N = 8192), with many the drain.  128 rows, N = 8192, s = 16: 180 us
+// with three bf16 products per correlation, 158 us with one fp16 product.
 // The grid is launched cooperatively whenever a row tile has more than one CTA, so all CTAs that
 // wait for one another are resident.
 #include "exact_tc_common.cuh"
@@ -36,18 +37,18 @@ constexpr int UNIT = 64;                                  // atoms per TMA box; 
 constexpr int MAX_SLICES = TILE_M;                        // at most one CTA per row
 constexpr int CAND = 16;                                  // candidates a row may have before the whole dictionary is re-scored
 
-// Keys of one row over one column half of a slice: the four largest and the atoms of the first three.
-struct __align__(8) Entry {
+// Keys of one row over one column half of a slice: the five largest and the atoms of the first four.
+struct __align__(16) Entry {
     uint32_t k[4];
-    uint32_t n01, n2;
+    uint32_t k4, n01, n23, pad;
 };
 
 template <int D_>
 struct GridSmem {
-    static constexpr int kStages = D_ == 128 ? 4 : 5;
+    static constexpr int kStages = 5;
     static constexpr int kATileBytes = TILE_M * D_ * 2;
     static constexpr int kStageBytes = TILE_N * STAGE_CH * 2;
-    alignas(1024) uint8_t A[2][kATileBytes];              // [high, low]
+    alignas(1024) uint8_t A[kATileBytes];
     alignas(1024) uint8_t B[kStages][kStageBytes];
     // of the rows settled here: the largest key, the atoms inside the band, their number
     uint32_t top_key[TILE_M];
@@ -78,9 +79,10 @@ struct GridArgs {
     int coef_dtype;
     int64_t ldc;
     double* Rd;             // [tiles * 128][d] fp64 residual rows
-    uint32_t* Rh;           // [tiles * 128][d / 2] bf16 high parts of the scaled rows, two channels per word
-    uint32_t* Rl;           // low parts
-    float* band;            // [tiles * 128] of the scaled rows
+    uint32_t* Rh;           // [tiles * 128][d / 2] the scaled rows as fp16, two channels per word
+    float2* band;           // [tiles * 128] band and norm of the scaled rows
+    const DictPart* parts;  // [n_parts] bounds of the dictionary
+    int n_parts;
     Entry* entries;         // [tiles][128][2 * slices]
     uint32_t* counters;     // [tiles * 32], zero at launch
     int slices;
@@ -125,7 +127,7 @@ __device__ __forceinline__ bool meet(uint32_t* counter, uint32_t target, int sli
 
 template <int D_>
 __global__ void __launch_bounds__(NT, 1)
-encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid_constant__ CUtensorMap tmap_lo, const GridArgs a) {
+encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridArgs a) {
     using S = GridSmem<D_>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     if ((smem_u32(smem_raw) & 1023u) != 0) {              // the swizzled tiles need this; never seen otherwise
@@ -145,7 +147,6 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
     constexpr int KH = D_ / STAGE_CH;
     constexpr int KSTEPS = STAGE_CH / UMMA_K;
     constexpr int STAGES = S::kStages;
-    constexpr int NSTG = 2 * KH;
     const WaitCtx wc{&sm.abort, a.status, a.wait_limit_ns};
 
     if (threadIdx.x == 0) {
@@ -174,14 +175,13 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
     if (warp == PRODUCER_WARP) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_hi)) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_lo)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_d)) : "memory");
             uint32_t p = 0;
             bool ok = true;
             for (int g = 0; g < a.s && ok; ++g) {
                 for (int t = 0; t < T && ok; ++t) {
                     const int w = min(TILE_N, width - t * TILE_N);
-                    for (int hp = 0; hp < NSTG; ++hp, ++p) {
+                    for (int h = 0; h < KH; ++h, ++p) {
                         const int stage = p % STAGES;
                         if (!wait_bounded_suspended(&sm.empty_b[stage], ((p / STAGES) & 1) ^ 1, wc, 2000)) {
                             ok = false;
@@ -190,8 +190,8 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                         // atoms past N arrive as zeros and count as bytes
                         mbar_expect_tx(&sm.full_b[stage], static_cast<uint32_t>(w) * STAGE_CH * 2);
                         for (int u = 0; u < w / UNIT; ++u)
-                            tma_load_2d(&sm.B[stage][u * (UNIT * STAGE_CH * 2)], (hp & 1) ? &tmap_lo : &tmap_hi, (hp >> 1) * STAGE_CH,
-                                        n_first + t * TILE_N + u * UNIT, &sm.full_b[stage]);
+                            tma_load_2d(&sm.B[stage][u * (UNIT * STAGE_CH * 2)], &tmap_d, h * STAGE_CH, n_first + t * TILE_N + u * UNIT,
+                                        &sm.full_b[stage]);
                     }
                 }
             }
@@ -206,7 +206,7 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         {
             uint32_t p = 0, accn = 0;
@@ -216,37 +216,28 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                     ok = false;
                     break;
                 }
-                for (int t = 0; t < T && ok; ++t, ++accn, p += NSTG) {
+                for (int t = 0; t < T && ok; ++t, ++accn, p += KH) {
                     const int acc = accn & 1;             // the accumulators take the tiles in turn
-                    const uint32_t idesc = instr_desc_bf16(TILE_M, min(TILE_N, width - t * TILE_N));
+                    const uint32_t idesc = instr_desc_f16(TILE_M, min(TILE_N, width - t * TILE_N));
                     if (!warp_wait_bounded(&sm.acc_empty[acc], ((accn >> 1) & 1) ^ 1, wc)) {
                         ok = false;
                         break;
                     }
                     const uint32_t d_tmem = tmem_d + acc * TILE_N;
-                    for (int hp = 0; hp < NSTG; ++hp) {
-                        const uint32_t ps = p + hp;
+                    for (int h = 0; h < KH; ++h) {
+                        const uint32_t ps = p + h;
                         const int stage = ps % STAGES;
-                        const int h = hp >> 1;
                         if (!warp_wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                         const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
-                        const uint64_t ah = make_smem_desc(smem_u32(&sm.A[0][h * (TILE_M * 128)]));
-                        const uint64_t al = make_smem_desc(smem_u32(&sm.A[1][h * (TILE_M * 128)]));
+                        const uint64_t a0 = make_smem_desc(smem_u32(&sm.A[h * (TILE_M * 128)]));
 #pragma unroll
                         for (int k = 0; k < KSTEPS; ++k) {
                             const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                            umma_bf16(d_tmem, ah + off, b0 + off, idesc, (hp | k) ? 1u : 0u);
-                        }
-                        if ((hp & 1) == 0) {              // high parts of the atoms: the low parts of the rows meet them too
-#pragma unroll
-                            for (int k = 0; k < KSTEPS; ++k) {
-                                const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                                umma_bf16(d_tmem, al + off, b0 + off, idesc, 1u);
-                            }
+                            umma_f16(d_tmem, a0 + off, b0 + off, idesc, (h | k) ? 1u : 0u);
                         }
                         umma_commit(&sm.empty_b[stage]);
                     }
@@ -272,26 +263,26 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
         // rows settled here: slice, slice + slices, ...; the k-th by warp k % 8, lane group k / 8 % 4, pass k / 32
         const int n_own = rows_here > slice ? (rows_here - slice + slices - 1) / slices : 0;
         const int n_ent = 2 * slices;                     // entries of a row
+        const DictBounds db = dict_bounds(a.parts, a.n_parts, lane);
         uint32_t* counter = a.counters + tile * 32;
         uint32_t target = 0;
         bool ok = true;
         uint32_t accn = 0;
-        // An fp64 row, the parts of its scaled form and its band to the scratch arrays, by the eight lanes of a row (all lanes
+        // An fp64 row, its scaled form as fp16 and its band to the scratch arrays, by the eight lanes of a row (all lanes
         // of the warp call; only those with `has` write).
         auto put_row = [&](const double (&R)[CH], int64_t row, bool has) {
-            const double nn = group8_sum(norm2_share<CH>(R));
-            if (!has) return;
-            float band;
-            const double scale = row_scale(nn, band);
+            float norm, err2 = 0.f;
+            const double scale = row_scale(group8_sum(norm2_share<CH>(R)), norm);
 #pragma unroll
             for (int k = 0; k < CH / 2; ++k) {
-                uint32_t hi, lo;
-                split_pair(R[2 * k] * scale, R[2 * k + 1] * scale, hi, lo);
-                __stcg(reinterpret_cast<double2*>(a.Rd + row * D_) + 8 * k + l8, make_double2(R[2 * k], R[2 * k + 1]));
-                __stcg(a.Rh + row * (D_ / 2) + 8 * k + l8, hi);
-                __stcg(a.Rl + row * (D_ / 2) + 8 * k + l8, lo);
+                const uint32_t w = round_pair(R[2 * k] * scale, R[2 * k + 1] * scale, err2);
+                if (has) {
+                    __stcg(reinterpret_cast<double2*>(a.Rd + row * D_) + 8 * k + l8, make_double2(R[2 * k], R[2 * k + 1]));
+                    __stcg(a.Rh + row * (D_ / 2) + 8 * k + l8, w);
+                }
             }
-            if (l8 == 0) __stcg(a.band + row, band);
+            err2 = group8_sumf(err2);
+            if (has && l8 == 0) __stcg(a.band + row, make_float2(row_band(norm, err2, db), norm));
         };
         // ---- R_0 = x ----
         for (int k0 = 0; k0 < n_own; k0 += EPI / 8) {
@@ -306,29 +297,29 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
         ok = meet(counter, target += slices, slices, ok, wc);
 
         for (int g = 0; g < a.s && ok; ++g) {
-            // ---- the residual's parts into the operand tiles (rows past M: zeros, once) ----
+            // ---- the residual into the operand tile (rows past M: zeros, once) ----
             constexpr int CPR = D_ / 8;                   // 16-byte chunks of a row
-            constexpr int PER = 2 * TILE_M * CPR / EPI;
+            constexpr int PER = TILE_M * CPR / EPI;
             uint4 v[PER];
 #pragma unroll
             for (int u = 0; u < PER; ++u) {
                 const int f = threadIdx.x + u * EPI;
-                const int part = f / (TILE_M * CPR), r = f / CPR % TILE_M, c = f % CPR;
+                const int r = f / CPR, c = f % CPR;
                 v[u] = make_uint4(0u, 0u, 0u, 0u);
-                if (r < rows_here) v[u] = __ldcg(reinterpret_cast<const uint4*>((part ? a.Rl : a.Rh) + (row_base + r) * (D_ / 2)) + c);
+                if (r < rows_here) v[u] = __ldcg(reinterpret_cast<const uint4*>(a.Rh + (row_base + r) * (D_ / 2)) + c);
             }
-            const float band_own = r_own < rows_here ? __ldcg(a.band + row_base + r_own) : 0.f;
+            const float band_own = r_own < rows_here ? __ldcg(&a.band[row_base + r_own].x) : 0.f;
 #pragma unroll
             for (int u = 0; u < PER; ++u) {
                 const int f = threadIdx.x + u * EPI;
-                const int part = f / (TILE_M * CPR), r = f / CPR % TILE_M, c = f % CPR;
-                if (g == 0 || r < rows_here) *reinterpret_cast<uint4*>(&sm.A[part][swz_off(r, c)]) = v[u];
+                const int r = f / CPR, c = f % CPR;
+                if (g == 0 || r < rows_here) *reinterpret_cast<uint4*>(&sm.A[swz_off(r, c)]) = v[u];
             }
             fence_proxy_async_smem();
             mbar_arrive(&sm.res_ready);
 
-            // ---- sweep of this slice: top four keys of this thread's half row ----
-            Top4 top{0u, 0u, 0u, 0u, 0u, 0u, 0u};
+            // ---- sweep of this slice: top five keys of this thread's half row ----
+            Top5 top = top5_none();
             const float fband = band_own > 0.f ? band_own * 1.0625f : -1.f;
             for (int t = 0; t < T; ++t, ++accn) {
                 const int acc = accn & 1;
@@ -341,19 +332,18 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                 tc_fence_after();
                 const int w = min(TILE_N, width - t * TILE_N);
                 const uint32_t ta = taddr + acc * TILE_N + half * (w / 2);
-                const uint32_t id = static_cast<uint32_t>(2 * t + half);
                 uint64_t* back = &sm.acc_empty[acc];
-                drain(ta, w / UNIT, top, id, fband, back, lane);
+                drain(ta, w / UNIT, top, static_cast<uint32_t>(t), fband, back, lane);
             }
             if (ok && r_own < rows_here) {
                 auto atom = [&](uint32_t key, uint32_t id) {      // (an empty key's place is never used)
-                    const int t = static_cast<int>(id >> 1), w = min(TILE_N, width - t * TILE_N);
-                    return static_cast<uint32_t>(n_first + t * TILE_N + static_cast<int>(id & 1) * (w / 2) + 127 - static_cast<int>(key & 127u)) & 0xFFFFu;
+                    const int t = static_cast<int>(id), w = min(TILE_N, width - t * TILE_N);
+                    return static_cast<uint32_t>(n_first + t * TILE_N + half * (w / 2) + 127 - static_cast<int>(key & 127u)) & 0xFFFFu;
                 };
-                uint2* e = reinterpret_cast<uint2*>(a.entries + ((row_base + r_own) * n_ent + 2 * slice + half));
-                __stcg(e + 0, make_uint2(top.k0, top.k1));
-                __stcg(e + 1, make_uint2(top.k2, top.k3));
-                __stcg(e + 2, make_uint2(atom(top.k0, top.i0) | (atom(top.k1, top.i1) << 16), atom(top.k2, top.i2)));
+                uint4* e = reinterpret_cast<uint4*>(a.entries + ((row_base + r_own) * n_ent + 2 * slice + half));
+                __stcg(e + 0, make_uint4(top.k0, top.k1, top.k2, top.k3));
+                __stcg(e + 1, make_uint4(top.k4, atom(top.k0, top.i0) | (atom(top.k1, top.i1) << 16),
+                                         atom(top.k2, top.i2) | (atom(top.k3, top.i3) << 16), 0u));
             }
             ok = meet(counter, target += slices, slices, ok, wc);
             if (!ok) break;
@@ -362,7 +352,7 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
             // (an entry per thread and trip, at most two trips: rows x 2 slices <= 2 (127 + slices))
             constexpr int TRIPS = 2;
             Entry mine[TRIPS];
-            float band_of[TRIPS];
+            float2 band_of[TRIPS];
             if (threadIdx.x < TILE_M / 32) sm.unknown[threadIdx.x] = 0u;
             if (threadIdx.x < TILE_M) {
                 sm.top_key[threadIdx.x] = 0u;
@@ -371,13 +361,13 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
 #pragma unroll
             for (int u = 0; u < TRIPS; ++u) {
                 const int f = threadIdx.x + u * EPI;
-                mine[u] = Entry{{0u, 0u, 0u, 0u}, 0u, 0u};
-                band_of[u] = 0.f;
+                mine[u] = Entry{{0u, 0u, 0u, 0u}, 0u, 0u, 0u, 0u};
+                band_of[u] = make_float2(0.f, 0.f);
                 if (f < n_own * n_ent) {
                     const int64_t row = row_base + slice + f / n_ent * slices;
-                    const uint2* e = reinterpret_cast<const uint2*>(a.entries + (row * n_ent + f % n_ent));
-                    const uint2 e0 = __ldcg(e), e1 = __ldcg(e + 1), e2 = __ldcg(e + 2);
-                    mine[u] = Entry{{e0.x, e0.y, e1.x, e1.y}, e2.x, e2.y};
+                    const uint4* e = reinterpret_cast<const uint4*>(a.entries + (row * n_ent + f % n_ent));
+                    const uint4 e0 = __ldcg(e), e1 = __ldcg(e + 1);
+                    mine[u] = Entry{{e0.x, e0.y, e0.z, e0.w}, e1.x, e1.y, e1.z, 0u};
                     band_of[u] = __ldcg(a.band + row);
                 }
             }
@@ -393,14 +383,14 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                 const int f = threadIdx.x + u * EPI;
                 if (f >= n_own * n_ent) continue;
                 const int k = f / n_ent;
-                const float v0 = __uint_as_float(sm.top_key[k] & kKeyMask), band = band_of[u];
+                const float v0 = __uint_as_float(sm.top_key[k] & kKeyMask), band = band_of[u].x;
                 if (!(v0 > 0.f) || a.N == 1 || v0 - __uint_as_float(mine[u].k[0] & kKeyMask) > band) continue;
-                // four of a half slice inside the band: there may be more; a band above everything: anything may be the pick
-                bool full = !(v0 > band) || (mine[u].k[3] != 0u && !(v0 - __uint_as_float(mine[u].k[3] & kKeyMask) > band));
+                // five of a half slice inside the band: there may be more; a band above everything: anything may be the pick
+                bool full = !(v0 > band) || (mine[u].k4 != 0u && !(v0 - __uint_as_float(mine[u].k4 & kKeyMask) > band));
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const uint32_t key = mine[u].k[i];
-                    const uint32_t n = i == 0 ? mine[u].n01 & 0xFFFFu : i == 1 ? mine[u].n01 >> 16 : mine[u].n2;
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t key = mine[u].k[i], n2 = i < 2 ? mine[u].n01 : mine[u].n23;
+                    const uint32_t n = (i & 1) ? n2 >> 16 : n2 & 0xFFFFu;
                     if (key != 0u && !(v0 - __uint_as_float(key & kKeyMask) > band) && n < static_cast<uint32_t>(a.N)) {
                         const int slot = atomicAdd(&sm.n_cand[k], 1);
                         if (slot < CAND)
@@ -411,7 +401,7 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                 }
                 if (full) {
                     atomicOr(&sm.unknown[k >> 5], 1u << (k & 31));
-                    sm.limit[k] = relative_limit(v0, band);   // (every writer of a row writes the same)
+                    sm.limit[k] = relative_limit(v0, band, band_of[u].y, db);   // (every writer of a row writes the same)
                 }
             }
             epilogue_barrier();
@@ -446,8 +436,6 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                         R[2 * c] = x.x;
                         R[2 * c + 1] = x.y;
                     }
-                    const float band = __ldcg(a.band + row);
-                    const float v0 = __uint_as_float(sm.top_key[kk] & kKeyMask);
                     const bool open = (sm.unknown[kk >> 5] >> (kk & 31)) & 1u;
                     int cnt = min(sm.n_cand[kk], CAND);   // none: an all-zero sweep (or NaN, or one atom) picks atom 0
                     int n = cnt > 0 ? sm.cand[kk][0] : 0;
@@ -480,9 +468,8 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __gr
                     load_atom<CH>(a.D + static_cast<int64_t>(n) * D_, l8, at);
                     const double c = group8_sum(slice_dot<CH>(R, at));
 #ifdef CSR_DEBUG_CHECKS
-                    const double nr = sqrt(group8_sum(norm2_share<CH>(R)));   // as in encode_exact_tc.cu
-                    if (l8 == 0 && has && cnt == 1 && band > 0.f)
-                        atomicMax(a.diag, __float_as_uint(fabsf(v0 / (band / (kBandRel * 1.001f)) - static_cast<float>(fabs(c) / nr))));
+                    const float2 bn = __ldcg(a.band + row);
+                    check_value<CH>(a.diag, R, at, c, __uint_as_float(sm.top_key[kk] & kKeyMask), bn.x, bn.y, db, l8, has && round == 0 && cnt == 1);
 #endif
                     if (l8 == 0 && has) {
                         a.out_idx[row * a.ldc + g] = static_cast<uint16_t>(n);
@@ -516,7 +503,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 int tiles_of(int64_t M) { return static_cast<int>((M + TILE_M - 1) / TILE_M); }
 
 template <int D_>
-int run(const CUtensorMap& mh, const CUtensorMap& ml, const GridArgs& g, int grid, cudaStream_t stream) {
+int run(const CUtensorMap& map, const GridArgs& g, int grid, cudaStream_t stream) {
     const size_t smem = sizeof(GridSmem<D_>);
     cudaError_t e = cudaFuncSetAttribute(encode_exact_grid_kernel<D_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
@@ -530,7 +517,7 @@ int run(const CUtensorMap& mh, const CUtensorMap& ml, const GridArgs& g, int gri
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g.slices > 1 ? 1 : 0;                  // a lone CTA per row tile waits for nobody
-    e = cudaLaunchKernelEx(&cfg, encode_exact_grid_kernel<D_>, mh, ml, g);
+    e = cudaLaunchKernelEx(&cfg, encode_exact_grid_kernel<D_>, map, g);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return kGridLaunchRefused;                        // nothing ran: the caller takes the other engine
@@ -550,12 +537,12 @@ int exact_grid_slices(int64_t M, int N) {
 
 size_t exact_grid_scratch_bytes(int64_t M, int d, int N) {
     const size_t rows = (size_t)tiles_of(M) * TILE_M;
-    return rows * d * 8 + 2 * rows * d * 2 + align256(rows * 4) + align256(rows * 2 * exact_grid_slices(M, N) * sizeof(Entry));
+    return rows * d * 8 + rows * d * 2 + align256(rows * 8) + align256(rows * 2 * exact_grid_slices(M, N) * sizeof(Entry));
 }
 size_t exact_grid_counter_words(int64_t M) { return (size_t)tiles_of(M) * 32; }
 
-int launch_encode_exact_grid(const EncodeArgs& a, void* hi, void* lo, void* scratch, uint32_t* counters, uint32_t* status,
-                             uint32_t* diag) {
+int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* dict_parts, int n_parts, void* scratch, uint32_t* counters,
+                             uint32_t* status, uint32_t* diag) {
     const size_t rows = (size_t)tiles_of(a.M) * TILE_M;
     char* p = static_cast<char*>(scratch);
     GridArgs g;
@@ -574,21 +561,20 @@ int launch_encode_exact_grid(const EncodeArgs& a, void* hi, void* lo, void* scra
     p += rows * a.d * 8;
     g.Rh = reinterpret_cast<uint32_t*>(p);
     p += rows * a.d * 2;
-    g.Rl = reinterpret_cast<uint32_t*>(p);
-    p += rows * a.d * 2;
-    g.band = reinterpret_cast<float*>(p);
-    p += align256(rows * 4);
+    g.band = reinterpret_cast<float2*>(p);
+    p += align256(rows * 8);
+    g.parts = static_cast<const DictPart*>(dict_parts);
+    g.n_parts = n_parts;
     g.entries = reinterpret_cast<Entry*>(p);
     g.counters = counters;
     g.slices = exact_grid_slices(a.M, a.N);
     g.status = status;
     g.diag = diag;
     g.wait_limit_ns = options().wait_limit_ns;
-    CUtensorMap mh, ml;
-    if (int rc = part_map(&mh, hi, a.N, a.d, UNIT)) return rc;
-    if (int rc = part_map(&ml, lo, a.N, a.d, UNIT)) return rc;
+    CUtensorMap map;
+    if (int rc = dict_map(&map, dict_f16, a.N, a.d, UNIT)) return rc;
     const int grid = tiles_of(a.M) * g.slices;
-    return a.d == 128 ? run<128>(mh, ml, g, grid, a.stream) : run<64>(mh, ml, g, grid, a.stream);
+    return a.d == 128 ? run<128>(map, g, grid, a.stream) : run<64>(map, g, grid, a.stream);
 }
 
 }  // namespace csr

@@ -1,39 +1,34 @@
 // Correctness-mode matching pursuit (paper Eq. 2-4) with the sweep on the sm_100a tensor cores.
 //
-// The picks must be those of an fp64 evaluation of the pursuit.  A bf16 product cannot decide
-// them, but three can bound them: with r = rh + rl and d = dh + dl (each part bf16, the low part
-// the rounded remainder), rh*dh + rl*dh + rh*dl differs from r*d by at most 3 * 2^-18 |r d| per
-// channel, so the sum over the channels is within 1.2e-5 ||R|| ||d|| of the exact correlation; the
-// tensor core adds the exact bf16 products in fp32.  Every correlation of a sweep is therefore
-// known to within a band of a few 1e-5 ||R||, which decides all rows but the few whose two
-// largest |correlations| are closer than that; for those the candidates are re-scored in fp64.
+// The picks must be those of an fp64 evaluation of the pursuit.  An fp16 product cannot decide
+// them, but it can bound them: with r = r' + e and d = d' + f (r', d' the fp16 values the tensor cores
+// read), a correlation r.d differs from r'.d' by at most ||e|| max ||d|| + ||r'|| max ||f||, and all of these
+// norms are known (row_band in exact_tc_common.cuh): about 4e-4 ||R||, plus what the fp32 accumulation adds.
+// So every correlation of a sweep is known to within a band of about 8e-4 ||R||, which decides 95 % of
+// the rows; for the others the candidates inside the band are re-scored in fp64.
 //
 // One persistent CTA per SM owns two tiles of 128 rows for all s iterations:
 //   - the fp64 residuals live in a per-CTA scratch area in global memory (256 KB, L2 resident);
-//     the bf16 high and low parts of the row, scaled by a power of two to a norm in [1, 2), are the
-//     tcgen05.mma A operands in shared memory (K-major, 128-byte swizzle, 2 row tiles x 2 parts);
-//   - the dictionary's high and low parts (two bf16 arrays made once per call) stream through a
-//     ring of 32 KB stages fetched by TMA: 64 channels of 256 atoms of one part per stage.  A
-//     stage of high parts feeds four groups of MMAs (both parts of both row tiles), a stage of low
-//     parts two (the high parts of both row tiles);
+//     the rows as fp16, scaled by a power of two to a norm in [1, 2), are the
+//     tcgen05.mma A operands in shared memory (K-major, 128-byte swizzle, 2 row tiles);
+//   - the dictionary's fp16 copy (made once per call) streams through a ring of 32 KB stages fetched
+//     by TMA: 64 channels of 256 atoms per stage, used by both row tiles;
 //   - each row tile has one 256-column fp32 accumulator in TMEM.  All eight epilogue warps drain
 //     every accumulator: warp w reads the 32 TMEM lanes of w % 4 and the 128 columns of w / 4, i.e.
 //     all of them sit in registers after one round of loads and the accumulator goes straight back
-//     to the tensor core.  Each thread keeps the four largest keys of its half row, a key being
+//     to the tensor core.  Each thread keeps the five largest keys of its half row, a key being
 //     |value| with its seven lowest mantissa bits replaced by the column's tag, and where the
-//     largest three came from.  Groups of eight values are first reduced to their largest
+//     largest four came from.  Groups of eight values are first reduced to their largest
 //     magnitude and only groups within the band of the running maximum are inserted;
 //   - at the end of a sweep the halves meet in shared memory, and each warp settles its 32 rows,
 //     eight lanes per row: rows whose best and second-best keys are further apart than the band
-//     take the best; otherwise the candidates inside the band (the first three of either half)
-//     are compared in fp64; rows where the fourth of a half is inside too are searched for in the
+//     take the best; otherwise the candidates inside the band (the first four of either half)
+//     are compared in fp64; rows where the fifth of a half is inside too are searched for in the
 //     whole dictionary (fp32 filter, then fp64) by the eight warps together.  Coefficient (Eq. 2,
 //     signed) and residual update (Eq. 4) are fp64, as in the plain-ALU encoder.
-// What bounds it: the MMAs (6144 cycles per 256 atoms and pair of row tiles; the operand reads from
-// shared memory take 165 cycles per 128 x 256 x 16 MMA instead of 128) and about 30 us per sweep
-// for the settling of 256 rows.  Rows with more candidates than known used to be the
-// warp's own job, 450 us for N = 4096, about once in 300000 row-steps: a wave of 37888 rows took 765
-// or 1210 us; it takes 750 us now.
+// What bounds it: the epilogue and the settling, no longer the MMAs (2048 cycles per 256 atoms and pair of row tiles).
+// Three bf16 products per correlation, whose band was 2^-12 ||R||, took 6144: 100000 rows, N = 4096, s = 8,
+// 2441 us so and 2195 us with one fp16 product; a training step of 65536 rows (N = 8192, s = 8) 2992 and 2332 us.
 // Warp roles: 0-7 epilogue, 8 TMA producer, 9 TMEM owner and MMA issuer.  All waits are bounded.
 #include "exact_tc_common.cuh"
 
@@ -47,19 +42,16 @@ constexpr int PRODUCER_WARP = 8;
 constexpr int MMA_WARP = 9;
 constexpr int ROWS = 2 * TILE_M;                          // rows a CTA holds at a time
 constexpr uint32_t TMEM_COLS = 512;
-constexpr uint32_t kInstrDesc = instr_desc_bf16(TILE_M, TILE_N);
-#ifndef CSR_TC_GROUP128
-#define CSR_TC_GROUP128 2                                 // measured: 12-17 % faster than 1 at d = 128
-#endif
+constexpr uint32_t kInstrDesc = instr_desc_f16(TILE_M, TILE_N);
 
 template <int D_>
 struct TcSmem {
-    static constexpr int kStages = D_ == 128 ? 3 : 4;
-    static constexpr int kATileBytes = TILE_M * D_ * 2;          // one part of one row tile
+    static constexpr int kStages = D_ == 128 ? 4 : 5;
+    static constexpr int kATileBytes = TILE_M * D_ * 2;
     static constexpr int kStageBytes = TILE_N * STAGE_CH * 2;
-    alignas(1024) uint8_t A[2][2][kATileBytes];                  // [row tile][high, low]
+    alignas(1024) uint8_t A[2][kATileBytes];
     alignas(1024) uint8_t B[kStages][kStageBytes];
-    uint32_t xchg[5][TILE_M];                                    // one half's top four of a row tile (and the rows' bands)
+    uint32_t xchg[6][TILE_M];                                    // one half's top five of a row tile (and the rows' bands)
     uint64_t full_b[kStages];
     uint64_t empty_b[kStages];
     uint64_t acc_full[2];
@@ -72,8 +64,7 @@ struct TcSmem {
 
 template <int D_>
 __global__ void __launch_bounds__(NT, 1)
-encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid_constant__ CUtensorMap tmap_lo,
-                       const float* __restrict__ D, const void* __restrict__ X, int x_dtype, int64_t ldx, int64_t M, int N, int s,
+encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPart* __restrict__ parts, int n_parts, const float* __restrict__ D, const void* __restrict__ X, int x_dtype, int64_t ldx, int64_t M, int N, int s,
                        uint16_t* __restrict__ out_idx, void* __restrict__ out_coef, int coef_dtype, int64_t ldc,
                        double* __restrict__ Rd_all, uint32_t* status, [[maybe_unused]] uint32_t* diag,
                        unsigned long long wait_limit_ns) {
@@ -92,9 +83,6 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
     constexpr int KH = D_ / STAGE_CH;                       // 64-channel blocks per row
     constexpr int KSTEPS = STAGE_CH / UMMA_K;
     constexpr int STAGES = S::kStages;
-    constexpr int NSTG = 2 * KH;                            // stages per dictionary tile
-    constexpr int GROUP = STAGES >= NSTG + 2 ? NSTG : CSR_TC_GROUP128;
-    static_assert(GROUP < STAGES && NSTG % GROUP == 0, "a group of stages must fit the ring with one stage to spare");
     const WaitCtx wc{&sm.abort, status, wait_limit_ns};
 
     if (threadIdx.x == 0) {
@@ -123,14 +111,13 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
     if (warp == PRODUCER_WARP) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_hi)) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_lo)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_d)) : "memory");
             uint32_t p = 0;
             bool ok = true;
             for (int64_t pair = blockIdx.x; pair < n_pairs && ok; pair += gridDim.x) {
                 for (int g = 0; g < s && ok; ++g) {
                     for (int t = 0; t < T && ok; ++t) {
-                        for (int hp = 0; hp < 2 * KH; ++hp, ++p) {
+                        for (int h = 0; h < KH; ++h, ++p) {
                             const int stage = p % STAGES;
                             if (!wait_bounded_suspended(&sm.empty_b[stage], ((p / STAGES) & 1) ^ 1, wc, 2000)) {
                                 ok = false;
@@ -138,8 +125,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                             }
                             // atoms past N arrive as zeros and count as bytes
                             mbar_expect_tx(&sm.full_b[stage], S::kStageBytes);
-                            tma_load_2d(&sm.B[stage][0], (hp & 1) ? &tmap_lo : &tmap_hi, (hp >> 1) * STAGE_CH, t * TILE_N,
-                                        &sm.full_b[stage]);
+                            tma_load_2d(&sm.B[stage][0], &tmap_d, h * STAGE_CH, t * TILE_N, &sm.full_b[stage]);
                         }
                     }
                 }
@@ -155,7 +141,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         {
             uint32_t p = 0, accn = 0, steps = 0;
@@ -166,48 +152,34 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                         ok = false;
                         break;
                     }
-                    // A dictionary tile is NSTG stages (high and low parts of each 64-channel block).
-                    // Each row tile takes GROUP stages in a row before the other takes the same ones,
-                    // and a stage goes back to the producer after the second row tile's use: the
-                    // larger the group, the further apart the two accumulators complete (the epilogue
-                    // drains them one after the other), at the price of a shorter prefetch distance.
-                    for (int t = 0; t < T && ok; ++t, ++accn, p += NSTG) {
-                        for (int hp0 = 0; hp0 < NSTG && ok; hp0 += GROUP) {
-                            for (int tile = 0; tile < 2 && ok; ++tile) {
-                                for (int hp = hp0; hp < hp0 + GROUP; ++hp) {
-                                    const uint32_t ps = p + hp;
-                                    const int stage = ps % STAGES;
-                                    const int h = hp >> 1;
-                                    const bool low = hp & 1;      // this stage holds low parts of the atoms
-                                    if (tile == 0 && !warp_wait_bounded_suspended(&sm.full_b[stage], (ps / STAGES) & 1, wc, 1000)) {
-                                        ok = false;
-                                        break;
-                                    }
-                                    if (hp == 0 && !warp_wait_bounded_suspended(&sm.acc_empty[tile], (accn & 1) ^ 1, wc, 1000)) {
-                                        ok = false;
-                                        break;
-                                    }
-                                    tc_fence_after();
-                                    const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
-                                    const uint32_t d_tmem = tmem_d + tile * TILE_N;
-                                    const uint64_t ah = make_smem_desc(smem_u32(&sm.A[tile][0][h * (TILE_M * 128)]));
-                                    const uint64_t al = make_smem_desc(smem_u32(&sm.A[tile][1][h * (TILE_M * 128)]));
-#pragma unroll
-                                    for (int k = 0; k < KSTEPS; ++k) {
-                                        const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                                        umma_bf16(d_tmem, ah + off, b0 + off, kInstrDesc, (hp | k) ? 1u : 0u);
-                                    }
-                                    if (!low) {
-#pragma unroll
-                                        for (int k = 0; k < KSTEPS; ++k) {
-                                            const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                                            umma_bf16(d_tmem, al + off, b0 + off, kInstrDesc, 1u);
-                                        }
-                                    }
-                                    if (tile == 1) umma_commit(&sm.empty_b[stage]);
-                                    if (hp == NSTG - 1) umma_commit(&sm.acc_full[tile]);
-                                }
+                    // Each row tile takes all stages of a dictionary tile before the other takes the same ones: the
+                    // accumulators then complete a whole tile's MMAs apart, and the epilogue drains them one
+                    // after the other.
+                    for (int t = 0; t < T && ok; ++t, ++accn, p += KH) {
+                        for (int tile = 0; tile < 2 && ok; ++tile) {
+                            if (!warp_wait_bounded_suspended(&sm.acc_empty[tile], (accn & 1) ^ 1, wc, 1000)) {
+                                ok = false;
+                                break;
                             }
+                            const uint32_t d_tmem = tmem_d + tile * TILE_N;
+                            for (int h = 0; h < KH; ++h) {
+                                const uint32_t ps = p + h;
+                                const int stage = ps % STAGES;
+                                if (tile == 0 && !warp_wait_bounded_suspended(&sm.full_b[stage], (ps / STAGES) & 1, wc, 1000)) {
+                                    ok = false;
+                                    break;
+                                }
+                                tc_fence_after();
+                                const uint64_t a0 = make_smem_desc(smem_u32(&sm.A[tile][h * (TILE_M * 128)]));
+                                const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
+#pragma unroll
+                                for (int k = 0; k < KSTEPS; ++k) {
+                                    const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
+                                    umma_f16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
+                                }
+                                if (tile == 1) umma_commit(&sm.empty_b[stage]);
+                            }
+                            if (ok) umma_commit(&sm.acc_full[tile]);
                         }
                     }
                 }
@@ -229,12 +201,24 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
         const int l8 = lane & 7, grp = lane >> 3;
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + half * 128;
         double* Rd_cta = Rd_all + static_cast<int64_t>(blockIdx.x) * ROWS * D_;
-        uint8_t* Ahi = &sm.A[own_tile][0][0];
-        uint8_t* Alo = &sm.A[own_tile][1][0];
+        uint8_t* A_own = &sm.A[own_tile][0];
+        const DictBounds db = dict_bounds(parts, n_parts, lane);
         uint32_t accn = 0;
         bool ok = true;
         for (int64_t pair = blockIdx.x; pair < n_pairs && ok; pair += gridDim.x) {
-            float band = 0.f;                               // of row r_own of tile own_tile
+            float band = 0.f, norm = 0.f;                   // of row r_own of tile own_tile, scaled
+            // A row's new residual to memory; its norm and band to the lane that has the row (pass p's, if set in `rows`).
+            auto put_row = [&](const double (&R)[CH], int p, bool write, uint32_t rows) {
+                const int r = q * 32 + 4 * p + grp;
+                float nr;
+                const double scale = row_scale(group8_sum(norm2_share<CH>(R)), nr);
+                const float err2 = group8_sumf(store_residual<CH>(R, scale, Rd_cta + static_cast<int64_t>(own_tile * TILE_M + r) * D_, A_own, r, l8, write));
+                const float n_o = __shfl_sync(FULL, nr, (lane & 3) * 8), e_o = __shfl_sync(FULL, err2, (lane & 3) * 8);
+                if ((lane >> 2) == p && ((rows >> lane) & 1u)) {
+                    norm = n_o;
+                    band = row_band(n_o, e_o, db);
+                }
+            };
             // ---- R_0 = x ----
 #pragma unroll 1
             for (int p = 0; p < 8; ++p) {
@@ -248,18 +232,14 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
 #pragma unroll
                     for (int k = 0; k < CH; ++k) R[k] = 0.0;
                 }
-                float b;
-                const double scale = row_scale(group8_sum(norm2_share<CH>(R)), b);
-                store_residual<CH>(R, scale, Rd_cta + static_cast<int64_t>(own_tile * TILE_M + r) * D_, Ahi, Alo, r, l8);
-                const float b_o = __shfl_sync(FULL, b, (lane & 3) * 8);
-                if ((lane >> 2) == p) band = b_o;
+                put_row(R, p, true, FULL);
             }
             fence_proxy_async_smem();
             mbar_arrive(&sm.res_ready);
 
             for (int g = 0; g < s && ok; ++g) {
-                // ---- sweep: top four keys of this thread's half of two rows ----
-                Top4 st[2] = {Top4{0u, 0u, 0u, 0u, 0u, 0u, 0u}, Top4{0u, 0u, 0u, 0u, 0u, 0u, 0u}};
+                // ---- sweep: top five keys of this thread's half of two rows ----
+                Top5 st[2] = {top5_none(), top5_none()};
                 // the filter's bands of this thread's two rows: its own and the one the warp of the
                 // other row tile left in shared memory
                 float* band_x = reinterpret_cast<float*>(&sm.xchg[0][0]);
@@ -280,8 +260,8 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                             break;
                         }
                         tc_fence_after();
-                        Top4 qa = a ? st[1] : st[0];
-                        drain128(taddr + a * TILE_N, qa, static_cast<uint32_t>(2 * t + half), a ? fband[1] : fband[0], &sm.acc_empty[a], lane);
+                        Top5 qa = a ? st[1] : st[0];
+                        drain128(taddr + a * TILE_N, qa, static_cast<uint32_t>(t), a ? fband[1] : fband[0], &sm.acc_empty[a], lane);
                         if (a)
                             st[1] = qa;
                         else
@@ -289,18 +269,19 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                     }
                 }
                 // ---- bring the column halves together: warps 0-3 get row tile 0's, warps 4-7 row tile 1's ----
-                auto post = [&](const Top4& o) {
+                auto post = [&](const Top5& o) {
                     sm.xchg[0][r_own] = o.k0;
                     sm.xchg[1][r_own] = o.k1;
                     sm.xchg[2][r_own] = o.k2;
                     sm.xchg[3][r_own] = o.k3;
-                    sm.xchg[4][r_own] = o.i0 | (o.i1 << 10) | (o.i2 << 20);
+                    sm.xchg[4][r_own] = o.k4;
+                    sm.xchg[5][r_own] = o.i0 | (o.i1 << 8) | (o.i2 << 16) | (o.i3 << 24);   // (at most 256 tiles)
                 };
-                Top4 other{0u, 0u, 0u, 0u, 0u, 0u, 0u};
+                Top5 other = top5_none();
                 auto take = [&]() {
-                    const uint32_t ids = sm.xchg[4][r_own];
-                    other = Top4{sm.xchg[0][r_own], sm.xchg[1][r_own], sm.xchg[2][r_own], sm.xchg[3][r_own],
-                                 ids & 1023u,       (ids >> 10) & 1023u, (ids >> 20) & 1023u};
+                    const uint32_t ids = sm.xchg[5][r_own];
+                    other = Top5{sm.xchg[0][r_own], sm.xchg[1][r_own], sm.xchg[2][r_own], sm.xchg[3][r_own],
+                                 sm.xchg[4][r_own], ids & 255u,        (ids >> 8) & 255u, (ids >> 16) & 255u, ids >> 24};
                 };
                 if (half == 1) post(st[0]);
                 if (epilogue_barrier_any(!ok || sm.abort != 0)) {
@@ -313,29 +294,33 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                 epilogue_barrier();
                 if (half == 1) take();
                 epilogue_barrier();                         // (the exchange area is rewritten from here on)
-                // The row's candidates: the first three of either half (two 16-bit atoms per word), a bit in
-                // my_flags for each that is inside the band; bit 6: the fourth of a half is inside too, so there
+                // The row's candidates: the first four of either half (two 16-bit atoms per word), a bit in
+                // my_flags for each that is inside the band; kUnknown: the fifth of a half is inside too, so there
                 // may be more than are known (NaN counts as inside).
-                const Top4 mine = own_tile ? st[1] : st[0];
+                constexpr int kUnknown = 256;
+                const Top5 mine = own_tile ? st[1] : st[0];
                 const float v0 = fmaxf(__uint_as_float(mine.k0 & kKeyMask), __uint_as_float(other.k0 & kKeyMask));
-                uint32_t my_cand[3];
+                uint32_t my_cand[4];
                 int my_flags = 0, my_n1 = 0;                // an all-zero sweep picks atom 0
                 {
-                    const uint32_t key[6] = {mine.k0, mine.k1, mine.k2, other.k0, other.k1, other.k2};
-                    const int at[6] = {atom_of(mine.k0, mine.i0),   atom_of(mine.k1, mine.i1),   atom_of(mine.k2, mine.i2),
-                                       atom_of(other.k0, other.i0), atom_of(other.k1, other.i1), atom_of(other.k2, other.i2)};
+                    const uint32_t key[8] = {mine.k0, mine.k1, mine.k2, mine.k3, other.k0, other.k1, other.k2, other.k3};
+                    const uint32_t id[8] = {mine.i0, mine.i1, mine.i2, mine.i3, other.i0, other.i1, other.i2, other.i3};
+                    int at[8];
 #pragma unroll
-                    for (int i = 0; i < 3; ++i)
+                    for (int i = 0; i < 8; ++i)             // (mine: the columns of this warp's half)
+                        at[i] = static_cast<int>(id[i]) * TILE_N + (i < 4 ? half : half ^ 1) * 128 + 127 - static_cast<int>(key[i] & 127u);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
                         my_cand[i] = (static_cast<uint32_t>(at[2 * i]) & 0xFFFFu) | (static_cast<uint32_t>(at[2 * i + 1]) << 16);
                     if (v0 > 0.f && N > 1) {
 #pragma unroll
-                        for (int i = 5; i >= 0; --i)
+                        for (int i = 7; i >= 0; --i)
                             if (!(v0 - __uint_as_float(key[i] & kKeyMask) > band) && at[i] < N) {
                                 my_flags |= 1 << i;
                                 my_n1 = at[i];
                             }
-                        if (!(v0 - __uint_as_float(mine.k3 & kKeyMask) > band) || !(v0 - __uint_as_float(other.k3 & kKeyMask) > band))
-                            my_flags |= 64;
+                        if (!(v0 - __uint_as_float(mine.k4 & kKeyMask) > band) || !(v0 - __uint_as_float(other.k4 & kKeyMask) > band))
+                            my_flags |= kUnknown;
                     }
                 }
 
@@ -358,7 +343,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                 // Rows whose candidates are not all known are left for a second round: the eight warps search
                 // the dictionary for each of them together (a single warp took 450 us for 4096 atoms, and
                 // about one sweep of 37888 rows in eight has such a row).
-                const uint32_t unknown = __ballot_sync(FULL, (my_flags & 64) != 0);
+                const uint32_t unknown = __ballot_sync(FULL, (my_flags & kUnknown) != 0);
                 uint32_t todo = ~unknown;
 #pragma unroll 1
                 for (int round = 0; round < 2; ++round) {
@@ -367,7 +352,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                         float* limit = reinterpret_cast<float*>(lists + 8);
                         Rescored* found = reinterpret_cast<Rescored*>(lists + 8 + ROWS);
                         if (lane == 0) lists[warp] = unknown;
-                        if (my_flags & 64) limit[warp * 32 + lane] = relative_limit(v0, band);
+                        if (my_flags & kUnknown) limit[warp * 32 + lane] = relative_limit(v0, band, norm, db);
                         if (!epilogue_barrier_any(unknown != 0)) break;
 #pragma unroll 1
                         for (int w = 0; w < 8; ++w)
@@ -403,7 +388,6 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                         const int r = q * 32 + src;
                         const int64_t m = pair * ROWS + own_tile * TILE_M + r;
                         const bool has = (todo >> src) & 1u;
-                        double* Rrow = Rd_cta + static_cast<int64_t>(own_tile * TILE_M + r) * D_;
                         const bool cmp = (flags & (flags - 1)) != 0;         // this row has several candidates
                         if (__any_sync(FULL, cmp)) {        // their fp64 correlations decide, the lowest atom among equals
                             const int n_first = n;
@@ -411,9 +395,9 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                             double cbest = -1.0;
                             int nbest = n;
 #pragma unroll 1
-                            for (int i = 0; i < 6; ++i) {
+                            for (int i = 0; i < 8; ++i) {
                                 if (!((some >> i) & 1u)) continue;
-                                const uint32_t pair_of = __shfl_sync(FULL, i < 2 ? my_cand[0] : i < 4 ? my_cand[1] : my_cand[2], src);
+                                const uint32_t pair_of = __shfl_sync(FULL, i < 2 ? my_cand[0] : i < 4 ? my_cand[1] : i < 6 ? my_cand[2] : my_cand[3], src);
                                 const bool in = cmp && ((flags >> i) & 1);
                                 const int nc = in ? static_cast<int>((i & 1) ? pair_of >> 16 : pair_of & 0xFFFFu) : n;
                                 float ax[CH];
@@ -429,14 +413,8 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
                         }
                         const double c = group8_sum(slice_dot<CH>(R, a));
 #ifdef CSR_DEBUG_CHECKS
-                        {   // largest |tensor-core value - fp64 value| / ||R|| seen, as float bits
-                            const float vbo = __shfl_sync(FULL, v0, src), bo = __shfl_sync(FULL, band, src);
-                            const double nr = sqrt(group8_sum(norm2_share<CH>(R)));
-                            if (l8 == 0 && m < M && has && round == 0 && (flags & (flags - 1)) == 0 && bo > 0.f) {
-                                const float rel = fabsf(vbo / (bo / (kBandRel * 1.001f)) - static_cast<float>(fabs(c) / nr));
-                                atomicMax(diag, __float_as_uint(rel));
-                            }
-                        }
+                        check_value<CH>(diag, R, a, c, __shfl_sync(FULL, v0, src), __shfl_sync(FULL, band, src), __shfl_sync(FULL, norm, src), db, l8,
+                                        m < M && has && round == 0 && !cmp);
 #endif
                         if (l8 == 0 && m < M && has) {
                             out_idx[m * ldc + g] = static_cast<uint16_t>(n);
@@ -451,11 +429,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
 #pragma unroll
                                 for (int k = 0; k < CH; ++k) R[k] = fma(-c, static_cast<double>(a[k]), R[k]);
                             }
-                            float b;
-                            const double scale = row_scale(group8_sum(norm2_share<CH>(R)), b);
-                            if (has) store_residual<CH>(R, scale, Rrow, Ahi, Alo, r, l8);
-                            const float b_o = __shfl_sync(FULL, b, (lane & 3) * 8);
-                            if ((lane >> 2) == p && ((todo >> lane) & 1u)) band = b_o;
+                            put_row(R, p, has, todo);
                         }
                         n = n_nx;
                         flags = flags_nx;
@@ -483,23 +457,89 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_hi, const __grid
     }
 }
 
-// D (fp32, [N][d]) -> its bf16 high part and the bf16 rounding of the remainder, same layout; also
-// zeroes the words that the CTAs of a split row tile meet at.
-__global__ void split_dict_kernel(const float4* __restrict__ D, uint2* __restrict__ hi, uint2* __restrict__ lo, int64_t n_vec4,
-                                  uint32_t* __restrict__ zero, int n_zero) {
+// D (fp32, [N][d]) -> fp16 of `scale` times it, same layout, and each block's largest squared norms of an atom and of
+// what the rounding took from one (see DictBounds).  The scale is the power of two that brings the largest of 32
+// atoms spread over the dictionary to a norm in [1, 2): every block takes the same.  Atoms far larger than those
+// overflow; the error's norm is then infinite, as it is for them, and every row is searched for in fp64.  Atoms
+// that are not finite are left out of the norms: the sweep meets them as they are.  Also zeroes the words that the
+// CTAs of a split row tile meet at.  One warp per atom.
+template <int D_>
+__global__ void __launch_bounds__(256)
+dict_to_f16_kernel(const float* __restrict__ D, int N, uint32_t* __restrict__ out, DictPart* __restrict__ parts, uint32_t* __restrict__ zero,
+                   int n_zero) {
+    constexpr int PER = D_ / 64;                          // pairs of channels per lane
+    __shared__ float red[2][8];
+    __shared__ float first[8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_zero; i += gridDim.x * blockDim.x) zero[i] = 0u;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec4; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 v = D[i];
-        const float f[4] = {v.x, v.y, v.z, v.w};
-        uint32_t h[4], l[4];
+    auto load = [&](int n, float2 (&v)[PER]) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const __nv_bfloat16 hk = __float2bfloat16_rn(f[k]);
-            h[k] = __bfloat16_as_ushort(hk);
-            l[k] = __bfloat16_as_ushort(__float2bfloat16_rn(f[k] - __bfloat162float(hk)));
+        for (int k = 0; k < PER; ++k) v[k] = __ldg(reinterpret_cast<const float2*>(D + static_cast<int64_t>(n) * D_) + lane + 32 * k);
+    };
+    float big = 0.f;                                      // largest magnitude, then norm relative to it: no overflow on the way
+    {
+        float2 v[4][PER];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) load(static_cast<int>(static_cast<int64_t>(warp * 4 + j) * N / 32), v[j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float m = 0.f, ss = 0.f;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) m = fmaxf(m, fmaxf(fabsf(v[j][k].x), fabsf(v[j][k].y)));
+            for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+            if (!(m > 0.f) || !(m <= 3.0e38f)) continue;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const float x = v[j][k].x / m, y = v[j][k].y / m;
+                ss = fmaf(x, x, fmaf(y, y, ss));
+            }
+            for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(FULL, ss, o);
+            const float nrm = m * sqrtf(ss);
+            if (nrm <= 3.0e38f) big = fmaxf(big, nrm);    // (NaN channels: not taken)
         }
-        hi[i] = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
-        lo[i] = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
+    }
+    if (lane == 0) first[warp] = big;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) big = fmaxf(big, first[w]);
+    const int e = static_cast<int>(__float_as_uint(big) >> 23);           // biased exponent of the largest norm
+    const float scale = e >= 2 && e <= 252 ? __uint_as_float(static_cast<uint32_t>(254 - e) << 23) : 1.f;
+    float norm2 = 0.f, err2 = 0.f;
+    for (int n = blockIdx.x * 8 + warp; n < N; n += gridDim.x * 8) {
+        float2 v[PER];
+        load(n, v);
+        float nn = 0.f, ee = 0.f;
+        bool finite = true;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            finite = finite && fabsf(v[k].x) <= 3.4028234e38f && fabsf(v[k].y) <= 3.4028234e38f;
+            const float x = v[k].x * scale, y = v[k].y * scale;
+            const __half2 h = __floats2half2_rn(x, y);
+            const float2 w = __half22float2(h);
+            nn = fmaf(x, x, fmaf(y, y, nn));
+            ee = fmaf(x - w.x, x - w.x, fmaf(y - w.y, y - w.y, ee));
+            out[static_cast<int64_t>(n) * (D_ / 2) + lane + 32 * k] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        for (int o = 16; o; o >>= 1) {
+            nn += __shfl_xor_sync(FULL, nn, o);
+            ee += __shfl_xor_sync(FULL, ee, o);
+        }
+        if (!__all_sync(FULL, finite)) continue;
+        norm2 = fmaxf(norm2, nn);
+        err2 = fmaxf(err2, ee == ee ? ee : __int_as_float(0x7f800000));
+    }
+    if (lane == 0) {
+        red[0][warp] = norm2;
+        red[1][warp] = err2;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) {
+            norm2 = fmaxf(norm2, red[0][w]);
+            err2 = fmaxf(err2, red[1][w]);
+        }
+        parts[blockIdx.x] = DictPart{norm2, err2, scale, 0.f};
     }
 }
 
@@ -511,14 +551,13 @@ int ctas_for(int64_t M) {
 }
 
 template <int D_>
-int run(const EncodeArgs& a, const CUtensorMap& mh, const CUtensorMap& ml, double* Rd, uint32_t* status, uint32_t* diag) {
+int run(const EncodeArgs& a, const CUtensorMap& map, const DictPart* parts, int n_parts, double* Rd, uint32_t* status, uint32_t* diag) {
     const size_t smem = sizeof(TcSmem<D_>);
     cudaError_t e = cudaFuncSetAttribute(encode_exact_tc_kernel<D_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     const int grid = ctas_for(a.M);
-    encode_exact_tc_kernel<D_><<<grid, NT, smem, a.stream>>>(mh, ml, a.D, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx,
-                                                                     a.out_coef, a.coef_dtype, a.ld_code, Rd, status, diag,
-                                                                     options().wait_limit_ns);
+    encode_exact_tc_kernel<D_><<<grid, NT, smem, a.stream>>>(map, parts, n_parts, a.D, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx,
+                                                             a.out_coef, a.coef_dtype, a.ld_code, Rd, status, diag, options().wait_limit_ns);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "encode_exact_tc launch: %s", cudaGetErrorString(e));
     return CSR_OK;
@@ -555,7 +594,7 @@ size_t pair_scratch_bytes(int64_t M, int d) { return (size_t)ctas_for(M) * ROWS 
 
 }  // namespace
 
-// [high parts][low parts][counters of the two split launches][rows of the launch that is running]
+// [fp16 dictionary][its bounds][counters of the two split launches][rows of the launch that is running]
 size_t encode_exact_tc_scratch_bytes(int64_t M, int d, int N) {
     const Plan p = make_plan(M, N, false);
     size_t rows = pair_scratch_bytes(M, d), words = 0;    // (also what is needed where a split launch is refused)
@@ -565,7 +604,7 @@ size_t encode_exact_tc_scratch_bytes(int64_t M, int d, int N) {
         if (b > rows) rows = b;
         words += exact_grid_counter_words(m);
     }
-    return 2 * align1k((size_t)N * d * 2) + align1k(words * 4) + rows;
+    return align1k((size_t)N * d * 2) + align1k(kMaxDictParts * sizeof(DictPart)) + align1k(words * 4) + rows;
 }
 
 int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status, uint32_t* diag, bool pairs_only) {
@@ -574,21 +613,21 @@ int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status,
         return fail(CSR_ERR_ALIGNMENT, "internal: exact-mode scratch not 1024-byte aligned");
     const Plan plan = make_plan(a.M, a.N, pairs_only);
     char* base = static_cast<char*>(scratch);
-    const size_t part = align1k((size_t)a.N * a.d * 2);
-    void* hi = base;
-    void* lo = base + part;
-    uint32_t* counters = reinterpret_cast<uint32_t*>(base + 2 * part);
+    void* dict = base;
+    base += align1k((size_t)a.N * a.d * 2);
+    DictPart* parts = reinterpret_cast<DictPart*>(base);
+    base += align1k(kMaxDictParts * sizeof(DictPart));
+    uint32_t* counters = reinterpret_cast<uint32_t*>(base);
     size_t words = 0;
     for (int64_t m : plan.grid_rows)
         if (m) words += exact_grid_counter_words(m);
-    char* rows = base + 2 * part + align1k(words * 4);
-    const int64_t n_vec4 = (int64_t)a.N * a.d / 4;
-    int blocks = (int)((n_vec4 + 255) / 256);
-    if (blocks > 4 * sm_count()) blocks = 4 * sm_count();
-    split_dict_kernel<<<blocks, 256, 0, a.stream>>>(reinterpret_cast<const float4*>(a.D), static_cast<uint2*>(hi),
-                                                    static_cast<uint2*>(lo), n_vec4, counters, (int)words);
+    char* rows = base + align1k(words * 4);
+    int n_parts = (a.N + 7) / 8;
+    if (n_parts > kMaxDictParts) n_parts = kMaxDictParts;
+    auto to_f16 = a.d == 128 ? dict_to_f16_kernel<128> : dict_to_f16_kernel<64>;
+    to_f16<<<n_parts, 256, 0, a.stream>>>(a.D, a.N, static_cast<uint32_t*>(dict), parts, counters, (int)words);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "split_dict launch: %s", cudaGetErrorString(e));
+    if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "dict_to_f16 launch: %s", cudaGetErrorString(e));
     auto rows_from = [&](int64_t r0, int64_t m) {
         EncodeArgs b = a;
         b.X = static_cast<const char*>(a.X) + (size_t)r0 * a.ldx * dtype_size(a.x_dtype);
@@ -598,11 +637,10 @@ int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status,
         return b;
     };
     auto run_pairs = [&](const EncodeArgs& b) {
-        CUtensorMap mh, ml;
-        if (int rc = part_map(&mh, hi, a.N, a.d, TILE_N)) return rc;
-        if (int rc = part_map(&ml, lo, a.N, a.d, TILE_N)) return rc;
+        CUtensorMap map;
+        if (int rc = dict_map(&map, dict, a.N, a.d, TILE_N)) return rc;
         double* Rd = reinterpret_cast<double*>(rows);
-        return a.d == 128 ? run<128>(b, mh, ml, Rd, status, diag) : run<64>(b, mh, ml, Rd, status, diag);
+        return a.d == 128 ? run<128>(b, map, parts, n_parts, Rd, status, diag) : run<64>(b, map, parts, n_parts, Rd, status, diag);
     };
     if (plan.pair_rows)
         if (int rc = run_pairs(rows_from(0, plan.pair_rows))) return rc;
@@ -610,7 +648,7 @@ int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status,
     for (int64_t m : plan.grid_rows) {
         if (m == 0) continue;
         const EncodeArgs b = rows_from(r0, m);
-        int rc = launch_encode_exact_grid(b, hi, lo, rows, counters, status, diag);
+        int rc = launch_encode_exact_grid(b, dict, parts, n_parts, rows, counters, status, diag);
         if (rc == kGridLaunchRefused) rc = run_pairs(b);
         if (rc != CSR_OK) return rc;
         counters += exact_grid_counter_words(m);

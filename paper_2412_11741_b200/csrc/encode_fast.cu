@@ -524,7 +524,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         if constexpr (ONE) {
             // one row tile; the CTA's dictionary tiles go to the two accumulators in turn
@@ -557,7 +557,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
 #pragma unroll
                         for (int k = 0; k < KSTEPS; ++k) {
                             const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                            umma_bf16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
+                            umma_f16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
                         }
                         umma_commit(&sm.empty_b[stage]);
                     }
@@ -604,7 +604,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                                 for (int k = 0; k < KSTEPS; ++k) {
                                     // 16 channels = 32 bytes inside a 128-byte swizzled row
                                     const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                                    umma_bf16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
+                                    umma_f16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
                                 }
                                 // the second row tile is the last reader of a stage
                                 if (tile == 1) umma_commit(&sm.empty_b[stage]);

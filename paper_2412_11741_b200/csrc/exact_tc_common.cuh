@@ -1,7 +1,7 @@
 // Pieces shared by the two tensor-core encoders of the correctness mode (one CTA per pair of row
-// tiles for all atoms; the dictionary split across the CTAs of one launch for fewer rows): the
-// running top four of a row's correlations, fp64 residual rows as bf16 operand parts, the fp64
-// arithmetic of the picks.
+// tiles for all atoms; the dictionary split across the CTAs of one launch for fewer rows): the fp16
+// operands and the bound of what their rounding does to a correlation, the running top five of a row's
+// correlations, the fp64 arithmetic of the picks.
 #pragma once
 
 #include <cuda.h>
@@ -20,26 +20,53 @@ constexpr int UMMA_K = 16;
 constexpr int STAGE_CH = 64;
 constexpr uint32_t kKeyMask = 0x7FFFFF80u;                // |value| without its seven lowest mantissa bits
 constexpr uint32_t FULL = 0xffffffffu;
-// Half-width of the undecided zone relative to ||R||: twice the error of a tensor-core
-// correlation (the split's 1.2e-5 plus the fp32 accumulation of 3 d products in groups of 16)
-// plus the 2^-16 relative truncation of the keys.
-constexpr float kBandRel = 1.0f / 4096.0f;
+// What the tensor cores' fp32 accumulation of d exact products of fp16 values (in groups of 16) may add to
+// the error of a correlation, relative to ||R|| and the largest norm of an atom.  Measured (checked
+// build): below a quarter of it.
+constexpr float kAccumRel = 1.0f / 32768.0f;
+
+// The dictionary as the sweeps read it: fp16, times a power of two; largest norm of a (scaled) atom and
+// of what the rounding took from one.
+struct DictBounds {
+    float norm, err, scale;
+};
+// One block's share of them, as dict_to_f16_kernel leaves it.
+constexpr int kMaxDictParts = 296;
+struct DictPart {
+    float norm2, err2, scale, pad;
+};
+// All of them put together; every lane of a warp calls and gets the result (at most ten loads a lane).
+__device__ __forceinline__ DictBounds dict_bounds(const DictPart* __restrict__ parts, int n_parts, int lane) {
+    float norm2 = 0.f, err2 = 0.f;
+    for (int i = lane; i < n_parts; i += 32) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(parts) + i);
+        norm2 = fmaxf(norm2, v.x);
+        err2 = fmaxf(err2, v.y);
+    }
+    for (int o = 16; o; o >>= 1) {
+        norm2 = fmaxf(norm2, __shfl_xor_sync(FULL, norm2, o));
+        err2 = fmaxf(err2, __shfl_xor_sync(FULL, err2, o));
+    }
+    return DictBounds{sqrtf(norm2) * 1.0001f, sqrtf(err2) * 1.0001f, __ldg(&parts[0].scale)};
+}
 
 __device__ __forceinline__ uint32_t swz_off(int r, int chunk) {
     const int kblock = chunk >> 3, cc = chunk & 7;
     return kblock * (TILE_M * 128) + (r >> 3) * 1024 + (r & 7) * 128 + ((cc ^ (r & 7)) << 4);
 }
 
-// The four largest keys seen, in descending order, and the places (2 * dictionary tile + column
-// half) the first three came from.
-struct Top4 {
-    uint32_t k0, k1, k2, k3;
-    uint32_t i0, i1, i2;
+// The five largest keys seen, in descending order, and the dictionary tiles the first four came from.
+struct Top5 {
+    uint32_t k0, k1, k2, k3, k4;
+    uint32_t i0, i1, i2, i3;
 };
+__device__ __forceinline__ Top5 top5_none() { return Top5{0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}; }
 
-__device__ __forceinline__ void top4_insert(Top4& q, uint32_t k, uint32_t id) {
-    const bool p0 = k > q.k0, p1 = k > q.k1, p2 = k > q.k2;
-    q.k3 = p2 ? q.k2 : max(q.k3, k);
+__device__ __forceinline__ void top5_insert(Top5& q, uint32_t k, uint32_t id) {
+    const bool p0 = k > q.k0, p1 = k > q.k1, p2 = k > q.k2, p3 = k > q.k3;
+    q.k4 = p3 ? q.k3 : max(q.k4, k);
+    q.k3 = p2 ? q.k2 : (p3 ? k : q.k3);
+    q.i3 = p2 ? q.i2 : (p3 ? id : q.i3);
     q.k2 = p1 ? q.k1 : (p2 ? k : q.k2);
     q.i2 = p1 ? q.i1 : (p2 ? id : q.i2);
     q.k1 = p0 ? q.k0 : (p1 ? k : q.k1);
@@ -59,11 +86,11 @@ __device__ __forceinline__ float absmax3(float a, float b, float c) {
 // for nearly every lane that gets here.  A value more than the band above the running maximum leaves
 // everything seen so far outside the band, so it simply becomes the only entry.  Returns the new
 // state and threshold.
-struct Top4Thr {
-    Top4 q;
+struct Top5Thr {
+    Top5 q;
     float thr;
 };
-static __device__ __noinline__ Top4Thr insert_group(Top4 q, float thr, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, uint32_t v4,
+static __device__ __noinline__ Top5Thr insert_group(Top5 q, float thr, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, uint32_t v4,
                                                     uint32_t v5, uint32_t v6, uint32_t v7, uint32_t tag, uint32_t id, float band) {
     // Keys whose last three bits are the place in the group (a lower column wins among equals); the
     // chains are kept short: a call is waited for, two warps per scheduler cannot cover it.
@@ -79,17 +106,17 @@ static __device__ __noinline__ Top4Thr insert_group(Top4 q, float thr, uint32_t 
         if (!(val >= thr)) break;
         const uint32_t key = best | rest;
         if (val > __uint_as_float(q.k0 & kKeyMask) + band)
-            q = Top4{key, 0u, 0u, 0u, id, 0u, 0u};
+            q = Top5{key, 0u, 0u, 0u, 0u, id, 0u, 0u, 0u};
         else
-            top4_insert(q, key, id);
+            top5_insert(q, key, id);
         thr = __uint_as_float(q.k0 & kKeyMask) - band;
 #pragma unroll
         for (int j = 0; j < 8; ++j) k[j] = k[j] == best ? 0u : k[j];
     }
-    return Top4Thr{q, thr};
+    return Top5Thr{q, thr};
 }
 
-// Folds 32 columns of this thread's row into its top four; `tag0` is the tag of v[0] (tags fall
+// Folds 32 columns of this thread's row into its top five; `tag0` is the tag of v[0] (tags fall
 // with the column so that the lowest column wins among equal magnitudes).  Eight values at a
 // time are first reduced to their largest magnitude (half an instruction each) and only a group
 // that reaches `thr`, the running maximum less the band, is inserted (a call: the sweep's code has
@@ -97,17 +124,17 @@ static __device__ __noinline__ Top4Thr insert_group(Top4 q, float thr, uint32_t 
 // final maximum was within the band of the running one when it came by, so what the filter
 // drops can never matter.
 template <int J = 0>
-__device__ __forceinline__ void chunk_top4(const uint32_t (&v)[32], Top4& q, uint32_t id, uint32_t tag0, float& thr, float band) {
+__device__ __forceinline__ void chunk_top5(const uint32_t (&v)[32], Top5& q, uint32_t id, uint32_t tag0, float& thr, float band) {
     if constexpr (J < 32) {
         const float ga = absmax3(__uint_as_float(v[J]), __uint_as_float(v[J + 1]), __uint_as_float(v[J + 2]));
         const float gb = absmax3(__uint_as_float(v[J + 3]), __uint_as_float(v[J + 4]), __uint_as_float(v[J + 5]));
         const float gc = absmax3(__uint_as_float(v[J + 6]), __uint_as_float(v[J + 7]), ga);
         if (fmaxf(gb, gc) >= thr) {
-            const Top4Thr r = insert_group(q, thr, v[J], v[J + 1], v[J + 2], v[J + 3], v[J + 4], v[J + 5], v[J + 6], v[J + 7], tag0 - J, id, band);
+            const Top5Thr r = insert_group(q, thr, v[J], v[J + 1], v[J + 2], v[J + 3], v[J + 4], v[J + 5], v[J + 6], v[J + 7], tag0 - J, id, band);
             q = r.q;
             thr = r.thr;
         }
-        chunk_top4<J + 8>(v, q, id, tag0, thr, band);
+        chunk_top5<J + 8>(v, q, id, tag0, thr, band);
     }
 }
 
@@ -116,7 +143,7 @@ __device__ __forceinline__ void chunk_top4(const uint32_t (&v)[32], Top4& q, uin
 // instruction cache.  No load is in flight while a group is inserted (the call may move registers).
 // `band`: that of the row, a little widened; negative for a row that is all zero (nothing is
 // inserted and atom 0 is taken).
-__device__ __forceinline__ void drain(uint32_t taddr, int chunks, Top4& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
+__device__ __forceinline__ void drain(uint32_t taddr, int chunks, Top5& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
     float thr = __uint_as_float(q.k0 & kKeyMask) - band;
     uint32_t tag0 = 127u;
 #pragma unroll 1
@@ -136,15 +163,15 @@ __device__ __forceinline__ void drain(uint32_t taddr, int chunks, Top4& q, uint3
             __syncwarp();
             if (lane == 0) mbar_arrive(acc_empty);
         }
-        chunk_top4(v0, q, id, tag0, thr, band);
-        if (c + 1 < chunks) chunk_top4(v1, q, id, tag0 - 32u, thr, band);
+        chunk_top5(v0, q, id, tag0, thr, band);
+        if (c + 1 < chunks) chunk_top5(v1, q, id, tag0 - 32u, thr, band);
         tag0 -= 64u;
     }
 }
 
 // The same for 128 columns, handed back as soon as all of them are in registers: for an accumulator that
 // the tensor core is waiting for.
-__device__ __forceinline__ void drain128(uint32_t taddr, Top4& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
+__device__ __forceinline__ void drain128(uint32_t taddr, Top5& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
     uint32_t v0[32], v1[32], v2[32], v3[32];
     tmem_ld32(taddr + 0, v0);
     tmem_ld32(taddr + 32, v1);
@@ -158,14 +185,10 @@ __device__ __forceinline__ void drain128(uint32_t taddr, Top4& q, uint32_t id, f
     __syncwarp();
     if (lane == 0) mbar_arrive(acc_empty);
     float thr = __uint_as_float(q.k0 & kKeyMask) - band;
-    chunk_top4(v0, q, id, 127u, thr, band);
-    chunk_top4(v1, q, id, 95u, thr, band);
-    chunk_top4(v2, q, id, 63u, thr, band);
-    chunk_top4(v3, q, id, 31u, thr, band);
-}
-
-__device__ __forceinline__ int atom_of(uint32_t key, uint32_t id) {
-    return static_cast<int>(id) * 128 + (127 - static_cast<int>(key & 127u));
+    chunk_top5(v0, q, id, 127u, thr, band);
+    chunk_top5(v1, q, id, 95u, thr, band);
+    chunk_top5(v2, q, id, 63u, thr, band);
+    chunk_top5(v3, q, id, 31u, thr, band);
 }
 
 // Barrier of the 256 epilogue threads that also tells every one of them whether any of them
@@ -224,14 +247,23 @@ __device__ __forceinline__ double slice_dot(const double (&R)[CH], const float (
     return (c0 + c1) + (c2 + c3);
 }
 
-// bf16 high and low parts of two neighbouring channels, one word of each.
-__device__ __forceinline__ void split_pair(double r0, double r1, uint32_t& hi, uint32_t& lo) {
+// Two neighbouring channels of a scaled row as fp16, one word, and what the rounding took from them squared, added to
+// `err2`.  (A value is brought to fp32 first: what that rounds off, 2^-24 of it, is far inside the allowance
+// of row_band.)
+__device__ __forceinline__ uint32_t round_pair(double r0, double r1, float& err2) {
     const float f0 = static_cast<float>(r0), f1 = static_cast<float>(r1);
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
-    const __nv_bfloat16 l0 = __float2bfloat16_rn(f0 - __bfloat162float(h0));
-    const __nv_bfloat16 l1 = __float2bfloat16_rn(f1 - __bfloat162float(h1));
-    hi = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
-    lo = static_cast<uint32_t>(__bfloat16_as_ushort(l0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(l1)) << 16);
+    const __half2 h = __floats2half2_rn(f0, f1);
+    const float2 w = __half22float2(h);
+    const float e0 = f0 - w.x, e1 = f1 - w.y;
+    err2 = fmaf(e0, e0, err2);
+    err2 = fmaf(e1, e1, err2);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float group8_sumf(float v) {
+    v += __shfl_xor_sync(FULL, v, 1);
+    v += __shfl_xor_sync(FULL, v, 2);
+    v += __shfl_xor_sync(FULL, v, 4);
+    return v;
 }
 
 // This lane's share of ||R||^2.
@@ -246,37 +278,76 @@ __device__ __forceinline__ double norm2_share(const double (&R)[CH]) {
     return n0 + n1;
 }
 
-// What a row is multiplied by before it is split into parts, from its ||R||^2: the power of two that brings
-// ||R|| into [1, 2), so that the parts, the sweep's values and the band keep their precision at any
+// What a row is multiplied by before it is rounded to fp16, from its ||R||^2: the power of two that brings
+// ||R|| into [1, 2), so that the operands, the sweep's values and the band keep their precision at any
 // norm (the keys of a sweep are only compared with one another and with the band, all in the same
-// unit, and a power of two leaves every bit of them as it is).  `band` gets the undecided zone in that
-// unit: 0 for a row of zeros; Inf or NaN, and no scaling, for a row that is not finite.
-__device__ __forceinline__ double row_scale(double nn, float& band) {
+// unit, and a power of two leaves every bit of them as it is).  `norm` gets ||R|| in that unit:
+// 0 for a row of zeros; Inf or NaN, and no scaling, for a row that is not finite.
+__device__ __forceinline__ double row_scale(double nn, float& norm) {
     const int e = (__double2hiint(nn) >> 20) & 0x7FF;
     const double scale = e == 0 || e == 0x7FF ? 1.0 : __hiloint2double((1023 - ((e - 1023) >> 1)) << 20, 0);
-    band = e == 0 ? 0.f : kBandRel * sqrtf(static_cast<float>(nn * scale * scale)) * 1.001f;
+    norm = e == 0 ? 0.f : sqrtf(static_cast<float>(nn * scale * scale));
     return scale;
 }
+// Half-width of the undecided zone of a row, in the sweep's unit, from its norm and the norm of what rounding it to
+// fp16 took from it: twice the error of a correlation, plus the 2^-16 relative truncation of the keys.  With
+// r = r' + e and d = d' + f (r', d' the fp16 values), r.d - r'.d' = e.d + r'.f, which is at most
+// ||e|| max ||d|| + ||r'|| max ||f|| (Cauchy-Schwarz): these norms are taken, not assumed, and come to 4e-4 ||R|| for
+// unit atoms (a rounding error is 1.9e-4 of its value in the mean square), less than half of what the formats alone
+// would promise.
+__device__ __forceinline__ float row_band(float norm, float err2, const DictBounds& b) {
+    const float err = sqrtf(err2);
+    const float half = fmaf(err, b.norm, fmaf(norm + err, b.err, kAccumRel * norm * b.norm));
+    return norm > 0.f || norm != norm ? 1.001f * fmaf(2.f, half, norm * b.norm * (1.f / 65536.f)) : 0.f;
+}
 // From which |correlation| on, relative to ||R||, an atom can be the pick, for a sweep whose largest value was `v0`
-// (both in the sweep's unit): that value less the band, and half a band for the search's fp32 rounding.
-__device__ __forceinline__ float relative_limit(float v0, float band) { return (v0 - 1.5f * band) * (kBandRel * 1.001f / band); }
+// (in the sweep's unit, as band and norm): that value less the band, and half a band for the search's fp32
+// rounding.
+__device__ __forceinline__ float relative_limit(float v0, float band, float norm, const DictBounds& b) {
+    return (v0 - 1.5f * band) / (norm * b.scale);
+}
 
-// Writes this lane's CH residual values: fp64 to the scratch row (`row`: its first element), bf16 high and
-// low parts of `scale` times them into the operand tiles.
+// Writes this lane's CH residual values: fp64 to the scratch row (`row`: its first element), `scale` times them as fp16
+// to the operand tile.  Returns this lane's share of the rounding's squared norm.
 template <int CH>
-__device__ __forceinline__ void store_residual(const double (&R)[CH], double scale, double* __restrict__ row, uint8_t* Ahi, uint8_t* Alo,
-                                               int r, int l8) {
+__device__ __forceinline__ float store_residual(const double (&R)[CH], double scale, double* __restrict__ row, uint8_t* A, int r, int l8,
+                                                bool write) {
+    float err2 = 0.f;
 #pragma unroll
     for (int k = 0; k < CH / 2; ++k) {
-        reinterpret_cast<double2*>(row)[8 * k + l8] = make_double2(R[2 * k], R[2 * k + 1]);
-        uint32_t hi, lo;
-        split_pair(R[2 * k] * scale, R[2 * k + 1] * scale, hi, lo);
-        // channels 2 (8 k + l8), +1: 16-byte chunk 2 k + l8 / 4 of the row, word l8 % 4 of it
-        const uint32_t off = swz_off(r, 2 * k + (l8 >> 2)) + (l8 & 3) * 4;
-        *reinterpret_cast<uint32_t*>(Ahi + off) = hi;
-        *reinterpret_cast<uint32_t*>(Alo + off) = lo;
+        const uint32_t w = round_pair(R[2 * k] * scale, R[2 * k + 1] * scale, err2);
+        if (write) {
+            reinterpret_cast<double2*>(row)[8 * k + l8] = make_double2(R[2 * k], R[2 * k + 1]);
+            // channels 2 (8 k + l8), +1: 16-byte chunk 2 k + l8 / 4 of the row, word l8 % 4 of it
+            *reinterpret_cast<uint32_t*>(A + swz_off(r, 2 * k + (l8 >> 2)) + (l8 & 3) * 4) = w;
+        }
+    }
+    return err2;
+}
+
+#ifdef CSR_DEBUG_CHECKS
+// For a pick taken without re-scoring, with `v` its key's value: what the tensor core's own arithmetic contributed (against the
+// fp64 sum of the same fp16 operands, relative to ||R|| and the largest atom) and how much of half the band the
+// whole deviation from the fp64 correlation `c` used up.  Both raise words of `diag` (float bits).  Eight lanes of a row call.
+template <int CH>
+__device__ __forceinline__ void check_value(uint32_t* diag, const double (&R)[CH], const float (&a)[CH], double c, float v, float band, float norm,
+                                            const DictBounds& b, int l8, bool count) {
+    float unused;
+    const double scale = row_scale(group8_sum(norm2_share<CH>(R)), unused);
+    double p = 0.0;
+#pragma unroll
+    for (int k = 0; k < CH; ++k)
+        p = fma(static_cast<double>(__half2float(__float2half_rn(static_cast<float>(R[k] * scale)))),
+                static_cast<double>(__half2float(__float2half_rn(a[k] * b.scale))), p);
+    p = fabs(group8_sum(p));
+    if (l8 == 0 && count && band > 0.f) {
+        const float own = static_cast<float>(fabs(v - p)) / (norm * b.norm);
+        const float use = static_cast<float>(fabs(v - fabs(c) * scale * b.scale)) / (0.5f * band);
+        atomicMax(diag, __float_as_uint(own));
+        atomicMax(diag + 1, __float_as_uint(use));
     }
 }
+#endif
 
 // Elements `off` and `off + 1` of X widened to fp64.
 __device__ __forceinline__ void load_x2(const void* X, int x_dtype, int64_t off, double& x0, double& x1) {
@@ -412,16 +483,16 @@ inline EncodeTiledFn tensor_map_encoder() {
     return fn;
 }
 
-// One bf16 part of the dictionary, [N][d]: boxes of box_atoms atoms x 64 channels, 128-byte swizzle;
+// The dictionary's fp16 copy, [N][d]: boxes of box_atoms atoms x 64 channels, 128-byte swizzle;
 // atoms past N read as zeros.
-inline int part_map(CUtensorMap* map, void* base, int N, int d, int box_atoms) {
+inline int dict_map(CUtensorMap* map, void* base, int N, int d, int box_atoms) {
     EncodeTiledFn encode = tensor_map_encoder();
     if (!encode) return fail(CSR_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
     const cuuint64_t gdim[2] = {(cuuint64_t)d, (cuuint64_t)N};
     const cuuint64_t gstride[1] = {(cuuint64_t)d * 2};
     const cuuint32_t box[2] = {STAGE_CH, (cuuint32_t)box_atoms};
     const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, gdim, gstride, box, estr,
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, base, gdim, gstride, box, estr,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(CSR_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);

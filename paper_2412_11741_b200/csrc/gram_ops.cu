@@ -160,7 +160,7 @@ gram_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
             }
         }
     } else if (warp == MMA_WARP) {
-        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         {
             bool ok = warp_wait_bounded(&sm.a_full, 0, wc);
@@ -180,9 +180,9 @@ gram_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ C
 #pragma unroll
                     for (int k = 0; k < KBLK / 16; ++k) {
                         const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);       // 16 elements = 32 bytes
-                        umma_bf16(d_tmem, ah + off, bh + off, kIdesc, (kb | k) ? 1u : 0u);
-                        umma_bf16(d_tmem, ah + off, bl + off, kIdesc, 1u);
-                        umma_bf16(d_tmem, al + off, bh + off, kIdesc, 1u);
+                        umma_f16(d_tmem, ah + off, bh + off, kIdesc, (kb | k) ? 1u : 0u);
+                        umma_f16(d_tmem, ah + off, bl + off, kIdesc, 1u);
+                        umma_f16(d_tmem, al + off, bh + off, kIdesc, 1u);
                     }
                 }
                 umma_commit(&sm.b_empty[b]);
@@ -336,7 +336,7 @@ grad_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constant__ 
             }
         }
     } else if (warp == MMA_WARP) {
-        // (the whole warp runs this, one elected lane issues: see umma_bf16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         {
             bool ok = true;
@@ -353,9 +353,9 @@ grad_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constant__ 
 #pragma unroll
                 for (int k = 0; k < KBLK / 16; ++k) {
                     const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                    umma_bf16(tmem_d, ah + off, bh + off, kIdesc, (p | k) ? 1u : 0u);
-                    umma_bf16(tmem_d, ah + off, bl + off, kIdesc, 1u);
-                    umma_bf16(tmem_d, al + off, bh + off, kIdesc, 1u);
+                    umma_f16(tmem_d, ah + off, bh + off, kIdesc, (p | k) ? 1u : 0u);
+                    umma_f16(tmem_d, ah + off, bl + off, kIdesc, 1u);
+                    umma_f16(tmem_d, al + off, bh + off, kIdesc, 1u);
                 }
                 umma_commit(&sm.empty[st]);
             }

@@ -129,13 +129,13 @@ __device__ __forceinline__ void tmem_relinquish() {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 operands, fp32 accumulate.  The whole warp calls, converged, with
+// D[tmem] (+)= A[smem] * B[smem]^T, bf16 or fp16 operands (`idesc` says which), fp32 accumulate.  The whole warp calls, converged, with
 // the same arguments, and one elected lane issues: in code that only lane 0 runs, every MMA first has
 // to move its descriptors to the uniform registers the instruction takes, 116 cycles a piece, 168
 // when the other warps are busy too, more than the 128 x 256 x 16 MMA itself takes.  Measured, 128
 // MMAs in a row per SM with eight warps reading tensor memory: 178 cycles per MMA from lane 0,
 // 139 with the election (128 is the tensor core's own rate).
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(
         "{\n"
@@ -202,9 +202,12 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr) {
     return desc;
 }
 
-// Instruction descriptor of tcgen05.mma kind::f16: fp32 accumulator, bf16 A and B, both K-major.
+// Instruction descriptors of tcgen05.mma kind::f16: fp32 accumulator, A and B both bf16 or both fp16, both K-major.
+__host__ __device__ constexpr uint32_t instr_desc_f16(int m, int n) {
+    return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
+}
 __host__ __device__ constexpr uint32_t instr_desc_bf16(int m, int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
+    return instr_desc_f16(m, n) | (1u << 7) | (1u << 10);
 }
 
 struct WaitCtx {
