@@ -3,8 +3,8 @@
 // HBM traffic per row is 4*s bytes of codes in and d * sizeof(out) bytes out; the s atom rows a
 // row needs are gathered from the dictionary, which is a few MB and stays in L2, so from about
 // s = 4 up the kernel is bound by the L2 -> SM gather (s * d * sizeof(atom) bytes per row) or, with
-// fp16 atoms up to about s = 8, by instruction issue (0.71 per cycle at s = 8; 139 us for 2^20 rows at
-// N = 8192, 132 at N = 512, where the L1 holds the dictionary), not by HBM.  Two things follow:
+// fp16 atoms up to about s = 8, by instruction issue (0.71 per cycle at s = 8; with the dictionary in the L1, N = 512, nearly
+// all of the time is left), not by HBM.  Two things follow:
 //   - the atoms can be gathered from the fp16 copy of a prepared dictionary (csr_dict_create)
 //     instead of the fp32 master: half the gathered bytes, and with fp16 coefficients (the
 //     stored form) the products need no unpacking at all: fma.rn.f32.f16 multiplies two fp16
@@ -38,52 +38,81 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// The 16 bytes of an atom a lane holds: four fp32 channels, or eight fp16 channels.
-template <bool F16>
-struct Piece;
-template <>
-struct Piece<false> {
-    static constexpr int CH = 4;
-    static __device__ __forceinline__ void axpy(float (&a)[4], float c, const uint4& v) {
-        a[0] = fmaf(c, __uint_as_float(v.x), a[0]);
-        a[1] = fmaf(c, __uint_as_float(v.y), a[1]);
-        a[2] = fmaf(c, __uint_as_float(v.z), a[2]);
-        a[3] = fmaf(c, __uint_as_float(v.w), a[3]);
-    }
-};
-// acc0 += c * low half of w, acc1 += c * high half of w: fp16 x fp16 products are exact in
-// fp32, the sum is rounded once (the same value as fmaf on the widened operands).
-__device__ __forceinline__ void fma2_f16(float& acc0, float& acc1, uint32_t w, uint16_t c) {
+// Sums are kept in pairs of neighbouring channels.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pair(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpair(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ void fma_pair(f32x2& acc, float c, float a0, float a1) {
+    float lo, hi;
+    unpair(acc, lo, hi);
+    acc = pair(fmaf(c, a0, lo), fmaf(c, a1, hi));
+}
+// acc += c * the two halves of w: fp16 x fp16 products are exact in fp32, the sum is rounded once (the same value as
+// fmaf on the widened operands).  (Widened operands and the packed fma.rn.f32x2: 176 us against 146 for 2^20 rows,
+// s = 8, N = 8192.)
+__device__ __forceinline__ void fma2_f16(f32x2& acc, uint32_t w, uint16_t c) {
+    float a0, a1;
+    unpair(acc, a0, a1);
     asm("{\n"
         ".reg .b16 lo, hi;\n"
         "mov.b32 {lo, hi}, %2;\n"
         "fma.rn.f32.f16 %0, lo, %3, %0;\n"
         "fma.rn.f32.f16 %1, hi, %3, %1;\n"
         "}\n"
-        : "+f"(acc0), "+f"(acc1)
+        : "+f"(a0), "+f"(a1)
         : "r"(w), "h"(c));
+    acc = pair(a0, a1);
 }
+
+// The 16 bytes of an atom a lane holds: four fp32 channels, or eight fp16 channels.
+template <bool F16>
+struct Piece;
+template <>
+struct Piece<false> {
+    static constexpr int CH = 4;
+    static __device__ __forceinline__ void axpy(f32x2 (&a)[2], float c, const uint4& v) {
+        fma_pair(a[0], c, __uint_as_float(v.x), __uint_as_float(v.y));
+        fma_pair(a[1], c, __uint_as_float(v.z), __uint_as_float(v.w));
+    }
+};
 template <>
 struct Piece<true> {
     static constexpr int CH = 8;
     // fp32 coefficient: the atom's halves are widened first
-    static __device__ __forceinline__ void axpy(float (&a)[8], float c, const uint4& v) {
+    static __device__ __forceinline__ void axpy(f32x2 (&a)[4], float c, const uint4& v) {
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[q]));
-            a[2 * q] = fmaf(c, f.x, a[2 * q]);
-            a[2 * q + 1] = fmaf(c, f.y, a[2 * q + 1]);
+            fma_pair(a[q], c, f.x, f.y);
         }
     }
     // fp16 coefficient, as stored
-    static __device__ __forceinline__ void axpy(float (&a)[8], uint16_t c, const uint4& v) {
-        fma2_f16(a[0], a[1], v.x, c);
-        fma2_f16(a[2], a[3], v.y, c);
-        fma2_f16(a[4], a[5], v.z, c);
-        fma2_f16(a[6], a[7], v.w, c);
+    static __device__ __forceinline__ void axpy(f32x2 (&a)[4], uint16_t c, const uint4& v) {
+        fma2_f16(a[0], v.x, c);
+        fma2_f16(a[1], v.y, c);
+        fma2_f16(a[2], v.z, c);
+        fma2_f16(a[3], v.w, c);
     }
 };
+// Byte offset of the atom whose index is the low or high half of a word of two.  Where an atom is 256 bytes the
+// index's two bytes are put above the lane's (its place in the atom, l * 16): one instruction; elsewhere the lane's
+// place is in the base.  With this and two indices clamped at a time, 2^20 rows, s = 8, fp16 atoms, N = 8192 take 139 us
+// instead of 144 (an index unpacked, clamped and widened on its own each).
+template <int ROW_BYTES>
+__device__ __forceinline__ uint32_t piece_lo(uint32_t w, uint32_t lane_off) {
+    if constexpr (ROW_BYTES == 256) return __byte_perm(w, lane_off, 0x7104);
+    return (w & 0xFFFFu) * ROW_BYTES;
+}
+template <int ROW_BYTES>
+__device__ __forceinline__ uint32_t piece_hi(uint32_t w, uint32_t lane_off) {
+    if constexpr (ROW_BYTES == 256) return __byte_perm(w, lane_off, 0x7324);
+    return (w >> 16) * ROW_BYTES;
+}
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi, int out_dtype) {
     if (out_dtype == CSR_DTYPE_BF16) {
@@ -144,7 +173,7 @@ __device__ __forceinline__ void stage_codes(uint16_t* s_idx, unsigned char* s_co
 template <int CH, int LPR, typename P>
 __device__ __forceinline__ void rows_generic(const uint4* __restrict__ Dl, const uint16_t* ci, const unsigned char* cc,
                                              int cbytes, int s, int N, const int (&r)[PP], const bool (&valid)[PP],
-                                             float (&acc)[PP][CH], [[maybe_unused]] uint32_t* status) {
+                                             f32x2 (&acc)[PP][CH / 2], [[maybe_unused]] uint32_t* status) {
     for (int g0 = 0; g0 < s; g0 += INFLIGHT) {
         uint4 v[PP][INFLIGHT];
         float c[PP][INFLIGHT];
@@ -174,15 +203,18 @@ __device__ __forceinline__ void rows_generic(const uint4* __restrict__ Dl, const
 }
 
 // The same for s a multiple of four and rows that all exist: the codes of four steps come out
-// of shared memory with one 8-byte load per array (16 bytes for fp32 coefficients), and nothing
-// is predicated.
+// of shared memory with one 8-byte load per array (16 bytes for fp32 coefficients), two indices are
+// clamped at a time, and nothing is predicated.
 template <int CH, int LPR, typename P, bool COEF16>
-__device__ __forceinline__ void rows_by_four(const uint4* __restrict__ Dl, const uint16_t* ci, const unsigned char* cc, int s,
-                                             int N, const int (&r)[PP], float (&acc)[PP][CH], [[maybe_unused]] uint32_t* status) {
+__device__ __forceinline__ void rows_by_four(const void* __restrict__ Dict, uint32_t lane_off, const uint16_t* ci, const unsigned char* cc,
+                                             int s, int N, const int (&r)[PP], f32x2 (&acc)[PP][CH / 2], [[maybe_unused]] uint32_t* status) {
     static_assert(INFLIGHT == 4, "four steps per trip");
     constexpr bool RAW16 = COEF16 && CH == 8;             // fp16 coefficients meet fp16 atoms: no conversion
     using CoefT = typename std::conditional<RAW16, uint16_t, float>::type;
-    const int nmax = N - 1;
+    constexpr int ROW = LPR * 16;
+    const uint32_t nmax = static_cast<uint32_t>(N - 1), nmax2 = nmax | (nmax << 16);
+    const char* base = static_cast<const char*>(Dict) + (ROW == 256 ? 0u : lane_off);
+    const auto piece = [&](uint32_t off) { return __ldg(reinterpret_cast<const uint4*>(base + off)); };
     for (int g0 = 0; g0 < s; g0 += 4) {
         uint4 v[PP][4];
         CoefT c[PP][4];
@@ -210,16 +242,14 @@ __device__ __forceinline__ void rows_by_four(const uint4* __restrict__ Dl, const
                 c[w][2] = cw.z;
                 c[w][3] = cw.w;
             }
-            const int i0 = min(static_cast<int>(iw.x & 0xFFFFu), nmax), i1 = min(static_cast<int>(iw.x >> 16), nmax);
-            const int i2 = min(static_cast<int>(iw.y & 0xFFFFu), nmax), i3 = min(static_cast<int>(iw.y >> 16), nmax);
 #ifdef CSR_DEBUG_CHECKS
-            if (static_cast<int>(max(max(iw.x & 0xFFFFu, iw.x >> 16), max(iw.y & 0xFFFFu, iw.y >> 16))) > nmax)
-                atomicOr(status, kStatusBounds);
+            if (max(max(iw.x & 0xFFFFu, iw.x >> 16), max(iw.y & 0xFFFFu, iw.y >> 16)) > nmax) atomicOr(status, kStatusBounds);
 #endif
-            v[w][0] = __ldg(Dl + static_cast<uint32_t>(i0 * LPR));
-            v[w][1] = __ldg(Dl + static_cast<uint32_t>(i1 * LPR));
-            v[w][2] = __ldg(Dl + static_cast<uint32_t>(i2 * LPR));
-            v[w][3] = __ldg(Dl + static_cast<uint32_t>(i3 * LPR));
+            const uint32_t i01 = __vminu2(iw.x, nmax2), i23 = __vminu2(iw.y, nmax2);
+            v[w][0] = piece(piece_lo<ROW>(i01, lane_off));
+            v[w][1] = piece(piece_hi<ROW>(i01, lane_off));
+            v[w][2] = piece(piece_lo<ROW>(i23, lane_off));
+            v[w][3] = piece(piece_hi<ROW>(i23, lane_off));
         }
 #pragma unroll
         for (int w = 0; w < PP; ++w)
@@ -232,7 +262,7 @@ __device__ __forceinline__ void rows_by_four(const uint4* __restrict__ Dl, const
 // gives): three steps per trip, no step of four left half empty.
 template <int CH, int LPR, typename P, bool COEF16>
 __device__ __forceinline__ void rows_by_three(const uint4* __restrict__ Dl, const uint16_t* ci, const unsigned char* cc, int s,
-                                              int N, const int (&r)[PP], float (&acc)[PP][CH], [[maybe_unused]] uint32_t* status) {
+                                              int N, const int (&r)[PP], f32x2 (&acc)[PP][CH / 2], [[maybe_unused]] uint32_t* status) {
     constexpr bool RAW16 = COEF16 && CH == 8;
     using CoefT = typename std::conditional<RAW16, uint16_t, float>::type;
     const int nmax = N - 1;
@@ -286,7 +316,7 @@ reconstruct_kernel(const void* __restrict__ Dict, const uint16_t* __restrict__ i
     auto s_coef = [&](int which) { return mine + which * (stride_i + stride_c) + stride_i; };
 
     const int sub = lane / LPR, l = lane % LPR;
-    const uint4* Dl = static_cast<const uint4*>(Dict) + l;  // this lane's 16 bytes of atom 0; an atom row is LPR pieces
+    [[maybe_unused]] const uint4* Dl = static_cast<const uint4*>(Dict) + l;  // this lane's 16 bytes of atom 0; an atom row is LPR pieces
     const int64_t n_units = (M + rw - 1) / rw;            // units of rw rows
     const int64_t unit_step = (int64_t)gridDim.x * (NT / 32);
 
@@ -310,20 +340,20 @@ reconstruct_kernel(const void* __restrict__ Dict, const uint16_t* __restrict__ i
         for (int p = 0; p * RPP < rows; p += PP) {
             int r[PP];
             bool valid[PP];
-            float acc[PP][CH];
+            f32x2 acc[PP][CH / 2];
 #pragma unroll
             for (int w = 0; w < PP; ++w) {
                 r[w] = (p + w) * RPP + sub;               // row inside the unit
                 valid[w] = r[w] < rows;
                 if (BY != By::Any) r[w] = min(r[w], rows - 1);   // (a row past the end repeats the last one and is not stored)
 #pragma unroll
-                for (int k = 0; k < CH; ++k) acc[w][k] = 0.f;
+                for (int k = 0; k < CH / 2; ++k) acc[w][k] = 0ull;
             }
             if constexpr (BY == By::Four) {
                 if (cbytes == 2)
-                    rows_by_four<CH, LPR, P, true>(Dl, ci, cc, s, N, r, acc, status);
+                    rows_by_four<CH, LPR, P, true>(Dict, static_cast<uint32_t>(l) * 16u, ci, cc, s, N, r, acc, status);
                 else
-                    rows_by_four<CH, LPR, P, false>(Dl, ci, cc, s, N, r, acc, status);
+                    rows_by_four<CH, LPR, P, false>(Dict, static_cast<uint32_t>(l) * 16u, ci, cc, s, N, r, acc, status);
             } else if constexpr (BY == By::Three) {
                 if (cbytes == 2)
                     rows_by_three<CH, LPR, P, true>(Dl, ci, cc, s, N, r, acc, status);
@@ -334,7 +364,12 @@ reconstruct_kernel(const void* __restrict__ Dict, const uint16_t* __restrict__ i
             }
 #pragma unroll
             for (int w = 0; w < PP; ++w)
-                if (valid[w]) store_out<CH>(X_hat, out_dtype, (u * rw + r[w]) * ldxh + l * CH, acc[w]);
+                if (valid[w]) {
+                    float f[CH];
+#pragma unroll
+                    for (int k = 0; k < CH / 2; ++k) unpair(acc[w][k], f[2 * k], f[2 * k + 1]);
+                    store_out<CH>(X_hat, out_dtype, (u * rw + r[w]) * ldxh + l * CH, f);
+                }
         }
         __syncwarp();                                      // the buffer may be refilled
     }
