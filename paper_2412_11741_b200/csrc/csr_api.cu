@@ -694,7 +694,7 @@ int csr_dict_train_step(const csr_train_params_t* p) {
     if (!aligned16(p->D) || !aligned16(p->X) || (reinterpret_cast<uintptr_t>(p->losses) % 8))
         return fail(CSR_ERR_ALIGNMENT, "D and X must be 16-byte aligned, losses 8-byte aligned");
     if (!(p->lr >= 0.f) || !(p->beta >= 0.f)) return fail(CSR_ERR_INVALID_ARG, "lr and beta must be >= 0");
-    // scratch layout: [encoder's own region][idx][coef][grad_mse][grad_div]
+    // scratch layout: [encoder's own region][idx][coef][the step's own]
     size_t enc = (encode_fast_workspace_bytes(p->d, p->N) + 1023) / 1024 * 1024;
     if (p->M > 0 && encode_fast_split_applies(p->M, p->N)) enc += encode_fast_split_scratch_bytes(p->M, p->d, p->N);
     if (p->M > 0 && encode_exact_split_applies(p->M, p->N)) {
@@ -708,10 +708,8 @@ int csr_dict_train_step(const csr_train_params_t* p) {
     enc = (enc + 1023) / 1024 * 1024;
     const size_t idx_b = ((size_t)p->M * p->s * 2 + 255) / 256 * 256;
     const size_t coef_b = ((size_t)p->M * p->s * 4 + 255) / 256 * 256;
-    const size_t g_b = ((size_t)p->N * p->d * 4 + 255) / 256 * 256;
-    const size_t div_b = div_grad_scratch_bytes(p->N, p->d);
     void* base = nullptr;
-    if (int rc = ensure_work(enc + idx_b + coef_b + 2 * g_b + div_b, &base, static_cast<cudaStream_t>(p->stream))) return rc;
+    if (int rc = ensure_work(enc + idx_b + coef_b + dict_train_scratch_bytes(p->N, p->d), &base, static_cast<cudaStream_t>(p->stream))) return rc;
     char* q = static_cast<char*>(align_up(static_cast<char*>(base) + kStatusBytes, 1024)) + enc;
     TrainArgs a;
     a.D = static_cast<float*>(p->D);
@@ -724,9 +722,6 @@ int csr_dict_train_step(const csr_train_params_t* p) {
     a.idx = reinterpret_cast<uint16_t*>(q);
     a.coef = reinterpret_cast<float*>(q + idx_b);
     a.grad_mse = reinterpret_cast<float*>(q + idx_b + coef_b);
-    a.grad_div = reinterpret_cast<float*>(q + idx_b + coef_b + g_b);
-    a.div_scratch = q + idx_b + coef_b + 2 * g_b;
-    a.status = static_cast<uint32_t*>(base);
     a.losses = p->losses;
     a.lr = p->lr;
     a.beta = p->beta;
