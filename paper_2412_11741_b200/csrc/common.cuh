@@ -46,6 +46,7 @@ struct EncodeArgs {
     int64_t ld_code;   // elements between consecutive rows of out_idx and of out_coef (>= s)
     cudaStream_t stream;
     float load = 1.f;  // rows in flight on the GPU beside these, these included, as a multiple of M (grouped calls)
+    bool after_copy = false;   // the launch before this one on the stream is the dictionary's conversion (prepare_fast_dictionary)
 };
 
 // fp32-operand matching pursuit with fp64 re-scoring of unresolved picks.

@@ -405,6 +405,7 @@ int encode_device(const csr_encode_params_t* p, bool shared_scratch = true, cons
     if (!status) status = static_cast<uint32_t*>(base);
     char* scratch = static_cast<char*>(align_up(static_cast<char*>(base) + kStatusBytes, 1024));
     if (int rc = prepare_fast_dictionary(a.D, a.N, a.d, scratch, a.stream)) return rc;
+    a.after_copy = true;
     return launch_encode_fast_prepared(a, scratch, status, split ? scratch + dict_b : nullptr);
 }
 

@@ -299,14 +299,23 @@ __device__ __forceinline__ void pick_and_update(uint8_t* Atile, int q, int lane,
 }
 
 // ---------------------------------------------------------------------------------------
-// dictionary preparation: fp32 -> bf16 copy, same [N][d] layout
+// dictionary preparation: fp32 -> bf16 copy, same [N][d] layout, zeros up to a multiple of eight atoms
 // ---------------------------------------------------------------------------------------
-__global__ void dict_to_bf16_kernel(const float4* __restrict__ src, uint2* __restrict__ dst, int64_t n_vec4) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec4; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 v = src[i];
-        uint2 o;
-        o.x = pack_bf16(v.x, v.y);
-        o.y = pack_bf16(v.z, v.w);
+// The encoder that follows may be launched with programmatic stream serialization (EncodeArgs::after_copy): its CTAs come
+// up beside this kernel's, load their rows and wait for its end before they touch the copy.  4160 fp32 rows, N = 1024,
+// s = 8: 45.1 us one after the other, 42.0 so; 100003 rows, N = 5001, d = 64, whose padding was a launch of its own: 432 -> 428.
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__global__ void dict_to_bf16_kernel(const float4* __restrict__ src, uint2* __restrict__ dst, int64_t n_vec4, int64_t n_padded) {
+    next_may_start();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_padded; i += (int64_t)gridDim.x * blockDim.x) {
+        uint2 o = make_uint2(0u, 0u);
+        if (i < n_vec4) {
+            const float4 v = src[i];
+            o.x = pack_bf16(v.x, v.y);
+            o.y = pack_bf16(v.z, v.w);
+        }
         dst[i] = o;
     }
 }
@@ -494,6 +503,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap_d)) : "memory");
+            wait_for_previous();                              // the bf16 copy
             uint32_t p = 0;
             bool ok = true;
             for (int64_t pair = pair_first; pair < n_pairs && ok; pair += pair_step) {
@@ -688,6 +698,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
             }
             fence_proxy_async_smem();
             mbar_arrive(&sm.res_ready[tile]);
+            wait_for_previous();                              // (the picks read the copy too)
 
             for (int g = 0; g < s && ok; ++g) {
                 // ---- sweep: running arg-max of |correlation| over all atom tiles ----
@@ -925,6 +936,7 @@ encode_few_kernel(const uint16_t* __restrict__ Db, const void* __restrict__ X, i
         sm.abort = 0;
         fence_barrier_init();
     }
+    wait_for_previous();
     // ---- this warp's atoms ----
     const int a0 = (cta * RT_WARPS + warp) * (MT * 16);   // atoms a0 + 16 mt + l4 (+ 8)
     uint32_t A[MT][KT][4];
@@ -1157,6 +1169,13 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int clus
     cfg.numAttrs = 1;
 }
 
+// Adds to cfg that its CTAs may come up before the kernel in front of them has ended.
+void beside_previous(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    ++cfg.numAttrs;
+}
+
 // How many clusters of `cluster_ctas` CTAs of the encoder the device holds at once (0: none,
 // or clusters of that size cannot be launched here).  Asked once per size.
 template <int D_, int G>
@@ -1210,9 +1229,10 @@ int launch(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db, uin
                      : n_splits > 1  ? (int)(n_pairs * n_splits)
                                      : (int)(n_pairs < (int64_t)sm_count() ? n_pairs : (int64_t)sm_count());
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cluster_config<D_, G>(cfg, attr, tile_splits > 1 ? tile_splits : 1, grid, smem, a.stream);
     if (tile_splits <= 1) cfg.numAttrs = 0;
+    if (a.after_copy) beside_previous(cfg, attr);
     e = cudaLaunchKernelEx(&cfg, kernel, tmap, Db, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx, a.out_coef, a.coef_dtype,
                            a.ld_code, vec_codes, key_mask, status, tile_splits > 0 ? tile_splits : n_splits, partial,
                            options().wait_limit_ns);
@@ -1335,10 +1355,11 @@ int launch_few(const EncodeArgs& a, const uint16_t* Db, uint32_t* status) {
     if (e == cudaSuccess) {
         const uint32_t key_mask = ~static_cast<uint32_t>(TILE_N / G - 1);
         cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         cluster_config<D_, G>(cfg, attr, n_ctas, (int)((a.M + 8 * NTL - 1) / (8 * NTL)) * n_ctas, 0, a.stream);
         cfg.blockDim = dim3(RT_THREADS, 1, 1);
         if (n_ctas == 1) cfg.numAttrs = 0;
+        if (a.after_copy) beside_previous(cfg, attr);
         e = cudaLaunchKernelEx(&cfg, kernel, Db, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx, a.out_coef, a.coef_dtype, a.ld_code,
                                key_mask, status, n_ctas, options().wait_limit_ns);
     }
@@ -1362,6 +1383,7 @@ int launch_planned(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t*
     const RowPlan p = options().fast_split == 0 ? plan_rows<D_, G>(a.M, a.N, a.load) : RowPlan{a.M, {0, 0}, {0, 0}, 0.f};
     auto rows_from = [&](int64_t r0, int64_t m) {
         EncodeArgs b = a;
+        b.after_copy = a.after_copy && r0 == 0;            // (the launches after the first follow an encoder)
         b.X = static_cast<const char*>(a.X) + (size_t)r0 * a.ldx * dtype_size(a.x_dtype);
         b.out_idx = a.out_idx + r0 * a.ld_code;
         b.out_coef = static_cast<char*>(a.out_coef) + (size_t)r0 * a.ld_code * (a.coef_dtype == CSR_DTYPE_F16 ? 2 : 4);
@@ -1417,6 +1439,7 @@ int run_split_g(const EncodeArgs& a, const CUtensorMap& tmap, const uint16_t* Db
     const int64_t chunks = a.M * (D_ / 8);
     rows_to_bf16_kernel<D_><<<(unsigned)((chunks + 255) / 256), 256, 0, a.stream>>>(a.X, a.x_dtype, a.ldx, a.M, Rb);
     EncodeArgs b = a;
+    b.after_copy = false;
     b.X = Rb;
     b.x_dtype = CSR_DTYPE_BF16;
     b.ldx = D_;
@@ -1457,18 +1480,13 @@ size_t encode_fast_workspace_bytes(int d, int N) { return (size_t)padded_atoms(N
 int prepare_fast_dictionary(const float* D, int N, int d, void* workspace, cudaStream_t stream) {
     if ((reinterpret_cast<uintptr_t>(workspace) & 1023u) != 0)
         return fail(CSR_ERR_ALIGNMENT, "internal: dictionary scratch not 1024-byte aligned");
-    const int64_t n_vec4 = (int64_t)N * d / 4;
-    int blocks = (int)((n_vec4 + 255) / 256);
+    const int64_t n_vec4 = (int64_t)N * d / 4, n_padded = (int64_t)padded_atoms(N) * d / 4;
+    int blocks = (int)((n_padded + 255) / 256);
     if (blocks > 4 * sm_count()) blocks = 4 * sm_count();
-    dict_to_bf16_kernel<<<blocks, 256, 0, stream>>>(reinterpret_cast<const float4*>(D), reinterpret_cast<uint2*>(workspace),
-                                                    n_vec4);
+    dict_to_bf16_kernel<<<blocks, 256, 0, stream>>>(reinterpret_cast<const float4*>(D), reinterpret_cast<uint2*>(workspace), n_vec4,
+                                                    n_padded);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "dict_to_bf16 launch: %s", cudaGetErrorString(e));
-    const int n_pad = padded_atoms(N);
-    if (n_pad > N) {
-        e = cudaMemsetAsync(static_cast<char*>(workspace) + (size_t)N * d * 2, 0, (size_t)(n_pad - N) * d * 2, stream);
-        if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-    }
     return CSR_OK;
 }
 
@@ -1511,7 +1529,9 @@ int load_fast_kernels(int d, int N) {
 int launch_encode_fast(const EncodeArgs& a, void* workspace, uint32_t* status) {
     if (a.M == 0) return CSR_OK;
     if (int rc = prepare_fast_dictionary(a.D, a.N, a.d, workspace, a.stream)) return rc;
-    return launch_encode_fast_prepared(a, workspace, status, nullptr);
+    EncodeArgs b = a;
+    b.after_copy = true;
+    return launch_encode_fast_prepared(b, workspace, status, nullptr);
 }
 
 int launch_encode_fast_prepared(const EncodeArgs& a, const void* dict_bf16, uint32_t* status, void* split_scratch) {
