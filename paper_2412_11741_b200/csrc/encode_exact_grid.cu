@@ -6,7 +6,7 @@
 // (row tiles) x (slices of the dictionary), at most one CTA per SM, and all s iterations run in one
 // launch.  Per iteration
 //   - every CTA loads its tile's 128 residual rows as fp16 (32 KB from the L2), multiplies them with
-//     its slice by the same fp16 product per correlation, and every thread keeps the five
+//     its slice by the same fp16 product per correlation, and every thread keeps the
 //     largest keys of its half row (drain as in encode_exact_tc.cu);
 //   - the keys go to a scratch array, the CTAs of the row tile meet (counter in global memory,
 //     bounded wait);
@@ -35,12 +35,12 @@ constexpr int MMA_WARP = 9;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int UNIT = 64;                                  // atoms per TMA box; slices are whole units
 constexpr int MAX_SLICES = TILE_M;                        // at most one CTA per row
-constexpr int CAND = 16;                                  // candidates a row may have before the whole dictionary is re-scored
+constexpr int CAND = 16;                                  // groups a row may have inside the band before the whole dictionary is re-scored
 
-// Keys of one row over one column half of a slice: the five largest and the atoms of the first four.
-struct __align__(16) Entry {
+// Keys of one row over one column half of a slice: the four largest and the groups of the first three, by their first atom.
+struct __align__(8) Entry {
     uint32_t k[4];
-    uint32_t k4, n01, n23, pad;
+    uint32_t n01, n2;
 };
 
 template <int D_>
@@ -50,7 +50,7 @@ struct GridSmem {
     static constexpr int kStageBytes = TILE_N * STAGE_CH * 2;
     alignas(1024) uint8_t A[kATileBytes];
     alignas(1024) uint8_t B[kStages][kStageBytes];
-    // of the rows settled here: the largest key, the atoms inside the band, their number
+    // of the rows settled here: the largest key, the groups inside the band by their first atoms, their number
     uint32_t top_key[TILE_M];
     uint16_t cand[TILE_M][CAND];
     int n_cand[TILE_M];
@@ -81,7 +81,8 @@ struct GridArgs {
     double* Rd;             // [tiles * 128][d] fp64 residual rows
     uint32_t* Rh;           // [tiles * 128][d / 2] the scaled rows as fp16, two channels per word
     float2* band;           // [tiles * 128] band and norm of the scaled rows
-    const DictPart* parts;  // [n_parts] bounds of the dictionary
+    const uint16_t* dict;   // [N][d] the dictionary's scaled fp16 copy
+    const DictPart* parts;  // [n_parts] its bounds
     int n_parts;
     Entry* entries;         // [tiles][128][2 * slices]
     uint32_t* counters;     // [tiles * 32], zero at launch
@@ -254,6 +255,7 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
     } else {
         // ------------------------------ epilogue ------------------------------
         constexpr int CH = D_ / 8;                        // channels per lane when eight lanes share a row
+        constexpr int G = kGroup<D_>;
         const int q = warp & 3, half = warp >> 2;         // TMEM lane quarter, column half
         const int r_own = q * 32 + lane;                  // the row of the tile whose correlations this thread sees
         const int l8 = lane & 7, grp = lane >> 3;
@@ -318,8 +320,8 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
             fence_proxy_async_smem();
             mbar_arrive(&sm.res_ready);
 
-            // ---- sweep of this slice: top five keys of this thread's half row ----
-            Top5 top = top5_none();
+            // ---- sweep of this slice: the largest keys of this thread's half row ----
+            Tops top = no_tops();
             const float fband = band_own > 0.f ? band_own * 1.0625f : -1.f;
             for (int t = 0; t < T; ++t, ++accn) {
                 const int acc = accn & 1;
@@ -333,17 +335,25 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
                 const int w = min(TILE_N, width - t * TILE_N);
                 const uint32_t ta = taddr + acc * TILE_N + half * (w / 2);
                 uint64_t* back = &sm.acc_empty[acc];
-                drain(ta, w / UNIT, top, static_cast<uint32_t>(t), fband, back, lane);
+                const uint32_t id = static_cast<uint32_t>(t);
+                if (w == TILE_N)
+                    drain<G, 4>(ta, top, id, fband, back, lane);
+                else if (w == 3 * UNIT)
+                    drain<G, 3>(ta, top, id, fband, back, lane);
+                else if (w == 2 * UNIT)
+                    drain<G, 2>(ta, top, id, fband, back, lane);
+                else
+                    drain<G, 1>(ta, top, id, fband, back, lane);
             }
             if (ok && r_own < rows_here) {
-                auto atom = [&](uint32_t key, uint32_t id) {      // (an empty key's place is never used)
+                auto start = [&](uint32_t key, uint32_t id) {     // (an empty key's place is never used)
                     const int t = static_cast<int>(id), w = min(TILE_N, width - t * TILE_N);
-                    return static_cast<uint32_t>(n_first + t * TILE_N + half * (w / 2) + 127 - static_cast<int>(key & 127u)) & 0xFFFFu;
+                    return static_cast<uint32_t>(n_first + t * TILE_N + half * (w / 2) + static_cast<int>(key & 31u) * G) & 0xFFFFu;
                 };
-                uint4* e = reinterpret_cast<uint4*>(a.entries + ((row_base + r_own) * n_ent + 2 * slice + half));
-                __stcg(e + 0, make_uint4(top.k0, top.k1, top.k2, top.k3));
-                __stcg(e + 1, make_uint4(top.k4, atom(top.k0, top.i0) | (atom(top.k1, top.i1) << 16),
-                                         atom(top.k2, top.i2) | (atom(top.k3, top.i3) << 16), 0u));
+                uint2* e = reinterpret_cast<uint2*>(a.entries + ((row_base + r_own) * n_ent + 2 * slice + half));
+                __stcg(e + 0, make_uint2(top.k0, top.k1));
+                __stcg(e + 1, make_uint2(top.k2, top.k3));
+                __stcg(e + 2, make_uint2(start(top.k0, top.i0) | (start(top.k1, top.i1) << 16), start(top.k2, top.i2)));
             }
             ok = meet(counter, target += slices, slices, ok, wc);
             if (!ok) break;
@@ -361,13 +371,13 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
 #pragma unroll
             for (int u = 0; u < TRIPS; ++u) {
                 const int f = threadIdx.x + u * EPI;
-                mine[u] = Entry{{0u, 0u, 0u, 0u}, 0u, 0u, 0u, 0u};
+                mine[u] = Entry{{0u, 0u, 0u, 0u}, 0u, 0u};
                 band_of[u] = make_float2(0.f, 0.f);
                 if (f < n_own * n_ent) {
                     const int64_t row = row_base + slice + f / n_ent * slices;
-                    const uint4* e = reinterpret_cast<const uint4*>(a.entries + (row * n_ent + f % n_ent));
-                    const uint4 e0 = __ldcg(e), e1 = __ldcg(e + 1);
-                    mine[u] = Entry{{e0.x, e0.y, e0.z, e0.w}, e1.x, e1.y, e1.z, 0u};
+                    const uint2* e = reinterpret_cast<const uint2*>(a.entries + (row * n_ent + f % n_ent));
+                    const uint2 e0 = __ldcg(e), e1 = __ldcg(e + 1), e2 = __ldcg(e + 2);
+                    mine[u] = Entry{{e0.x, e0.y, e1.x, e1.y}, e2.x, e2.y};
                     band_of[u] = __ldcg(a.band + row);
                 }
             }
@@ -385,12 +395,12 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
                 const int k = f / n_ent;
                 const float v0 = __uint_as_float(sm.top_key[k] & kKeyMask), band = band_of[u].x;
                 if (!(v0 > 0.f) || a.N == 1 || v0 - __uint_as_float(mine[u].k[0] & kKeyMask) > band) continue;
-                // five of a half slice inside the band: there may be more; a band above everything: anything may be the pick
-                bool full = !(v0 > band) || (mine[u].k4 != 0u && !(v0 - __uint_as_float(mine[u].k4 & kKeyMask) > band));
+                // four of a half slice inside the band: there may be more; a band above everything: anything may be the pick
+                bool full = !(v0 > band) || (mine[u].k[3] != 0u && !(v0 - __uint_as_float(mine[u].k[3] & kKeyMask) > band));
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint32_t key = mine[u].k[i], n2 = i < 2 ? mine[u].n01 : mine[u].n23;
-                    const uint32_t n = (i & 1) ? n2 >> 16 : n2 & 0xFFFFu;
+                for (int i = 0; i < 3; ++i) {
+                    const uint32_t key = mine[u].k[i];
+                    const uint32_t n = i == 0 ? mine[u].n01 & 0xFFFFu : i == 1 ? mine[u].n01 >> 16 : mine[u].n2;
                     if (key != 0u && !(v0 - __uint_as_float(key & kKeyMask) > band) && n < static_cast<uint32_t>(a.N)) {
                         const int slot = atomicAdd(&sm.n_cand[k], 1);
                         if (slot < CAND)
@@ -437,39 +447,38 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
                         R[2 * c + 1] = x.y;
                     }
                     const bool open = (sm.unknown[kk >> 5] >> (kk & 31)) & 1u;
-                    int cnt = min(sm.n_cand[kk], CAND);   // none: an all-zero sweep (or NaN, or one atom) picks atom 0
+                    const int cnt = min(sm.n_cand[kk], CAND);   // none: an all-zero sweep (or NaN, or one atom) picks atom 0
                     int n = cnt > 0 ? sm.cand[kk][0] : 0;
+                    [[maybe_unused]] bool single = false;
                     if (round == 1) {                     // searched for by all warps: nothing left to decide
                         n = has ? sm.found_n[kk] : 0;
-                        cnt = 0;
-                    } else if (open) {
-                        has = false;
-                        cnt = min(cnt, 1);
-                    }
-                    const bool cmp = cnt > 1;        // several candidates: their fp64 correlations decide, the lowest atom among equals
-                    if (__any_sync(FULL, cmp)) {
-                        const int most = static_cast<int>(__reduce_max_sync(FULL, cmp ? static_cast<unsigned>(cnt) : 0u));
-                        double cbest = -1.0;
-                        int nbest = n;
+                    } else {
+                        // the pick's atom within its group; where that does not decide it, fp64 over all groups, a row at a time
+                        if (open) has = false;
+                        GroupAtoms<D_> ga;
+                        ga.load(a.dict, n, a.N, l8);
+                        uint4 r[D_ / 64];
+#pragma unroll
+                        for (int j = 0; j < D_ / 64; ++j) r[j] = *reinterpret_cast<const uint4*>(&sm.A[swz_off(slice + kk * slices, l8 + 8 * j)]);
+                        const uint32_t bits = (inside(ga.value(r, n, a.N, l8), __ldcg(&a.band[row].x)) >> (8 * grp)) & 255u;
+                        const int first = bits == 0u ? 0 : G == 8 ? __ffs(bits) - 1 : (__ffs(bits) - 1) / 2;
+                        single = cnt == 1 && bits != 0u && (bits >> (G == 8 ? first : 2 * first)) <= (G == 8 ? 1u : 3u);
+                        if (single) n += first;
 #pragma unroll 1
-                        for (int ci = 0; ci < most; ++ci) {
-                            const int nc = cmp ? sm.cand[kk][min(ci, cnt - 1)] : n;
-                            float ax[CH];
-                            load_atom<CH>(a.D + static_cast<int64_t>(nc) * D_, l8, ax);
-                            const double cc = fabs(group8_sum(slice_dot<CH>(R, ax)));
-                            if (cc > cbest || (cc == cbest && nc < nbest)) {
-                                cbest = cc;
-                                nbest = nc;
-                            }
+                        for (uint32_t left = __ballot_sync(FULL, has && cnt > 0 && !single && l8 == 0); left; left &= left - 1) {
+                            const int src = __ffs(left) - 1;
+                            const int k2 = __shfl_sync(FULL, kk, src);
+                            const int found = decide<D_>(a.D, a.N, a.Rd + (row_base + slice + k2 * slices) * D_, min(sm.n_cand[k2], CAND),
+                                                         [&](int i) { return static_cast<int>(sm.cand[k2][i]); }, lane);
+                            if (grp == (src >> 3)) n = found;
                         }
-                        if (cmp) n = nbest;
                     }
                     float at[CH];
                     load_atom<CH>(a.D + static_cast<int64_t>(n) * D_, l8, at);
                     const double c = group8_sum(slice_dot<CH>(R, at));
 #ifdef CSR_DEBUG_CHECKS
                     const float2 bn = __ldcg(a.band + row);
-                    check_value<CH>(a.diag, R, at, c, __uint_as_float(sm.top_key[kk] & kKeyMask), bn.x, bn.y, db, l8, has && round == 0 && cnt == 1);
+                    check_value<CH>(a.diag, R, at, c, __uint_as_float(sm.top_key[kk] & kKeyMask), bn.x, bn.y, db, l8, has && single);
 #endif
                     if (l8 == 0 && has) {
                         a.out_idx[row * a.ldc + g] = static_cast<uint16_t>(n);
@@ -563,6 +572,7 @@ int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* di
     p += rows * a.d * 2;
     g.band = reinterpret_cast<float2*>(p);
     p += align256(rows * 8);
+    g.dict = static_cast<const uint16_t*>(dict_f16);
     g.parts = static_cast<const DictPart*>(dict_parts);
     g.n_parts = n_parts;
     g.entries = reinterpret_cast<Entry*>(p);

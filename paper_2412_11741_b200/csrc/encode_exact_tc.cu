@@ -16,18 +16,21 @@
 //   - each row tile has one 256-column fp32 accumulator in TMEM.  All eight epilogue warps drain
 //     every accumulator: warp w reads the 32 TMEM lanes of w % 4 and the 128 columns of w / 4, i.e.
 //     all of them sit in registers after one round of loads and the accumulator goes straight back
-//     to the tensor core.  Each thread keeps the five largest keys of its half row, a key being
-//     |value| with its seven lowest mantissa bits replaced by the column's tag, and where the
-//     largest four came from.  Groups of eight values are first reduced to their largest
-//     magnitude and only groups within the band of the running maximum are inserted;
+//     to the tensor core.  Groups of adjacent atoms (kGroup) are reduced to their largest magnitude, a key being
+//     that with its five lowest mantissa bits replaced by the group's number, and each thread keeps the tile's three
+//     largest keys, all without a branch; those within the band of the row's running maximum then join
+//     the four largest keys of its half row (three of them with the tile they came from);
 //   - at the end of a sweep the halves meet in shared memory, and each warp settles its 32 rows,
-//     eight lanes per row: rows whose best and second-best keys are further apart than the band
-//     take the best; otherwise the candidates inside the band (the first four of either half)
-//     are compared in fp64; rows where the fifth of a half is inside too are searched for in the
+//     eight lanes per row: the values of the group with the largest key are computed again from the fp16 operands.  Rows
+//     whose best atom is further than the band above the rest of its group and above every other group
+//     take it; otherwise all atoms of the groups inside the band (the first three of either half) are compared in
+//     fp64, a row at a time by the warp; rows where the fourth of a half is inside too are searched for in the
 //     whole dictionary (fp32 filter, then fp64) by the eight warps together.  Coefficient (Eq. 2,
 //     signed) and residual update (Eq. 4) are fp64, as in the plain-ALU encoder.
-// What bounds it: the epilogue and the settling, no longer the MMAs (2048 cycles per 256 atoms and pair of row tiles).
-// Three bf16 products per correlation, whose band was 2^-12 ||R||, took 6144: 100000 rows, N = 4096, s = 8,
+// What bounds it: at N = 4096 a sweep takes 44000 cycles (2048 of 2700 per 256 atoms are MMAs), the gathers of the groups
+// 10000, what fp64 decides 8000, the settling 28000.  With the five largest keys kept value by value, a branch per
+// eight of them, a sweep took 101000 (5000 a tile): 100000 rows, N = 4096, s = 8, 1916 us so and 1388 us now;
+// a training step (65536 rows, N = 8192, s = 8) 1872 and 1394.  Three bf16 products per correlation, whose band was 2^-12 ||R||, took 6144: 100000 rows, N = 4096, s = 8,
 // 2441 us so and 2195 us with one fp16 product; a training step of 65536 rows (N = 8192, s = 8) 2992 and 2332 us.
 // Warp roles: 0-7 epilogue, 8 TMA producer, 9 TMEM owner and MMA issuer.  All waits are bounded.
 #include "exact_tc_common.cuh"
@@ -51,7 +54,7 @@ struct TcSmem {
     static constexpr int kStageBytes = TILE_N * STAGE_CH * 2;
     alignas(1024) uint8_t A[2][kATileBytes];
     alignas(1024) uint8_t B[kStages][kStageBytes];
-    uint32_t xchg[6][TILE_M];                                    // one half's top five of a row tile (and the rows' bands)
+    uint32_t xchg[5][TILE_M];                                    // one half's largest keys of a row tile (and the rows' bands)
     uint64_t full_b[kStages];
     uint64_t empty_b[kStages];
     uint64_t acc_full[2];
@@ -64,7 +67,7 @@ struct TcSmem {
 
 template <int D_>
 __global__ void __launch_bounds__(NT, 1)
-encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPart* __restrict__ parts, int n_parts, const float* __restrict__ D, const void* __restrict__ X, int x_dtype, int64_t ldx, int64_t M, int N, int s,
+encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* __restrict__ dict, const DictPart* __restrict__ parts, int n_parts, const float* __restrict__ D, const void* __restrict__ X, int x_dtype, int64_t ldx, int64_t M, int N, int s,
                        uint16_t* __restrict__ out_idx, void* __restrict__ out_coef, int coef_dtype, int64_t ldc,
                        double* __restrict__ Rd_all, uint32_t* status, [[maybe_unused]] uint32_t* diag,
                        unsigned long long wait_limit_ns) {
@@ -194,6 +197,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
     } else {
         // ------------------------------ epilogue ------------------------------
         constexpr int CH = D_ / 8;                          // channels per lane when eight lanes share a row
+        constexpr int G = kGroup<D_>;
         const int q = warp & 3;                             // TMEM lane quarter
         const int half = warp >> 2;                         // column half drained by this warp
         const int own_tile = warp >> 2;                     // row tile whose rows this warp settles
@@ -238,8 +242,8 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
             mbar_arrive(&sm.res_ready);
 
             for (int g = 0; g < s && ok; ++g) {
-                // ---- sweep: top five keys of this thread's half of two rows ----
-                Top5 st[2] = {top5_none(), top5_none()};
+                // ---- sweep: the largest keys of this thread's half of two rows ----
+                Tops st[2] = {no_tops(), no_tops()};
                 // the filter's bands of this thread's two rows: its own and the one the warp of the
                 // other row tile left in shared memory
                 float* band_x = reinterpret_cast<float*>(&sm.xchg[0][0]);
@@ -260,8 +264,8 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
                             break;
                         }
                         tc_fence_after();
-                        Top5 qa = a ? st[1] : st[0];
-                        drain128(taddr + a * TILE_N, qa, static_cast<uint32_t>(t), a ? fband[1] : fband[0], &sm.acc_empty[a], lane);
+                        Tops qa = a ? st[1] : st[0];
+                        drain<G, 4>(taddr + a * TILE_N, qa, static_cast<uint32_t>(t), a ? fband[1] : fband[0], &sm.acc_empty[a], lane);
                         if (a)
                             st[1] = qa;
                         else
@@ -269,19 +273,18 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
                     }
                 }
                 // ---- bring the column halves together: warps 0-3 get row tile 0's, warps 4-7 row tile 1's ----
-                auto post = [&](const Top5& o) {
+                auto post = [&](const Tops& o) {
                     sm.xchg[0][r_own] = o.k0;
                     sm.xchg[1][r_own] = o.k1;
                     sm.xchg[2][r_own] = o.k2;
                     sm.xchg[3][r_own] = o.k3;
-                    sm.xchg[4][r_own] = o.k4;
-                    sm.xchg[5][r_own] = o.i0 | (o.i1 << 8) | (o.i2 << 16) | (o.i3 << 24);   // (at most 256 tiles)
+                    sm.xchg[4][r_own] = o.i0 | (o.i1 << 8) | (o.i2 << 16);   // (at most 256 tiles)
                 };
-                Top5 other = top5_none();
+                Tops other = no_tops();
                 auto take = [&]() {
-                    const uint32_t ids = sm.xchg[5][r_own];
-                    other = Top5{sm.xchg[0][r_own], sm.xchg[1][r_own], sm.xchg[2][r_own], sm.xchg[3][r_own],
-                                 sm.xchg[4][r_own], ids & 255u,        (ids >> 8) & 255u, (ids >> 16) & 255u, ids >> 24};
+                    const uint32_t ids = sm.xchg[4][r_own];
+                    other = Tops{sm.xchg[0][r_own], sm.xchg[1][r_own], sm.xchg[2][r_own], sm.xchg[3][r_own],
+                                 ids & 255u,        (ids >> 8) & 255u, ids >> 16};
                 };
                 if (half == 1) post(st[0]);
                 if (epilogue_barrier_any(!ok || sm.abort != 0)) {
@@ -294,43 +297,81 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
                 epilogue_barrier();
                 if (half == 1) take();
                 epilogue_barrier();                         // (the exchange area is rewritten from here on)
-                // The row's candidates: the first four of either half (two 16-bit atoms per word), a bit in
-                // my_flags for each that is inside the band; kUnknown: the fifth of a half is inside too, so there
-                // may be more than are known (NaN counts as inside).
-                constexpr int kUnknown = 256;
-                const Top5 mine = own_tile ? st[1] : st[0];
+                // The row's groups: the first three of either half, a bit in my_flags for each that is inside the band;
+                // kUnknown: the fourth of a half is inside too, so there may be more than are known (NaN counts as inside).
+                constexpr int kUnknown = 64;
+                const Tops mine = own_tile ? st[1] : st[0];
                 const float v0 = fmaxf(__uint_as_float(mine.k0 & kKeyMask), __uint_as_float(other.k0 & kKeyMask));
-                uint32_t my_cand[4];
-                int my_flags = 0, my_n1 = 0;                // an all-zero sweep picks atom 0
+                int my_start[6], my_flags = 0, my_n1 = 0, my_first = 0;   // an all-zero sweep picks atom 0
                 {
-                    const uint32_t key[8] = {mine.k0, mine.k1, mine.k2, mine.k3, other.k0, other.k1, other.k2, other.k3};
-                    const uint32_t id[8] = {mine.i0, mine.i1, mine.i2, mine.i3, other.i0, other.i1, other.i2, other.i3};
-                    int at[8];
+                    const uint32_t key[6] = {mine.k0, mine.k1, mine.k2, other.k0, other.k1, other.k2};
+                    const uint32_t id[6] = {mine.i0, mine.i1, mine.i2, other.i0, other.i1, other.i2};
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)             // (mine: the columns of this warp's half)
-                        at[i] = static_cast<int>(id[i]) * TILE_N + (i < 4 ? half : half ^ 1) * 128 + 127 - static_cast<int>(key[i] & 127u);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        my_cand[i] = (static_cast<uint32_t>(at[2 * i]) & 0xFFFFu) | (static_cast<uint32_t>(at[2 * i + 1]) << 16);
+                    for (int i = 0; i < 6; ++i)             // (mine: the columns of this warp's half)
+                        my_start[i] = static_cast<int>(id[i]) * TILE_N + (i < 3 ? half : half ^ 1) * 128 + static_cast<int>(key[i] & 31u) * G;
                     if (v0 > 0.f && N > 1) {
 #pragma unroll
-                        for (int i = 7; i >= 0; --i)
-                            if (!(v0 - __uint_as_float(key[i] & kKeyMask) > band) && at[i] < N) {
+                        for (int i = 5; i >= 0; --i)
+                            if (!(v0 - __uint_as_float(key[i] & kKeyMask) > band) && my_start[i] < N) {
                                 my_flags |= 1 << i;
-                                my_n1 = at[i];
+                                my_first = my_start[i];
                             }
-                        if (!(v0 - __uint_as_float(mine.k4 & kKeyMask) > band) || !(v0 - __uint_as_float(other.k4 & kKeyMask) > band))
+                        if (!(v0 - __uint_as_float(mine.k3 & kKeyMask) > band) || !(v0 - __uint_as_float(other.k3 & kKeyMask) > band))
                             my_flags |= kUnknown;
+                    }
+                }
+
+                // ---- the pick's atom within its group; a wave of passes' gathers in flight together ----
+                bool open = false;                          // this lane's row is for fp64 to decide
+                {
+                    constexpr int CK = D_ / 64, WAVE = 32 / (G * CK);
+#pragma unroll 1
+                    for (int w0 = 0; w0 < 8; w0 += WAVE) {
+                        GroupAtoms<D_> at[WAVE];
+                        int n0[WAVE];
+#pragma unroll
+                        for (int u = 0; u < WAVE; ++u) {
+                            n0[u] = __shfl_sync(FULL, my_first, 4 * (w0 + u) + grp);
+                            at[u].load(dict, n0[u], N, l8);
+                        }
+#pragma unroll
+                        for (int u = 0; u < WAVE; ++u) {
+                            const int src = 4 * (w0 + u) + grp;
+                            uint4 r[CK];
+#pragma unroll
+                            for (int j = 0; j < CK; ++j) r[j] = *reinterpret_cast<const uint4*>(A_own + swz_off(q * 32 + src, l8 + 8 * j));
+                            const uint32_t in = inside(at[u].value(r, n0[u], N, l8), __shfl_sync(FULL, band, src));
+                            if ((lane >> 2) == w0 + u && my_flags != 0) {
+                                const uint32_t bits = (in >> (8 * (lane & 3))) & 255u;
+                                const int first = bits == 0u ? 0 : G == 8 ? __ffs(bits) - 1 : (__ffs(bits) - 1) / 2;
+                                my_n1 = my_first + first;   // (no value at all: a row that is not finite)
+                                open = bits == 0u || (bits >> (G == 8 ? first : 2 * first)) > (G == 8 ? 1u : 3u) || (my_flags & (my_flags - 1)) != 0;
+                            }
+                        }
+                    }
+#pragma unroll 1
+                    for (uint32_t left = __ballot_sync(FULL, open && (my_flags & kUnknown) == 0); left; left &= left - 1) {
+                        const int src = __ffs(left) - 1;
+                        int st6[6];
+#pragma unroll
+                        for (int i = 0; i < 6; ++i) st6[i] = __shfl_sync(FULL, my_start[i], src);
+                        const int f = __shfl_sync(FULL, my_flags, src);
+                        const int n = decide<D_>(D, N, Rd_cta + static_cast<int64_t>(own_tile * TILE_M + q * 32 + src) * D_, __popc(f), [&](int i) {
+                            int k = f;
+                            for (int j = 0; j < i; ++j) k &= k - 1;
+                            const int at = __ffs(k) - 1;
+                            return at == 0 ? st6[0] : at == 1 ? st6[1] : at == 2 ? st6[2] : at == 3 ? st6[3] : at == 4 ? st6[4] : st6[5];
+                        }, lane);
+                        if (lane == src) my_n1 = n;
                     }
                 }
 
                 // ---- settle the 32 rows of this warp, eight lanes per row, four rows per pass; the
                 // next pass's residual rows and atoms are requested before this pass is worked on
                 // (one copy of the code: it has to stay in the instruction cache next to the sweep) ----
-                auto fetch = [&](int p, int& n, int& flags, double (&R)[CH], float (&a)[CH]) {
+                auto fetch = [&](int p, int& n, double (&R)[CH], float (&a)[CH]) {
                     const int src = 4 * p + grp;
                     n = __shfl_sync(FULL, my_n1, src);
-                    flags = __shfl_sync(FULL, my_flags, src);
                     const double* Rrow = Rd_cta + static_cast<int64_t>(own_tile * TILE_M + q * 32 + src) * D_;
 #pragma unroll
                     for (int k = 0; k < CH / 2; ++k) {
@@ -364,19 +405,18 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
                             }
                         epilogue_barrier();                 // (the next sweep's bands go to the same words)
                         todo = unknown;
-                        my_flags = 0;
                     }
-                    int n, flags;
+                    int n;
                     double R[CH];
                     float a[CH];
-                    fetch(0, n, flags, R, a);
+                    fetch(0, n, R, a);
 #pragma unroll 1
                     for (int p = 0; p < 8; ++p) {
-                        int n_nx = 0, flags_nx = 0;
+                        int n_nx = 0;
                         double R_nx[CH];
                         float a_nx[CH];
                         if (p + 1 < 8) {
-                            fetch(p + 1, n_nx, flags_nx, R_nx, a_nx);
+                            fetch(p + 1, n_nx, R_nx, a_nx);
                         } else {
 #pragma unroll
                             for (int k = 0; k < CH; ++k) {
@@ -388,33 +428,11 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
                         const int r = q * 32 + src;
                         const int64_t m = pair * ROWS + own_tile * TILE_M + r;
                         const bool has = (todo >> src) & 1u;
-                        const bool cmp = (flags & (flags - 1)) != 0;         // this row has several candidates
-                        if (__any_sync(FULL, cmp)) {        // their fp64 correlations decide, the lowest atom among equals
-                            const int n_first = n;
-                            const uint32_t some = __reduce_or_sync(FULL, static_cast<uint32_t>(flags));
-                            double cbest = -1.0;
-                            int nbest = n;
-#pragma unroll 1
-                            for (int i = 0; i < 8; ++i) {
-                                if (!((some >> i) & 1u)) continue;
-                                const uint32_t pair_of = __shfl_sync(FULL, i < 2 ? my_cand[0] : i < 4 ? my_cand[1] : i < 6 ? my_cand[2] : my_cand[3], src);
-                                const bool in = cmp && ((flags >> i) & 1);
-                                const int nc = in ? static_cast<int>((i & 1) ? pair_of >> 16 : pair_of & 0xFFFFu) : n;
-                                float ax[CH];
-                                load_atom<CH>(D + static_cast<int64_t>(nc) * D_, l8, ax);
-                                const double cc = fabs(group8_sum(slice_dot<CH>(R, ax)));
-                                if (in && (cc > cbest || (cc == cbest && nc < nbest))) {
-                                    cbest = cc;
-                                    nbest = nc;
-                                }
-                            }
-                            if (cmp) n = nbest;
-                            if (__any_sync(FULL, n != n_first)) load_atom<CH>(D + static_cast<int64_t>(n) * D_, l8, a);
-                        }
                         const double c = group8_sum(slice_dot<CH>(R, a));
 #ifdef CSR_DEBUG_CHECKS
+                        const bool was_open = __shfl_sync(FULL, open, src);   // (every lane takes part)
                         check_value<CH>(diag, R, a, c, __shfl_sync(FULL, v0, src), __shfl_sync(FULL, band, src), __shfl_sync(FULL, norm, src), db, l8,
-                                        m < M && has && round == 0 && !cmp);
+                                        m < M && has && round == 0 && !was_open);
 #endif
                         if (l8 == 0 && m < M && has) {
                             out_idx[m * ldc + g] = static_cast<uint16_t>(n);
@@ -432,7 +450,6 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const DictPar
                             put_row(R, p, has, todo);
                         }
                         n = n_nx;
-                        flags = flags_nx;
 #pragma unroll
                         for (int k = 0; k < CH; ++k) {
                             R[k] = R_nx[k];
@@ -551,12 +568,12 @@ int ctas_for(int64_t M) {
 }
 
 template <int D_>
-int run(const EncodeArgs& a, const CUtensorMap& map, const DictPart* parts, int n_parts, double* Rd, uint32_t* status, uint32_t* diag) {
+int run(const EncodeArgs& a, const CUtensorMap& map, const uint16_t* dict, const DictPart* parts, int n_parts, double* Rd, uint32_t* status, uint32_t* diag) {
     const size_t smem = sizeof(TcSmem<D_>);
     cudaError_t e = cudaFuncSetAttribute(encode_exact_tc_kernel<D_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     const int grid = ctas_for(a.M);
-    encode_exact_tc_kernel<D_><<<grid, NT, smem, a.stream>>>(map, parts, n_parts, a.D, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx,
+    encode_exact_tc_kernel<D_><<<grid, NT, smem, a.stream>>>(map, dict, parts, n_parts, a.D, a.X, a.x_dtype, a.ldx, a.M, a.N, a.s, a.out_idx,
                                                              a.out_coef, a.coef_dtype, a.ld_code, Rd, status, diag, options().wait_limit_ns);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "encode_exact_tc launch: %s", cudaGetErrorString(e));
@@ -640,7 +657,8 @@ int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status,
         CUtensorMap map;
         if (int rc = dict_map(&map, dict, a.N, a.d, TILE_N)) return rc;
         double* Rd = reinterpret_cast<double*>(rows);
-        return a.d == 128 ? run<128>(b, map, parts, n_parts, Rd, status, diag) : run<64>(b, map, parts, n_parts, Rd, status, diag);
+        const uint16_t* copy = static_cast<const uint16_t*>(dict);
+        return a.d == 128 ? run<128>(b, map, copy, parts, n_parts, Rd, status, diag) : run<64>(b, map, copy, parts, n_parts, Rd, status, diag);
     };
     if (plan.pair_rows)
         if (int rc = run_pairs(rows_from(0, plan.pair_rows))) return rc;

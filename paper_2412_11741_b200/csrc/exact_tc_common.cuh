@@ -1,6 +1,6 @@
 // Pieces shared by the two tensor-core encoders of the correctness mode (one CTA per pair of row
 // tiles for all atoms; the dictionary split across the CTAs of one launch for fewer rows): the fp16
-// operands and the bound of what their rounding does to a correlation, the running top five of a row's
+// operands and the bound of what their rounding does to a correlation, the groups of atoms that hold a row's largest
 // correlations, the fp64 arithmetic of the picks.
 #pragma once
 
@@ -18,7 +18,12 @@ constexpr int TILE_M = 128;
 constexpr int TILE_N = 256;
 constexpr int UMMA_K = 16;
 constexpr int STAGE_CH = 64;
-constexpr uint32_t kKeyMask = 0x7FFFFF80u;                // |value| without its seven lowest mantissa bits
+constexpr uint32_t kKeyMask = 0x7FFFFFE0u;                // |value| without its five lowest mantissa bits
+// Adjacent atoms that the sweep takes as one: it keeps their largest |correlation|; which of them that was is found
+// when the row is settled (2 KB of the dictionary's fp16 copy gathered per row at d = 128).  Groups of four at d = 128:
+// a training step of 65536 rows (N = 8192, s = 8) 1511 us, of eight 1394.
+template <int D_>
+constexpr int kGroup = 8;
 constexpr uint32_t FULL = 0xffffffffu;
 // What the tensor cores' fp32 accumulation of d exact products of fp16 values (in groups of 16) may add to
 // the error of a correlation, relative to ||R|| and the largest norm of an atom.  Measured (checked
@@ -55,18 +60,17 @@ __device__ __forceinline__ uint32_t swz_off(int r, int chunk) {
     return kblock * (TILE_M * 128) + (r >> 3) * 1024 + (r & 7) * 128 + ((cc ^ (r & 7)) << 4);
 }
 
-// The five largest keys seen, in descending order, and the dictionary tiles the first four came from.
-struct Top5 {
-    uint32_t k0, k1, k2, k3, k4;
-    uint32_t i0, i1, i2, i3;
+// The largest keys of groups seen, in descending order, and the dictionary tiles the first three came from.  A key is a
+// group's largest |value| with the group's number inside the thread's part of a dictionary tile in its five lowest bits.
+struct Tops {
+    uint32_t k0, k1, k2, k3;
+    uint32_t i0, i1, i2;
 };
-__device__ __forceinline__ Top5 top5_none() { return Top5{0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}; }
+__device__ __forceinline__ Tops no_tops() { return Tops{0u, 0u, 0u, 0u, 0u, 0u, 0u}; }
 
-__device__ __forceinline__ void top5_insert(Top5& q, uint32_t k, uint32_t id) {
-    const bool p0 = k > q.k0, p1 = k > q.k1, p2 = k > q.k2, p3 = k > q.k3;
-    q.k4 = p3 ? q.k3 : max(q.k4, k);
-    q.k3 = p2 ? q.k2 : (p3 ? k : q.k3);
-    q.i3 = p2 ? q.i2 : (p3 ? id : q.i3);
+__device__ __forceinline__ void tops_insert(Tops& q, uint32_t k, uint32_t id) {
+    const bool p0 = k > q.k0, p1 = k > q.k1, p2 = k > q.k2;
+    q.k3 = p2 ? q.k2 : max(q.k3, k);
     q.k2 = p1 ? q.k1 : (p2 ? k : q.k2);
     q.i2 = p1 ? q.i1 : (p2 ? id : q.i2);
     q.k1 = p0 ? q.k0 : (p1 ? k : q.k1);
@@ -81,126 +85,79 @@ __device__ __forceinline__ float absmax3(float a, float b, float c) {
     return r;
 }
 
-// What the filter lets through and new_best did not settle, one copy for all groups of eight: keys `k0` .. `k7` whose last
-// three bits are the place in the group, `rest` the other bits of its tags.  Inserts from the largest down until what is
-// left is below the rising threshold.  A value more than the band above the running maximum leaves
-// everything seen so far outside the band, so it simply becomes the only entry.  Returns the new
-// state and threshold.
-struct Top5Thr {
-    Top5 q;
-    float thr;
+// The three largest keys of a thread's part of one dictionary tile.
+struct Three {
+    uint32_t a, b, c;
 };
-static __device__ __noinline__ Top5Thr insert_group(Top5 q, float thr, uint32_t k0, uint32_t k1, uint32_t k2, uint32_t k3, uint32_t k4,
-                                                    uint32_t k5, uint32_t k6, uint32_t k7, uint32_t rest, uint32_t id, float band) {
-    uint32_t k[8] = {k0, k1, k2, k3, k4, k5, k6, k7};
-#pragma unroll 1
-    for (int trip = 0; trip < 8; ++trip) {
-        const uint32_t a = __vimax3_u32(k[0], k[1], k[2]), b = __vimax3_u32(k[3], k[4], k[5]);
-        const uint32_t best = max(__vimax3_u32(k[6], k[7], a), b);
-        const float val = __uint_as_float(best & kKeyMask);
-        if (!(val >= thr)) break;
-        const uint32_t key = best | rest;
-        if (val > __uint_as_float(q.k0 & kKeyMask) + band)
-            q = Top5{key, 0u, 0u, 0u, 0u, id, 0u, 0u, 0u};
-        else
-            top5_insert(q, key, id);
-        thr = __uint_as_float(q.k0 & kKeyMask) - band;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) k[j] = k[j] == best ? 0u : k[j];
-    }
-    return Top5Thr{q, thr};
+// Two more keys: nine two- and three-input minima and maxima, no branch.
+__device__ __forceinline__ void fold2(Three& q, uint32_t g, uint32_t h) {
+    const uint32_t x = max(g, h), y = min(g, h);
+    const uint32_t s = min(q.a, x), u = max(q.b, y), w = min(q.b, y);
+    q.a = max(q.a, x);
+    q.c = __vimax3_u32(q.c, w, min(s, u));
+    q.b = max(s, u);
 }
-
-// Folds 32 columns of this thread's row into its top five; `tag0` is the tag of v[0] (tags fall
-// with the column so that the lowest column wins among equal magnitudes).  Eight values at a
-// time are first reduced to their largest magnitude (half an instruction each) and only a group
-// that reaches `thr`, the running maximum less the band, is looked at: whatever ends up within the band of the
-// final maximum was within the band of the running one when it came by, so what the filter
-// drops can never matter.  Nearly always the group's largest is then more than the band above the running
-// maximum and above the rest of its group: it becomes the only entry (the second largest of the group is found by
-// subtracting the largest from all keys: it turns to zero and the others stay in order).  Everything else
-// is a call: the sweep's code has to stay small enough for the instruction cache.  100000 rows, N = 4096, s = 8: 2195 us
-// with a call for every group that the filter lets through, 1916 us so.
-template <int J = 0>
-__device__ __forceinline__ void chunk_top5(const uint32_t (&v)[32], Top5& q, uint32_t id, uint32_t tag0, float& thr, float band) {
+// Key of the G values from v[J] on (a NaN counts as nothing).
+template <int G, int J>
+__device__ __forceinline__ uint32_t key_of(const uint32_t (&v)[32], uint32_t tag) {
+    auto f = [&](int j) { return __uint_as_float(v[J + j]); };
+    float m = absmax3(f(0), f(1), f(2));
+    if constexpr (G == 4)
+        m = absmax3(m, f(3), 0.f);
+    else
+        m = absmax3(absmax3(f(3), f(4), f(5)), absmax3(f(6), f(7), m), 0.f);
+    return (__float_as_uint(m) & kKeyMask) | tag;
+}
+// 32 columns, whose first group has number T0.
+template <int G, int T0, int J = 0>
+__device__ __forceinline__ void fold32(const uint32_t (&v)[32], Three& q) {
     if constexpr (J < 32) {
-        const float ga = absmax3(__uint_as_float(v[J]), __uint_as_float(v[J + 1]), __uint_as_float(v[J + 2]));
-        const float gb = absmax3(__uint_as_float(v[J + 3]), __uint_as_float(v[J + 4]), __uint_as_float(v[J + 5]));
-        const float gc = absmax3(__uint_as_float(v[J + 6]), __uint_as_float(v[J + 7]), ga);
-        if (fmaxf(gb, gc) >= thr) {
-            uint32_t k[8], u[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) k[j] = (v[J + j] & kKeyMask) | static_cast<uint32_t>(7 - j);
-            const uint32_t best = max(__vimax3_u32(k[6], k[7], __vimax3_u32(k[0], k[1], k[2])), __vimax3_u32(k[3], k[4], k[5]));
-#pragma unroll
-            for (int j = 0; j < 8; ++j) u[j] = k[j] - best;
-            const uint32_t next = best + max(__vimax3_u32(u[6], u[7], __vimax3_u32(u[0], u[1], u[2])), __vimax3_u32(u[3], u[4], u[5]));
-            const uint32_t rest = tag0 - J - 7u;          // tags of a group are consecutive, the last a multiple of eight
-            const float val = __uint_as_float(best & kKeyMask), limit = val - band;
-            if (limit > __uint_as_float(q.k0 & kKeyMask) && limit > __uint_as_float(next & kKeyMask)) {
-                q = Top5{best | rest, 0u, 0u, 0u, 0u, id, 0u, 0u, 0u};
-                thr = limit;
-            } else {
-                const Top5Thr r = insert_group(q, thr, k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7], rest, id, band);
-                q = r.q;
-                thr = r.thr;
-            }
+        fold2(q, key_of<G, J>(v, T0 + J / G), key_of<G, J + G>(v, T0 + J / G + 1));
+        fold32<G, T0, J + 2 * G>(v, q);
+    }
+}
+// A tile's three largest into the row's: whatever ends up within the band of the final maximum was within the band of
+// the running one when it came by, so what stays out can never matter.  A key more than the band above the
+// running maximum leaves everything seen so far outside the band and becomes the only one.  The tile's third is not known to be the
+// last inside the band: it counts as one too many.  `band`: that of the row, a little widened; negative for a row that is all zero
+// (nothing is taken and atom 0 is picked).
+__device__ __forceinline__ void merge(Tops& q, const Three& l, uint32_t id, float band) {
+    auto val = [](uint32_t k) { return __uint_as_float(k & kKeyMask); };
+    if (val(l.a) >= val(q.k0) - band) {
+        if (val(l.a) - band > val(q.k0))
+            q = Tops{l.a, 0u, 0u, 0u, id, 0u, 0u};
+        else
+            tops_insert(q, l.a, id);
+        const float thr = val(q.k0) - band;
+        if (val(l.b) >= thr) {
+            tops_insert(q, l.b, id);
+            if (val(l.c) >= thr) q.k3 = max(q.k3, l.c);
         }
-        chunk_top5<J + 8>(v, q, id, tag0, thr, band);
     }
 }
 
-// Folds `chunks` x 32 columns of an accumulator into `q`, 64 at a time, and hands the accumulator back
-// when the last have arrived.  Rolled: with all 128 columns' code in line the sweep outgrows the
-// instruction cache.  No load is in flight while a group is inserted (the call may move registers).
-// `band`: that of the row, a little widened; negative for a row that is all zero (nothing is
-// inserted and atom 0 is taken).
-__device__ __forceinline__ void drain(uint32_t taddr, int chunks, Top5& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
-    float thr = __uint_as_float(q.k0 & kKeyMask) - band;
-    uint32_t tag0 = 127u;
-#pragma unroll 1
-    for (int c = 0; c < chunks; c += 2) {
-        uint32_t v0[32], v1[32];
-        tmem_ld32(taddr + 32 * c, v0);
-        if (c + 1 < chunks) {
-            tmem_ld32(taddr + 32 * (c + 1), v1);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v1[j] = 0u;
-        }
-        tmem_wait_ld(v0);
-        reg_fence(v1);
-        if (c + 2 >= chunks) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty);
-        }
-        chunk_top5(v0, q, id, tag0, thr, band);
-        if (c + 1 < chunks) chunk_top5(v1, q, id, tag0 - 32u, thr, band);
-        tag0 -= 64u;
-    }
-}
-
-// The same for 128 columns, handed back as soon as all of them are in registers: for an accumulator that
-// the tensor core is waiting for.
-__device__ __forceinline__ void drain128(uint32_t taddr, Top5& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
+// Folds a thread's 32 * CHUNKS columns of an accumulator into its row's `q` and hands the accumulator back as soon as all of them
+// are in registers.
+template <int G, int CHUNKS>
+__device__ __forceinline__ void drain(uint32_t taddr, Tops& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
     uint32_t v0[32], v1[32], v2[32], v3[32];
     tmem_ld32(taddr + 0, v0);
-    tmem_ld32(taddr + 32, v1);
-    tmem_ld32(taddr + 64, v2);
-    tmem_ld32(taddr + 96, v3);
+    if constexpr (CHUNKS > 1) tmem_ld32(taddr + 32, v1);
+    if constexpr (CHUNKS > 2) tmem_ld32(taddr + 64, v2);
+    if constexpr (CHUNKS > 3) tmem_ld32(taddr + 96, v3);
     tmem_wait_ld(v0);
-    reg_fence(v1);
-    reg_fence(v2);
-    reg_fence(v3);
+    if constexpr (CHUNKS > 1) reg_fence(v1);
+    if constexpr (CHUNKS > 2) reg_fence(v2);
+    if constexpr (CHUNKS > 3) reg_fence(v3);
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(acc_empty);
-    float thr = __uint_as_float(q.k0 & kKeyMask) - band;
-    chunk_top5(v0, q, id, 127u, thr, band);
-    chunk_top5(v1, q, id, 95u, thr, band);
-    chunk_top5(v2, q, id, 63u, thr, band);
-    chunk_top5(v3, q, id, 31u, thr, band);
+    Three l{0u, 0u, 0u};
+    fold32<G, 0>(v0, l);
+    if constexpr (CHUNKS > 1) fold32<G, 32 / G>(v1, l);
+    if constexpr (CHUNKS > 2) fold32<G, 64 / G>(v2, l);
+    if constexpr (CHUNKS > 3) fold32<G, 96 / G>(v3, l);
+    merge(q, l, id, band);
 }
 
 // Barrier of the 256 epilogue threads that also tells every one of them whether any of them
@@ -302,7 +259,7 @@ __device__ __forceinline__ double row_scale(double nn, float& norm) {
     return scale;
 }
 // Half-width of the undecided zone of a row, in the sweep's unit, from its norm and the norm of what rounding it to
-// fp16 took from it: twice the error of a correlation, plus the 2^-16 relative truncation of the keys.  With
+// fp16 took from it: twice the error of a correlation, plus the 2^-18 relative truncation of the keys (and half as much again for the fp32 rounding of their differences).  With
 // r = r' + e and d = d' + f (r', d' the fp16 values), r.d - r'.d' = e.d + r'.f, which is at most
 // ||e|| max ||d|| + ||r'|| max ||f|| (Cauchy-Schwarz): these norms are taken, not assumed, and come to 4e-4 ||R|| for
 // unit atoms (a rounding error is 1.9e-4 of its value in the mean square), less than half of what the formats alone
@@ -310,7 +267,7 @@ __device__ __forceinline__ double row_scale(double nn, float& norm) {
 __device__ __forceinline__ float row_band(float norm, float err2, const DictBounds& b) {
     const float err = sqrtf(err2);
     const float half = fmaf(err, b.norm, fmaf(norm + err, b.err, kAccumRel * norm * b.norm));
-    return norm > 0.f || norm != norm ? 1.001f * fmaf(2.f, half, norm * b.norm * (1.f / 65536.f)) : 0.f;
+    return norm > 0.f || norm != norm ? 1.001f * fmaf(2.f, half, norm * b.norm * (1.f / 131072.f)) : 0.f;
 }
 // From which |correlation| on, relative to ||R||, an atom can be the pick, for a sweep whose largest value was `v0`
 // (in the sweep's unit, as band and norm): that value less the band, and half a band for the search's fp32
@@ -378,6 +335,112 @@ __device__ __forceinline__ void load_x2(const void* X, int x_dtype, int64_t off,
             x1 = f.y;
         }
     }
+}
+
+// acc += the products of two pairs of fp16 values, exact, each sum rounded once.
+__device__ __forceinline__ void fma2_f16(float& acc0, float& acc1, uint32_t a, uint32_t b) {
+    asm("{\n"
+        ".reg .b16 al, ah, bl, bh;\n"
+        "mov.b32 {al, ah}, %2;\n"
+        "mov.b32 {bl, bh}, %3;\n"
+        "fma.rn.f32.f16 %0, al, bl, %0;\n"
+        "fma.rn.f32.f16 %1, ah, bh, %1;\n"
+        "}\n"
+        : "+f"(acc0), "+f"(acc1)
+        : "r"(a), "r"(b));
+}
+// The sweep's values of one group again: eight lanes per row, lane l8 holds 16-byte chunks l8 + 8 j of the G atoms and of the row.
+template <int D_>
+struct GroupAtoms {
+    static constexpr int G = kGroup<D_>, CK = D_ / 64;
+    uint4 a[G][CK];
+    __device__ __forceinline__ void load(const uint16_t* __restrict__ dict, int n0, int N, int l8) {
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            const uint4* src = reinterpret_cast<const uint4*>(dict + static_cast<int64_t>(min(n0 + i, N - 1)) * D_);
+#pragma unroll
+            for (int j = 0; j < CK; ++j) a[i][j] = __ldg(src + l8 + 8 * j);
+        }
+    }
+    // |r . d| of atom `atom(l8)` of the group, to this lane; negative for one past the dictionary's end.
+    static __device__ __forceinline__ int atom(int l8) { return G == 8 ? l8 : l8 >> 1; }
+    __device__ __forceinline__ float value(const uint4 (&r)[CK], int n0, int N, int l8) const {
+        float e[G];
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            float x = 0.f, y = 0.f;
+#pragma unroll
+            for (int j = 0; j < CK; ++j) {
+                fma2_f16(x, y, r[j].x, a[i][j].x);
+                fma2_f16(x, y, r[j].y, a[i][j].y);
+                fma2_f16(x, y, r[j].z, a[i][j].z);
+                fma2_f16(x, y, r[j].w, a[i][j].w);
+            }
+            e[i] = x + y;
+        }
+        // a lane keeps half of its atoms at each step and sends the other half's sums to the lane that keeps those
+#pragma unroll
+        for (int h = G / 2, bit = 4; bit > 0; bit >>= 1, h >>= 1) {
+            if (h > 0) {
+                const bool up = l8 & bit;
+#pragma unroll
+                for (int i = 0; i < h; ++i) {
+                    const float keep = up ? e[i + h] : e[i], send = up ? e[i] : e[i + h];
+                    e[i] = keep + __shfl_xor_sync(FULL, send, bit);
+                }
+            } else {
+                e[0] += __shfl_xor_sync(FULL, e[0], bit);
+            }
+        }
+        return n0 + atom(l8) < N ? fabsf(e[0]) : -1.f;
+    }
+};
+// Of the group's values, a bit for each lane of the warp whose atom is within the band of its row's largest.
+__device__ __forceinline__ uint32_t inside(float value, float band) {
+    float m = value;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+    return __ballot_sync(FULL, value >= 0.f && !(m - value > band));
+}
+// One row by the whole warp: the atom of largest fp64 |R . d| in the groups start(0) .. start(groups - 1), the lowest among equals.
+template <int D_, typename F>
+__device__ __forceinline__ int decide(const float* __restrict__ D, int N, const double* Rrow, int groups, F&& start, int lane) {
+    constexpr int CH = D_ / 8;
+    const int l8 = lane & 7, grp = lane >> 3;
+    double R[CH];
+#pragma unroll
+    for (int k = 0; k < CH / 2; ++k) {
+        const double2 v = __ldcg(reinterpret_cast<const double2*>(Rrow) + 8 * k + l8);
+        R[2 * k] = v.x;
+        R[2 * k + 1] = v.y;
+    }
+    double best = -1.0;
+    int bn = 0;
+#pragma unroll 1
+    for (int i = 0; i < groups; ++i) {
+        const int n0 = start(i);
+#pragma unroll 1
+        for (int a = 0; a < kGroup<D_>; a += 4) {
+            const int n = n0 + a + grp;
+            float at[CH];
+            load_atom<CH>(D + static_cast<int64_t>(min(n, N - 1)) * D_, l8, at);
+            const double c = fabs(group8_sum(slice_dot<CH>(R, at)));
+            if (n < N && (c > best || (c == best && n < bn))) {
+                best = c;
+                bn = n;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+        const double ob = __shfl_xor_sync(FULL, best, o);
+        const int on = __shfl_xor_sync(FULL, bn, o);
+        if (ob > best || (ob == best && on < bn)) {
+            best = ob;
+            bn = on;
+        }
+    }
+    return bn;
 }
 
 // Arg-max of |R . d_n| over the atoms [n0, n1) for one row, by one warp (all lanes call): its share

@@ -110,3 +110,38 @@ def test_atoms_that_are_not_finite_are_met_as_they_are(csr, engine):
     finally:
         csr.csr_set_option("exact_engine", 0)
     assert torch.equal(keep[0].view(torch.int16), got[0].view(torch.int16)) and torch.equal(keep[1], got[1])
+
+
+@pytest.mark.parametrize("engine", [0, 2])
+@pytest.mark.parametrize("M,N,d", [(6, 1000, 128), (130, 515, 64), (700, 2100, 128), (3000, 1030, 64)])
+@pytest.mark.parametrize("apart", [1, 3, 8, 130])
+def test_near_ties_within_and_across_groups(csr, engine, M, N, d, apart):
+    """The sweep keeps the largest of eight adjacent atoms: atoms almost alike at the same place of their group, in the same group
+    and further apart, closer than the sweep can tell and not closer than fp64 can; exact copies go to the lower one."""
+    g = torch.Generator(device=DEV).manual_seed(N + apart)
+    D = torch.randn(N, d, device=DEV, generator=g)
+    near = torch.arange(16, N - apart, 2 * apart + 17, device=DEV)
+    D[near + apart] = D[near] + 10.0 ** torch.empty(len(near), 1, device=DEV).uniform_(-6, -2, generator=g) * torch.randn(len(near), d, device=DEV, generator=g)
+    D = torch.nn.functional.normalize(D, dim=1)
+    D[9], D[9 + apart] = D[8], -D[8]
+    D = D.contiguous()
+    pick = near[torch.randint(0, len(near), (M,), device=DEV, generator=g)]
+    X = (D[pick] * (1.0 + torch.rand(M, 1, device=DEV, generator=g)) + 0.02 * torch.randn(M, d, device=DEV, generator=g)).contiguous()
+    X[0] = -2.0 * D[8]
+    csr.csr_set_option("exact_engine", engine)
+    try:
+        idx, coef = csr.csr_encode_ex(D, X, 3, mode=csr.CSR_MODE_FP32_EXACT, coef_dtype=torch.float32)
+        assert csr.csr_device_status() == csr.CSR_OK
+    finally:
+        csr.csr_set_option("exact_engine", 0)
+    got = idx.view(torch.int16).long() & 0xFFFF
+    assert int(got[0, 0]) == 8
+    Dd, R = D.double(), X.double()
+    for k in range(3):                                     # each pick is a largest correlation of fp64's, to fp64's own rounding
+        corr = (R @ Dd.T).abs()
+        best = corr.max(dim=1).values
+        mine = corr.gather(1, got[:, k:k + 1])[:, 0]
+        assert bool((best - mine <= 128 * 2.0 ** -52 * R.norm(dim=1)).all())
+        c = (R * Dd[got[:, k]]).sum(1)
+        assert torch.allclose(coef[:, k].double(), c, rtol=2.0 ** -22, atol=1e-13)
+        R = R - c[:, None] * Dd[got[:, k]]
