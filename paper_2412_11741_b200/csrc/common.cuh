@@ -68,13 +68,13 @@ int launch_encode_exact_split(const EncodeArgs& a, void* scratch);
 // what is left over the same way as few rows.  `pairs_only`: pairs of row tiles whatever M is.
 size_t encode_exact_tc_scratch_bytes(int64_t M, int d, int N);
 int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status, uint32_t* diag, bool pairs_only);
-// The split engine's pieces: CTAs per row tile (0: too many rows), scratch, counter words (zeroed by the
-// caller), launch on the dictionary's scaled fp16 copy and its bounds; kGridLaunchRefused when the driver refuses it.
+// The split engine's pieces: CTAs per row tile (0: too many rows), scratch, words that the CTAs meet at and leave for one
+// another (zeroed by the caller), launch on the dictionary's scaled fp16 copy and its bounds; kGridLaunchRefused when the driver refuses it.
 constexpr int kGridLaunchRefused = 1;                      // internal: not a CSR_ERR_* code
 int exact_grid_slices(int64_t M, int N);
-size_t exact_grid_scratch_bytes(int64_t M, int d, int N);
-size_t exact_grid_counter_words(int64_t M);
-int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* dict_parts, int n_parts, void* scratch, uint32_t* counters,
+size_t exact_grid_scratch_bytes(int64_t M, int d);
+size_t exact_grid_word_bytes(int64_t M, int N);
+int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* dict_parts, int n_parts, void* scratch, void* words,
                              uint32_t* status, uint32_t* diag);
 
 // tcgen05 bf16 matching pursuit.  `workspace` holds the bf16 copy of D (N*d*2 bytes,

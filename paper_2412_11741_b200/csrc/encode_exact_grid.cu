@@ -8,17 +8,20 @@
 //   - every CTA loads its tile's 128 residual rows as fp16 (32 KB from the L2), multiplies them with
 //     its slice by the same fp16 product per correlation, and every thread keeps the
 //     largest keys of its half row (drain as in encode_exact_tc.cu);
-//   - the keys go to a scratch array, the CTAs of the row tile meet (counter in global memory,
-//     bounded wait);
+//   - the keys go to a scratch array, tagged with the iteration, and are taken from there as they come;
 //   - the rows of the tile are dealt out to its CTAs, eight lanes settle a row: the largest key
 //     over all slices, everything inside the band re-scored in fp64, fp64 coefficient and residual
-//     update; the new fp16 rows go back to the scratch array and the CTAs meet again.
+//     update; the new fp16 rows go back to the scratch array and the CTAs meet (counter in global memory, bounded
+//     wait).
 // The fp64 rows, bands and fp16 rows live in L2-resident scratch.  The dictionary stages of the next
 // iteration are fetched while the rows are being settled.
 //
-// What bounds it: with few rows the chain of dependent steps (A load, MMA, drain, meeting, settle,
-// meeting: 9 to 10 us an iteration at 16 to 128 rows, N = 8192), with many the drain.  128 rows, N = 8192, s = 16: 180 us
-// with three bf16 products per correlation, 158 us with one fp16 product.
+// What bounds it: with few rows the chain of dependent steps, in cycles of an iteration at 128 rows, N = 8192: the rows' load
+// 1800, the sweep 2500, the keys on their way 2100, their maximum and band 1800, fp64 3000, the meeting 3500; with many
+// the settling (26000 of 128 rows, beside a sweep of 23000 at N = 4096).  128 rows, N = 8192, s = 16: 180 us with three bf16
+// products per correlation, 158 us with one fp16 product, 147 us with the branch-free drain, keys taken as they come
+// instead of behind a second meeting and fp64 for all atoms of the group at once.  (The rows as tagged words too, instead of the
+// meeting: 192 us, and 299 us when every thread polled all of its words.)
 // The grid is launched cooperatively whenever a row tile has more than one CTA, so all CTAs that
 // wait for one another are resident.
 #include "exact_tc_common.cuh"
@@ -37,11 +40,72 @@ constexpr int UNIT = 64;                                  // atoms per TMA box; 
 constexpr int MAX_SLICES = TILE_M;                        // at most one CTA per row
 constexpr int CAND = 16;                                  // groups a row may have inside the band before the whole dictionary is re-scored
 
+// What a CTA leaves of its keys for the others: 16 bytes written and read at once, the last word the number of the
+// iteration they are for, from 1.  The reader takes them as soon as they carry the number that it waits for: no fence and
+// no second trip to the L2, as after a barrier.  They are written again only when every CTA of the tile has
+// passed the meeting after the settling, that is, has read them.
+struct Word {
+    uint32_t x, y, z, tag;
+};
+__device__ __forceinline__ void put_word(Word* p, const Word& v) {
+    asm volatile(
+        "{\n"
+        ".reg .b64 lo, hi;\n"
+        ".reg .b128 t;\n"
+        "mov.b64 lo, {%1, %2};\n"
+        "mov.b64 hi, {%3, %4};\n"
+        "mov.b128 t, {lo, hi};\n"
+        "st.relaxed.gpu.global.b128 [%0], t;\n"
+        "}\n" ::"l"(p),
+        "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.tag)
+        : "memory");
+}
+__device__ __forceinline__ Word get_word(const Word* p) {
+    Word v;
+    asm volatile(
+        "{\n"
+        ".reg .b64 lo, hi;\n"
+        ".reg .b128 t;\n"
+        "ld.relaxed.gpu.global.b128 t, [%4];\n"
+        "mov.b128 {lo, hi}, t;\n"
+        "mov.b64 {%0, %1}, lo;\n"
+        "mov.b64 {%2, %3}, hi;\n"
+        "}\n"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.tag)
+        : "l"(p)
+        : "memory");
+    return v;
+}
 // Keys of one row over one column half of a slice: the four largest and the groups of the first three, by their first atom.
-struct __align__(8) Entry {
+struct Entry {
     uint32_t k[4];
     uint32_t n01, n2;
 };
+constexpr int ENTRY_WORDS = 2;
+
+// Takes an entry once it carries `tag`.  Bounded like every wait; false: given up.
+__device__ __forceinline__ bool take_entry(const Word* p, uint32_t tag, const WaitCtx& w, Entry& e) {
+    unsigned long long t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        const Word a = get_word(p), b = get_word(p + 1);
+        if (a.tag == tag && b.tag == tag) {
+            e = Entry{{a.x, a.y, b.x, b.y}, a.z, b.z};
+            return true;
+        }
+        bool out = w.limit_ns == 0 || it >= (1u << 28);
+        if (!out && (it & 15u) == 0) {
+            if (*w.abort) return false;
+            const unsigned long long t = globaltimer_ns();
+            if (t0 == 0) t0 = t;
+            out = t - t0 > w.limit_ns;
+        }
+        if (out) {
+            *w.abort = 1;
+            atomicOr(w.status, kStatusTimeout);
+            return false;
+        }
+    }
+}
 
 template <int D_>
 struct GridSmem {
@@ -84,7 +148,7 @@ struct GridArgs {
     const uint16_t* dict;   // [N][d] the dictionary's scaled fp16 copy
     const DictPart* parts;  // [n_parts] its bounds
     int n_parts;
-    Entry* entries;         // [tiles][128][2 * slices]
+    Word* entries;          // [tiles][128][2 * slices][ENTRY_WORDS], tags zero at launch
     uint32_t* counters;     // [tiles * 32], zero at launch
     int slices;
     uint32_t* status;
@@ -255,7 +319,6 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
     } else {
         // ------------------------------ epilogue ------------------------------
         constexpr int CH = D_ / 8;                        // channels per lane when eight lanes share a row
-        constexpr int G = kGroup<D_>;
         const int q = warp & 3, half = warp >> 2;         // TMEM lane quarter, column half
         const int r_own = q * 32 + lane;                  // the row of the tile whose correlations this thread sees
         const int l8 = lane & 7, grp = lane >> 3;
@@ -273,18 +336,30 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
         // An fp64 row, its scaled form as fp16 and its band to the scratch arrays, by the eight lanes of a row (all lanes
         // of the warp call; only those with `has` write).
         auto put_row = [&](const double (&R)[CH], int64_t row, bool has) {
-            float norm, err2 = 0.f;
-            const double scale = row_scale(group8_sum(norm2_share<CH>(R)), norm);
+            const Operand<CH> o = to_operand<CH>(R);
+            if (!has) return;
 #pragma unroll
             for (int k = 0; k < CH / 2; ++k) {
-                const uint32_t w = round_pair(R[2 * k] * scale, R[2 * k + 1] * scale, err2);
-                if (has) {
-                    __stcg(reinterpret_cast<double2*>(a.Rd + row * D_) + 8 * k + l8, make_double2(R[2 * k], R[2 * k + 1]));
-                    __stcg(a.Rh + row * (D_ / 2) + 8 * k + l8, w);
-                }
+                __stcg(reinterpret_cast<double2*>(a.Rd + row * D_) + 8 * k + l8, make_double2(R[2 * k], R[2 * k + 1]));
+                __stcg(a.Rh + row * (D_ / 2) + 8 * k + l8, o.w[k]);
             }
-            err2 = group8_sumf(err2);
-            if (has && l8 == 0) __stcg(a.band + row, make_float2(row_band(norm, err2, db), norm));
+            if (l8 == 0) __stcg(a.band + row, make_float2(row_band(o.norm, o.err2, db), o.norm));
+        };
+        auto put_code = [&](int64_t row, int g, int n, double c) {
+            a.out_idx[row * a.ldc + g] = static_cast<uint16_t>(n);
+            const float cf = static_cast<float>(c);
+            if (a.coef_dtype == CSR_DTYPE_F16)
+                reinterpret_cast<__half*>(a.out_coef)[row * a.ldc + g] = __float2half_rn(cf);
+            else
+                reinterpret_cast<float*>(a.out_coef)[row * a.ldc + g] = cf;
+        };
+        auto load_row = [&](int64_t row, double (&R)[CH]) {
+#pragma unroll
+            for (int c = 0; c < CH / 2; ++c) {
+                const double2 x = __ldcg(reinterpret_cast<const double2*>(a.Rd + row * D_) + 8 * c + l8);
+                R[2 * c] = x.x;
+                R[2 * c + 1] = x.y;
+            }
         };
         // ---- R_0 = x ----
         for (int k0 = 0; k0 < n_own; k0 += EPI / 8) {
@@ -337,26 +412,24 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
                 uint64_t* back = &sm.acc_empty[acc];
                 const uint32_t id = static_cast<uint32_t>(t);
                 if (w == TILE_N)
-                    drain<G, 4>(ta, top, id, fband, back, lane);
+                    drain<4>(ta, top, id, fband, back, lane);
                 else if (w == 3 * UNIT)
-                    drain<G, 3>(ta, top, id, fband, back, lane);
+                    drain<3>(ta, top, id, fband, back, lane);
                 else if (w == 2 * UNIT)
-                    drain<G, 2>(ta, top, id, fband, back, lane);
+                    drain<2>(ta, top, id, fband, back, lane);
                 else
-                    drain<G, 1>(ta, top, id, fband, back, lane);
+                    drain<1>(ta, top, id, fband, back, lane);
             }
             if (ok && r_own < rows_here) {
                 auto start = [&](uint32_t key, uint32_t id) {     // (an empty key's place is never used)
                     const int t = static_cast<int>(id), w = min(TILE_N, width - t * TILE_N);
                     return static_cast<uint32_t>(n_first + t * TILE_N + half * (w / 2) + static_cast<int>(key & 31u) * G) & 0xFFFFu;
                 };
-                uint2* e = reinterpret_cast<uint2*>(a.entries + ((row_base + r_own) * n_ent + 2 * slice + half));
-                __stcg(e + 0, make_uint2(top.k0, top.k1));
-                __stcg(e + 1, make_uint2(top.k2, top.k3));
-                __stcg(e + 2, make_uint2(start(top.k0, top.i0) | (start(top.k1, top.i1) << 16), start(top.k2, top.i2)));
+                Word* e = a.entries + ((row_base + r_own) * n_ent + 2 * slice + half) * ENTRY_WORDS;
+                const uint32_t tag = static_cast<uint32_t>(g) + 1u;
+                put_word(e, Word{top.k0, top.k1, start(top.k0, top.i0) | (start(top.k1, top.i1) << 16), tag});
+                put_word(e + 1, Word{top.k2, top.k3, start(top.k2, top.i2), tag});
             }
-            ok = meet(counter, target += slices, slices, ok, wc);
-            if (!ok) break;
 
             // ---- this CTA's rows: largest key over all slices, then what lies inside its band ----
             // (an entry per thread and trip, at most two trips: rows x 2 slices <= 2 (127 + slices))
@@ -372,20 +445,35 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
             for (int u = 0; u < TRIPS; ++u) {
                 const int f = threadIdx.x + u * EPI;
                 mine[u] = Entry{{0u, 0u, 0u, 0u}, 0u, 0u};
-                band_of[u] = make_float2(0.f, 0.f);
-                if (f < n_own * n_ent) {
-                    const int64_t row = row_base + slice + f / n_ent * slices;
-                    const uint2* e = reinterpret_cast<const uint2*>(a.entries + (row * n_ent + f % n_ent));
-                    const uint2 e0 = __ldcg(e), e1 = __ldcg(e + 1), e2 = __ldcg(e + 2);
-                    mine[u] = Entry{{e0.x, e0.y, e1.x, e1.y}, e2.x, e2.y};
-                    band_of[u] = __ldcg(a.band + row);
-                }
+                band_of[u] = f < n_own * n_ent ? __ldcg(a.band + row_base + slice + f / n_ent * slices) : make_float2(0.f, 0.f);
             }
-            epilogue_barrier();
+            // (a warp that has at most one row keeps it at hand: what it needs next are only the atoms)
+            double R[CH];
+            if (n_own <= EPI / 32) load_row(row_base + slice + min(warp, max(n_own - 1, 0)) * slices, R);
 #pragma unroll
             for (int u = 0; u < TRIPS; ++u) {
                 const int f = threadIdx.x + u * EPI;
-                if (f < n_own * n_ent) atomicMax(&sm.top_key[f / n_ent], mine[u].k[0]);
+                if (ok && f < n_own * n_ent)
+                    ok = take_entry(a.entries + ((row_base + slice + f / n_ent * slices) * n_ent + f % n_ent) * ENTRY_WORDS,
+                                    static_cast<uint32_t>(g) + 1u, wc, mine[u]);
+            }
+            if (epilogue_barrier_any(!ok || sm.abort != 0)) {
+                ok = false;
+                break;
+            }
+#pragma unroll
+            for (int u = 0; u < TRIPS; ++u) {
+                const int f = threadIdx.x + u * EPI;
+                const bool in = f < n_own * n_ent;
+                // (where all of a warp's entries are one row's, their maximum goes there once)
+                const int k = in ? f / n_ent : -1;
+                const uint32_t top = mine[u].k[0];
+                if (__all_sync(FULL, k == __shfl_sync(FULL, k, 0))) {
+                    const uint32_t most = __reduce_max_sync(FULL, top);
+                    if (lane == 0 && in) atomicMax(&sm.top_key[k], most);
+                } else if (in) {
+                    atomicMax(&sm.top_key[k], top);
+                }
             }
             epilogue_barrier();
 #pragma unroll
@@ -416,9 +504,67 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
             }
             epilogue_barrier();
 
-            // ---- settle them, rows with unknown candidates in a second round ----
+            // ---- settle them: a row per warp, its lane groups an atom each ... ----
+            const bool single_rows = n_own <= EPI / 32;
+            if (single_rows && warp < n_own && !((sm.unknown[0] >> warp) & 1u)) {
+                const int64_t row = row_base + slice + warp * slices;
+                const int cnt = min(sm.n_cand[warp], CAND);   // none: an all-zero sweep (or NaN, or one atom) picks atom 0
+                double best = -1.0, c = 0.0;
+                float at[CH];
+                int n = 0;
+                if (cnt == 0) {
+                    load_atom<CH>(a.D, l8, at);
+                    c = group8_sum(slice_dot<CH>(R, at));
+                }
 #pragma unroll 1
-            for (int round = 0; round < 2; ++round) {
+                for (int i = 0; i < cnt; ++i) {
+                    const int n0 = sm.cand[warp][i];
+                    float x[2][CH];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) load_atom<CH>(a.D + static_cast<int64_t>(min(n0 + 4 * h + grp, a.N - 1)) * D_, l8, x[h]);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int nh = n0 + 4 * h + grp;
+                        const double ch = group8_sum(slice_dot<CH>(R, x[h]));
+                        if (nh < a.N && (fabs(ch) > best || (fabs(ch) == best && nh < n))) {
+                            best = fabs(ch);
+                            c = ch;
+                            n = nh;
+#pragma unroll
+                            for (int k = 0; k < CH; ++k) at[k] = x[h][k];
+                        }
+                    }
+                }
+                // the lane group that has the pick (the lowest atom among equal values) goes on with it
+                double top = best;
+                int low = n;
+#pragma unroll
+                for (int o = 8; o < 32; o <<= 1) {
+                    const double ob = __shfl_xor_sync(FULL, top, o);
+                    const int on = __shfl_xor_sync(FULL, low, o);
+                    if (ob > top || (ob == top && on < low)) {
+                        top = ob;
+                        low = on;
+                    }
+                }
+                const uint32_t won = __ballot_sync(FULL, best == top && n == low);   // (nothing but NaN: every group has atom 0 and -1)
+                const bool has = won != 0u && grp == (__ffs(won) - 1) / 8;
+                if (top < 0.0 && cnt > 0) {
+                    load_atom<CH>(a.D, l8, at);
+                    c = group8_sum(slice_dot<CH>(R, at));
+                }
+                if (l8 == 0 && has) put_code(row, g, n, c);
+                if (g + 1 < a.s) {
+                    double ad[CH];
+                    widen<CH>(at, ad);
+#pragma unroll
+                    for (int k = 0; k < CH; ++k) R[k] = fma(-c, ad[k], R[k]);
+                    put_row(R, row, has);
+                }
+            }
+            // ---- ... or eight lanes per row; rows with unknown candidates in a second round ----
+#pragma unroll 1
+            for (int round = single_rows ? 1 : 0; round < 2; ++round) {
                 if (round == 1) {
                     epilogue_barrier();
                     if ((sm.unknown[0] | sm.unknown[1] | sm.unknown[2] | sm.unknown[3]) == 0u) break;
@@ -439,13 +585,7 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
                     if (!__any_sync(FULL, has)) continue;
                     const int kk = k < n_own ? k : 0;         // (lane groups without a row repeat one and write nothing)
                     const int64_t row = row_base + slice + kk * slices;
-                    double R[CH];
-#pragma unroll
-                    for (int c = 0; c < CH / 2; ++c) {
-                        const double2 x = __ldcg(reinterpret_cast<const double2*>(a.Rd + row * D_) + 8 * c + l8);
-                        R[2 * c] = x.x;
-                        R[2 * c + 1] = x.y;
-                    }
+                    load_row(row, R);
                     const bool open = (sm.unknown[kk >> 5] >> (kk & 31)) & 1u;
                     const int cnt = min(sm.n_cand[kk], CAND);   // none: an all-zero sweep (or NaN, or one atom) picks atom 0
                     int n = cnt > 0 ? sm.cand[kk][0] : 0;
@@ -461,9 +601,8 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
 #pragma unroll
                         for (int j = 0; j < D_ / 64; ++j) r[j] = *reinterpret_cast<const uint4*>(&sm.A[swz_off(slice + kk * slices, l8 + 8 * j)]);
                         const uint32_t bits = (inside(ga.value(r, n, a.N, l8), __ldcg(&a.band[row].x)) >> (8 * grp)) & 255u;
-                        const int first = bits == 0u ? 0 : G == 8 ? __ffs(bits) - 1 : (__ffs(bits) - 1) / 2;
-                        single = cnt == 1 && bits != 0u && (bits >> (G == 8 ? first : 2 * first)) <= (G == 8 ? 1u : 3u);
-                        if (single) n += first;
+                        single = cnt == 1 && __popc(bits) == 1;
+                        if (single) n += __ffs(bits) - 1;
 #pragma unroll 1
                         for (uint32_t left = __ballot_sync(FULL, has && cnt > 0 && !single && l8 == 0); left; left &= left - 1) {
                             const int src = __ffs(left) - 1;
@@ -475,22 +614,17 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
                     }
                     float at[CH];
                     load_atom<CH>(a.D + static_cast<int64_t>(n) * D_, l8, at);
-                    const double c = group8_sum(slice_dot<CH>(R, at));
+                    double ad[CH];
+                    widen<CH>(at, ad);
+                    const double c = group8_sum(slice_dot<CH>(R, ad));
 #ifdef CSR_DEBUG_CHECKS
                     const float2 bn = __ldcg(a.band + row);
                     check_value<CH>(a.diag, R, at, c, __uint_as_float(sm.top_key[kk] & kKeyMask), bn.x, bn.y, db, l8, has && single);
 #endif
-                    if (l8 == 0 && has) {
-                        a.out_idx[row * a.ldc + g] = static_cast<uint16_t>(n);
-                        const float cf = static_cast<float>(c);
-                        if (a.coef_dtype == CSR_DTYPE_F16)
-                            reinterpret_cast<__half*>(a.out_coef)[row * a.ldc + g] = __float2half_rn(cf);
-                        else
-                            reinterpret_cast<float*>(a.out_coef)[row * a.ldc + g] = cf;
-                    }
+                    if (l8 == 0 && has) put_code(row, g, n, c);
                     if (g + 1 < a.s) {
 #pragma unroll
-                        for (int c2 = 0; c2 < CH; ++c2) R[c2] = fma(-c, static_cast<double>(at[c2]), R[c2]);
+                        for (int c2 = 0; c2 < CH; ++c2) R[c2] = fma(-c, ad[c2], R[c2]);
                         put_row(R, row, has);
                     }
                 }
@@ -544,13 +678,16 @@ int exact_grid_slices(int64_t M, int N) {
     return s < MAX_SLICES ? s : MAX_SLICES;
 }
 
-size_t exact_grid_scratch_bytes(int64_t M, int d, int N) {
+size_t exact_grid_scratch_bytes(int64_t M, int d) {
     const size_t rows = (size_t)tiles_of(M) * TILE_M;
-    return rows * d * 8 + rows * d * 2 + align256(rows * 8) + align256(rows * 2 * exact_grid_slices(M, N) * sizeof(Entry));
+    return rows * d * 8 + rows * d * 2 + align256(rows * 8);
 }
-size_t exact_grid_counter_words(int64_t M) { return (size_t)tiles_of(M) * 32; }
+// [counters][entries]
+size_t exact_grid_word_bytes(int64_t M, int N) {
+    return (size_t)tiles_of(M) * 128 + (size_t)tiles_of(M) * TILE_M * 2 * exact_grid_slices(M, N) * ENTRY_WORDS * sizeof(Word);
+}
 
-int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* dict_parts, int n_parts, void* scratch, uint32_t* counters,
+int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* dict_parts, int n_parts, void* scratch, void* words,
                              uint32_t* status, uint32_t* diag) {
     const size_t rows = (size_t)tiles_of(a.M) * TILE_M;
     char* p = static_cast<char*>(scratch);
@@ -575,8 +712,8 @@ int launch_encode_exact_grid(const EncodeArgs& a, void* dict_f16, const void* di
     g.dict = static_cast<const uint16_t*>(dict_f16);
     g.parts = static_cast<const DictPart*>(dict_parts);
     g.n_parts = n_parts;
-    g.entries = reinterpret_cast<Entry*>(p);
-    g.counters = counters;
+    g.counters = static_cast<uint32_t*>(words);
+    g.entries = reinterpret_cast<Word*>(static_cast<char*>(words) + (size_t)tiles_of(a.M) * 128);
     g.slices = exact_grid_slices(a.M, a.N);
     g.status = status;
     g.diag = diag;

@@ -16,7 +16,7 @@
 //   - each row tile has one 256-column fp32 accumulator in TMEM.  All eight epilogue warps drain
 //     every accumulator: warp w reads the 32 TMEM lanes of w % 4 and the 128 columns of w / 4, i.e.
 //     all of them sit in registers after one round of loads and the accumulator goes straight back
-//     to the tensor core.  Groups of adjacent atoms (kGroup) are reduced to their largest magnitude, a key being
+//     to the tensor core.  Groups of eight adjacent atoms are reduced to their largest magnitude, a key being
 //     that with its five lowest mantissa bits replaced by the group's number, and each thread keeps the tile's three
 //     largest keys, all without a branch; those within the band of the row's running maximum then join
 //     the four largest keys of its half row (three of them with the tile they came from);
@@ -27,10 +27,8 @@
 //     fp64, a row at a time by the warp; rows where the fourth of a half is inside too are searched for in the
 //     whole dictionary (fp32 filter, then fp64) by the eight warps together.  Coefficient (Eq. 2,
 //     signed) and residual update (Eq. 4) are fp64, as in the plain-ALU encoder.
-// What bounds it: at N = 4096 a sweep takes 44000 cycles (2048 of 2700 per 256 atoms are MMAs), the gathers of the groups
-// 10000, what fp64 decides 8000, the settling 28000.  With the five largest keys kept value by value, a branch per
-// eight of them, a sweep took 101000 (5000 a tile): 100000 rows, N = 4096, s = 8, 1916 us so and 1388 us now;
-// a training step (65536 rows, N = 8192, s = 8) 1872 and 1394.  Three bf16 products per correlation, whose band was 2^-12 ||R||, took 6144: 100000 rows, N = 4096, s = 8,
+// What bounds it: the epilogue and the settling, no longer the MMAs (2048 cycles per 256 atoms and pair of row tiles).
+// Three bf16 products per correlation, whose band was 2^-12 ||R||, took 6144: 100000 rows, N = 4096, s = 8,
 // 2441 us so and 2195 us with one fp16 product; a training step of 65536 rows (N = 8192, s = 8) 2992 and 2332 us.
 // Warp roles: 0-7 epilogue, 8 TMA producer, 9 TMEM owner and MMA issuer.  All waits are bounded.
 #include "exact_tc_common.cuh"
@@ -197,7 +195,6 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
     } else {
         // ------------------------------ epilogue ------------------------------
         constexpr int CH = D_ / 8;                          // channels per lane when eight lanes share a row
-        constexpr int G = kGroup<D_>;
         const int q = warp & 3;                             // TMEM lane quarter
         const int half = warp >> 2;                         // column half drained by this warp
         const int own_tile = warp >> 2;                     // row tile whose rows this warp settles
@@ -214,10 +211,17 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
             // A row's new residual to memory; its norm and band to the lane that has the row (pass p's, if set in `rows`).
             auto put_row = [&](const double (&R)[CH], int p, bool write, uint32_t rows) {
                 const int r = q * 32 + 4 * p + grp;
-                float nr;
-                const double scale = row_scale(group8_sum(norm2_share<CH>(R)), nr);
-                const float err2 = group8_sumf(store_residual<CH>(R, scale, Rd_cta + static_cast<int64_t>(own_tile * TILE_M + r) * D_, A_own, r, l8, write));
-                const float n_o = __shfl_sync(FULL, nr, (lane & 3) * 8), e_o = __shfl_sync(FULL, err2, (lane & 3) * 8);
+                const Operand<CH> o = to_operand<CH>(R);
+                if (write) {
+                    double2* row = reinterpret_cast<double2*>(Rd_cta + static_cast<int64_t>(own_tile * TILE_M + r) * D_);
+#pragma unroll
+                    for (int k = 0; k < CH / 2; ++k) {
+                        row[8 * k + l8] = make_double2(R[2 * k], R[2 * k + 1]);
+                        // channels 2 (8 k + l8), +1: 16-byte chunk 2 k + l8 / 4 of the row, word l8 % 4 of it
+                        *reinterpret_cast<uint32_t*>(A_own + swz_off(r, 2 * k + (l8 >> 2)) + (l8 & 3) * 4) = o.w[k];
+                    }
+                }
+                const float n_o = __shfl_sync(FULL, o.norm, (lane & 3) * 8), e_o = __shfl_sync(FULL, o.err2, (lane & 3) * 8);
                 if ((lane >> 2) == p && ((rows >> lane) & 1u)) {
                     norm = n_o;
                     band = row_band(n_o, e_o, db);
@@ -265,7 +269,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
                         }
                         tc_fence_after();
                         Tops qa = a ? st[1] : st[0];
-                        drain<G, 4>(taddr + a * TILE_N, qa, static_cast<uint32_t>(t), a ? fband[1] : fband[0], &sm.acc_empty[a], lane);
+                        drain<4>(taddr + a * TILE_N, qa, static_cast<uint32_t>(t), a ? fband[1] : fband[0], &sm.acc_empty[a], lane);
                         if (a)
                             st[1] = qa;
                         else
@@ -314,7 +318,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
                         for (int i = 5; i >= 0; --i)
                             if (!(v0 - __uint_as_float(key[i] & kKeyMask) > band) && my_start[i] < N) {
                                 my_flags |= 1 << i;
-                                my_first = my_start[i];
+                                my_n1 = my_first = my_start[i];
                             }
                         if (!(v0 - __uint_as_float(mine.k3 & kKeyMask) > band) || !(v0 - __uint_as_float(other.k3 & kKeyMask) > band))
                             my_flags |= kUnknown;
@@ -343,9 +347,8 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
                             const uint32_t in = inside(at[u].value(r, n0[u], N, l8), __shfl_sync(FULL, band, src));
                             if ((lane >> 2) == w0 + u && my_flags != 0) {
                                 const uint32_t bits = (in >> (8 * (lane & 3))) & 255u;
-                                const int first = bits == 0u ? 0 : G == 8 ? __ffs(bits) - 1 : (__ffs(bits) - 1) / 2;
-                                my_n1 = my_first + first;   // (no value at all: a row that is not finite)
-                                open = bits == 0u || (bits >> (G == 8 ? first : 2 * first)) > (G == 8 ? 1u : 3u) || (my_flags & (my_flags - 1)) != 0;
+                                if (bits != 0u) my_n1 = my_first + __ffs(bits) - 1;
+                                open = __popc(bits) != 1 || (my_flags & (my_flags - 1)) != 0;   // (no value at all: a row that is not finite)
                             }
                         }
                     }
@@ -428,9 +431,11 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
                         const int r = q * 32 + src;
                         const int64_t m = pair * ROWS + own_tile * TILE_M + r;
                         const bool has = (todo >> src) & 1u;
-                        const double c = group8_sum(slice_dot<CH>(R, a));
+                        double ad[CH];
+                        widen<CH>(a, ad);
+                        const double c = group8_sum(slice_dot<CH>(R, ad));
 #ifdef CSR_DEBUG_CHECKS
-                        const bool was_open = __shfl_sync(FULL, open, src);   // (every lane takes part)
+                        const bool was_open = __shfl_sync(FULL, open, src);
                         check_value<CH>(diag, R, a, c, __shfl_sync(FULL, v0, src), __shfl_sync(FULL, band, src), __shfl_sync(FULL, norm, src), db, l8,
                                         m < M && has && round == 0 && !was_open);
 #endif
@@ -445,7 +450,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
                         if (g + 1 < s) {
                             if (has) {
 #pragma unroll
-                                for (int k = 0; k < CH; ++k) R[k] = fma(-c, static_cast<double>(a[k]), R[k]);
+                                for (int k = 0; k < CH; ++k) R[k] = fma(-c, ad[k], R[k]);
                             }
                             put_row(R, p, has, todo);
                         }
@@ -479,16 +484,16 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
 // atoms spread over the dictionary to a norm in [1, 2): every block takes the same.  Atoms far larger than those
 // overflow; the error's norm is then infinite, as it is for them, and every row is searched for in fp64.  Atoms
 // that are not finite are left out of the norms: the sweep meets them as they are.  Also zeroes the words that the
-// CTAs of a split row tile meet at.  One warp per atom.
+// CTAs of a split row tile meet at and leave for one another.  One warp per atom.
 template <int D_>
 __global__ void __launch_bounds__(256)
-dict_to_f16_kernel(const float* __restrict__ D, int N, uint32_t* __restrict__ out, DictPart* __restrict__ parts, uint32_t* __restrict__ zero,
+dict_to_f16_kernel(const float* __restrict__ D, int N, uint32_t* __restrict__ out, DictPart* __restrict__ parts, uint4* __restrict__ zero,
                    int n_zero) {
     constexpr int PER = D_ / 64;                          // pairs of channels per lane
     __shared__ float red[2][8];
     __shared__ float first[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_zero; i += gridDim.x * blockDim.x) zero[i] = 0u;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_zero; i += gridDim.x * blockDim.x) zero[i] = make_uint4(0u, 0u, 0u, 0u);
     auto load = [&](int n, float2 (&v)[PER]) {
 #pragma unroll
         for (int k = 0; k < PER; ++k) v[k] = __ldg(reinterpret_cast<const float2*>(D + static_cast<int64_t>(n) * D_) + lane + 32 * k);
@@ -611,17 +616,17 @@ size_t pair_scratch_bytes(int64_t M, int d) { return (size_t)ctas_for(M) * ROWS 
 
 }  // namespace
 
-// [fp16 dictionary][its bounds][counters of the two split launches][rows of the launch that is running]
+// [fp16 dictionary][its bounds][words of the two split launches][rows of the launch that is running]
 size_t encode_exact_tc_scratch_bytes(int64_t M, int d, int N) {
     const Plan p = make_plan(M, N, false);
     size_t rows = pair_scratch_bytes(M, d), words = 0;    // (also what is needed where a split launch is refused)
     for (int64_t m : p.grid_rows) {
         if (m == 0) continue;
-        const size_t b = exact_grid_scratch_bytes(m, d, N);
+        const size_t b = exact_grid_scratch_bytes(m, d);
         if (b > rows) rows = b;
-        words += exact_grid_counter_words(m);
+        words += exact_grid_word_bytes(m, N);
     }
-    return align1k((size_t)N * d * 2) + align1k(kMaxDictParts * sizeof(DictPart)) + align1k(words * 4) + rows;
+    return align1k((size_t)N * d * 2) + align1k(kMaxDictParts * sizeof(DictPart)) + align1k(words) + rows;
 }
 
 int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status, uint32_t* diag, bool pairs_only) {
@@ -634,15 +639,15 @@ int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status,
     base += align1k((size_t)a.N * a.d * 2);
     DictPart* parts = reinterpret_cast<DictPart*>(base);
     base += align1k(kMaxDictParts * sizeof(DictPart));
-    uint32_t* counters = reinterpret_cast<uint32_t*>(base);
-    size_t words = 0;
+    char* words = base;
+    size_t n_words = 0;
     for (int64_t m : plan.grid_rows)
-        if (m) words += exact_grid_counter_words(m);
-    char* rows = base + align1k(words * 4);
+        if (m) n_words += exact_grid_word_bytes(m, a.N);
+    char* rows = base + align1k(n_words);
     int n_parts = (a.N + 7) / 8;
     if (n_parts > kMaxDictParts) n_parts = kMaxDictParts;
     auto to_f16 = a.d == 128 ? dict_to_f16_kernel<128> : dict_to_f16_kernel<64>;
-    to_f16<<<n_parts, 256, 0, a.stream>>>(a.D, a.N, static_cast<uint32_t*>(dict), parts, counters, (int)words);
+    to_f16<<<n_parts, 256, 0, a.stream>>>(a.D, a.N, static_cast<uint32_t*>(dict), parts, reinterpret_cast<uint4*>(words), (int)(n_words / 16));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(CSR_ERR_CUDA, "dict_to_f16 launch: %s", cudaGetErrorString(e));
     auto rows_from = [&](int64_t r0, int64_t m) {
@@ -666,10 +671,10 @@ int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status,
     for (int64_t m : plan.grid_rows) {
         if (m == 0) continue;
         const EncodeArgs b = rows_from(r0, m);
-        int rc = launch_encode_exact_grid(b, dict, parts, n_parts, rows, counters, status, diag);
+        int rc = launch_encode_exact_grid(b, dict, parts, n_parts, rows, words, status, diag);
         if (rc == kGridLaunchRefused) rc = run_pairs(b);
         if (rc != CSR_OK) return rc;
-        counters += exact_grid_counter_words(m);
+        words += exact_grid_word_bytes(m, a.N);
         r0 += m;
     }
     return CSR_OK;

@@ -22,8 +22,7 @@ constexpr uint32_t kKeyMask = 0x7FFFFFE0u;                // |value| without its
 // Adjacent atoms that the sweep takes as one: it keeps their largest |correlation|; which of them that was is found
 // when the row is settled (2 KB of the dictionary's fp16 copy gathered per row at d = 128).  Groups of four at d = 128:
 // a training step of 65536 rows (N = 8192, s = 8) 1511 us, of eight 1394.
-template <int D_>
-constexpr int kGroup = 8;
+constexpr int G = 8;
 constexpr uint32_t FULL = 0xffffffffu;
 // What the tensor cores' fp32 accumulation of d exact products of fp16 values (in groups of 16) may add to
 // the error of a correlation, relative to ||R|| and the largest norm of an atom.  Measured (checked
@@ -98,22 +97,18 @@ __device__ __forceinline__ void fold2(Three& q, uint32_t g, uint32_t h) {
     q.b = max(s, u);
 }
 // Key of the G values from v[J] on (a NaN counts as nothing).
-template <int G, int J>
+template <int J>
 __device__ __forceinline__ uint32_t key_of(const uint32_t (&v)[32], uint32_t tag) {
     auto f = [&](int j) { return __uint_as_float(v[J + j]); };
-    float m = absmax3(f(0), f(1), f(2));
-    if constexpr (G == 4)
-        m = absmax3(m, f(3), 0.f);
-    else
-        m = absmax3(absmax3(f(3), f(4), f(5)), absmax3(f(6), f(7), m), 0.f);
+    const float m = absmax3(absmax3(f(3), f(4), f(5)), absmax3(f(6), f(7), absmax3(f(0), f(1), f(2))), 0.f);
     return (__float_as_uint(m) & kKeyMask) | tag;
 }
 // 32 columns, whose first group has number T0.
-template <int G, int T0, int J = 0>
+template <int T0, int J = 0>
 __device__ __forceinline__ void fold32(const uint32_t (&v)[32], Three& q) {
     if constexpr (J < 32) {
-        fold2(q, key_of<G, J>(v, T0 + J / G), key_of<G, J + G>(v, T0 + J / G + 1));
-        fold32<G, T0, J + 2 * G>(v, q);
+        fold2(q, key_of<J>(v, T0 + J / G), key_of<J + G>(v, T0 + J / G + 1));
+        fold32<T0, J + 2 * G>(v, q);
     }
 }
 // A tile's three largest into the row's: whatever ends up within the band of the final maximum was within the band of
@@ -137,46 +132,67 @@ __device__ __forceinline__ void merge(Tops& q, const Three& l, uint32_t id, floa
 }
 
 // Folds a thread's 32 * CHUNKS columns of an accumulator into its row's `q` and hands the accumulator back as soon as all of them
-// are in registers.
-template <int G, int CHUNKS>
+// are in registers; HALVES: 64 at a time, for a kernel whose threads have few.
+template <int CHUNKS, bool HALVES = false>
 __device__ __forceinline__ void drain(uint32_t taddr, Tops& q, uint32_t id, float band, uint64_t* acc_empty, int lane) {
-    uint32_t v0[32], v1[32], v2[32], v3[32];
-    tmem_ld32(taddr + 0, v0);
-    if constexpr (CHUNKS > 1) tmem_ld32(taddr + 32, v1);
-    if constexpr (CHUNKS > 2) tmem_ld32(taddr + 64, v2);
-    if constexpr (CHUNKS > 3) tmem_ld32(taddr + 96, v3);
-    tmem_wait_ld(v0);
-    if constexpr (CHUNKS > 1) reg_fence(v1);
-    if constexpr (CHUNKS > 2) reg_fence(v2);
-    if constexpr (CHUNKS > 3) reg_fence(v3);
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(acc_empty);
     Three l{0u, 0u, 0u};
-    fold32<G, 0>(v0, l);
-    if constexpr (CHUNKS > 1) fold32<G, 32 / G>(v1, l);
-    if constexpr (CHUNKS > 2) fold32<G, 64 / G>(v2, l);
-    if constexpr (CHUNKS > 3) fold32<G, 96 / G>(v3, l);
+    auto back = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty);
+    };
+    if constexpr (HALVES) {
+        static_assert(CHUNKS == 4, "two halves of two chunks");
+        uint32_t v0[32], v1[32];
+        tmem_ld32(taddr + 0, v0);
+        tmem_ld32(taddr + 32, v1);
+        tmem_wait_ld(v0);
+        reg_fence(v1);
+        fold32<0>(v0, l);
+        fold32<32 / G>(v1, l);
+        tmem_ld32(taddr + 64, v0);
+        tmem_ld32(taddr + 96, v1);
+        tmem_wait_ld(v0);
+        reg_fence(v1);
+        back();
+        fold32<64 / G>(v0, l);
+        fold32<96 / G>(v1, l);
+    } else {
+        uint32_t v0[32], v1[32], v2[32], v3[32];
+        tmem_ld32(taddr + 0, v0);
+        if constexpr (CHUNKS > 1) tmem_ld32(taddr + 32, v1);
+        if constexpr (CHUNKS > 2) tmem_ld32(taddr + 64, v2);
+        if constexpr (CHUNKS > 3) tmem_ld32(taddr + 96, v3);
+        tmem_wait_ld(v0);
+        if constexpr (CHUNKS > 1) reg_fence(v1);
+        if constexpr (CHUNKS > 2) reg_fence(v2);
+        if constexpr (CHUNKS > 3) reg_fence(v3);
+        back();
+        fold32<0>(v0, l);
+        if constexpr (CHUNKS > 1) fold32<32 / G>(v1, l);
+        if constexpr (CHUNKS > 2) fold32<64 / G>(v2, l);
+        if constexpr (CHUNKS > 3) fold32<96 / G>(v3, l);
+    }
     merge(q, l, id, band);
 }
 
-// Barrier of the 256 epilogue threads that also tells every one of them whether any of them
+// Barrier of 256 epilogue threads (`bar`: its number) that also tells every one of them whether any of them
 // passed `pred`.
-__device__ __forceinline__ bool epilogue_barrier_any(bool pred) {
+__device__ __forceinline__ bool epilogue_barrier_any(bool pred, int bar = 1) {
     uint32_t r;
     asm volatile(
         "{\n"
         ".reg .pred p, q;\n"
         "setp.ne.u32 q, %1, 0;\n"
-        "bar.red.or.pred p, 1, 256, q;\n"
+        "bar.red.or.pred p, %2, 256, q;\n"
         "selp.u32 %0, 1, 0, p;\n"
         "}\n"
         : "=r"(r)
-        : "r"(static_cast<uint32_t>(pred))
+        : "r"(static_cast<uint32_t>(pred)), "r"(bar)
         : "memory");
     return r != 0;
 }
-__device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void epilogue_barrier(int bar = 1) { asm volatile("bar.sync %0, 256;" ::"r"(bar) : "memory"); }
 
 __device__ __forceinline__ double group8_sum(double v) {
     v += __shfl_xor_sync(FULL, v, 1);
@@ -204,23 +220,33 @@ __device__ __forceinline__ void load_atom(const float* __restrict__ atom, int l8
 }
 // (four running sums: a single chain of fp64 FMAs would wait out the pipe's latency CH times)
 template <int CH>
-__device__ __forceinline__ double slice_dot(const double (&R)[CH], const float (&a)[CH]) {
+__device__ __forceinline__ double slice_dot(const double (&R)[CH], const double (&a)[CH]) {
     double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
 #pragma unroll
     for (int k = 0; k < CH; k += 4) {
-        c0 = fma(R[k], static_cast<double>(a[k]), c0);
-        c1 = fma(R[k + 1], static_cast<double>(a[k + 1]), c1);
-        c2 = fma(R[k + 2], static_cast<double>(a[k + 2]), c2);
-        c3 = fma(R[k + 3], static_cast<double>(a[k + 3]), c3);
+        c0 = fma(R[k], a[k], c0);
+        c1 = fma(R[k + 1], a[k + 1], c1);
+        c2 = fma(R[k + 2], a[k + 2], c2);
+        c3 = fma(R[k + 3], a[k + 3], c3);
     }
     return (c0 + c1) + (c2 + c3);
+}
+template <int CH>
+__device__ __forceinline__ void widen(const float (&a)[CH], double (&ad)[CH]) {
+#pragma unroll
+    for (int k = 0; k < CH; ++k) ad[k] = static_cast<double>(a[k]);
+}
+template <int CH>
+__device__ __forceinline__ double slice_dot(const double (&R)[CH], const float (&a)[CH]) {
+    double ad[CH];
+    widen<CH>(a, ad);
+    return slice_dot<CH>(R, ad);
 }
 
 // Two neighbouring channels of a scaled row as fp16, one word, and what the rounding took from them squared, added to
 // `err2`.  (A value is brought to fp32 first: what that rounds off, 2^-24 of it, is far inside the allowance
 // of row_band.)
-__device__ __forceinline__ uint32_t round_pair(double r0, double r1, float& err2) {
-    const float f0 = static_cast<float>(r0), f1 = static_cast<float>(r1);
+__device__ __forceinline__ uint32_t round_pair(float f0, float f1, float& err2) {
     const __half2 h = __floats2half2_rn(f0, f1);
     const float2 w = __half22float2(h);
     const float e0 = f0 - w.x, e1 = f1 - w.y;
@@ -276,22 +302,41 @@ __device__ __forceinline__ float relative_limit(float v0, float band, float norm
     return (v0 - 1.5f * band) / (norm * b.scale);
 }
 
-// Writes this lane's CH residual values: fp64 to the scratch row (`row`: its first element), `scale` times them as fp16
-// to the operand tile.  Returns this lane's share of the rounding's squared norm.
+// This lane's CH residual values as the sweep takes them: scaled, fp16, two channels per word; the row's norm and what the rounding
+// took from it squared (of all eight lanes of the row).  All lanes of a warp call.  Rows of ordinary norm are scaled and
+// measured in fp32: fp64 operations and conversions are what the settling has least of, and nothing here needs more than a few
+// bits of the norm.
 template <int CH>
-__device__ __forceinline__ float store_residual(const double (&R)[CH], double scale, double* __restrict__ row, uint8_t* A, int r, int l8,
-                                                bool write) {
-    float err2 = 0.f;
+struct Operand {
+    uint32_t w[CH / 2];
+    float norm, err2;
+};
+template <int CH>
+__device__ __forceinline__ Operand<CH> to_operand(const double (&R)[CH]) {
+    Operand<CH> o;
+    float f[CH], n0 = 0.f, n1 = 0.f, err2 = 0.f;
 #pragma unroll
     for (int k = 0; k < CH / 2; ++k) {
-        const uint32_t w = round_pair(R[2 * k] * scale, R[2 * k + 1] * scale, err2);
-        if (write) {
-            reinterpret_cast<double2*>(row)[8 * k + l8] = make_double2(R[2 * k], R[2 * k + 1]);
-            // channels 2 (8 k + l8), +1: 16-byte chunk 2 k + l8 / 4 of the row, word l8 % 4 of it
-            *reinterpret_cast<uint32_t*>(A + swz_off(r, 2 * k + (l8 >> 2)) + (l8 & 3) * 4) = w;
-        }
+        f[2 * k] = static_cast<float>(R[2 * k]);
+        f[2 * k + 1] = static_cast<float>(R[2 * k + 1]);
+        n0 = fmaf(f[2 * k], f[2 * k], n0);
+        n1 = fmaf(f[2 * k + 1], f[2 * k + 1], n1);
     }
-    return err2;
+    const float nn = group8_sumf(n0 + n1);
+    if (__all_sync(FULL, nn >= 0x1p-60f && nn <= 0x1p60f)) {
+        const int e = static_cast<int>(__float_as_uint(nn) >> 23) - 127;
+        const float scale = __uint_as_float(static_cast<uint32_t>(127 - (e >> 1)) << 23);
+        o.norm = sqrtf(nn) * scale;
+#pragma unroll
+        for (int k = 0; k < CH / 2; ++k) o.w[k] = round_pair(f[2 * k] * scale, f[2 * k + 1] * scale, err2);
+    } else {
+        const double scale = row_scale(group8_sum(norm2_share<CH>(R)), o.norm);
+#pragma unroll
+        for (int k = 0; k < CH / 2; ++k)
+            o.w[k] = round_pair(static_cast<float>(R[2 * k] * scale), static_cast<float>(R[2 * k + 1] * scale), err2);
+    }
+    o.err2 = group8_sumf(err2);
+    return o;
 }
 
 #ifdef CSR_DEBUG_CHECKS
@@ -301,8 +346,7 @@ __device__ __forceinline__ float store_residual(const double (&R)[CH], double sc
 template <int CH>
 __device__ __forceinline__ void check_value(uint32_t* diag, const double (&R)[CH], const float (&a)[CH], double c, float v, float band, float norm,
                                             const DictBounds& b, int l8, bool count) {
-    float unused;
-    const double scale = row_scale(group8_sum(norm2_share<CH>(R)), unused);
+    const double scale = exp2(rint(log2(static_cast<double>(norm) / sqrt(group8_sum(norm2_share<CH>(R))))));   // the power of two that was taken
     double p = 0.0;
 #pragma unroll
     for (int k = 0; k < CH; ++k)
@@ -352,7 +396,7 @@ __device__ __forceinline__ void fma2_f16(float& acc0, float& acc1, uint32_t a, u
 // The sweep's values of one group again: eight lanes per row, lane l8 holds 16-byte chunks l8 + 8 j of the G atoms and of the row.
 template <int D_>
 struct GroupAtoms {
-    static constexpr int G = kGroup<D_>, CK = D_ / 64;
+    static constexpr int CK = D_ / 64;
     uint4 a[G][CK];
     __device__ __forceinline__ void load(const uint16_t* __restrict__ dict, int n0, int N, int l8) {
 #pragma unroll
@@ -362,8 +406,7 @@ struct GroupAtoms {
             for (int j = 0; j < CK; ++j) a[i][j] = __ldg(src + l8 + 8 * j);
         }
     }
-    // |r . d| of atom `atom(l8)` of the group, to this lane; negative for one past the dictionary's end.
-    static __device__ __forceinline__ int atom(int l8) { return G == 8 ? l8 : l8 >> 1; }
+    // |r . d| of the group's atom l8, to this lane; negative for one past the dictionary's end.
     __device__ __forceinline__ float value(const uint4 (&r)[CK], int n0, int N, int l8) const {
         float e[G];
 #pragma unroll
@@ -380,19 +423,15 @@ struct GroupAtoms {
         }
         // a lane keeps half of its atoms at each step and sends the other half's sums to the lane that keeps those
 #pragma unroll
-        for (int h = G / 2, bit = 4; bit > 0; bit >>= 1, h >>= 1) {
-            if (h > 0) {
-                const bool up = l8 & bit;
+        for (int h = 4; h > 0; h >>= 1) {
+            const bool up = l8 & h;
 #pragma unroll
-                for (int i = 0; i < h; ++i) {
-                    const float keep = up ? e[i + h] : e[i], send = up ? e[i] : e[i + h];
-                    e[i] = keep + __shfl_xor_sync(FULL, send, bit);
-                }
-            } else {
-                e[0] += __shfl_xor_sync(FULL, e[0], bit);
+            for (int i = 0; i < h; ++i) {
+                const float keep = up ? e[i + h] : e[i], send = up ? e[i] : e[i + h];
+                e[i] = keep + __shfl_xor_sync(FULL, send, h);
             }
         }
-        return n0 + atom(l8) < N ? fabsf(e[0]) : -1.f;
+        return n0 + l8 < N ? fabsf(e[0]) : -1.f;
     }
 };
 // Of the group's values, a bit for each lane of the warp whose atom is within the band of its row's largest.
@@ -419,12 +458,13 @@ __device__ __forceinline__ int decide(const float* __restrict__ D, int N, const 
 #pragma unroll 1
     for (int i = 0; i < groups; ++i) {
         const int n0 = start(i);
-#pragma unroll 1
-        for (int a = 0; a < kGroup<D_>; a += 4) {
-            const int n = n0 + a + grp;
-            float at[CH];
-            load_atom<CH>(D + static_cast<int64_t>(min(n, N - 1)) * D_, l8, at);
-            const double c = fabs(group8_sum(slice_dot<CH>(R, at)));
+        float at[2][CH];                                  // four atoms at a time, eight lanes each
+#pragma unroll
+        for (int h = 0; h < 2; ++h) load_atom<CH>(D + static_cast<int64_t>(min(n0 + 4 * h + grp, N - 1)) * D_, l8, at[h]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int n = n0 + 4 * h + grp;
+            const double c = fabs(group8_sum(slice_dot<CH>(R, at[h])));
             if (n < N && (c > best || (c == best && n < bn))) {
                 best = c;
                 bn = n;
@@ -524,22 +564,22 @@ struct Rescored {
     double val;
     int n, pad;
 };
-// One row over the whole dictionary by the 256 epilogue threads (all call): the pick, to every thread.
+// One row over the whole dictionary by 256 epilogue threads (all call; `warp`: 0 to 7): the pick, to every thread.
 template <int D_>
 __device__ __forceinline__ int rescore_row(const float* __restrict__ D, int N, const double* Rrow, float thresh, Rescored* found, int warp,
-                                           int lane) {
+                                           int lane, int bar = 1) {
     const int per = ((N + 7) / 8 + 15) / 16 * 16;
     const int n0 = min(warp * per, N), n1 = min(n0 + per, N);
     Rescored r{-1.0, 0, 0};
     if (n0 < n1) r.val = rescore_part<D_>(D, n0, n1, Rrow, thresh, lane, &r.n);
     if (lane == 0) found[warp] = r;
-    epilogue_barrier();
+    epilogue_barrier(bar);
     Rescored top{-1.0, 0, 0};
     for (int w = 0; w < 8; ++w) {                         // atoms ascend with the warp: the first of equal values is the lowest
         const Rescored o = found[w];
         if (o.val > top.val) top = o;
     }
-    epilogue_barrier();
+    epilogue_barrier(bar);
     return top.n;
 }
 
