@@ -587,26 +587,27 @@ int run(const EncodeArgs& a, const CUtensorMap& map, const uint16_t* dict, const
 
 // How M rows are run: `pair_rows` of them as pairs of row tiles, one CTA each for the whole
 // dictionary, then up to two launches of one row tile per CTA whose CTAs split the dictionary.
-// A wave of pairs takes the time of two waves of single row tiles (the tensor cores bound both),
-// a row tile split over c CTAs 1/c of one.  Whole waves of pairs come first (they read the
-// dictionary half as often); the last, partial one is replaced wherever that saves at least a
-// quarter of it.  Measured at N = 4096, s = 8, d = 128 in us (cold caches, the dictionary's split and the
-// launches included), this plan against pairs only: 2048 rows 155 / 744, 9472 284 / 747, 18944
-// 415 / 753, 20000 540 / 755, 24224 652 / 759, 27648 691 / 759 (where the second launch would not split
-// its tiles any more, pairs are as good and are taken), 37888 769.  Few rows at N = 8192, s = 16: 16 rows
-// 157 us, 128 rows 189, 512 rows 237, 4096 rows 511, against 474, 339, 1672 and 6567 for the plain-ALU
-// encoder with its launch pair per iteration and 2090 to 2350 for pairs.
+// A wave of pairs costs less than two waves of single row tiles (39 against 29 us an iteration at N = 1024, d = 128, plus
+// 1.2 and 0.7 us per 256 atoms), and the last, partial wave is replaced wherever single tiles take less.  Up to one tile per
+// SM they always do.  With more, a second launch follows, and it has to be short: its tiles' dictionary is cut into at least
+// least_slices() slices each.  Measured at s = 6, d = 128 in us (warm L2, preparation included), two launches / pairs for
+// 18944 + 128 k rows: N = 1024: k = 8 (16 slices) 230 / 238, 24 (six) 247 / 228; N = 4096: six 333 / 376, four 382 / 380,
+// three 417 / 382; N = 8192: four 462 / 512, three 542 / 513; N = 16384: three 751 / 826, two 808 / 828; N = 32768: three
+// 1459 / 1443, two 1549 / 1459.  d = 64: N = 1024 sixteen 179 / 196, ten 218 / 197; N = 2048 six 237 / 238, five 257 / 233; N = 4096
+// four 307 / 323, three 313 / 292; N = 8192 three 398 / 423, two 419 / 425; N = 16384 two 662 / 714; N = 32768 two 1133 / 1314.
 struct Plan {
     int64_t pair_rows;
     int64_t grid_rows[2];
 };
-Plan make_plan(int64_t M, int N, bool pairs_only) {
+int least_slices(int d, int N) { return N < 2048 ? 16 : N < 4096 ? 8 : N < 16384 ? 4 : d == 64 ? 2 : 3; }
+
+Plan make_plan(int64_t M, int d, int N, bool pairs_only) {
     Plan p{M, {0, 0}};
     if (pairs_only) return p;
     const int64_t sms = sm_count(), wave = sms * ROWS;
     const int64_t rest = M % wave, tiles = (rest + TILE_M - 1) / TILE_M;
     const int64_t over = tiles > sms ? tiles - sms : 0;   // row tiles of the second launch
-    if (tiles == 0 || (over > 0 && exact_grid_slices(over * TILE_M, N) < 2)) return p;
+    if (tiles == 0 || (over > 0 && exact_grid_slices(over * TILE_M, N) < least_slices(d, N))) return p;
     p.pair_rows = M - rest;
     p.grid_rows[0] = over > 0 ? sms * TILE_M : rest;
     p.grid_rows[1] = rest - p.grid_rows[0];
@@ -618,7 +619,7 @@ size_t pair_scratch_bytes(int64_t M, int d) { return (size_t)ctas_for(M) * ROWS 
 
 // [fp16 dictionary][its bounds][words of the two split launches][rows of the launch that is running]
 size_t encode_exact_tc_scratch_bytes(int64_t M, int d, int N) {
-    const Plan p = make_plan(M, N, false);
+    const Plan p = make_plan(M, d, N, false);
     size_t rows = pair_scratch_bytes(M, d), words = 0;    // (also what is needed where a split launch is refused)
     for (int64_t m : p.grid_rows) {
         if (m == 0) continue;
@@ -633,7 +634,7 @@ int launch_encode_exact_tc(const EncodeArgs& a, void* scratch, uint32_t* status,
     if (a.M == 0) return CSR_OK;
     if ((reinterpret_cast<uintptr_t>(scratch) & 1023u) != 0)
         return fail(CSR_ERR_ALIGNMENT, "internal: exact-mode scratch not 1024-byte aligned");
-    const Plan plan = make_plan(a.M, a.N, pairs_only);
+    const Plan plan = make_plan(a.M, a.d, a.N, pairs_only);
     char* base = static_cast<char*>(scratch);
     void* dict = base;
     base += align1k((size_t)a.N * a.d * 2);

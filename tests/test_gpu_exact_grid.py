@@ -58,6 +58,23 @@ def test_split_engine_equals_the_pair_engine(csr, M, N, d, s, dtype):
         assert rep.ok, rep.detail
 
 
+@pytest.mark.parametrize("over,N,d", [(1, 1024, 128), (9, 1023, 64), (10, 1024, 128), (18, 2048, 64), (19, 2300, 128), (37, 4096, 64), (38, 4100, 128)])
+def test_second_launch_of_single_tiles(csr, over, N, d):
+    """More row tiles than SMs by `over`, on both sides of where the second launch has too few slices: the codes of pairs."""
+    M = 128 * torch.cuda.get_device_properties(0).multi_processor_count + 128 * over - 5
+    g = torch.Generator(device=DEV).manual_seed(M + N)
+    D = torch.nn.functional.normalize(torch.randn(N, d, device=DEV, generator=g), dim=1).contiguous()
+    X = torch.randn(M, d, device=DEV, generator=g).to(torch.bfloat16)
+    idx, coef = csr.csr_encode_ex(D, X, 2, mode=csr.CSR_MODE_FP32_EXACT, coef_dtype=torch.float32)
+    csr.csr_set_option("exact_engine", 2)
+    try:
+        idx2, coef2 = csr.csr_encode_ex(D, X, 2, mode=csr.CSR_MODE_FP32_EXACT, coef_dtype=torch.float32)
+    finally:
+        csr.csr_set_option("exact_engine", 0)
+    assert csr.csr_device_status() == csr.CSR_OK
+    assert np.array_equal(_np(idx), _np(idx2)) and torch.equal(coef, coef2)
+
+
 def test_split_engine_writes_strided_codes_and_reads_strided_rows(csr):
     g = torch.Generator(device=DEV).manual_seed(3)
     D = torch.nn.functional.normalize(torch.randn(1000, 64, device=DEV, generator=g), dim=1).contiguous()
