@@ -210,7 +210,6 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
     const int n_first = u0 * UNIT, width = (u1 - u0) * UNIT;   // this CTA's atoms (slices <= units: never empty)
     const int T = (width + TILE_N - 1) / TILE_N;          // accumulator tiles of a sweep, the last 64 .. 256 wide
     constexpr int KH = D_ / STAGE_CH;
-    constexpr int KSTEPS = STAGE_CH / UMMA_K;
     constexpr int STAGES = S::kStages;
     const WaitCtx wc{&sm.abort, a.status, a.wait_limit_ns};
 
@@ -271,7 +270,7 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        // (the whole warp runs this, one elected lane issues: see umma_f16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16_block)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         {
             uint32_t p = 0, accn = 0;
@@ -299,14 +298,11 @@ encode_exact_grid_kernel(const __grid_constant__ CUtensorMap tmap_d, const GridA
                         tc_fence_after();
                         const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
                         const uint64_t a0 = make_smem_desc(smem_u32(&sm.A[h * (TILE_M * 128)]));
-#pragma unroll
-                        for (int k = 0; k < KSTEPS; ++k) {
-                            const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                            umma_f16(d_tmem, a0 + off, b0 + off, idesc, (h | k) ? 1u : 0u);
-                        }
-                        umma_commit(&sm.empty_b[stage]);
+                        if (h < KH - 1)
+                            umma_f16_block(d_tmem, a0, b0, idesc, h, &sm.empty_b[stage]);
+                        else
+                            umma_f16_block(d_tmem, a0, b0, idesc, h, &sm.empty_b[stage], &sm.acc_full[acc]);
                     }
-                    if (ok) umma_commit(&sm.acc_full[acc]);
                 }
             }
             if (!ok) {

@@ -82,7 +82,6 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
     const int T = (N + TILE_N - 1) / TILE_N;
     const int64_t n_pairs = (M + ROWS - 1) / ROWS;
     constexpr int KH = D_ / STAGE_CH;                       // 64-channel blocks per row
-    constexpr int KSTEPS = STAGE_CH / UMMA_K;
     constexpr int STAGES = S::kStages;
     const WaitCtx wc{&sm.abort, status, wait_limit_ns};
 
@@ -142,7 +141,7 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        // (the whole warp runs this, one elected lane issues: see umma_f16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16_block)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         {
             uint32_t p = 0, accn = 0, steps = 0;
@@ -157,30 +156,30 @@ encode_exact_tc_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_
                     // accumulators then complete a whole tile's MMAs apart, and the epilogue drains them one
                     // after the other.
                     for (int t = 0; t < T && ok; ++t, ++accn, p += KH) {
-                        for (int tile = 0; tile < 2 && ok; ++tile) {
-                            if (!warp_wait_bounded_suspended(&sm.acc_empty[tile], (accn & 1) ^ 1, wc, 1000)) {
-                                ok = false;
-                                break;
-                            }
+#pragma unroll
+                        for (int tile = 0; tile < 2; ++tile) {
+                            ok = warp_wait_bounded_suspended(&sm.acc_empty[tile], (accn & 1) ^ 1, wc, 1000);
                             const uint32_t d_tmem = tmem_d + tile * TILE_N;
+#pragma unroll
                             for (int h = 0; h < KH; ++h) {
                                 const uint32_t ps = p + h;
                                 const int stage = ps % STAGES;
-                                if (tile == 0 && !warp_wait_bounded_suspended(&sm.full_b[stage], (ps / STAGES) & 1, wc, 1000)) {
-                                    ok = false;
-                                    break;
-                                }
+                                if (tile == 0 && ok) ok = warp_wait_bounded_suspended(&sm.full_b[stage], (ps / STAGES) & 1, wc, 1000);
+                                if (!ok) break;
                                 tc_fence_after();
                                 const uint64_t a0 = make_smem_desc(smem_u32(&sm.A[tile][h * (TILE_M * 128)]));
                                 const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
-#pragma unroll
-                                for (int k = 0; k < KSTEPS; ++k) {
-                                    const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                                    umma_f16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
-                                }
-                                if (tile == 1) umma_commit(&sm.empty_b[stage]);
+                                // (the second row tile is the last reader of a stage)
+                                if (h < KH - 1 && tile == 0)
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h);
+                                else if (h < KH - 1)
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.empty_b[stage]);
+                                else if (tile == 0)
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.acc_full[tile]);
+                                else
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.empty_b[stage], &sm.acc_full[tile]);
                             }
-                            if (ok) umma_commit(&sm.acc_full[tile]);
+                            if (!ok) break;
                         }
                     }
                 }

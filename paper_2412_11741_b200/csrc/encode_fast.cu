@@ -70,7 +70,6 @@ using namespace tc;
 
 constexpr int TILE_M = 128;
 constexpr int TILE_N = 256;                           // atoms per accumulator / per MMA instruction
-constexpr int UMMA_K = 16;
 constexpr int STAGE_CH = 64;                          // channels per dictionary stage (one 128-byte row)
 constexpr int STAGES = 4;
 constexpr int NT = 320;
@@ -461,7 +460,6 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
     const int64_t pair_first = n_splits > 1 ? blockIdx.x / n_splits : blockIdx.x;
     const int64_t pair_step = n_splits > 1 ? gridDim.x / n_splits : gridDim.x;
     constexpr int KH = D_ / STAGE_CH;                       // stages per dictionary tile
-    constexpr int KSTEPS = STAGE_CH / UMMA_K;               // MMAs per stage
     constexpr int CHUNKS = D_ / 8;                          // 16-byte chunks per row
     constexpr int NG = TILE_N / G;                          // arg-max groups per accumulator
     const WaitCtx wc{&sm.abort, status, wait_limit_ns};
@@ -534,7 +532,7 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------ MMA issuer ------------------------------
-        // (the whole warp runs this, one elected lane issues: see umma_f16)
+        // (the whole warp runs this, one elected lane issues: see umma_f16_block)
         const uint32_t tmem_d = warp_uniform(tmem_base);
         if constexpr (ONE) {
             // one row tile; the CTA's dictionary tiles go to the two accumulators in turn
@@ -564,17 +562,12 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
                         tc_fence_after();
                         const uint64_t a0 = make_smem_desc(smem_u32(&sm.A[0][h * (TILE_M * 128)]));
                         const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
-#pragma unroll
-                        for (int k = 0; k < KSTEPS; ++k) {
-                            const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                            umma_f16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
-                        }
-                        umma_commit(&sm.empty_b[stage]);
+                        if (h < KH - 1)
+                            umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.empty_b[stage]);
+                        else
+                            umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.empty_b[stage], &sm.acc_full[acc]);
                     }
-                    if (ok) {
-                        umma_commit(&sm.acc_full[acc]);
-                        ++accn[acc];
-                    }
+                    if (ok) ++accn[acc];
                 }
             }
             if (!ok) {
@@ -589,37 +582,31 @@ encode_fast_kernel(const __grid_constant__ CUtensorMap tmap_d, const uint16_t* _
             for (int64_t pair = pair_first; pair < n_pairs && ok; pair += pair_step) {
                 for (int g = 0; g < s && ok; ++g, ++steps) {
                     for (int t = t_begin; t < T && ok; t += t_step, p += KH, ++accn) {
-                        for (int tile = 0; tile < 2 && ok; ++tile) {
-                            if (t == t_begin && !warp_wait_bounded(&sm.res_ready[tile], steps & 1, wc)) {
-                                ok = false;
-                                break;
-                            }
-                            if (!warp_wait_bounded(&sm.acc_empty[tile], (accn & 1) ^ 1, wc)) {
-                                ok = false;
-                                break;
-                            }
+#pragma unroll
+                        for (int tile = 0; tile < 2; ++tile) {
+                            if (t == t_begin) ok = warp_wait_bounded(&sm.res_ready[tile], steps & 1, wc);
+                            if (ok) ok = warp_wait_bounded(&sm.acc_empty[tile], (accn & 1) ^ 1, wc);
                             const uint32_t d_tmem = tmem_d + tile * TILE_N;
 #pragma unroll
                             for (int h = 0; h < KH; ++h) {
                                 const uint32_t ps = p + h;
                                 const int stage = ps % STAGES;
-                                if (tile == 0 && !warp_wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc)) {
-                                    ok = false;
-                                    break;
-                                }
+                                if (tile == 0 && ok) ok = warp_wait_bounded(&sm.full_b[stage], (ps / STAGES) & 1, wc);
+                                if (!ok) break;
                                 tc_fence_after();
                                 const uint64_t a0 = make_smem_desc(smem_u32(&sm.A[tile][h * (TILE_M * 128)]));
                                 const uint64_t b0 = make_smem_desc(smem_u32(&sm.B[stage][0]));
-#pragma unroll
-                                for (int k = 0; k < KSTEPS; ++k) {
-                                    // 16 channels = 32 bytes inside a 128-byte swizzled row
-                                    const uint64_t off = static_cast<uint64_t>((k * 32) >> 4);
-                                    umma_f16(d_tmem, a0 + off, b0 + off, kInstrDesc, (h | k) ? 1u : 0u);
-                                }
-                                // the second row tile is the last reader of a stage
-                                if (tile == 1) umma_commit(&sm.empty_b[stage]);
+                                // (the second row tile is the last reader of a stage)
+                                if (h < KH - 1 && tile == 0)
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h);
+                                else if (h < KH - 1)
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.empty_b[stage]);
+                                else if (tile == 0)
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.acc_full[tile]);
+                                else
+                                    umma_f16_block(d_tmem, a0, b0, kInstrDesc, h, &sm.empty_b[stage], &sm.acc_full[tile]);
                             }
-                            if (ok) umma_commit(&sm.acc_full[tile]);
+                            if (!ok) break;
                         }
                     }
                 }

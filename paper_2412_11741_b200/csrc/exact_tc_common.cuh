@@ -16,7 +16,6 @@ using namespace tc;
 
 constexpr int TILE_M = 128;
 constexpr int TILE_N = 256;
-constexpr int UMMA_K = 16;
 constexpr int STAGE_CH = 64;
 constexpr uint32_t kKeyMask = 0x7FFFFFE0u;                // |value| without its five lowest mantissa bits
 // Adjacent atoms that the sweep takes as one: it keeps their largest |correlation|; which of them that was is found

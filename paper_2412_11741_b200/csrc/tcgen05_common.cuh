@@ -129,22 +129,63 @@ __device__ __forceinline__ void tmem_relinquish() {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 or fp16 operands (`idesc` says which), fp32 accumulate.  The whole warp calls, converged, with
-// the same arguments, and one elected lane issues: in code that only lane 0 runs, every MMA first has
+// D[tmem] (+)= A[smem] * B[smem]^T for one 64-channel block of both operands (bf16 or fp16, `idesc` says which; fp32 accumulate):
+// four MMAs, 32 bytes apart in the swizzled rows, then a commit (umma_commit) to each barrier given.  The whole warp
+// calls, converged, with the same arguments, and one elected lane issues: in code that only lane 0 runs, every MMA first has
 // to move its descriptors to the uniform registers the instruction takes, 116 cycles a piece, 168
 // when the other warps are busy too, more than the 128 x 256 x 16 MMA itself takes.  Measured, 128
 // MMAs in a row per SM with eight warps reading tensor memory: 178 cycles per MMA from lane 0,
-// 139 with the election (128 is the tensor core's own rate).
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
+// 139 with the election (128 is the tensor core's own rate).  One election for a block instead of one for each MMA and commit
+// shortens the issuing warp's chain per row tile (615 cycles in a copy with clocks, while a d = 64 tile's MMAs take 512): 262144 rows,
+// N = 4096, s = 8: 1798 -> 1748 us; 100003 rows, N = 5001, d = 64, s = 6: 428 -> 424; exact mode, 100000 rows, N = 4096, s = 8: 1278 -> 1256.
+// (An issuing warp per accumulator: 2154 and 477 us.  The tensor core takes the MMAs of two warps in turn, so that both accumulators
+// complete, and are drained, at the same time.)
+__device__ __forceinline__ void umma_f16_block(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n"
-        ".reg .pred p, e;\n"
+        ".reg .pred p, e, t;\n"
+        "setp.ne.b32 p, %10, 0;\n"
+        "setp.eq.b32 t, 0, 0;\n"
         "elect.sync _|e, 0xffffffff;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %9, p;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %6, %9, t;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %3, %7, %9, t;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %8, %9, t;\n"
+        "}\n" ::"r"(d_tmem), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "r"(idesc),
+        "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void umma_f16_block(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate, uint64_t* bar0) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p, e, t;\n"
+        "setp.ne.b32 p, %10, 0;\n"
+        "setp.eq.b32 t, 0, 0;\n"
+        "elect.sync _|e, 0xffffffff;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %9, p;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %6, %9, t;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %3, %7, %9, t;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %8, %9, t;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%11];\n"
+        "}\n" ::"r"(d_tmem), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "r"(idesc),
+        "r"(accumulate), "r"(smem_u32(bar0))
+        : "memory");
+}
+__device__ __forceinline__ void umma_f16_block(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate, uint64_t* bar0, uint64_t* bar1) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p, e, t;\n"
+        "setp.ne.b32 p, %10, 0;\n"
+        "setp.eq.b32 t, 0, 0;\n"
+        "elect.sync _|e, 0xffffffff;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %9, p;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %6, %9, t;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %3, %7, %9, t;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %8, %9, t;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%11];\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%12];\n"
+        "}\n" ::"r"(d_tmem), "l"(a), "l"(a + 2), "l"(a + 4), "l"(a + 6), "l"(b), "l"(b + 2), "l"(b + 4), "l"(b + 6), "r"(idesc),
+        "r"(accumulate), "r"(smem_u32(bar0)), "r"(smem_u32(bar1))
         : "memory");
 }
 // The mbarrier gets one arrival once every tcgen05.mma issued so far by the elected lane is done (the
